@@ -184,8 +184,10 @@ aiq_status_t launch_qlinear_tc(const LayerJob& job, int N, int K, int M, void* w
 // weight_bytes: packed weights + scales + biases of all jobs (for the profile's byte count)
 aiq_status_t launch_conv(const ConvGeom& g, const LayerJob* jobs_dev, int n_jobs,
                          const float* net_input, double weight_bytes, cudaStream_t s);
-aiq_status_t launch_depthwise(const ConvGeom& g, const LayerJob* jobs_dev, int n_jobs,
-                              const float* net_input, double weight_bytes, cudaStream_t s);
+// Depthwise 3x3 (depthwise.cu).  `map`: CUtensorMap over the input slot (channels, hi | lo, columns, padded rows, images).
+aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions, void* map_out);
+aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
+                              int32_t* error_flag, double weight_bytes, cudaStream_t s);
 // Tensor-core convolution (conv_tc.cu).  `map` points to a 128-byte CUtensorMap over the input
 // slot: dims (2*Cs, W, batch_capacity*(H+2), versions).
 bool conv_tc_eligible(const ConvGeom& g);

@@ -1,439 +1,450 @@
 // Depthwise 3x3 convolution (stride 1 or 2, pad 1) with bias, residual and activation.
 //
-// The layer moves 8 bytes per output element for 18 FLOP: it is bound by memory traffic, so
-// the kernel is organised around wide, coalesced accesses and input reuse in registers:
-//   - a thread owns 8 consecutive channels (16-byte loads: one for the hi and one for the lo
-//     half of a split pixel, two for a float32 pixel) and 4 consecutive output columns;
-//   - for each of the 3 input rows it loads the 6 (stride 1) or 9 (stride 2) input columns
-//     its 4 outputs need once and feeds all taps from registers;
-//   - work items (output row, column group, channel octet) are flattened with the channel
-//     octet fastest, so consecutive lanes touch consecutive 16-byte units whatever the
-//     channel count (32 .. 960 in MobileNetV2);
-//   - the 9 x C expanded weights, scales and biases sit in shared memory; blocks are
-//     persistent (grid-stride over items).
+// The layer moves 8 bytes per output element for 18 FLOP: it is bound by memory traffic, so the
+// kernel is organised around bytes in flight and instructions per element:
+//   - input rows arrive in a ring of shared-memory stages by TMA, several rows ahead of their use (a
+//     stage = one padded row of NI images x a column tile x a slab of Cb channels; columns outside
+//     the map are filled with zeros, rows outside it are the physical padding rows of the tensor),
+//     so the loads in flight do not depend on how many warps are resident;
+//   - a thread owns 4 consecutive channels and COLS consecutive output columns of one image and walks
+//     down the rows: each input row feeds the (up to three) output rows it belongs to, an input value is
+//     unpacked once per thread, and the 36 weights stay in registers (a block keeps its channel slab);
+//   - products are packed float32 pairs (two lanes per instruction).
+// The kernels this one replaced loaded their inputs from global memory in each thread (one row per
+// thread, or rows walked by a thread): 43 instructions per element and the loads of three blocks in
+// flight, 2.7 TB/s on MobileNetV2-CIFAR at batch 256, and every block expanded the weights of all
+// channels into shared memory first, which was most of the 13 us of a single-image launch.
 // Rows 0 and Ho+1 of every output image (the physical padding rows) are written as zeros.
-//
-// Two kernels share this organisation.  depthwise3x3_kernel gives a thread one output row of
-// its columns: every output row re-reads its three input rows (from L1 / L2), which is fine
-// for small launches that need the parallelism.  depthwise3x3_walk_kernel gives a thread up to
-// 16 consecutive output rows: it walks down the input rows once, each row feeding the (up to
-// three) output rows it belongs to.
-#include "common.cuh"
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+#include <type_traits>
 
 namespace aiq {
 
 namespace {
 
-constexpr int kDwThreads = 256;
-constexpr int kDwCols = 2;        // output columns per thread
-constexpr int kWalkCh = 4;        // channels per thread of the row-walking kernel
+constexpr int kDwThreads = 256;                     // compute threads at most; one more warp issues the copies
+constexpr int kDwMaxStages = 8;
+constexpr int kDwCols = 2;                          // output columns per thread
+constexpr int kDwMaxColGroups = 56;                 // column groups of a block: its input box stays within 256 columns
 
+struct DwParams {
+  int B, H, W, Ho, Wo, C, Cs, act;
+  int Cb, CQ;               // channels of a slab, its quads
+  int XG, n_ct;             // column groups of a block, column tiles of a row
+  int NI, n_ig;             // images of a block, image groups
+  int rb, n_rb;             // output rows of a block, row blocks
+  int n_slabs, n_units;     // units: slab fastest, then column tile, row block, image group
+  int Wb;                   // input columns of a stage
+  int stages, box_bytes, stage_bytes;   // bytes a copy brings; stages start on 128-byte boundaries
+  int batch_capacity;       // images per version of the input slot
+  int32_t* error_flag;
+};
+
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// hi and lo halves of four channels -> two packed float pairs (a bfloat16 is the upper half of a float)
+__device__ __forceinline__ void join4(uint2 h, uint2 l, uint64_t* v) {
+  v[0] = add2(pack2(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xFFFF0000u)),
+              pack2(__uint_as_float(l.x << 16), __uint_as_float(l.x & 0xFFFF0000u)));
+  v[1] = add2(pack2(__uint_as_float(h.y << 16), __uint_as_float(h.y & 0xFFFF0000u)),
+              pack2(__uint_as_float(l.y << 16), __uint_as_float(l.y & 0xFFFF0000u)));
+}
+
+// Four channels of one pixel in shared memory: [hi(Cb) | lo(Cb)] bfloat16 or Cb floats.
 template <int FMT>
-__device__ __forceinline__ void load8(const void* __restrict__ base, size_t pixel, int c, int Cs, float* v) {
+__device__ __forceinline__ void read4(const uint8_t* p, int Cb, uint64_t* v) {
   if (FMT == ACT_SPLIT) {
-    const __nv_bfloat16* px = static_cast<const __nv_bfloat16*>(base) + pixel * 2 * Cs;
-    const uint4 h = __ldg(reinterpret_cast<const uint4*>(px + c));
-    const uint4 l = __ldg(reinterpret_cast<const uint4*>(px + Cs + c));
-    const uint32_t hw[4] = {h.x, h.y, h.z, h.w}, lw[4] = {l.x, l.y, l.z, l.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {          // a bfloat16 is the upper half of a float
-      v[2 * i] = __uint_as_float(hw[i] << 16) + __uint_as_float(lw[i] << 16);
-      v[2 * i + 1] = __uint_as_float(hw[i] & 0xFFFF0000u) + __uint_as_float(lw[i] & 0xFFFF0000u);
-    }
+    join4(*reinterpret_cast<const uint2*>(p), *reinterpret_cast<const uint2*>(p + 2 * Cb), v);
   } else {
-    const float* px = static_cast<const float*>(base) + pixel * Cs + c;
-    const float4 a = __ldg(reinterpret_cast<const float4*>(px)), b = __ldg(reinterpret_cast<const float4*>(px) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
+    v[0] = t.x; v[1] = t.y;
   }
 }
 
+// The same four channels of a pixel in global memory (lo_off: bytes from the hi to the lo half).
 template <int FMT>
-__device__ __forceinline__ void store8(void* __restrict__ base, size_t pixel, int c, int Cs, const float* v) {
+__device__ __forceinline__ void load4(const uint8_t* __restrict__ p, uint32_t lo_off, uint64_t* v) {
   if (FMT == ACT_SPLIT) {
-    __nv_bfloat16* px = static_cast<__nv_bfloat16*>(base) + pixel * 2 * Cs;
-    uint32_t hw[4], lw[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      // hi = bf16_rn(v), lo = bf16_rn(v - hi), two values per packed conversion (the roundings of split_bf16)
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-      hw[i] = *reinterpret_cast<const uint32_t*>(&h);
-      const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * i] - __uint_as_float(hw[i] << 16),
-                                                     v[2 * i + 1] - __uint_as_float(hw[i] & 0xFFFF0000u));
-      lw[i] = *reinterpret_cast<const uint32_t*>(&l);
-    }
-    *reinterpret_cast<uint4*>(px + c) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-    *reinterpret_cast<uint4*>(px + Cs + c) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+    join4(__ldg(reinterpret_cast<const uint2*>(p)), __ldg(reinterpret_cast<const uint2*>(p + lo_off)), v);
   } else {
-    float* px = static_cast<float*>(base) + pixel * Cs + c;
-    *reinterpret_cast<float4*>(px) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(px + 4) = make_float4(v[4], v[5], v[6], v[7]);
-  }
-}
-
-// Expanded weights [9][Cs], scales [Cs] and biases [Cs] of one job -> shared memory.  A thread
-// takes whole channels: the first tap brings the packed row (32 elements, 16 .. 128 bytes) into
-// L1 and the other eight taps hit it, and the channels of a thread are independent loads.
-__device__ __forceinline__ void stage_dw_params(const LayerJob& job, int Cout, int Cs, float* wsm, float* ssm, float* bsm) {
-  const int wrow_bytes = 32 * job.bits / 8;              // K = 9 pads to 32 elements
-#pragma unroll 4
-  for (int c = threadIdx.x; c < Cs; c += kDwThreads) {
-    const bool real = c < Cout;
-    const uint8_t* row = job.w + (size_t)(real ? c : 0) * wrow_bytes;
-#pragma unroll
-    for (int tap = 0; tap < 9; ++tap) wsm[tap * Cs + c] = real ? load_element(row, tap, job.bits) : 0.f;
-    ssm[c] = real ? job.scale[c] : 0.f;
-    bsm[c] = real ? job.bias[c] : 0.f;
-  }
-}
-
-template <int FMT, int STRIDE>
-__global__ void __launch_bounds__(kDwThreads, 4)
-depthwise3x3_kernel(ConvGeom g, const LayerJob* __restrict__ jobs) {
-  extern __shared__ __align__(16) float dsm[];          // [9][Cs] weights, [Cs] scale, [Cs] bias
-  const LayerJob job = jobs[blockIdx.y];
-  const int Cs = g.Cs_out;                               // == Cs_in
-  float* wsm = dsm;
-  float* ssm = dsm + 9 * Cs;
-  float* bsm = ssm + Cs;
-  stage_dw_params(job, g.Cout, Cs, wsm, ssm, bsm);
-  __syncthreads();
-
-  constexpr int IN_COLS = (kDwCols - 1) * STRIDE + 3;    // 6 or 9 input columns per thread
-  const int octs = Cs / 8;
-  const int col_groups = (g.Wo + kDwCols - 1) / kDwCols;
-  const int rows_out = g.B * (g.Ho + 2);
-  const long long n_items = (long long)rows_out * col_groups * octs;
-  for (long long item = (long long)blockIdx.x * kDwThreads + threadIdx.x; item < n_items;
-       item += (long long)gridDim.x * kDwThreads) {
-    const int oct = (int)(item % octs);
-    const long long rest = item / octs;
-    const int cg = (int)(rest % col_groups);
-    const int jr = (int)(rest / col_groups);             // padded output row (image, y')
-    const int b = jr / (g.Ho + 2), oyp = jr - b * (g.Ho + 2);
-    const int c = oct * 8, ox0 = cg * kDwCols;
-    float acc[kDwCols][8];
-#pragma unroll
-    for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc[x][i] = 0.f;
-    const bool interior = oyp >= 1 && oyp <= g.Ho;
-    if (interior) {
-#pragma unroll
-      for (int r = 0; r < 3; ++r) {
-        const int iy = (oyp - 1) * STRIDE - 1 + r;       // unpadded input row
-        if (iy < 0 || iy >= g.H) continue;
-        const size_t row_pix = (size_t)(b * (g.H + 2) + iy + 1) * g.W;
-        float in[IN_COLS][8];
-#pragma unroll
-        for (int xx = 0; xx < IN_COLS; ++xx) {
-          const int ix = ox0 * STRIDE - 1 + xx;
-          if (ix >= 0 && ix < g.W) {
-            load8<FMT>(job.in, row_pix + ix, c, Cs, in[xx]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) in[xx][i] = 0.f;
-          }
-        }
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const float4 w0 = *reinterpret_cast<const float4*>(wsm + (r * 3 + t) * Cs + c);
-          const float4 w1 = *reinterpret_cast<const float4*>(wsm + (r * 3 + t) * Cs + c + 4);
-          const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-          for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc[x][i] = fmaf(in[x * STRIDE + t][i], wv[i], acc[x][i]);
-        }
-      }
-    }
-    const float4 s0 = *reinterpret_cast<const float4*>(ssm + c), s1 = *reinterpret_cast<const float4*>(ssm + c + 4);
-    const float4 b0 = *reinterpret_cast<const float4*>(bsm + c), b1 = *reinterpret_cast<const float4*>(bsm + c + 4);
-    const float sc[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-    const float bi[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-    for (int x = 0; x < kDwCols; ++x) {
-      const int ox = ox0 + x;
-      if (ox >= g.Wo) break;
-      const size_t opix = (size_t)jr * g.Wo + ox;
-      float v[8];
-      if (interior) {
-        float rs[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        if (job.res) load8<FMT>(job.res, opix, c, Cs, rs);
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-          v[i] = (c + i < g.Cout) ? apply_act(fmaf(acc[x][i], sc[i], bi[i]) + rs[i], g.act) : 0.f;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = 0.f;
-      }
-      store8<FMT>(job.out, opix, c, Cs, v);
-    }
-  }
-}
-
-
-// Four channels of one pixel (the unit of the row-walking kernel).  `p` points at the group's
-// first channel in the pixel (split format: in the hi half; the lo half is lo_off bytes on).
-template <int FMT>
-__device__ __forceinline__ void load4(const uint8_t* __restrict__ p, uint32_t lo_off, float* v) {
-  if (FMT == ACT_SPLIT) {
-    const uint2 h = __ldg(reinterpret_cast<const uint2*>(p));
-    const uint2 l = __ldg(reinterpret_cast<const uint2*>(p + lo_off));
-    v[0] = __uint_as_float(h.x << 16) + __uint_as_float(l.x << 16);            // a bfloat16 is the upper half of a float
-    v[1] = __uint_as_float(h.x & 0xFFFF0000u) + __uint_as_float(l.x & 0xFFFF0000u);
-    v[2] = __uint_as_float(h.y << 16) + __uint_as_float(l.y << 16);
-    v[3] = __uint_as_float(h.y & 0xFFFF0000u) + __uint_as_float(l.y & 0xFFFF0000u);
-  } else {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = pack2(t.x, t.y); v[1] = pack2(t.z, t.w);
   }
 }
 
 template <int FMT>
 __device__ __forceinline__ void store4(uint8_t* __restrict__ p, uint32_t lo_off, const float* v) {
   if (FMT == ACT_SPLIT) {
-    uint32_t hw[2], lw[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      // hi = bf16_rn(v), lo = bf16_rn(v - hi), two values per packed conversion (the roundings of split_bf16)
-      const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-      hw[i] = *reinterpret_cast<const uint32_t*>(&h);
-      const __nv_bfloat162 l = __floats2bfloat162_rn(v[2 * i] - __uint_as_float(hw[i] << 16),
-                                                     v[2 * i + 1] - __uint_as_float(hw[i] & 0xFFFF0000u));
-      lw[i] = *reinterpret_cast<const uint32_t*>(&l);
-    }
-    *reinterpret_cast<uint2*>(p) = make_uint2(hw[0], hw[1]);
-    *reinterpret_cast<uint2*>(p + lo_off) = make_uint2(lw[0], lw[1]);
+    uint2 h, l;
+    split_pair(v[0], v[1], h.x, l.x);
+    split_pair(v[2], v[3], h.y, l.y);
+    *reinterpret_cast<uint2*>(p) = h;
+    *reinterpret_cast<uint2*>(p + lo_off) = l;
   } else {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
   }
 }
 
-// Row-walking kernel.  A thread owns kWalkCh = 4 channels x kDwCols output columns and walks down up to
-// `rb` consecutive output rows of one image, loading every input row once:
-//   stride 1: input row y feeds output rows y - 1 (tap row 2), y (tap row 1) and y + 1 (tap row
-//             0), held in three accumulator sets whose roles rotate from row to row;
-//   stride 2: output row j takes input rows 2j - 1, 2j, 2j + 1; row 2j + 1 is also the first
-//             tap row of output j + 1, whose product is carried over.
-// The row loop is a real loop (three rotated copies of the body at stride 1), so the code stays
-// small whatever `rb` is.  Input rows -1 and H are the physical padding rows of the image, which
-// every kernel writes as zeros: they are loaded like any other row.
-// acc[x][i] (+)= sum_t in[x * STRIDE + t][i] * w[(r, t)][c + i]
-template <int STRIDE, bool ACCUMULATE>
-__device__ __forceinline__ void dw_tap_row(const float* __restrict__ wsm, int Cs, int c, int r,
-                                           const float (&in)[(kDwCols - 1) * STRIDE + 3][kWalkCh], float (&acc)[kDwCols][kWalkCh]) {
-#pragma unroll
-  for (int t = 0; t < 3; ++t) {
-    const float4 w0 = *reinterpret_cast<const float4*>(wsm + (r * 3 + t) * Cs + c);
-    const float wv[kWalkCh] = {w0.x, w0.y, w0.z, w0.w};
-#pragma unroll
-    for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-      for (int i = 0; i < kWalkCh; ++i) {
-        const float prev = (ACCUMULATE || t > 0) ? acc[x][i] : 0.f;
-        acc[x][i] = fmaf(in[x * STRIDE + t][i], wv[i], prev);
-      }
-  }
+struct DwUnit { int slab, ox0, oy0, n_out, img0; };     // ox0: first output column of the tile
+template <int COLS>
+__device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int u) {
+  DwUnit d;
+  d.slab = u % p.n_slabs;
+  u /= p.n_slabs;
+  d.ox0 = (u % p.n_ct) * p.XG * COLS;
+  u /= p.n_ct;
+  d.oy0 = (u % p.n_rb) * p.rb;
+  d.n_out = min(p.rb, p.Ho - d.oy0);
+  d.img0 = (u / p.n_rb) * p.NI;
+  return d;
 }
 
-template <int FMT, int STRIDE>
-__global__ void __launch_bounds__(kDwThreads, 3)
-depthwise3x3_walk_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, int rb) {
-  extern __shared__ __align__(16) float dsm[];          // [9][Cs] weights, [Cs] scale, [Cs] bias
+// COLS output columns per thread: 2 (four output columns save a third of the unpacking at stride 1, but
+// three rows of accumulators beside the weights then spill at two blocks per SM).
+template <int FMT, int STRIDE, int COLS>
+__global__ void __launch_bounds__(kDwThreads + 32, 2)
+depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, const LayerJob* __restrict__ jobs) {
+  extern __shared__ __align__(128) uint8_t smem_raw[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~(uintptr_t)127);
   const LayerJob job = jobs[blockIdx.y];
-  const int Cs = g.Cs_out;                               // == Cs_in
-  float* wsm = dsm;
-  float* ssm = dsm + 9 * Cs;
-  float* bsm = ssm + Cs;
-  stage_dw_params(job, g.Cout, Cs, wsm, ssm, bsm);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int n_compute = (int)blockDim.x - 32;          // whole warps; the last warp issues the copies
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ring + p.stages * p.stage_bytes);
+  const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kDwMaxStages;
+  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * kDwMaxStages);
+
+  if (tid == 0) {
+    for (int i = 0; i < p.stages; ++i) {
+      mbar_init(bar_full + 8 * i, 1);
+      mbar_init(bar_empty + 8 * i, n_compute / 32);
+    }
+    *s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   __syncthreads();
 
-  constexpr int IN_COLS = (kDwCols - 1) * STRIDE + 3;    // input columns per thread
-  const int octs = Cs / kWalkCh;                         // channel groups
-  const int col_groups = (g.Wo + kDwCols - 1) / kDwCols;
-  const int row_blocks = (g.Ho + rb - 1) / rb;
-  const size_t pix_bytes = (size_t)4 * Cs;               // a pixel: [hi(Cs) | lo(Cs)] bfloat16 or Cs floats
-  const uint32_t lo_off = 2u * Cs;                       // split format: bytes from the hi to the lo half
-  const uint32_t in_pitch = (uint32_t)(g.W * pix_bytes), out_pitch = (uint32_t)(g.Wo * pix_bytes);
-  const bool clamp = g.act != AIQ_ACT_NONE;              // relu: [0, inf), relu6: [0, 6]
-  const float act_hi = g.act == AIQ_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
-  const long long n_items = (long long)g.B * row_blocks * col_groups * octs;
-  for (long long item = (long long)blockIdx.x * kDwThreads + threadIdx.x; item < n_items;
-       item += (long long)gridDim.x * kDwThreads) {
-    const int oct = (int)(item % octs);
-    long long rest = item / octs;
-    const int cg = (int)(rest % col_groups);
-    rest /= col_groups;
-    const int rbk = (int)(rest % row_blocks);
-    const int b = (int)(rest / row_blocks);
-    const int c = oct * kWalkCh, ox0 = cg * kDwCols;
-    const uint32_t ch_off = (uint32_t)c * (FMT == ACT_SPLIT ? 2u : 4u);   // bytes from a pixel to its channel c
-    const int oy0 = rbk * rb;                            // first (unpadded) output row of the block
-    const int n_out = min(rb, g.Ho - oy0);               // output rows of this block
-    const size_t out_row0 = (size_t)b * (g.Ho + 2);      // padded output row 0 of the image
-    const size_t in_row0 = (size_t)b * (g.H + 2) + 1;    // padded input row of unpadded row 0
-    const int ix0 = ox0 * STRIDE - 1;
+  if (tid >= n_compute) {
+    // ---- producer: padded input rows oy0 * STRIDE .. of every unit of this block, in order -----------
+    if (lane == 0) {
+      bool alive = true;
+      uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
+      for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
+        const DwUnit d = dw_unit<COLS>(p, u);
+        const int n_rows = (d.n_out - 1) * STRIDE + 3;
+        const int img = job.in_version * p.batch_capacity + d.img0;
+        for (int r = 0; r < n_rows; ++r) {
+          alive = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+          if (!alive) break;
+          issued |= 1u << stage;
+          issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+          mbar_expect_tx(bar_full + 8 * stage, (uint32_t)p.box_bytes);
+          asm volatile(
+              "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+              ::"r"(smem_u32(ring) + stage * p.stage_bytes), "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(bar_full + 8 * stage),
+              "r"(d.slab * p.Cb), "r"(0), "r"(d.ox0 * STRIDE - 1), "r"(d.oy0 * STRIDE + r), "r"(img)
+              : "memory");
+          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
+        }
+      }
+      for (int i = 0; i < p.stages; ++i)               // copies in flight must land before the CTA exits
+        if (issued & (1u << i)) {
+          const long long t0 = clock64();
+          while (!mbar_try_wait(bar_full + 8 * i, (issued_phase >> i) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
+        }
+    }
+    return;
+  }
 
-    // Addresses are kept as running pointers: one per input column, stepped by a row after every
-    // load (a column outside the image points at a pixel of the image's first padding row, which
-    // holds zeros, and does not move), one for the output row and one for the residual row.
-    const uint8_t* colp[IN_COLS];
-    uint32_t colstep[IN_COLS];
-    {
-      const uint8_t* in_base = static_cast<const uint8_t*>(job.in) + ch_off;
-      const size_t first_row = in_row0 + (size_t)(oy0 * STRIDE) - 1;      // padded row of m = 0 (>= in_row0 - 1)
+  // ---- compute: thread = (image of the group, column group, channel quad), quad fastest ---------------
+  const int q = tid % p.CQ, xg = (tid / p.CQ) % p.XG, ni = tid / (p.CQ * p.XG);
+  const bool worker = ni < p.NI;                         // the last warp may have idle lanes
+  const int slab = (int)blockIdx.x % p.n_slabs;          // the grid is a multiple of the slabs: fixed for this block
+  const int c = slab * p.Cb + q * 4;
+  const size_t pix_bytes = (size_t)4 * p.Cs;             // [hi(Cs) | lo(Cs)] bfloat16 or Cs floats
+  const uint32_t lo_off = 2u * p.Cs;
+  const uint32_t ch_off = (uint32_t)c * (FMT == ACT_SPLIT ? 2u : 4u);
+  const uint32_t out_pitch = (uint32_t)(p.Wo * pix_bytes);
+  const uint32_t col_bytes = 4u * p.Cb;                  // a pixel of the slab in shared memory
+  const bool clamp = p.act != AIQ_ACT_NONE;              // relu: [0, inf), relu6: [0, 6]
+  const float act_hi = p.act == AIQ_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
+
+  uint64_t w[9][2], sc[2], bi[2];                        // weights, scale and bias of the four channels
+  {
+    float t[9][4], s4[4], b4[4];
+    const int wrow_bytes = 32 * job.bits / 8;            // K = 9 pads to 32 elements
 #pragma unroll
-      for (int xx = 0; xx < IN_COLS; ++xx) {
-        const int ix = ix0 + xx;
-        const bool inside = ix >= 0 && ix < g.W;
-        colp[xx] = in_base + (inside ? first_row * g.W + ix : (in_row0 - 1) * g.W) * pix_bytes;
-        colstep[xx] = inside ? in_pitch : 0u;
+    for (int i = 0; i < 4; ++i) {
+      const bool real = worker && c + i < p.C;           // padding channels: zero weights, scale and bias
+      const uint8_t* row = job.w + (size_t)(real ? c + i : 0) * wrow_bytes;
+      uint4 r0 = __ldg(reinterpret_cast<const uint4*>(row)), r1 = r0, r2 = r0;
+      if (job.bits >= 16) r1 = __ldg(reinterpret_cast<const uint4*>(row) + 1);
+      if (job.bits == 32) r2 = __ldg(reinterpret_cast<const uint4*>(row) + 2);
+      const uint32_t words[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        float v;
+        if (job.bits == 4) v = (float)((int)(((words[k >> 3] >> (4 * (k & 7))) & 0xFu) ^ 8u) - 8);
+        else if (job.bits == 8) v = (float)(int)(int8_t)((words[k >> 2] >> (8 * (k & 3))) & 0xFFu);
+        else if (job.bits == 16) v = __half2float(__ushort_as_half((unsigned short)((words[k >> 1] >> (16 * (k & 1))) & 0xFFFFu)));
+        else v = __uint_as_float(words[k]);
+        t[k][i] = real ? v : 0.f;
+      }
+      s4[i] = real ? __ldg(job.scale + c + i) : 0.f;
+      b4[i] = real ? __ldg(job.bias + c + i) : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) { w[k][0] = pack2(t[k][0], t[k][1]); w[k][1] = pack2(t[k][2], t[k][3]); }
+    sc[0] = pack2(s4[0], s4[1]); sc[1] = pack2(s4[2], s4[3]);
+    bi[0] = pack2(b4[0], b4[1]); bi[1] = pack2(b4[2], b4[3]);
+  }
+
+  constexpr int IN_COLS = (COLS - 1) * STRIDE + 3;
+  const uint8_t* my_cols = ring + (size_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
+                           (size_t)q * (FMT == ACT_SPLIT ? 8 : 16);
+  uint32_t stage = 0, phase = 0;
+  bool alive = true;
+  // The next padded row: wait, accumulate it as tap row RA into `a`, RB into `b` and RC into `cc` (-1: not
+  // at all; the first contribution to `cc` is written, not added) and hand the stage back.
+  auto row = [&](auto ra, auto rb_, auto rc, uint64_t (&a)[COLS][2], uint64_t (&b)[COLS][2], uint64_t (&cc)[COLS][2]) -> bool {
+    constexpr int RA = decltype(ra)::value, RB = decltype(rb_)::value, RC = decltype(rc)::value;
+    alive = mbar_wait_warp(bar_full + 8 * stage, phase, s_abort, p.error_flag);
+    if (!alive) return false;
+    const uint8_t* src = my_cols + stage * p.stage_bytes;
+#pragma unroll
+    for (int xx = 0; xx < IN_COLS; ++xx) {
+      uint64_t v[2];
+      read4<FMT>(src + xx * col_bytes, p.Cb, v);
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        if ((xx - t) % STRIDE != 0 || xx < t || (xx - t) / STRIDE >= COLS) continue;
+        const int x = (xx - t) / STRIDE;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (RA >= 0) a[x][i] = fma2(v[i], w[(RA < 0 ? 0 : RA) * 3 + t][i], a[x][i]);
+          if (RB >= 0) b[x][i] = fma2(v[i], w[(RB < 0 ? 0 : RB) * 3 + t][i], b[x][i]);
+          if (RC >= 0) cc[x][i] = fma2(v[i], w[(RC < 0 ? 0 : RC) * 3 + t][i], t == 0 ? 0ull : cc[x][i]);
+        }
       }
     }
-    auto load_next_row = [&](float (&in)[IN_COLS][kWalkCh]) {
-#pragma unroll
-      for (int xx = 0; xx < IN_COLS; ++xx) {
-        load4<FMT>(colp[xx], lo_off, in[xx]);
-        colp[xx] += colstep[xx];
-      }
-    };
-    uint8_t* outp = static_cast<uint8_t*>(job.out) + ch_off + ((out_row0 + oy0 + 1) * g.Wo + ox0) * pix_bytes;
-    const uint8_t* resp = job.res ? static_cast<const uint8_t*>(job.res) + (outp - static_cast<uint8_t*>(job.out)) : nullptr;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the reads above before the next copy's writes
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_empty + 8 * stage);
+    if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
+    return true;
+  };
+  using I0 = std::integral_constant<int, 0>;
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  using IN = std::integral_constant<int, -1>;
 
+  for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
+    const DwUnit d = dw_unit<COLS>(p, u);
+    const int b = d.img0 + ni, ox = d.ox0 + xg * COLS;
+    const bool writes = worker && b < p.B && c < p.Cs && ox < p.Wo;
+    uint8_t* outp = static_cast<uint8_t*>(job.out) + ch_off + (((size_t)b * (p.Ho + 2) + d.oy0 + 1) * p.Wo + ox) * pix_bytes;
+    const uint8_t* resp = job.res ? static_cast<const uint8_t*>(job.res) + (outp - static_cast<uint8_t*>(job.out)) : nullptr;
     // finish and store the next output row (rows are emitted in order) from its accumulators
-    auto emit = [&](const float (&acc)[kDwCols][kWalkCh]) {
-      const float4 s0 = *reinterpret_cast<const float4*>(ssm + c);
-      const float4 b0 = *reinterpret_cast<const float4*>(bsm + c);
-      const float sc[kWalkCh] = {s0.x, s0.y, s0.z, s0.w};
-      const float bi[kWalkCh] = {b0.x, b0.y, b0.z, b0.w};
+    auto emit = [&](const uint64_t (&acc)[COLS][2]) {
+      if (writes) {
 #pragma unroll
-      for (int x = 0; x < kDwCols; ++x) {
-        if (ox0 + x >= g.Wo) break;
-        float v[kWalkCh];
+        for (int x = 0; x < COLS; ++x) {
+          if (ox + x >= p.Wo) break;
+          uint64_t r[2] = {fma2(acc[x][0], sc[0], bi[0]), fma2(acc[x][1], sc[1], bi[1])};
+          if (resp) {
+            uint64_t rs[2];
+            load4<FMT>(resp + x * pix_bytes, lo_off, rs);
+            r[0] = add2(r[0], rs[0]);
+            r[1] = add2(r[1], rs[1]);
+          }
+          const float2 e0 = unpack2(r[0]), e1 = unpack2(r[1]);
+          float v[4] = {e0.x, e0.y, e1.x, e1.y};
+          if (clamp) {
 #pragma unroll
-        for (int i = 0; i < kWalkCh; ++i) v[i] = fmaf(acc[x][i], sc[i], bi[i]);
-        if (resp) {
-          float rs[kWalkCh];
-          load4<FMT>(resp + x * pix_bytes, lo_off, rs);
-#pragma unroll
-          for (int i = 0; i < kWalkCh; ++i) v[i] += rs[i];
+            for (int i = 0; i < 4; ++i) v[i] = fminf(fmaxf(v[i], 0.f), act_hi);
+          }
+          store4<FMT>(outp + x * pix_bytes, lo_off, v);   // padding channels: zero weights and bias give zero
         }
-        if (clamp) {
-#pragma unroll
-          for (int i = 0; i < kWalkCh; ++i) v[i] = fminf(fmaxf(v[i], 0.f), act_hi);
-        }
-        if (c + kWalkCh > g.Cout) {                      // padding channels stay zero
-#pragma unroll
-          for (int i = 0; i < kWalkCh; ++i)
-            if (c + i >= g.Cout) v[i] = 0.f;
-        }
-        store4<FMT>(outp + x * pix_bytes, lo_off, v);
       }
       outp += out_pitch;
       if (resp) resp += out_pitch;
     };
-
     if (STRIDE == 1) {
-      // k-th input row of the block = unpadded row oy0 - 1 + k, k = 0 .. n_out + 1.  a0 / a1 / a2
-      // belong to output rows oy0 + k - 2 / k - 1 / k; a0 is complete after this row.
-      auto step = [&](int k, float (&a0)[kDwCols][kWalkCh], float (&a1)[kDwCols][kWalkCh], float (&a2)[kDwCols][kWalkCh]) {
-        float in[IN_COLS][kWalkCh];
-        load_next_row(in);                               // unpadded row oy0 - 1 + k (-1 .. H)
-        // rows that belong to a neighbouring block are accumulated too and never stored
-        dw_tap_row<STRIDE, true>(wsm, Cs, c, 2, in, a0);
-        dw_tap_row<STRIDE, true>(wsm, Cs, c, 1, in, a1);
-        dw_tap_row<STRIDE, false>(wsm, Cs, c, 0, in, a2);
-        if (k >= 2) emit(a0);
-      };
-      float A[kDwCols][kWalkCh], B[kDwCols][kWalkCh], C[kDwCols][kWalkCh];
+      // input row k of the block (padded row oy0 + k) is tap row 2 / 1 / 0 of output rows k - 2 / k - 1 / k
+      uint64_t A[COLS][2], Bq[COLS][2], Cq[COLS][2];
 #pragma unroll
-      for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-        for (int i = 0; i < kWalkCh; ++i) A[x][i] = B[x][i] = 0.f;
-      const int n_rows = n_out + 2;
+      for (int x = 0; x < COLS; ++x) A[x][0] = A[x][1] = Bq[x][0] = Bq[x][1] = 0ull;
+      const int n_rows = d.n_out + 2;
       for (int k = 0; k < n_rows; k += 3) {
-        step(k, A, B, C);
-        if (k + 1 < n_rows) step(k + 1, B, C, A);
-        if (k + 2 < n_rows) step(k + 2, C, A, B);
+        if (!row(I2(), I1(), I0(), A, Bq, Cq)) break;
+        if (k >= 2) emit(A);
+        if (k + 1 < n_rows) {
+          if (!row(I2(), I1(), I0(), Bq, Cq, A)) break;
+          if (k + 1 >= 2) emit(Bq);
+        }
+        if (k + 2 < n_rows) {
+          if (!row(I2(), I1(), I0(), Cq, A, Bq)) break;
+          emit(Cq);
+        }
       }
     } else {
-      // output row j of the block takes unpadded input rows 2 (oy0 + j) - 1, .., + 1
-      float acc[kDwCols][kWalkCh], carry[kDwCols][kWalkCh];
-      float in[IN_COLS][kWalkCh];
+      // output row j takes padded rows 2 j, 2 j + 1, 2 j + 2; row 2 j + 2 is also the first of output j + 1
+      uint64_t acc[COLS][2], next[COLS][2];
+      row(IN(), IN(), I0(), acc, acc, next);
+      for (int j = 0; j < d.n_out && alive; ++j) {
 #pragma unroll
-      for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-        for (int i = 0; i < kWalkCh; ++i) carry[x][i] = 0.f;
-      load_next_row(in);                                 // unpadded row 2 oy0 - 1
-      dw_tap_row<STRIDE, false>(wsm, Cs, c, 0, in, carry);
-      for (int j = 0; j < n_out; ++j) {
-        load_next_row(in);                               // rows 2 (oy0 + j) and, below, + 1 (<= H)
-#pragma unroll
-        for (int x = 0; x < kDwCols; ++x)
-#pragma unroll
-          for (int i = 0; i < kWalkCh; ++i) acc[x][i] = carry[x][i];
-        dw_tap_row<STRIDE, true>(wsm, Cs, c, 1, in, acc);
-        load_next_row(in);
-        dw_tap_row<STRIDE, true>(wsm, Cs, c, 2, in, acc);
-        dw_tap_row<STRIDE, false>(wsm, Cs, c, 0, in, carry);
+        for (int x = 0; x < COLS; ++x) { acc[x][0] = next[x][0]; acc[x][1] = next[x][1]; }
+        if (!row(I1(), IN(), IN(), acc, acc, acc)) break;
+        if (!row(I2(), IN(), I0(), acc, acc, next)) break;
         emit(acc);
       }
     }
     // the two physical padding rows of the image, by the first and the last row block
-    if (rbk == 0 || rbk == row_blocks - 1) {
-      const float zero[kWalkCh] = {0, 0, 0, 0};
+    if (writes) {
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
-        if (side == 0 ? rbk != 0 : rbk != row_blocks - 1) continue;
-        const size_t jr = out_row0 + (side == 0 ? 0 : g.Ho + 1);
+        if (side == 0 ? d.oy0 != 0 : d.oy0 + d.n_out != p.Ho) continue;
+        uint8_t* z = static_cast<uint8_t*>(job.out) + ch_off +
+                     (((size_t)b * (p.Ho + 2) + (side == 0 ? 0 : p.Ho + 1)) * p.Wo + ox) * pix_bytes;
 #pragma unroll
-        for (int x = 0; x < kDwCols; ++x)
-          if (ox0 + x < g.Wo)
-            store4<FMT>(static_cast<uint8_t*>(job.out) + ch_off + (jr * g.Wo + ox0 + x) * pix_bytes, lo_off, zero);
+        for (int x = 0; x < COLS; ++x)
+          if (ox + x < p.Wo) store4<FMT>(z + x * pix_bytes, lo_off, zero);
       }
     }
   }
 }
 
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiledFn dw_encode_fn() {
+  static std::atomic<EncodeTiledFn> fn{nullptr};
+  if (EncodeTiledFn f = fn.load(std::memory_order_acquire)) return f;
+  void* sym = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  fn.store(reinterpret_cast<EncodeTiledFn>(sym), std::memory_order_release);
+  return reinterpret_cast<EncodeTiledFn>(sym);
+}
+
+// The part of the launch shape the tensor map depends on: slab width, column groups, images of a stage.
+struct DwShape { int cols, Cb, XG, NI, Wb; };
+DwShape dw_shape(const ConvGeom& g, int batch_capacity) {
+  DwShape s = {};
+  s.cols = kDwCols;
+  const int xg = (g.Wo + s.cols - 1) / s.cols;
+  // the widest slab that divides the padded channels (wide slabs: long contiguous runs of the tensor), but
+  // narrower ones where a row of the map then fits one block, down to 32 channels
+  s.Cb = 16;
+  for (int cb : {32, 48, 64})
+    if (g.Cs_out % cb == 0 && (s.Cb < 32 || (cb / 4) * xg <= kDwThreads)) s.Cb = cb;
+  s.XG = std::min(xg, std::min(kDwMaxColGroups, kDwThreads / (s.Cb / 4)));
+  s.XG = (xg + (xg + s.XG - 1) / s.XG - 1) / ((xg + s.XG - 1) / s.XG);    // column tiles of equal width
+  // narrow maps: several images side by side fill the block (8 at most)
+  s.NI = std::max(1, std::min(std::min(8, batch_capacity), kDwThreads / (s.Cb / 4 * s.XG)));
+  s.Wb = (s.XG * s.cols - 1) * g.stride + 3;
+  return s;
+}
+
 }  // namespace
 
-aiq_status_t launch_depthwise(const ConvGeom& g, const LayerJob* jobs_dev, int n_jobs,
-                              const float* /*net_input*/, double weight_bytes, cudaStream_t s) {
+aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions, void* map_out) {
+  EncodeTiledFn enc = dw_encode_fn();
+  if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+  const DwShape s = dw_shape(g, batch_capacity);
+  const bool split = g.act_format == ACT_SPLIT;
+  // (channel, hi | lo, column, padded row, image over all versions); float32 pixels have one part
+  const cuuint64_t pix = 4ull * g.Cs_in, row = pix * g.W;
+  cuuint64_t dims[5] = {(cuuint64_t)g.Cs_in, split ? 2ull : 1ull, (cuuint64_t)g.W, (cuuint64_t)g.H + 2, (cuuint64_t)n_versions * batch_capacity};
+  cuuint64_t strides[4] = {split ? 2ull * g.Cs_in : pix, pix, row, row * (g.H + 2)};
+  cuuint32_t box[5] = {(cuuint32_t)s.Cb, split ? 2u : 1u, (cuuint32_t)s.Wb, 1u, (cuuint32_t)s.NI};
+  cuuint32_t one[5] = {1, 1, 1, 1, 1};
+  const CUresult r = enc(static_cast<CUtensorMap*>(map_out), split ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                         5, const_cast<void*>(slot_base), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled (depthwise) failed with code %d", (int)r);
+  return AIQ_OK;
+}
+
+aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
+                              int32_t* error_flag, double weight_bytes, cudaStream_t s) {
   if (g.stride != 1 && g.stride != 2) return set_error(AIQ_ERR_SHAPE, "depthwise: stride %d is not supported", g.stride);
-  const int Cs = g.Cs_out;
-  const size_t smem = (size_t)11 * Cs * sizeof(float);
   DeviceProps props;
   if (aiq_status_t st = current_device_props(&props)) return st;
-  const int n_sms = props.n_sms;
-  if (smem > 48 * 1024) return set_error(AIQ_ERR_SHAPE, "depthwise: %d channels need %zu bytes of shared memory", g.Cout, smem);
-  const int col_groups = (g.Wo + kDwCols - 1) / kDwCols;
-  // Rows per thread of the row-walking kernel: the image height cut into the fewest blocks of at
-  // most 16 rows, of equal height where it divides.  The kernel is used when it still gives
-  // every SM a block of threads; smaller launches need the parallelism of one row per thread.
-  const int n_blk = (g.Ho + 15) / 16;
-  const int rb = (g.Ho + n_blk - 1) / n_blk;
-  const long long items_rows = (long long)g.B * n_blk * col_groups * (Cs / kWalkCh);
-  const bool walk_rows = items_rows >= (long long)n_sms * kDwThreads;
-  const long long n_items = walk_rows ? items_rows : (long long)g.B * (g.Ho + 2) * col_groups * (Cs / 8);
-  long long blocks = (n_items + kDwThreads - 1) / kDwThreads;
-  const long long cap = (long long)n_sms * (walk_rows ? 3 : 4);   // persistent: as many blocks as are resident
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  dim3 grid((unsigned)blocks, n_jobs);
+  const DwShape sh = dw_shape(g, batch_capacity);
+  DwParams p = {};
+  p.B = g.B; p.H = g.H; p.W = g.W; p.Ho = g.Ho; p.Wo = g.Wo; p.C = g.Cout; p.Cs = g.Cs_out; p.act = g.act;
+  p.Cb = sh.Cb; p.CQ = sh.Cb / 4; p.XG = sh.XG; p.NI = sh.NI; p.Wb = sh.Wb;
+  const int col_groups = (g.Wo + sh.cols - 1) / sh.cols;
+  p.n_ct = (col_groups + sh.XG - 1) / sh.XG;
+  p.n_ig = (g.B + sh.NI - 1) / sh.NI;
+  p.n_slabs = (g.Cs_out + sh.Cb - 1) / sh.Cb;
+  p.batch_capacity = batch_capacity;
+  p.error_flag = error_flag;
+  p.box_bytes = sh.NI * sh.Wb * sh.Cb * 4;
+  p.stage_bytes = (int)align_up((size_t)p.box_bytes, 128);
+  const int threads = (p.CQ * p.XG * p.NI + 31) / 32 * 32 + 32;
+  // two blocks per SM, each with as many rows in flight as fit (at most 8)
+  const int per_cta = (props.smem_optin + 1024) / 2 - 1024;
+  const int fixed = 128 + (2 * kDwMaxStages + 1) * 8;
+  p.stages = std::min(kDwMaxStages, (per_cta - fixed) / p.stage_bytes);
+  if (p.stages < 2) return set_error(AIQ_ERR_SHAPE, "depthwise: %d bytes per input row do not fit shared memory", p.stage_bytes);
+  const int smem = p.stages * p.stage_bytes + fixed;
+  // Row blocks: whole images where they fill the GPU (no halo rows read twice), else blocks of rows, down to
+  // two, until every SM has work.
+  const long long columns = (long long)p.n_ig * p.n_ct * p.n_slabs * n_jobs;
+  const int want = (int)std::min<long long>((2ll * props.n_sms + columns - 1) / columns, (g.Ho + 1) / 2);
+  p.rb = (g.Ho + std::max(want, 1) - 1) / std::max(want, 1);
+  p.n_rb = (g.Ho + p.rb - 1) / p.rb;
+  p.n_units = p.n_ig * p.n_rb * p.n_ct * p.n_slabs;
+  // Blocks: a multiple of the slabs (a block then keeps its weights in registers).  The number is the one
+  // whose last wave is fullest, counted in units plus a start-up of about two units per block.
+  const int resident = 2 * props.n_sms;
+  const int per_slab = p.n_units / p.n_slabs;
+  int best_k = 1;
+  double best = 1e300;
+  for (int k = 1; k <= per_slab; ++k) {
+    const long long ctas = (long long)k * p.n_slabs * n_jobs;
+    const double waves = (double)((ctas + resident - 1) / resident);
+    const double cost = waves * ((per_slab + k - 1) / k + 2.0 / (p.rb * g.stride + 2));
+    if (cost < best * 0.999) { best = cost; best_k = k; }
+    if (ctas > 16ll * resident) break;
+  }
+  const dim3 grid((unsigned)(best_k * p.n_slabs), n_jobs);
   LaunchScope scope(AIQ_KERNEL_DEPTHWISE, s, 18.0 * g.B * g.Ho * g.Wo * g.Cout * n_jobs,
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                    (double)g.B * g.Ho * g.Wo * g.Cout));
-  if (walk_rows) {
-#define AIQ_DWR(FMT_, ST_) depthwise3x3_walk_kernel<FMT_, ST_><<<grid, kDwThreads, smem, s>>>(g, jobs_dev, rb)
-    if (g.act_format == ACT_SPLIT) { if (g.stride == 1) AIQ_DWR(ACT_SPLIT, 1); else AIQ_DWR(ACT_SPLIT, 2); }
-    else { if (g.stride == 1) AIQ_DWR(ACT_F32, 1); else AIQ_DWR(ACT_F32, 2); }
-#undef AIQ_DWR
-    AIQ_LAUNCH_CHECK("depthwise3x3_walk");
-    return AIQ_OK;
-  }
-#define AIQ_DW(FMT_, ST_) depthwise3x3_kernel<FMT_, ST_><<<grid, kDwThreads, smem, s>>>(g, jobs_dev)
-  if (g.act_format == ACT_SPLIT) { if (g.stride == 1) AIQ_DW(ACT_SPLIT, 1); else AIQ_DW(ACT_SPLIT, 2); }
-  else { if (g.stride == 1) AIQ_DW(ACT_F32, 1); else AIQ_DW(ACT_F32, 2); }
+  const CUtensorMap& m = *static_cast<const CUtensorMap*>(map);
+#define AIQ_DW(FMT_, ST_, COLS_)                                                                       \
+  do {                                                                                                 \
+    AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_>), per_cta);                          \
+    depthwise3x3_kernel<FMT_, ST_, COLS_><<<grid, threads, smem, s>>>(m, p, jobs_dev);                  \
+  } while (0)
+  if (g.act_format == ACT_SPLIT) { if (g.stride == 1) AIQ_DW(ACT_SPLIT, 1, kDwCols); else AIQ_DW(ACT_SPLIT, 2, kDwCols); }
+  else { if (g.stride == 1) AIQ_DW(ACT_F32, 1, kDwCols); else AIQ_DW(ACT_F32, 2, kDwCols); }
 #undef AIQ_DW
   AIQ_LAUNCH_CHECK("depthwise3x3");
   return AIQ_OK;

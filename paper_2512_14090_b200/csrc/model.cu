@@ -878,6 +878,12 @@ static aiq_status_t build_plan(const aiq_model* m, const uint8_t* schemes, int S
           if (st != AIQ_OK) return st;
         }
       }
+      if (li.d.kind == AIQ_LAYER_DEPTHWISE) {
+        const LayerInfo& src = m->layers[li.d.input];
+        aiq_status_t st = depthwise_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B,
+                                               plan.lp[li.d.input].n_versions, &lp.maps[0]);
+        if (st != AIQ_OK) return st;
+      }
       for (int v : vorder) {
         LayerJob j = {};
         const int bits = std::get<0>(keys[v]);
@@ -1003,7 +1009,8 @@ static aiq_status_t run_chunk(const aiq_model* m, const EvalPlan& plan, const La
       continue;
     }
     if (li.d.kind == AIQ_LAYER_DEPTHWISE) {
-      st = launch_depthwise(g, jobs_dev + lp.job_first, lp.n_versions, x_chunk, lp.weight_bytes, stream);
+      st = launch_depthwise(g, &lp.maps[0], jobs_dev + lp.job_first, lp.n_versions, plan.batch_capacity, m->status_word,
+                            lp.weight_bytes, stream);
       if (st != AIQ_OK) return st;
       continue;
     }

@@ -59,7 +59,32 @@ struct LaunchScope {
   ~LaunchScope();
   int slot_;
   cudaStream_t stream_;
+  bool chain;              // chain_pays(bytes), for launch_chained
 };
+
+// Launch of a kernel that is part of a chain on one stream (the layers of a forward pass): its blocks may become
+// resident, and run the part of their set-up that does not depend on the chain, while the kernel before drains.
+// Every such kernel calls chain_wait() in every block before it touches anything an earlier kernel of the chain
+// reads or writes, and chain_release() once its own set-up is done (a kernel that allocates tensor memory only after
+// it has it: a later kernel's block could otherwise take the columns an earlier one is waiting for).
+// `chain`: whether to do so at all (chain_pays); the kernel is the same either way.
+bool chain_pays(double bytes);
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// What a kernel of the chain reads of an earlier one's results: an ordinary load, not the read-only path, whose lines
+// may be older than the wait and which the compiler may move above it.
+template <typename T>
+__device__ __forceinline__ T ld_chain(const T* p) { return *p; }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 inline bool bits_ok(int bits) { return bits == 4 || bits == 8 || bits == 16 || bits == 32; }
 inline int padded_k(int K) { return (K + 31) / 32 * 32; }

@@ -21,10 +21,10 @@ constexpr int BK = 16;
 
 enum { IN_NCHW = 0, IN_SPLIT_VEC = 1, IN_SPLIT_SCALAR = 2 };
 
-__device__ __forceinline__ float4 load_split4(const __nv_bfloat16* __restrict__ pix, int c, int Cs) {
+__device__ __forceinline__ float4 load_split4(const __nv_bfloat16* pix, int c, int Cs) {
   // 4 consecutive channels of one pixel: hi and lo halves are 8-byte loads
-  const uint2 h = __ldg(reinterpret_cast<const uint2*>(pix + c));
-  const uint2 l = __ldg(reinterpret_cast<const uint2*>(pix + Cs + c));
+  const uint2 h = ld_chain(reinterpret_cast<const uint2*>(pix + c));
+  const uint2 l = ld_chain(reinterpret_cast<const uint2*>(pix + Cs + c));
   const __nv_bfloat162 h0 = *reinterpret_cast<const __nv_bfloat162*>(&h.x);
   const __nv_bfloat162 h1 = *reinterpret_cast<const __nv_bfloat162*>(&h.y);
   const __nv_bfloat162 l0 = *reinterpret_cast<const __nv_bfloat162*>(&l.x);
@@ -52,18 +52,18 @@ __device__ __forceinline__ void store_split4(__nv_bfloat16* __restrict__ pix, in
 // Element access of an activation tensor in either storage format.  A pixel is 4*Cs bytes
 // in both: Cs floats (ACT_F32) or [hi Cs | lo Cs] bfloat16 (ACT_SPLIT).
 template <int FMT>
-__device__ __forceinline__ float4 act_load4(const void* __restrict__ base, size_t pixel, int c, int Cs) {
+__device__ __forceinline__ float4 act_load4(const void* base, size_t pixel, int c, int Cs) {
   if (FMT == ACT_SPLIT)
     return load_split4(static_cast<const __nv_bfloat16*>(base) + pixel * 2 * Cs, c, Cs);
-  return __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(base) + pixel * Cs + c));
+  return ld_chain(reinterpret_cast<const float4*>(static_cast<const float*>(base) + pixel * Cs + c));
 }
 template <int FMT>
-__device__ __forceinline__ float act_load1(const void* __restrict__ base, size_t pixel, int c, int Cs) {
+__device__ __forceinline__ float act_load1(const void* base, size_t pixel, int c, int Cs) {
   if (FMT == ACT_SPLIT) {
     const __nv_bfloat16* px = static_cast<const __nv_bfloat16*>(base) + pixel * 2 * Cs;
     return __bfloat162float(px[c]) + __bfloat162float(px[Cs + c]);
   }
-  return __ldg(static_cast<const float*>(base) + pixel * Cs + c);
+  return ld_chain(static_cast<const float*>(base) + pixel * Cs + c);
 }
 template <int FMT>
 __device__ __forceinline__ void act_store4(void* __restrict__ base, size_t pixel, int c, int Cs, float4 v) {
@@ -125,6 +125,7 @@ conv_igemm_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, const float* __
   constexpr int B_PER_THREAD = (BK * BN + kConvThreads - 1) / kConvThreads;
   float b_reg[B_PER_THREAD];
   const int wrow_bytes = ((g.K + 31) / 32 * 32) * job.bits / 8;
+  chain_release();
 
   auto fetch = [&](int slice) {
     const int k0 = slice * BK;
@@ -217,6 +218,7 @@ conv_igemm_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, const float* __
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
 
+  chain_wait();
   fetch(0);
   stash(0);
   __syncthreads();
@@ -293,9 +295,9 @@ aiq_status_t launch_conv_tile(const ConvGeom& g, const LayerJob* jobs, int n_job
 #define AIQ_CONV_LAUNCH(MODE)                                                                        \
   do {                                                                                              \
     if (g.act_format == ACT_SPLIT)                                                                  \
-      conv_igemm_kernel<BM, BN, TM, TN, MODE, ACT_SPLIT><<<grid, kConvThreads, 0, s>>>(g, jobs, net_input); \
+      AIQ_CUDA_TRY(launch_chained(scope.chain, conv_igemm_kernel<BM, BN, TM, TN, MODE, ACT_SPLIT>, grid, dim3(kConvThreads), 0, s, g, jobs, net_input)); \
     else                                                                                            \
-      conv_igemm_kernel<BM, BN, TM, TN, MODE, ACT_F32><<<grid, kConvThreads, 0, s>>>(g, jobs, net_input);   \
+      AIQ_CUDA_TRY(launch_chained(scope.chain, conv_igemm_kernel<BM, BN, TM, TN, MODE, ACT_F32>, grid, dim3(kConvThreads), 0, s, g, jobs, net_input));   \
   } while (0)
   if (in_mode == IN_SPLIT_VEC) AIQ_CONV_LAUNCH(IN_SPLIT_VEC);
   else if (in_mode == IN_SPLIT_SCALAR) AIQ_CONV_LAUNCH(IN_SPLIT_SCALAR);
@@ -335,6 +337,8 @@ conv_stem_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, const float* __r
     bsm[n] = n < g.Cout ? job.bias[n] : 0.f;
   }
   __syncthreads();
+  chain_release();
+  chain_wait();
 
   const int rows_out = g.Ho + 2;
   const long long M = (long long)g.B * rows_out * g.Wo;      // padded output pixels
@@ -403,6 +407,8 @@ conv_stem_rs_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, const float* 
   }
   for (int n = threadIdx.x; n < COUT; n += kStemThreads) { ssm[n] = job.scale[n]; bsm[n] = job.bias[n]; }
   __syncthreads();
+  chain_release();
+  chain_wait();
 
   const int G = rs_group_images_dev(g.Wo);
   const int Bp = (g.B + 15) / 16 * 16;
@@ -507,6 +513,8 @@ conv_stem_rs_rows_kernel(ConvGeom g, const LayerJob* __restrict__ jobs, const fl
   for (int i = threadIdx.x; i < g.Cin * (kStemRows + 2) * G * 2; i += n_threads)    // the zero columns
     tile[(size_t)(i >> 1) * RS + ((i & 1) ? g.W + 1 : 0)] = 0.f;
   __syncthreads();
+  chain_release();
+  chain_wait();                                               // only the output depends on the kernels before
 
   const int img = threadIdx.x % G, ox = threadIdx.x / G;
   const size_t plane_bytes = (size_t)G * 16;
@@ -571,13 +579,13 @@ aiq_status_t launch_stem(const ConvGeom& g, const LayerJob* jobs, int n_jobs, co
       G * g.Wo <= 256 && (G * g.Wo) % 32 == 0 && smem + tile_bytes <= 100 * 1024) {
     AIQ_ENSURE_DYNAMIC_SMEM((conv_stem_rs_rows_kernel<COUT>), 100 * 1024);
     const dim3 rgrid((unsigned)(rs_padded_batch(g.B) / G * (g.Ho / kStemRows)), 1, n_jobs);
-    conv_stem_rs_rows_kernel<COUT><<<rgrid, G * g.Wo, smem + tile_bytes, s>>>(g, jobs, net_input);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_stem_rs_rows_kernel<COUT>, rgrid, dim3(G * g.Wo), smem + tile_bytes, s, g, jobs, net_input));
   } else if (g.act_format == ACT_RS)
-    conv_stem_rs_kernel<COUT><<<grid, kStemThreads, smem, s>>>(g, jobs, net_input);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_stem_rs_kernel<COUT>, grid, dim3(kStemThreads), smem, s, g, jobs, net_input));
   else if (g.act_format == ACT_SPLIT)
-    conv_stem_kernel<COUT, ACT_SPLIT><<<grid, kStemThreads, smem, s>>>(g, jobs, net_input);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_stem_kernel<COUT, ACT_SPLIT>, grid, dim3(kStemThreads), smem, s, g, jobs, net_input));
   else
-    conv_stem_kernel<COUT, ACT_F32><<<grid, kStemThreads, smem, s>>>(g, jobs, net_input);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_stem_kernel<COUT, ACT_F32>, grid, dim3(kStemThreads), smem, s, g, jobs, net_input));
   AIQ_LAUNCH_CHECK("conv_stem");
   return AIQ_OK;
 }
@@ -602,6 +610,8 @@ avgpool_kernel(const LayerJob* __restrict__ jobs, int H, int W, int C, int Cs) {
   const size_t p0 = ((size_t)b * (H + 2) + 1) * W;       // first interior pixel of image b
   const int ql = threadIdx.x % kPoolQuads, pl = threadIdx.x / kPoolQuads;
   const int c = (blockIdx.y * kPoolQuads + ql) * 4;
+  chain_release();
+  chain_wait();
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   if (c < Cs)
 #pragma unroll 4
@@ -637,10 +647,12 @@ avgpool_rs_kernel(const LayerJob* __restrict__ jobs, int B, int H, int W, int C)
   const size_t px_bytes = (size_t)(C / 4) * plane_bytes;
   const uint8_t* base = static_cast<const uint8_t*>(job.in) + (size_t)grp * H * W * px_bytes + (size_t)img * 16;
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  chain_release();
+  chain_wait();
   if (pl < PL)
     for (int i = pl; i < H * W; i += PL) {
-      const uint4 hv = __ldg(reinterpret_cast<const uint4*>(base + (size_t)i * px_bytes + (size_t)oc * plane_bytes));
-      const uint4 lv = __ldg(reinterpret_cast<const uint4*>(base + (size_t)i * px_bytes + (size_t)(octets + oc) * plane_bytes));
+      const uint4 hv = ld_chain(reinterpret_cast<const uint4*>(base + (size_t)i * px_bytes + (size_t)oc * plane_bytes));
+      const uint4 lv = ld_chain(reinterpret_cast<const uint4*>(base + (size_t)i * px_bytes + (size_t)(octets + oc) * plane_bytes));
       const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, lw[4] = {lv.x, lv.y, lv.z, lv.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
@@ -674,6 +686,8 @@ __global__ void argmax_count_kernel(const LayerJob* __restrict__ jobs, int B, in
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   int correct = 0;
+  chain_release();
+  chain_wait();
   if (b < B) {
     const float* lg = static_cast<const float*>(job.in) + (size_t)b * n_classes;
     float best = -INFINITY;
@@ -732,11 +746,11 @@ aiq_status_t launch_avgpool(const LayerJob* jobs_dev, int n_jobs, int B, int H, 
   LaunchScope scope(AIQ_KERNEL_POOL, s, (double)n_jobs * B * H * W * C,
                     4.0 * n_jobs * B * ((double)H * W * C + C));
   if (act_format == ACT_RS)
-    avgpool_rs_kernel<<<dim3(rs_padded_batch(B) / rs_group_images(W), 1, n_jobs), threads, 0, s>>>(jobs_dev, B, H, W, C);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, avgpool_rs_kernel, dim3(rs_padded_batch(B) / rs_group_images(W), 1, n_jobs), dim3(threads), 0, s, jobs_dev, B, H, W, C));
   else if (act_format == ACT_SPLIT)
-    avgpool_kernel<ACT_SPLIT><<<dim3(B, slabs, n_jobs), threads, 0, s>>>(jobs_dev, H, W, C, padded_channels(C));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, avgpool_kernel<ACT_SPLIT>, dim3(B, slabs, n_jobs), dim3(threads), 0, s, jobs_dev, H, W, C, padded_channels(C)));
   else
-    avgpool_kernel<ACT_F32><<<dim3(B, slabs, n_jobs), threads, 0, s>>>(jobs_dev, H, W, C, padded_channels(C));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, avgpool_kernel<ACT_F32>, dim3(B, slabs, n_jobs), dim3(threads), 0, s, jobs_dev, H, W, C, padded_channels(C)));
   AIQ_LAUNCH_CHECK("avgpool");
   return AIQ_OK;
 }
@@ -746,8 +760,8 @@ aiq_status_t launch_argmax_count(const LayerJob* jobs_dev, int n_jobs, int B, in
                                  long long preds_stride, long long img0, cudaStream_t s) {
   const int warps = 8;
   LaunchScope scope(AIQ_KERNEL_ARGMAX, s, 0.0, 4.0 * n_jobs * B * ((double)n_classes + 2));
-  argmax_count_kernel<<<dim3((B + warps - 1) / warps, 1, n_jobs), warps * 32, 0, s>>>(
-      jobs_dev, B, n_classes, labels, counts, preds, preds_stride, img0);
+  AIQ_CUDA_TRY(launch_chained(scope.chain, argmax_count_kernel, dim3((B + warps - 1) / warps, 1, n_jobs), dim3(warps * 32), 0, s,
+                              jobs_dev, B, n_classes, labels, counts, preds, preds_stride, img0));
   AIQ_LAUNCH_CHECK("argmax_count");
   return AIQ_OK;
 }

@@ -110,10 +110,12 @@ conv_pw_tc_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_const
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   bool alive = true;
+  chain_release();                                 // tensor memory is allocated (see launch_chained)
 
   if (warp == 0) {
     // ---- TMA producer -----------------------------------------------------------------------
     if (lane == 0) {
+      chain_wait();
       uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
       for (int tile = blockIdx.x; tile < n_tiles && alive; tile += gridDim.x) {
         for (int c = 0; c < n_chunks && alive; ++c) {
@@ -280,6 +282,7 @@ conv_pw_tc_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_const
     // 16 output channels (for layers that widen the channels the epilogue is most of the work).
     const int q = warp & 3;
     const int h = warp >= 10 ? 1 : 0;
+    chain_wait();                                      // the residual and the output slot
     int it = 0;
     for (int tile = blockIdx.x; tile < n_tiles && alive; tile += gridDim.x, ++it) {
       const int buf = it & 1;
@@ -304,8 +307,8 @@ conv_pw_tc_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_const
         const int n = n0 + c0;
         uint32_t rh[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rl[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         if (res && n < p.Cs_out) {
-          const uint4 a0 = __ldg(reinterpret_cast<const uint4*>(res + n)), a1 = __ldg(reinterpret_cast<const uint4*>(res + n) + 1);
-          const uint4 l0v = __ldg(reinterpret_cast<const uint4*>(res + p.Cs_out + n)), l1v = __ldg(reinterpret_cast<const uint4*>(res + p.Cs_out + n) + 1);
+          const uint4 a0 = ld_chain(reinterpret_cast<const uint4*>(res + n)), a1 = ld_chain(reinterpret_cast<const uint4*>(res + n) + 1);
+          const uint4 l0v = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out + n)), l1v = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out + n) + 1);
           rh[0] = a0.x; rh[1] = a0.y; rh[2] = a0.z; rh[3] = a0.w; rh[4] = a1.x; rh[5] = a1.y; rh[6] = a1.z; rh[7] = a1.w;
           rl[0] = l0v.x; rl[1] = l0v.y; rl[2] = l0v.z; rl[3] = l0v.w; rl[4] = l1v.x; rl[5] = l1v.y; rl[6] = l1v.z; rl[7] = l1v.w;
         }

@@ -364,6 +364,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   alive = alive && (*s_abort == 0);
+  chain_release();                                   // tensor memory is allocated (see launch_chained)
 
   // rows of the input that carry work: a 1x1 convolution at stride 2 only reads the even ones
   auto row_used = [&](int y) -> bool { return !(KS == 1 && STRIDE == 2 && (y & 1)); };
@@ -371,6 +372,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   // ---- roles ------------------------------------------------------------------------------
   if (warp == 0) {
     if (lane == 0 && alive) {
+      chain_wait();
       uint32_t stage = 0, phase = 0;
       uint32_t issued = 0, issued_phase = 0;
       for (int item = blockIdx.x; item < p.n_items && alive; item += gridDim.x) {
@@ -493,11 +495,12 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     auto load_res = [&](int k, int u, uint4* r) {
       int c0;
       const uint8_t* src = res_base + row_offset(k) + unit_offset(u, &c0);
-      r[0] = __ldg(reinterpret_cast<const uint4*>(src));
-      r[1] = __ldg(reinterpret_cast<const uint4*>(src + plane_bytes));
-      r[2] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)lo_plane0 * plane_bytes));
-      r[3] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(lo_plane0 + 1) * plane_bytes));
+      r[0] = ld_chain(reinterpret_cast<const uint4*>(src));
+      r[1] = ld_chain(reinterpret_cast<const uint4*>(src + plane_bytes));
+      r[2] = ld_chain(reinterpret_cast<const uint4*>(src + (size_t)lo_plane0 * plane_bytes));
+      r[3] = ld_chain(reinterpret_cast<const uint4*>(src + (size_t)(lo_plane0 + 1) * plane_bytes));
     };
+    chain_wait();                                      // the residual and the output slot
     if (res_base && total > 0 && alive) load_res(0, unit0, rres);
     for (int k = 0; k < total && alive; ++k) {
       const int il = k / rows_mine;
@@ -717,6 +720,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   alive = alive && (*s_abort == 0);
+  chain_release();                                     // tensor memory is allocated (see launch_chained)
 
   const int n_my_items = ((int)blockIdx.x < p.n_items) ? (p.n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   const int total = n_my_items * p.H;                  // rows this CTA streams, numbered g = item_local * H + y
@@ -729,6 +733,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
 
   if (warp == 0) {
     if (lane == 0 && alive) {
+      chain_wait();
       uint32_t issued = 0, issued_phase = 0;
       for (int g = 0; g < total && alive; ++g) {
         const int il = g / p.H, y = g - il * p.H;
@@ -809,6 +814,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
       t_col[u] = (second ? 256u : 0u) + (uint32_t)(xt * R * N + c0);
       cell[u] = (uint32_t)uph[u] * (uint32_t)p.a_lbo + (uint32_t)(ux[u] + 1) * 128u + (uint32_t)img * 16u;
     }
+    chain_wait();                                      // the output slot
     for (int g = h; g < total && alive; g += 2) {
       const int il = g / p.H, y = g - il * p.H;
       const int slot = g & (R - 1);
@@ -1030,7 +1036,8 @@ aiq_status_t launch_rs(const ConvGeom& g, const RsShape& sh, const CUtensorMap* 
                       2.0 * g.B * g.Ho * g.Wo * g.Cout * (double)(g.ks * g.ks * g.Cin) * n_jobs,
                       weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                      (pool_jobs ? 0.0 : (double)g.B * g.Ho * g.Wo * g.Cout)));
-    conv_rs_kernel<C, KS, STRIDE, PIECES><<<dim3(ctas, n_jobs, c.slices), c.threads, c.smem_bytes, s>>>(maps[0], maps[1], p, jobs_dev);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_rs_kernel<C, KS, STRIDE, PIECES>, dim3(ctas, n_jobs, c.slices), dim3(c.threads), c.smem_bytes, s,
+                                maps[0], maps[1], p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("conv_rs");
   return AIQ_OK;
@@ -1073,7 +1080,7 @@ aiq_status_t launch_rb(const ConvGeom& g, const CUtensorMap* map, const LayerJob
   {
     const double px = (double)g.B * g.H * g.W * C;
     LaunchScope scope(AIQ_KERNEL_CONV_TC, s, 2.0 * 2.0 * px * (9.0 * C) * n_jobs, weight_bytes + 4.0 * n_jobs * 2.0 * px);
-    conv_rs_block_kernel<C><<<dim3(ctas, n_jobs), kRbThreads, smem_bytes, s>>>(map[0], p, jobs_dev);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_rs_block_kernel<C>, dim3(ctas, n_jobs), dim3(kRbThreads), smem_bytes, s, map[0], p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("conv_rs_block");
   return AIQ_OK;

@@ -226,10 +226,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, TcParams p, const Lay
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
   alive = alive && (*s_abort == 0);            // the same answer in every thread
+  chain_release();                             // tensor memory is allocated (see launch_chained)
 
   // ---- roles ------------------------------------------------------------------------------
   if (warp == 0) {
     if (lane == 0 && alive) {
+      chain_wait();
       uint32_t stage = 0, phase = 0;
       uint32_t issued = 0, issued_phase = 0;       // per stage: a load was issued / parity of the last one
       for (int tile = blockIdx.x; tile < n_tiles && alive; tile += gridDim.x) {
@@ -421,11 +423,12 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, TcParams p, const Lay
 #pragma unroll
         for (int k = 0; k < RPL; ++k) {
           const int u = lane + 32 * k;
-          rpre[ii][k] = (jr >= 0 && u < 8 * UNITS) ? __ldg(reinterpret_cast<const uint4*>(src + unit_off(u)))
+          rpre[ii][k] = (jr >= 0 && u < 8 * UNITS) ? ld_chain(reinterpret_cast<const uint4*>(src + unit_off(u)))
                                                    : make_uint4(0u, 0u, 0u, 0u);
         }
       }
     };
+    chain_wait();                                  // the residual and the output slot
     if (job.res && (int)blockIdx.x < n_tiles && alive) fetch_residual(blockIdx.x);
     int it = 0;
     for (int tile = blockIdx.x; tile < n_tiles && alive; tile += gridDim.x, ++it) {
@@ -630,7 +633,8 @@ aiq_status_t launch_tc(const ConvGeom& g, const CUtensorMap& map, const LayerJob
                       2.0 * g.B * g.Ho * g.Wo * g.Cout * (double)(g.ks * g.ks * g.Cin) * n_jobs,
                       weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                      (double)g.B * g.Ho * g.Wo * g.Cout));
-    conv_tc_kernel<CS, N, KS, STRIDE, PIECES><<<dim3(ctas, n_jobs, slices), tc_threads(N), smem_bytes, s>>>(map, p, jobs_dev);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_tc_kernel<CS, N, KS, STRIDE, PIECES>, dim3(ctas, n_jobs, slices), dim3(tc_threads(N)), smem_bytes, s,
+                                map, p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("conv_tc");
   return AIQ_OK;
@@ -731,7 +735,7 @@ aiq_status_t launch_conv_pw_tc(const ConvGeom& g, const void* map, const void* o
   {
     LaunchScope scope(AIQ_KERNEL_CONV_TC, s, 2.0 * g.B * g.Ho * g.Wo * g.Cout * (double)g.Cin * n_jobs,
                       weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W + (double)g.B * g.Ho * g.Wo * g.Cout));
-    conv_pw_tc_kernel<<<dim3(ctas, n_jobs * p.n_ntiles), kPwThreads, smem_bytes, s>>>(m, mo, p, jobs_dev);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_pw_tc_kernel, dim3(ctas, n_jobs * p.n_ntiles), dim3(kPwThreads), smem_bytes, s, m, mo, p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("conv_pw_tc");
   return AIQ_OK;

@@ -84,11 +84,11 @@ __device__ __forceinline__ void read4(const uint8_t* p, int Cb, uint64_t* v) {
 
 // The same four channels of a pixel in global memory (lo_off: bytes from the hi to the lo half).
 template <int FMT>
-__device__ __forceinline__ void load4(const uint8_t* __restrict__ p, uint32_t lo_off, uint64_t* v) {
+__device__ __forceinline__ void load4(const uint8_t* p, uint32_t lo_off, uint64_t* v) {
   if (FMT == ACT_SPLIT) {
-    join4(__ldg(reinterpret_cast<const uint2*>(p)), __ldg(reinterpret_cast<const uint2*>(p + lo_off)), v);
+    join4(ld_chain(reinterpret_cast<const uint2*>(p)), ld_chain(reinterpret_cast<const uint2*>(p + lo_off)), v);
   } else {
-    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    const float4 t = ld_chain(reinterpret_cast<const float4*>(p));
     v[0] = pack2(t.x, t.y); v[1] = pack2(t.z, t.w);
   }
 }
@@ -143,10 +143,12 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  chain_release();
 
   if (tid >= n_compute) {
     // ---- producer: padded input rows oy0 * STRIDE .. of every unit of this block, in order -----------
     if (lane == 0) {
+      chain_wait();
       bool alive = true;
       uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
       for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
@@ -219,6 +221,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     bi[0] = pack2(b4[0], b4[1]); bi[1] = pack2(b4[2], b4[3]);
   }
 
+  chain_wait();                                          // the output slot may still be read by an earlier kernel
   constexpr int IN_COLS = (COLS - 1) * STRIDE + 3;
   const uint8_t* my_cols = ring + (size_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
                            (size_t)q * (FMT == ACT_SPLIT ? 8 : 16);
@@ -441,7 +444,7 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
 #define AIQ_DW(FMT_, ST_, COLS_)                                                                       \
   do {                                                                                                 \
     AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_>), per_cta);                          \
-    depthwise3x3_kernel<FMT_, ST_, COLS_><<<grid, threads, smem, s>>>(m, p, jobs_dev);                  \
+    AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<FMT_, ST_, COLS_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
   } while (0)
   if (g.act_format == ACT_SPLIT) { if (g.stride == 1) AIQ_DW(ACT_SPLIT, 1, kDwCols); else AIQ_DW(ACT_SPLIT, 2, kDwCols); }
   else { if (g.stride == 1) AIQ_DW(ACT_F32, 1, kDwCols); else AIQ_DW(ACT_F32, 2, kDwCols); }

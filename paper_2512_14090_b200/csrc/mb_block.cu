@@ -178,6 +178,7 @@ mb_block_kernel(MbParams p, const LayerJob* __restrict__ jobs) {
     tmem_alloc(smem_u32(s_tmem), (uint32_t)p.tmem_cols);
     tmem_relinquish();
   }
+  chain_wait();
   // input pixels of the band -> canonical planes, asynchronously (the border rows above / below an
   // image are stored in the tensor, so the run [pix0, pix0 + Ph) always exists)
   {
@@ -257,6 +258,7 @@ mb_block_kernel(MbParams p, const LayerJob* __restrict__ jobs) {
   __syncthreads();                                   // barriers initialised, band in place, tensor memory allocated
   tc_fence_after();
   const uint32_t tmem_base = *s_tmem;
+  chain_release();                                   // tensor memory is allocated (see launch_chained)
   if (tid == kMbLeader) {
     load_expand(0);
     load_coef(0);
@@ -438,8 +440,8 @@ mb_block_kernel(MbParams p, const LayerJob* __restrict__ jobs) {
       const int n = cg * 16;
       uint32_t rh[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rl[8] = {0, 0, 0, 0, 0, 0, 0, 0};
       if (res) {
-        const uint4 a0 = __ldg(reinterpret_cast<const uint4*>(res + n)), a1 = __ldg(reinterpret_cast<const uint4*>(res + n) + 1);
-        const uint4 l0 = __ldg(reinterpret_cast<const uint4*>(res + p.Cs_out + n)), l1 = __ldg(reinterpret_cast<const uint4*>(res + p.Cs_out + n) + 1);
+        const uint4 a0 = ld_chain(reinterpret_cast<const uint4*>(res + n)), a1 = ld_chain(reinterpret_cast<const uint4*>(res + n) + 1);
+        const uint4 l0 = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out + n)), l1 = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out + n) + 1);
         rh[0] = a0.x; rh[1] = a0.y; rh[2] = a0.z; rh[3] = a0.w; rh[4] = a1.x; rh[5] = a1.y; rh[6] = a1.z; rh[7] = a1.w;
         rl[0] = l0.x; rl[1] = l0.y; rl[2] = l0.z; rl[3] = l0.w; rl[4] = l1.x; rl[5] = l1.y; rl[6] = l1.z; rl[7] = l1.w;
       }
@@ -631,7 +633,7 @@ aiq_status_t launch_mb_block(const ConvGeom& ge, const ConvGeom& gd, const ConvG
     LaunchScope scope(AIQ_KERNEL_CONV_TC, s,
                       n_jobs * (2.0 * px_in * ge.Cin * ge.Cout + 2.0 * px_out * 9.0 * gd.Cout + 2.0 * px_out * gp.Cin * gp.Cout),
                       weight_bytes + 4.0 * n_jobs * (px_in * ge.Cin + px_out * gp.Cout));
-    mb_block_kernel<<<dim3((unsigned)(ge.B * c.bands), (unsigned)n_jobs), kMbThreads, c.smem_bytes, s>>>(p, jobs_dev);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, mb_block_kernel, dim3((unsigned)(ge.B * c.bands), (unsigned)n_jobs), dim3(kMbThreads), c.smem_bytes, s, p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("mb_block");
   return AIQ_OK;

@@ -59,11 +59,13 @@ qlinear_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K,
   const int warp = threadIdx.x >> 5;
   const int n0 = (blockIdx.x * kWarps + warp) * kRowsPerWarp;
   const int m0 = blockIdx.y * MT;
+  chain_release();
+  chain_wait();
   if (n0 >= N) return;
   const int Kpad = (K + 31) / 32 * 32;
   const size_t rb = (size_t)Kpad * BITS / 8;
   const int n_chunks = Kpad / E;
-  const float* __restrict__ x = static_cast<const float*>(job.in);
+  const float* x = static_cast<const float*>(job.in);
   const bool xvec = ((K & 3) == 0) && ((((uintptr_t)x) & 15) == 0);
 
   float acc[kRowsPerWarp][MT];
@@ -91,12 +93,12 @@ qlinear_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K,
         if (xvec && k0 + SE <= K) {
 #pragma unroll
           for (int v = 0; v < SE / 4; ++v) {
-            const float4 t = __ldg(reinterpret_cast<const float4*>(xp) + v);
+            const float4 t = ld_chain(reinterpret_cast<const float4*>(xp) + v);
             xv[m][4 * v] = t.x; xv[m][4 * v + 1] = t.y; xv[m][4 * v + 2] = t.z; xv[m][4 * v + 3] = t.w;
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < SE; ++j) xv[m][j] = (k0 + j < K) ? __ldg(xp + j) : 0.0f;
+          for (int j = 0; j < SE; ++j) xv[m][j] = (k0 + j < K) ? ld_chain(xp + j) : 0.0f;
         }
       }
 #pragma unroll
@@ -146,11 +148,11 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
   LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K * n_jobs,
                     n_jobs * ((double)N * row_bytes(K, BITS) + 4.0 * N + 4.0 * M * ((double)K + N)));
   if (M == 1) {
-    qlinear_kernel<BITS, 1><<<dim3(gx, 1, n_jobs), kWarps * 32, 0, s>>>(single, jobs_dev, N, K, M);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 1>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
   } else if (M == 2) {
-    qlinear_kernel<BITS, 2><<<dim3(gx, 1, n_jobs), kWarps * 32, 0, s>>>(single, jobs_dev, N, K, M);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 2>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
   } else {
-    qlinear_kernel<BITS, 4><<<dim3(gx, (M + 3) / 4, n_jobs), kWarps * 32, 0, s>>>(single, jobs_dev, N, K, M);
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 4>, dim3(gx, (M + 3) / 4, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
   }
   AIQ_LAUNCH_CHECK("qlinear");
   return AIQ_OK;

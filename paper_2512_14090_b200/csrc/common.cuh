@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <string.h>
 
 #include <atomic>
 
@@ -36,6 +37,30 @@ void count_launch();                         // per-thread launch counter (aiq_l
 // Properties of the current device (looked up once per device, then cached).
 struct DeviceProps { int dev, n_sms, smem_optin; };
 aiq_status_t current_device_props(DeviceProps* out);
+
+// Launch shapes are pure functions of a few sizes but cost microseconds to search, for each of 50 layers of a pass;
+// every thread keeps the last ones it computed (direct-mapped, 256 entries, a collision recomputes).
+// compute(Value*) -> bool; the value is kept only when it returns true.
+template <typename Value, int N>
+struct ConfigMemo {
+  struct Entry { int key[N]; bool used; Value value; };
+  template <typename F>
+  bool get(const int (&key)[N], Value* out, F compute) {
+    uint32_t h = 2166136261u;
+    for (int i = 0; i < N; ++i) h = (h ^ (uint32_t)key[i]) * 16777619u;
+    Entry& e = entries[(h ^ (h >> 15)) & 255u];
+    if (!e.used || memcmp(e.key, key, sizeof(key)) != 0) {
+      if (!compute(out)) return false;
+      memcpy(e.key, key, sizeof(key));
+      e.value = *out;
+      e.used = true;
+      return true;
+    }
+    *out = e.value;
+    return true;
+  }
+  Entry entries[256] = {};
+};
 
 // Opt-in of `kernel` to `bytes` of dynamic shared memory.  The attribute belongs to the
 // (kernel, device) pair, so the record of what has been set is kept per device; it is only

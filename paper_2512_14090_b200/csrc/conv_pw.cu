@@ -372,7 +372,7 @@ EncodeTiledFn pr_encode_fn() {
 // (about 12 clocks per channel); a block adds a set-up that grows with the weights it expands.  Blocks fill the GPU in
 // waves.
 struct PrConfig { int Nt, ew, stages, bufs, splits, tiles_per_cta, smem; };
-bool pr_config(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
+bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
   const int n_tiles = (g.B * (g.H + 2) * g.W + 127) / 128;
   const double K2 = 2.0 * g.Cs_in;
   double best = 1e300;
@@ -414,6 +414,12 @@ bool pr_config(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
     if (Nt == g.Cs_out) break;
   }
   return best < 1e300;
+}
+
+bool pr_config(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
+  static thread_local ConfigMemo<PrConfig, 8> memo;
+  const int key[8] = {g.B, g.H, g.W, g.Cs_in, g.Cs_out, n_jobs, pieces, props.dev};
+  return memo.get(key, out, [&](PrConfig* c) { return pr_search(g, n_jobs, pieces, props, c); });
 }
 
 template <int EW, int PIECES>

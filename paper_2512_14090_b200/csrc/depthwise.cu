@@ -7,8 +7,9 @@
 //     the map are filled with zeros, rows outside it are the physical padding rows of the tensor),
 //     so the loads in flight do not depend on how many warps are resident;
 //   - a thread owns 4 consecutive channels and COLS consecutive output columns of one image and walks
-//     down the rows: each input row feeds the (up to three) output rows it belongs to, an input value is
-//     unpacked once per thread, and the 36 weights stay in registers (a block keeps its channel slab);
+//     down the rows: each input row feeds the (up to three) output rows it belongs to, and an input value is
+//     unpacked once per thread.  A block keeps its channel slab, whose expanded weights, scales and biases
+//     sit in shared memory (beside three rows of accumulators they do not fit the registers);
 //   - products are packed float32 pairs (two lanes per instruction).
 // The kernels this one replaced loaded their inputs from global memory in each thread (one row per
 // thread, or rows walked by a thread): 43 instructions per element and the loads of three blocks in
@@ -24,9 +25,9 @@ namespace aiq {
 
 namespace {
 
-constexpr int kDwThreads = 256;                     // compute threads at most; one more warp issues the copies
+constexpr int kDwThreads = 224;                     // compute threads at most; one more warp issues the copies: eight warps
+                                                    // per block, so that two blocks per SM have 128 registers a thread
 constexpr int kDwMaxStages = 8;
-constexpr int kDwCols = 2;                          // output columns per thread
 constexpr int kDwMaxColGroups = 56;                 // column groups of a block: its input box stays within 256 columns
 
 struct DwParams {
@@ -55,6 +56,11 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
@@ -120,8 +126,10 @@ __device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int u) {
   return d;
 }
 
-// COLS output columns per thread: 2 (four output columns save a third of the unpacking at stride 1, but
-// three rows of accumulators beside the weights then spill at two blocks per SM).
+// COLS output columns per thread: 4 at stride 1 (small launches: 2, see dw_search_shape), 2 at stride 2.  What bounds the kernel is instructions: with two
+// columns a row cost 37 per output element at 0.46 issued per clock and scheduler (2.9 TB/s at 256 x 32 x 32 x 144
+// channels); four columns share six unpacked input columns (1.5 per output instead of 2), the per-row waiting and
+// the addresses.
 template <int FMT, int STRIDE, int COLS>
 __global__ void __launch_bounds__(kDwThreads + 32, 2)
 depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, const LayerJob* __restrict__ jobs) {
@@ -133,7 +141,30 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   uint64_t* bars = reinterpret_cast<uint64_t*>(ring + p.stages * p.stage_bytes);
   const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kDwMaxStages;
   volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * kDwMaxStages);
+  float* s_w = reinterpret_cast<float*>(ring + p.stages * p.stage_bytes + (2 * kDwMaxStages + 2) * 8);   // [9 taps, scale, bias][Cb]
+  const int slab = (int)blockIdx.x % p.n_slabs;          // the grid is a multiple of the slabs: fixed for this block
 
+  // expanded weights: a thread per channel of the slab
+  for (int i = tid; i < p.Cb; i += (int)blockDim.x) {
+    const int c = slab * p.Cb + i;
+    const bool real = c < p.C;                           // padding channels: zero weights, scale and bias
+    const uint8_t* row = job.w + (size_t)(real ? c : 0) * (32 * job.bits / 8);   // K = 9 pads to 32 elements
+    uint4 r0 = __ldg(reinterpret_cast<const uint4*>(row)), r1 = r0, r2 = r0;
+    if (job.bits >= 16) r1 = __ldg(reinterpret_cast<const uint4*>(row) + 1);
+    if (job.bits == 32) r2 = __ldg(reinterpret_cast<const uint4*>(row) + 2);
+    const uint32_t words[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      float v;
+      if (job.bits == 4) v = (float)((int)(((words[k >> 3] >> (4 * (k & 7))) & 0xFu) ^ 8u) - 8);
+      else if (job.bits == 8) v = (float)(int)(int8_t)((words[k >> 2] >> (8 * (k & 3))) & 0xFFu);
+      else if (job.bits == 16) v = __half2float(__ushort_as_half((unsigned short)((words[k >> 1] >> (16 * (k & 1))) & 0xFFFFu)));
+      else v = __uint_as_float(words[k]);
+      s_w[k * p.Cb + i] = real ? v : 0.f;
+    }
+    s_w[9 * p.Cb + i] = real ? __ldg(job.scale + c) : 0.f;
+    s_w[10 * p.Cb + i] = real ? __ldg(job.bias + c) : 0.f;
+  }
   if (tid == 0) {
     for (int i = 0; i < p.stages; ++i) {
       mbar_init(bar_full + 8 * i, 1);
@@ -181,7 +212,6 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   // ---- compute: thread = (image of the group, column group, channel quad), quad fastest ---------------
   const int q = tid % p.CQ, xg = (tid / p.CQ) % p.XG, ni = tid / (p.CQ * p.XG);
   const bool worker = ni < p.NI;                         // the last warp may have idle lanes
-  const int slab = (int)blockIdx.x % p.n_slabs;          // the grid is a multiple of the slabs: fixed for this block
   const int c = slab * p.Cb + q * 4;
   const size_t pix_bytes = (size_t)4 * p.Cs;             // [hi(Cs) | lo(Cs)] bfloat16 or Cs floats
   const uint32_t lo_off = 2u * p.Cs;
@@ -191,42 +221,17 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   const bool clamp = p.act != AIQ_ACT_NONE;              // relu: [0, inf), relu6: [0, 6]
   const float act_hi = p.act == AIQ_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
 
-  uint64_t w[9][2], sc[2], bi[2];                        // weights, scale and bias of the four channels
-  {
-    float t[9][4], s4[4], b4[4];
-    const int wrow_bytes = 32 * job.bits / 8;            // K = 9 pads to 32 elements
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const bool real = worker && c + i < p.C;           // padding channels: zero weights, scale and bias
-      const uint8_t* row = job.w + (size_t)(real ? c + i : 0) * wrow_bytes;
-      uint4 r0 = __ldg(reinterpret_cast<const uint4*>(row)), r1 = r0, r2 = r0;
-      if (job.bits >= 16) r1 = __ldg(reinterpret_cast<const uint4*>(row) + 1);
-      if (job.bits == 32) r2 = __ldg(reinterpret_cast<const uint4*>(row) + 2);
-      const uint32_t words[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
-#pragma unroll
-      for (int k = 0; k < 9; ++k) {
-        float v;
-        if (job.bits == 4) v = (float)((int)(((words[k >> 3] >> (4 * (k & 7))) & 0xFu) ^ 8u) - 8);
-        else if (job.bits == 8) v = (float)(int)(int8_t)((words[k >> 2] >> (8 * (k & 3))) & 0xFFu);
-        else if (job.bits == 16) v = __half2float(__ushort_as_half((unsigned short)((words[k >> 1] >> (16 * (k & 1))) & 0xFFFFu)));
-        else v = __uint_as_float(words[k]);
-        t[k][i] = real ? v : 0.f;
-      }
-      s4[i] = real ? __ldg(job.scale + c + i) : 0.f;
-      b4[i] = real ? __ldg(job.bias + c + i) : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 9; ++k) { w[k][0] = pack2(t[k][0], t[k][1]); w[k][1] = pack2(t[k][2], t[k][3]); }
-    sc[0] = pack2(s4[0], s4[1]); sc[1] = pack2(s4[2], s4[3]);
-    bi[0] = pack2(b4[0], b4[1]); bi[1] = pack2(b4[2], b4[3]);
-  }
-
   chain_wait();                                          // the output slot may still be read by an earlier kernel
   constexpr int IN_COLS = (COLS - 1) * STRIDE + 3;
   const uint8_t* my_cols = ring + (size_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
                            (size_t)q * (FMT == ACT_SPLIT ? 8 : 16);
   uint32_t stage = 0, phase = 0;
   bool alive = true;
+  const float* my_w = s_w + q * 4;
+  auto coef = [&](int k, uint64_t (&v)[2]) {             // the four channels of row k of s_w
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my_w + k * p.Cb);
+    v[0] = t.x; v[1] = t.y;
+  };
   // The next padded row: wait, accumulate it as tap row RA into `a`, RB into `b` and RC into `cc` (-1: not
   // at all; the first contribution to `cc` is written, not added) and hand the stage back.
   auto row = [&](auto ra, auto rb_, auto rc, uint64_t (&a)[COLS][2], uint64_t (&b)[COLS][2], uint64_t (&cc)[COLS][2]) -> bool {
@@ -234,23 +239,33 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     alive = mbar_wait_warp(bar_full + 8 * stage, phase, s_abort, p.error_flag);
     if (!alive) return false;
     const uint8_t* src = my_cols + stage * p.stage_bytes;
+    uint64_t v[IN_COLS][2];
 #pragma unroll
-    for (int xx = 0; xx < IN_COLS; ++xx) {
-      uint64_t v[2];
-      read4<FMT>(src + xx * col_bytes, p.Cb, v);
+    for (int xx = 0; xx < IN_COLS; ++xx) read4<FMT>(src + xx * col_bytes, p.Cb, v[xx]);
+    auto tap_row = [&](auto r_, auto fresh, uint64_t (&s)[COLS][2]) {
+      constexpr int R = decltype(r_)::value;
+      constexpr bool FRESH = decltype(fresh)::value;
 #pragma unroll
       for (int t = 0; t < 3; ++t) {
-        if ((xx - t) % STRIDE != 0 || xx < t || (xx - t) / STRIDE >= COLS) continue;
-        const int x = (xx - t) / STRIDE;
+        uint64_t w[2];
+        coef(R * 3 + t, w);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          if (RA >= 0) a[x][i] = fma2(v[i], w[(RA < 0 ? 0 : RA) * 3 + t][i], a[x][i]);
-          if (RB >= 0) b[x][i] = fma2(v[i], w[(RB < 0 ? 0 : RB) * 3 + t][i], b[x][i]);
-          if (RC >= 0) cc[x][i] = fma2(v[i], w[(RC < 0 ? 0 : RC) * 3 + t][i], t == 0 ? 0ull : cc[x][i]);
-        }
+        for (int x = 0; x < COLS; ++x)
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            s[x][i] = FRESH && t == 0 ? mul2(v[x * STRIDE + t][i], w[i]) : fma2(v[x * STRIDE + t][i], w[i], s[x][i]);
       }
+    };
+    if constexpr (RA >= 0) tap_row(ra, std::false_type(), a);
+    if constexpr (RB >= 0) tap_row(rb_, std::false_type(), b);
+    if constexpr (RC >= 0) tap_row(rc, std::true_type(), cc);
+    // The stage is handed back once its words have been used, not merely loaded: the accumulators of this row (every
+    // input column enters one of them) are operands of the empty statement before the arrival.
+#pragma unroll
+    for (int x = 0; x < COLS; ++x) {
+      if (RA >= 0) asm volatile("" ::"l"(a[x][0]), "l"(a[x][1]) : "memory");
+      else asm volatile("" ::"l"(cc[x][0]), "l"(cc[x][1]) : "memory");
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the reads above before the next copy's writes
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_empty + 8 * stage);
     if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
@@ -270,6 +285,9 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     // finish and store the next output row (rows are emitted in order) from its accumulators
     auto emit = [&](const uint64_t (&acc)[COLS][2]) {
       if (writes) {
+        uint64_t sc[2], bi[2];
+        coef(9, sc);
+        coef(10, bi);
 #pragma unroll
         for (int x = 0; x < COLS; ++x) {
           if (ox + x >= p.Wo) break;
@@ -355,22 +373,42 @@ EncodeTiledFn dw_encode_fn() {
 
 // The part of the launch shape the tensor map depends on: slab width, column groups, images of a stage.
 struct DwShape { int cols, Cb, XG, NI, Wb; };
-DwShape dw_shape(const ConvGeom& g, int batch_capacity) {
+DwShape dw_search_shape(const ConvGeom& g, int batch_capacity) {
   DwShape s = {};
-  s.cols = kDwCols;
+  // Four columns per thread at stride 1 where that gives every resident thread a row, else two: a small launch is
+  // bound by the chain of one row after the other, and half as many outputs per thread make a shorter one
+  // (MobileNetV2-CIFAR, one image: 341 us per pass with four columns, 318 with two).
+  s.cols = g.stride == 1 && (long long)batch_capacity * g.Ho * g.Wo * g.Cs_out >= 16ll * 65536 ? 4 : 2;
   const int xg = (g.Wo + s.cols - 1) / s.cols;
-  // the widest slab that divides the padded channels (wide slabs: long contiguous runs of the tensor), but
-  // narrower ones where a row of the map then fits one block, down to 32 channels
-  s.Cb = 16;
-  for (int cb : {32, 48, 64})
-    if (g.Cs_out % cb == 0 && (s.Cb < 32 || (cb / 4) * xg <= kDwThreads)) s.Cb = cb;
-  s.XG = std::min(xg, std::min(kDwMaxColGroups, kDwThreads / (s.Cb / 4)));
-  s.XG = (xg + (xg + s.XG - 1) / s.XG - 1) / ((xg + s.XG - 1) / s.XG);    // column tiles of equal width
-  // narrow maps: several images side by side fill the block (8 at most)
-  s.NI = std::max(1, std::min(std::min(8, batch_capacity), kDwThreads / (s.Cb / 4 * s.XG)));
+  // the slab width that keeps most of the threads on output columns that exist (ties: the widest, for long
+  // contiguous runs of the tensor); narrow maps put several images side by side, 8 at most
+  double best = 0.0;
+  for (int cb = 16; cb <= 256 && cb <= g.Cs_out; cb += 16) {
+    if (g.Cs_out % cb != 0 || cb / 4 > kDwThreads) continue;
+    int w = std::min(xg, std::min(kDwMaxColGroups, kDwThreads / (cb / 4)));
+    const int tiles = (xg + w - 1) / w;
+    w = (xg + tiles - 1) / tiles;                              // column tiles of equal width
+    const int ni = std::max(1, std::min(std::min(8, batch_capacity), kDwThreads / (cb / 4 * w)));
+    const int wb = (w * s.cols - 1) * g.stride + 3;
+    if (ni * wb * cb * 4 > 24 * 1024) continue;                // four rows in flight at two blocks per SM
+    // (a 16-channel slab reads and writes runs of 32 bytes, a 32-channel one of 64)
+    const double used = (double)(cb / 4) * w * ni * g.Wo / (tiles * w * s.cols) * (cb == 16 ? 0.75 : cb == 32 ? 0.9 : 1.0) *
+                        batch_capacity / ((batch_capacity + ni - 1) / ni * ni);
+    if (used >= best) { best = used; s.Cb = cb; s.XG = w; s.NI = ni; }
+  }
   s.Wb = (s.XG * s.cols - 1) * g.stride + 3;
   return s;
 }
+DwShape dw_shape(const ConvGeom& g, int batch_capacity) {
+  static thread_local ConfigMemo<DwShape, 5> memo;
+  const int key[5] = {g.Cs_out, g.Ho, g.Wo, g.stride, batch_capacity};
+  DwShape s;
+  memo.get(key, &s, [&](DwShape* out) { *out = dw_search_shape(g, batch_capacity); return true; });
+  return s;
+}
+
+// Rows of a block and blocks per slab (see launch_depthwise).
+struct DwSplit { int rb, n_rb, k; };
 
 }  // namespace
 
@@ -412,30 +450,45 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
   const int threads = (p.CQ * p.XG * p.NI + 31) / 32 * 32 + 32;
   // two blocks per SM, each with as many rows in flight as fit (at most 8)
   const int per_cta = (props.smem_optin + 1024) / 2 - 1024;
-  const int fixed = 128 + (2 * kDwMaxStages + 1) * 8;
+  const int fixed = 128 + (2 * kDwMaxStages + 2) * 8 + 11 * sh.Cb * 4;
   p.stages = std::min(kDwMaxStages, (per_cta - fixed) / p.stage_bytes);
   if (p.stages < 2) return set_error(AIQ_ERR_SHAPE, "depthwise: %d bytes per input row do not fit shared memory", p.stage_bytes);
-  const int smem = p.stages * p.stage_bytes + fixed;
-  // Row blocks: whole images where they fill the GPU (no halo rows read twice), else blocks of rows, down to
-  // two, until every SM has work.
-  const long long columns = (long long)p.n_ig * p.n_ct * p.n_slabs * n_jobs;
-  const int want = (int)std::min<long long>((2ll * props.n_sms + columns - 1) / columns, (g.Ho + 1) / 2);
-  p.rb = (g.Ho + std::max(want, 1) - 1) / std::max(want, 1);
-  p.n_rb = (g.Ho + p.rb - 1) / p.rb;
-  p.n_units = p.n_ig * p.n_rb * p.n_ct * p.n_slabs;
-  // Blocks: a multiple of the slabs (a block then keeps its weights in registers).  The number is the one
-  // whose last wave is fullest, counted in units plus a start-up of about two units per block.
+  // Row blocks and blocks per slab (the grid is a multiple of the slabs: a block then keeps its weights), chosen
+  // together: cost of a wave = input rows its blocks walk, halo rows included, and a start-up of about six rows;
+  // cutting images into row blocks pays where whole images would leave the last wave nearly empty (at 256 x 32 x 32 x
+  // 144 channels 192 of 296 resident blocks had work, each for two images) or are fewer than the blocks.
   const int resident = 2 * props.n_sms;
-  const int per_slab = p.n_units / p.n_slabs;
-  int best_k = 1;
-  double best = 1e300;
-  for (int k = 1; k <= per_slab; ++k) {
-    const long long ctas = (long long)k * p.n_slabs * n_jobs;
-    const double waves = (double)((ctas + resident - 1) / resident);
-    const double cost = waves * ((per_slab + k - 1) / k + 2.0 / (p.rb * g.stride + 2));
-    if (cost < best * 0.999) { best = cost; best_k = k; }
-    if (ctas > 16ll * resident) break;
-  }
+  const long long columns = (long long)p.n_ig * p.n_ct;        // units per slab and row block
+  static thread_local ConfigMemo<DwSplit, 8> memo;
+  const int key[8] = {g.Ho, g.stride, p.n_ig, p.n_ct, p.n_slabs, n_jobs, resident, 0};
+  DwSplit split;
+  memo.get(key, &split, [&](DwSplit* out) {
+    *out = {g.Ho, 1, 1};
+    double best = 1e300;
+    for (int n = 1; n <= g.Ho; n = n < 4 ? n + 1 : n + n / 2) {
+      const int rb = (g.Ho + n - 1) / n, n_rb = (g.Ho + rb - 1) / rb;
+      const long long per_slab = columns * n_rb;
+      const double rows = (rb - 1) * g.stride + 3;
+      for (int w = 1; w <= 5; ++w) {
+        long long k = w == 5 ? per_slab : (long long)w * resident / ((long long)p.n_slabs * n_jobs);
+        k = std::max(1ll, std::min(k, per_slab));
+        const long long each = (per_slab + k - 1) / k;
+        k = (per_slab + each - 1) / each;
+        const long long ctas = k * p.n_slabs * n_jobs;
+        const double cost = (double)((ctas + resident - 1) / resident) * (each * rows + 6.0);
+        if (cost < best * 0.999 && k * p.n_slabs < (1ll << 30)) { best = cost; *out = {rb, n_rb, (int)k}; }
+        if (k == per_slab) break;
+      }
+    }
+    return true;
+  });
+  p.rb = split.rb; p.n_rb = split.n_rb;
+  const int best_k = split.k;
+  p.n_units = p.n_ig * p.n_rb * p.n_ct * p.n_slabs;
+  // no more stages than rows a block walks (small launches: what is left of the SM is the next kernel's)
+  const long long block_rows = (long long)((p.n_units / p.n_slabs + best_k - 1) / best_k) * ((p.rb - 1) * g.stride + 3);
+  p.stages = (int)std::min<long long>(p.stages, std::max(2ll, block_rows));
+  const int smem = p.stages * p.stage_bytes + fixed;
   const dim3 grid((unsigned)(best_k * p.n_slabs), n_jobs);
   LaunchScope scope(AIQ_KERNEL_DEPTHWISE, s, 18.0 * g.B * g.Ho * g.Wo * g.Cout * n_jobs,
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
@@ -446,8 +499,11 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
     AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_>), per_cta);                          \
     AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<FMT_, ST_, COLS_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
   } while (0)
-  if (g.act_format == ACT_SPLIT) { if (g.stride == 1) AIQ_DW(ACT_SPLIT, 1, kDwCols); else AIQ_DW(ACT_SPLIT, 2, kDwCols); }
-  else { if (g.stride == 1) AIQ_DW(ACT_F32, 1, kDwCols); else AIQ_DW(ACT_F32, 2, kDwCols); }
+  if (g.act_format == ACT_SPLIT) {
+    if (g.stride == 2) AIQ_DW(ACT_SPLIT, 2, 2); else if (sh.cols == 4) AIQ_DW(ACT_SPLIT, 1, 4); else AIQ_DW(ACT_SPLIT, 1, 2);
+  } else {
+    if (g.stride == 2) AIQ_DW(ACT_F32, 2, 2); else if (sh.cols == 4) AIQ_DW(ACT_F32, 1, 4); else AIQ_DW(ACT_F32, 1, 2);
+  }
 #undef AIQ_DW
   AIQ_LAUNCH_CHECK("depthwise3x3");
   return AIQ_OK;

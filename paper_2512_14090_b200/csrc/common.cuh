@@ -279,24 +279,13 @@ aiq_status_t launch_mb_block(const ConvGeom& ge, const ConvGeom& gd, const ConvG
 bool conv_rs_block_eligible(const ConvGeom& g);
 aiq_status_t launch_conv_rs_block(const ConvGeom& g, const void* maps, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
                                   int32_t* error_flag, double weight_bytes, cudaStream_t s);
-// Pointwise (1x1, stride 1) tensor-core convolution with resident weights (conv_pw.cu), wherever the weights of 32
-// output channels fit shared memory.  `maps`: two CUtensorMaps (256 bytes), over the input and the output slot.
+// Pointwise (1x1, stride 1) tensor-core convolution for any channel count that is a multiple of 8, 16 at least
+// (conv_pw.cu).  `maps`: two CUtensorMaps (256 bytes), over the input and the output slot.
 bool conv_pw_eligible(const ConvGeom& g);
 aiq_status_t conv_pw_encode_maps(const ConvGeom& g, const void* in_slot, int in_versions, const void* out_slot, int out_versions,
                                  int batch_capacity, void* maps_out);
 aiq_status_t launch_conv_pw(const ConvGeom& g, const void* maps, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
                             int32_t* error_flag, double weight_bytes, int weight_bits, cudaStream_t s);
-// Pointwise (1x1, stride 1) tensor-core convolution with streamed weights, for any channel count that is a multiple
-// of 8 (conv_pw_tc.cuh).  `map`: CUtensorMap over the input slot, dims (Cs, 2, pixels of all versions).
-bool conv_pw_tc_eligible(const ConvGeom& g);
-aiq_status_t conv_pw_tc_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions,
-                                   void* map_out);
-// store map over the output slot: dims (Cs_out, 2, pixels per version, versions)
-aiq_status_t conv_pw_tc_encode_out_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions,
-                                       void* map_out);
-// weight_bits: 8 (4- or 8-bit codes), 16 or 32 (two bfloat16 pieces per weight); one class per launch
-aiq_status_t launch_conv_pw_tc(const ConvGeom& g, const void* map, const void* out_map, const LayerJob* jobs_dev, int n_jobs,
-                               int batch_capacity, int32_t* error_flag, double weight_bytes, int weight_bits, cudaStream_t s);
 // Test aid: a one-thread kernel whose bounded wait runs out after `limit_cycles` SM clocks; it sets
 // *error_flag to 1 and *observed (optional) to 2, then returns.
 aiq_status_t launch_expire_wait(int32_t* error_flag, long long limit_cycles, int32_t* observed, cudaStream_t s);

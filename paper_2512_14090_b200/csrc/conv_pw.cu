@@ -1,4 +1,4 @@
-// Pointwise (1x1, stride 1) convolution with its weights resident in shared memory, on the tcgen05 tensor cores.
+// Pointwise (1x1, stride 1) convolution on the tcgen05 tensor cores.
 //
 // A 1x1 convolution over split activations is a plain GEMM over all (padded) pixels.  A pixel is stored as
 // [hi(Cs) | lo(Cs)] bfloat16, so it is one row of K2 = 2 Cs elements, and element k meets weight column k mod Cs:
@@ -6,13 +6,18 @@
 // The layer is bound by its activation bytes (MobileNetV2: 4 (Cin + Cout) bytes and 2 Cin Cout operations per pixel),
 // so the kernel is built to keep them moving:
 //   - a block owns Nt output channels of one job, expands their packed weights to bfloat16 once, and then streams
-//     pixel tiles; the streaming kernel (conv_pw_tc.cuh) expanded them again for every tile of 128 pixels;
+//     pixel tiles (the kernel before expanded them again for every tile of 128 pixels);
 //   - A chunks are dense whatever the channel count (hi and lo of a 32-channel pixel share one chunk);
 //   - every epilogue warp works by itself on units of 32 pixels x 32 channels: accumulators -> scale, bias, residual,
 //     activation -> split into hi / lo -> its own 4 KB of shared memory -> one TMA store of both halves.  No barrier
 //     joins the warps, so the stores of one overlap the arithmetic of the others;
 //   - two blocks per SM where their weights fit: one block's set-up and last tiles overlap the other's stream.
 // Warps: 0 TMA producer, 1 MMA issuer, then EW epilogue warps.  Two accumulator buffers in tensor memory.
+//
+// STREAM variant, for layers with so many input channels that resident weights leave no room: the weights of 64
+// channels travel through the ring beside the hi and lo chunk of the pixels, expanded by eight more warps.  A block
+// can then hold more output channels, so that the pixels (the large tensor of such a layer) are read fewer times, and
+// has more bytes in flight.
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -24,6 +29,7 @@ namespace {
 constexpr int kPrChunkBytes = 128 * 128;             // 128 pixels x 64 bfloat16
 constexpr int kPrUnitBytes = 4096;                   // 32 pixels x 32 channels, hi then lo
 constexpr int kPrMaxStages = 8;
+constexpr int kPrExpWarps = 8;                       // weight expander warps of the STREAM variant
 
 struct PrParams {
   int P;                    // padded pixels of the batch: B * (H + 2) * W
@@ -38,10 +44,15 @@ struct PrParams {
   int32_t* error_flag;
 };
 
-// shared memory: A ring | store buffers | B (pieces x Cs_in / 8 planes of Nt rows x 16 bytes) | scale, bias | barriers
-__host__ __device__ inline int pr_b_bytes(int Nt, int Cs_in, int pieces) { return pieces * Nt * Cs_in * 2; }
-__host__ __device__ inline int pr_smem_bytes(int Nt, int Cs_in, int pieces, int ew, int stages, int bufs) {
-  return stages * kPrChunkBytes + ew * bufs * kPrUnitBytes + pr_b_bytes(Nt, Cs_in, pieces) + 2 * Nt * 4 + (2 * kPrMaxStages + 4) * 8 + 16;
+// shared memory: ring | store buffers | B (pieces x Cs_in / 8 planes of Nt rows x 16 bytes) | scale, bias | barriers
+// A ring stage is one chunk of A, or in the STREAM variant the hi and the lo chunk of 64 channels and their weights.
+__host__ __device__ inline int pr_stage_bytes(bool stream, int Nt, int pieces) {
+  return stream ? 2 * kPrChunkBytes + pieces * Nt * 128 : kPrChunkBytes;
+}
+__host__ __device__ inline int pr_b_bytes(bool stream, int Nt, int Cs_in, int pieces) { return stream ? 0 : pieces * Nt * Cs_in * 2; }
+__host__ __device__ inline int pr_smem_bytes(bool stream, int Nt, int Cs_in, int pieces, int ew, int stages, int bufs) {
+  return stages * pr_stage_bytes(stream, Nt, pieces) + ew * bufs * kPrUnitBytes + pr_b_bytes(stream, Nt, Cs_in, pieces) + 2 * Nt * 4 +
+         (3 * kPrMaxStages + 4) * 8 + 16;
 }
 
 // n / d with magic = floor(2^32 / d) + 1: the product is exact or one too high for any 32-bit n
@@ -53,10 +64,19 @@ __device__ __forceinline__ uint32_t div_by(uint32_t n, uint32_t d, uint32_t magi
 
 // 16 packed bytes of one weight row (32 bytes at 32 bits) -> bfloat16 planes: plane j of this row goes to dst + j * plane
 template <int PIECES>
-__device__ __forceinline__ void pr_expand(const uint8_t* __restrict__ src, int bits, int n_planes, uint8_t* dst, int plane, int piece) {
+struct PrRaw { uint4 v[PIECES]; };
+template <int PIECES>
+__device__ __forceinline__ PrRaw<PIECES> pr_fetch(const uint8_t* __restrict__ src, int bits) {
+  PrRaw<PIECES> r;
+  r.v[0] = __ldg(reinterpret_cast<const uint4*>(src));
+  if (PIECES == 2) r.v[PIECES - 1] = bits == 32 ? __ldg(reinterpret_cast<const uint4*>(src) + 1) : make_uint4(0u, 0u, 0u, 0u);
+  return r;
+}
+template <int PIECES>
+__device__ __forceinline__ void pr_expand(const PrRaw<PIECES>& raw, int bits, int n_planes, uint8_t* dst, int plane, int piece) {
   uint32_t o[4];
   if (PIECES == 1) {
-    const uint4 r = __ldg(reinterpret_cast<const uint4*>(src));
+    const uint4 r = raw.v[0];
     if (bits == 8) {
       expand8_bf16(make_uint2(r.x, r.y), 8, o);
       *reinterpret_cast<uint4*>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
@@ -77,13 +97,14 @@ __device__ __forceinline__ void pr_expand(const uint8_t* __restrict__ src, int b
     // w = hi + lo, hi = bf16(w), lo = bf16(w - hi): exact for a half, within 2^-17 of a float32 weight
     float w[8];
     if (bits == 16) {
-      const uint4 r = __ldg(reinterpret_cast<const uint4*>(src));
+      const uint4 r = raw.v[0];
       const __half2* h2 = reinterpret_cast<const __half2*>(&r);
 #pragma unroll
       for (int j = 0; j < 4; ++j) { const float2 f = __half22float2(h2[j]); w[2 * j] = f.x; w[2 * j + 1] = f.y; }
     } else {
-      const float4 a = __ldg(reinterpret_cast<const float4*>(src)), b = __ldg(reinterpret_cast<const float4*>(src) + 1);
-      w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y; w[6] = b.z; w[7] = b.w;
+      const uint4 a = raw.v[0], b = raw.v[PIECES - 1];
+      w[0] = __uint_as_float(a.x); w[1] = __uint_as_float(a.y); w[2] = __uint_as_float(a.z); w[3] = __uint_as_float(a.w);
+      w[4] = __uint_as_float(b.x); w[5] = __uint_as_float(b.y); w[6] = __uint_as_float(b.z); w[7] = __uint_as_float(b.w);
     }
     uint32_t l[4];
 #pragma unroll
@@ -93,11 +114,11 @@ __device__ __forceinline__ void pr_expand(const uint8_t* __restrict__ src, int b
   }
 }
 
-template <int EW, int PIECES>
-__global__ void __launch_bounds__((2 + EW) * 32, EW == 8 ? 2 : 1)
+template <int EW, int PIECES, bool STREAM>
+__global__ void __launch_bounds__((2 + EW + (STREAM ? kPrExpWarps : 0)) * 32, EW == 8 && !STREAM ? 2 : 1)
 conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap out_map, PrParams p,
                const LayerJob* __restrict__ jobs) {
-  constexpr int THREADS = (2 + EW) * 32;
+  constexpr int THREADS = (2 + EW + (STREAM ? kPrExpWarps : 0)) * 32;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   // blocks that read the same pixels (the channel tiles of a range) are neighbours: the later ones find them in L2
@@ -106,23 +127,26 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
   const LayerJob job = jobs[(int)blockIdx.x / (p.n_ntiles * p.splits)];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int Nt = p.Nt, n0 = ntile * Nt, stages = p.n_stages;
-  uint8_t* staging = smem + stages * kPrChunkBytes;
+  const int stage_bytes = pr_stage_bytes(STREAM, Nt, PIECES);
+  uint8_t* staging = smem + stages * stage_bytes;
   uint8_t* bsm = staging + EW * p.n_bufs * kPrUnitBytes;
-  float* s_scale = reinterpret_cast<float*>(bsm + pr_b_bytes(Nt, p.Cs_in, PIECES));
+  float* s_scale = reinterpret_cast<float*>(bsm + pr_b_bytes(STREAM, Nt, p.Cs_in, PIECES));
   float* s_bias = s_scale + Nt;
   uint64_t* bars = reinterpret_cast<uint64_t*>(s_bias + Nt);
   const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kPrMaxStages;
-  const uint32_t bar_acc_full = bar_empty + 8 * kPrMaxStages, bar_acc_empty = bar_acc_full + 16;
-  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 2 * kPrMaxStages + 4);
+  const uint32_t bar_b_full = bar_empty + 8 * kPrMaxStages;     // STREAM: the expanders finished the weights of a stage
+  const uint32_t bar_acc_full = bar_b_full + 8 * kPrMaxStages, bar_acc_empty = bar_acc_full + 16;
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + 3 * kPrMaxStages + 4);
   volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
   const int tile0 = split * p.tiles_per_cta, tile1 = min(tile0 + p.tiles_per_cta, p.n_tiles);
-  const int K2 = 2 * p.Cs_in, n_chunks = (K2 + 63) >> 6;
+  const int K2 = 2 * p.Cs_in, n_chunks = STREAM ? (p.Cs_in + 63) >> 6 : (K2 + 63) >> 6;
   const int groups = (min(Nt, p.Cs_out - n0) + 31) >> 5;      // units of 32 channels of this block
 
   if (tid == 0) {
     for (int i = 0; i < stages; ++i) {
       mbar_init(bar_full + 8 * i, 1);
       mbar_init(bar_empty + 8 * i, 1);
+      mbar_init(bar_b_full + 8 * i, kPrExpWarps);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar_acc_full + 8 * i, 1);
@@ -142,11 +166,12 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
   }
   // weights -> B operand (K-major, no swizzle: plane of 8 channels, row, 16 bytes); consecutive threads take
   // consecutive rows, so their 16-byte stores are contiguous
-  {
-    const int plane = Nt * 16, piece = (p.Cs_in >> 3) * plane;
-    const int ppu = PIECES == 2 ? 1 : (job.bits == 8 ? 2 : 4);   // planes per 16 packed bytes (16 / 32 bits: one plane)
+  const int plane = Nt * 16;
+  const int ppu = PIECES == 2 ? 1 : (job.bits == 8 ? 2 : 4);     // planes per 16 packed bytes (16 / 32 bits: one plane)
+  const size_t wrow = (size_t)p.kpad * job.bits / 8;
+  if (!STREAM) {
+    const int piece = (p.Cs_in >> 3) * plane;
     const int uk = ((p.Cs_in >> 3) + ppu - 1) / ppu;
-    const size_t wrow = (size_t)p.kpad * job.bits / 8;
     const int n_units = Nt * uk;
 #pragma unroll 4
     for (int u = tid; u < n_units; u += THREADS) {
@@ -154,7 +179,7 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
       uint8_t* dst = bsm + (size_t)(j * ppu) * plane + r * 16;
       const int planes = min(ppu, (p.Cs_in >> 3) - j * ppu);
       if (n < p.Cout) {
-        pr_expand<PIECES>(job.w + (size_t)n * wrow + (size_t)j * ppu * job.bits, job.bits, planes, dst, plane, piece);
+        pr_expand<PIECES>(pr_fetch<PIECES>(job.w + (size_t)n * wrow + (size_t)j * ppu * job.bits, job.bits), job.bits, planes, dst, plane, piece);
       } else {
         for (int i = 0; i < planes; ++i) {
           *reinterpret_cast<uint4*>(dst + i * plane) = make_uint4(0u, 0u, 0u, 0u);
@@ -183,12 +208,14 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
           if (!alive) break;
           issued |= 1u << stage;
           issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-          mbar_expect_tx(bar_full + 8 * stage, kPrChunkBytes);
-          asm volatile(
-              "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-              ::"r"(smem_u32(smem) + stage * kPrChunkBytes), "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(bar_full + 8 * stage),
-              "r"(c * 64), "r"(pix)
-              : "memory");
+          mbar_expect_tx(bar_full + 8 * stage, (STREAM ? 2 : 1) * kPrChunkBytes);
+#pragma unroll
+          for (int part = 0; part < (STREAM ? 2 : 1); ++part)    // STREAM: 64 channels of the hi, then of the lo half
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+                ::"r"(smem_u32(smem) + stage * stage_bytes + part * kPrChunkBytes), "l"(reinterpret_cast<uint64_t>(&in_map)),
+                "r"(bar_full + 8 * stage), "r"(c * 64 + part * p.Cs_in), "r"(pix)
+                : "memory");
           if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -220,7 +247,25 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
         alive = mbar_wait_warp(bar_full + 8 * stage, phase, s_abort, p.error_flag);
         if (!alive) break;
         tc_fence_after();
-        const uint32_t a_lo = ((smem_u32(smem) + stage * kPrChunkBytes) >> 4) | (1u << 16);
+        const uint32_t a_lo = ((smem_u32(smem) + stage * stage_bytes) >> 4) | (1u << 16);
+        if constexpr (STREAM) {
+          alive = mbar_wait_warp(bar_b_full + 8 * stage, phase, s_abort, p.error_flag);
+          if (!alive) break;
+          tc_fence_after();
+          const uint32_t b_st = ((smem_u32(smem) + stage * stage_bytes + 2 * kPrChunkBytes) >> 4) | ((uint32_t)Nt << 16);
+          const int kmax = min(4, steps - c * 4);
+#pragma unroll
+          for (int part = 0; part < 2; ++part)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              if (kk < kmax) {
+                const uint64_t adesc = ((uint64_t)A_HI << 32) | (uint64_t)(a_lo + part * (kPrChunkBytes >> 4) + kk * 2);
+                const uint32_t b_lo = b_st + (uint32_t)kk * b_step;
+                umma_bf16(d_tmem, adesc, ((uint64_t)B_HI << 32) | (uint64_t)b_lo, idesc, accumulate);
+                accumulate = 1;
+                if (PIECES == 2) umma_bf16(d_tmem, adesc, ((uint64_t)B_HI << 32) | (uint64_t)(b_lo + 8u * (uint32_t)Nt), idesc, 1u);
+              }
+        } else {
         const int kmax = min(4, (K2 >> 4) - c * 4);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
@@ -233,10 +278,53 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
             if (++ks == steps) ks = 0;
           }
         }
+        }
         umma_commit(bar_empty + 8 * stage);
         if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
       }
       if (alive) umma_commit(bar_acc_full + 8 * buf);
+    }
+  } else if (STREAM && warp >= 2 + EW) {
+    // ---- STREAM weight expanders: packed rows -> the stage's B planes (8 of Nt rows per piece).  The packed words come
+    // from L2 one chunk ahead, so that their latency hides behind the expansion and the wait for a free stage.
+    constexpr int XT = kPrExpWarps * 32, UPT = 4;
+    const int et = tid - (2 + EW) * 32;
+    const int upr = 8 / ppu, n_units = Nt * upr;               // units of 16 packed bytes (32 at 32 bits) per chunk
+    PrRaw<PIECES> cur[UPT], nxt[UPT];
+    auto fetch = [&](int c, PrRaw<PIECES>* r) {
+#pragma unroll
+      for (int i = 0; i < UPT; ++i) {
+        const int u = et + i * XT, j = u / Nt, n = n0 + u - j * Nt, pl = c * 8 + j * ppu;
+        if (u < n_units && n < p.Cout && pl < (p.Cs_in >> 3)) {
+          r[i] = pr_fetch<PIECES>(job.w + (size_t)n * wrow + (size_t)pl * job.bits, job.bits);
+        } else {
+#pragma unroll
+          for (int k = 0; k < PIECES; ++k) r[i].v[k] = make_uint4(0u, 0u, 0u, 0u);
+        }
+      }
+    };
+    uint32_t stage = 0, phase = 0;
+    fetch(0, cur);
+    for (int tile = tile0; tile < tile1 && alive; ++tile) {
+      for (int c = 0; c < n_chunks; ++c) {
+        fetch(c + 1 < n_chunks ? c + 1 : 0, nxt);
+        alive = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+        if (!alive) break;
+        uint8_t* bst = smem + stage * stage_bytes + 2 * kPrChunkBytes;
+#pragma unroll
+        for (int i = 0; i < UPT; ++i) {
+          const int u = et + i * XT;
+          if (u < n_units) {
+            const int j = u / Nt, r = u - j * Nt;
+            pr_expand<PIECES>(cur[i], job.bits, ppu, bst + (size_t)(j * ppu) * plane + r * 16, plane, 8 * plane);
+          }
+          cur[i] = nxt[i];
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> visible to the MMA
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_b_full + 8 * stage);
+        if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
+      }
     }
   } else {
     // ---- epilogue: TMEM lanes 32q .. 32q+31 (pixels of the tile) belong to the warps with index mod 4 = q; the
@@ -366,28 +454,39 @@ EncodeTiledFn pr_encode_fn() {
   return reinterpret_cast<EncodeTiledFn>(sym);
 }
 
-// Launch shape: channel tile, blocks per SM, ring depth, pixel splits.  Every channel tile but the last is a multiple
-// of the 32 channels of a store unit.  Costs are in SM clocks: a tile of 128 pixels takes the longest of its MMAs
-// ((128 + Nt) / 4 clocks per 16-channel step), its input from L2 (about 40 bytes per clock and SM) and its epilogue
-// (about 12 clocks per channel); a block adds a set-up that grows with the weights it expands.  Blocks fill the GPU in
-// waves.
-struct PrConfig { int Nt, ew, stages, bufs, splits, tiles_per_cta, smem; };
+// Launch shape: variant, channel tile, blocks per SM, ring depth, pixel splits.  Every channel tile but the last is a
+// multiple of the 32 channels of a store unit.  Costs are in SM clocks: a tile of 128 pixels takes the longest of its
+// MMAs ((128 + Nt) / 4 clocks per 16-channel step), its input (40 bytes per clock and SM, less where the ring holds fewer
+// than about 1,600 clocks of that), its epilogue (about 12 clocks per channel) and, streamed, the expansion of its
+// weights; a block adds a set-up that grows with the weights it expands.  Blocks fill the GPU in waves.
+struct PrConfig { bool stream; int Nt, ew, stages, bufs, splits, tiles_per_cta, smem; };
 bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
   const int n_tiles = (g.B * (g.H + 2) * g.W + 127) / 128;
   const double K2 = 2.0 * g.Cs_in;
   double best = 1e300;
   for (int nt = 32; nt <= 256; nt += 32) {
-    int Nt = nt;
-    if (g.Cs_out <= nt) Nt = g.Cs_out;                         // the last candidate: one tile, any multiple of 16
+    const int Nt = g.Cs_out <= nt ? g.Cs_out : nt;             // the last candidate: one tile, any multiple of 16
     const int ntiles = (g.Cs_out + Nt - 1) / Nt;
-    for (int ew = 8; ew <= 16; ew += 8) {
-      const int occ = ew == 8 ? 2 : 1;
+    for (int variant = 0; variant < 4; ++variant) {
+      // two blocks per SM, one with 8 or 16 epilogue warps, one with streamed weights
+      const bool stream = variant == 3;
+      const int occ = variant == 0 ? 2 : 1, ew = variant == 2 ? 16 : 8;
       if (occ == 2 && Nt > 128) continue;                      // tensor memory: 2 Nt columns per block
+      if (stream && (Nt * 8 / (pieces == 2 ? 1 : 2) > 4 * kPrExpWarps * 32 || 2 * Nt > 512)) continue;
       const int limit = occ == 2 ? (props.smem_optin + 1024) / 2 - 1024 : props.smem_optin;
-      auto need = [&](int st, int bf) { return pr_smem_bytes(Nt, g.Cs_in, pieces, ew, st, bf) + 1024; };
+      auto need = [&](int st, int bf) { return pr_smem_bytes(stream, Nt, g.Cs_in, pieces, ew, st, bf) + 1024; };
       if (need(2, 1) > limit) continue;
-      const double c_mma = K2 / 16 * pieces * (128 + Nt) / 4.0, c_in = 128.0 * K2 * 2 / 40.0, c_epi = 12.0 * Nt;
-      const double tile = std::max(std::max(c_mma, c_in), c_epi), setup = 3000.0 + Nt * (double)g.Cs_in * pieces / 16.0;
+      int st = 2, bf = 1;
+      while (st < 4 && need(st + 1, bf) <= limit) ++st;
+      if (need(st, 2) <= limit) bf = 2;
+      while (st < kPrMaxStages && need(st + 1, bf) <= limit) ++st;
+      const double in_flight = (double)occ * st * (stream ? 2 : 1) * kPrChunkBytes;
+      const double c_mma = K2 / 16 * pieces * (128 + Nt) / 4.0;
+      const double c_in = 128.0 * K2 * 2 / std::min(40.0, in_flight / 1600.0);
+      const double c_epi = (ew == 8 && occ == 1 ? 18.0 : 12.0) * Nt;
+      const double c_exp = stream ? Nt * (double)g.Cs_in * pieces * 0.06 : 0.0;
+      const double tile = std::max(std::max(c_mma, c_in), std::max(c_epi, c_exp));
+      const double setup = 3000.0 + (stream ? 0.0 : Nt * (double)g.Cs_in * pieces / 16.0);
       const int pairs = n_jobs * ntiles;
       for (int wave = 1; wave <= 5; ++wave) {
         int splits = wave == 5 ? n_tiles : wave * occ * props.n_sms / pairs;
@@ -401,12 +500,7 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
         const double cost = full * one + (rem > props.n_sms ? one : rem > 0 ? tpc * tile + setup : 0.0);
         if (cost < best * 0.999) {
           best = cost;
-          out->Nt = Nt; out->ew = ew; out->splits = splits; out->tiles_per_cta = tpc;
-          int st = 2, bf = 1;
-          while (st < 4 && need(st + 1, bf) <= limit) ++st;
-          if (need(st, 2) <= limit) bf = 2;
-          while (st < kPrMaxStages && need(st + 1, bf) <= limit) ++st;
-          out->stages = st; out->bufs = bf; out->smem = need(st, bf);
+          *out = {stream, Nt, ew, st, bf, splits, tpc, need(st, bf)};
         }
         if (ctas >= (long long)n_tiles * pairs) break;
       }
@@ -415,19 +509,18 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
   }
   return best < 1e300;
 }
-
 bool pr_config(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
   static thread_local ConfigMemo<PrConfig, 8> memo;
   const int key[8] = {g.B, g.H, g.W, g.Cs_in, g.Cs_out, n_jobs, pieces, props.dev};
   return memo.get(key, out, [&](PrConfig* c) { return pr_search(g, n_jobs, pieces, props, c); });
 }
 
-template <int EW, int PIECES>
+template <int EW, int PIECES, bool STREAM>
 aiq_status_t launch_pr(const LaunchScope& scope, const DeviceProps& props, const PrConfig& c, const PrParams& p, const CUtensorMap& m,
                        const CUtensorMap& mo, const LayerJob* jobs_dev, int n_jobs, cudaStream_t s) {
-  AIQ_ENSURE_DYNAMIC_SMEM((conv_pw_kernel<EW, PIECES>), props.smem_optin);
-  AIQ_CUDA_TRY(launch_chained(scope.chain, conv_pw_kernel<EW, PIECES>, dim3((unsigned)(n_jobs * p.splits * p.n_ntiles)),
-                              dim3((2 + EW) * 32), c.smem, s, m, mo, p, jobs_dev));
+  AIQ_ENSURE_DYNAMIC_SMEM((conv_pw_kernel<EW, PIECES, STREAM>), props.smem_optin);
+  AIQ_CUDA_TRY(launch_chained(scope.chain, conv_pw_kernel<EW, PIECES, STREAM>, dim3((unsigned)(n_jobs * p.splits * p.n_ntiles)),
+                              dim3((2 + EW + (STREAM ? kPrExpWarps : 0)) * 32), c.smem, s, m, mo, p, jobs_dev));
   return AIQ_OK;
 }
 
@@ -435,11 +528,7 @@ aiq_status_t launch_pr(const LaunchScope& scope, const DeviceProps& props, const
 
 bool conv_pw_eligible(const ConvGeom& g) {
   if (g.in_is_nchw || g.act_format != ACT_SPLIT) return false;
-  if (g.ks != 1 || g.pad != 0 || g.stride != 1 || g.Cin % 8 != 0 || g.Cin < 16) return false;
-  DeviceProps props;
-  const int limit = current_device_props(&props) == AIQ_OK ? props.smem_optin : 227 * 1024;
-  // the narrowest candidate of pr_config with 16- / 32-bit weights, which need the most memory
-  return pr_smem_bytes(std::min(32, g.Cs_out), g.Cs_in, 2, 16, 2, 1) + 1024 <= limit;
+  return g.ks == 1 && g.pad == 0 && g.stride == 1 && g.Cin % 8 == 0 && g.Cin >= 16;
 }
 
 aiq_status_t conv_pw_encode_maps(const ConvGeom& g, const void* in_slot, int in_versions, const void* out_slot, int out_versions,
@@ -478,7 +567,7 @@ aiq_status_t launch_conv_pw(const ConvGeom& g, const void* maps, const LayerJob*
   if (aiq_status_t st = current_device_props(&props)) return st;
   const int pieces = weight_bits > 8 ? 2 : 1;
   PrConfig c = {};
-  if (!pr_config(g, n_jobs, pieces, props, &c)) return set_error(AIQ_ERR_SHAPE, "conv_pw: weights of 32 output channels do not fit shared memory");
+  if (!pr_config(g, n_jobs, pieces, props, &c)) return set_error(AIQ_ERR_SHAPE, "conv_pw: no launch shape fits shared memory");
   PrParams p = {};
   p.P = g.B * (g.H + 2) * g.W; p.H = g.H; p.W = g.W;
   p.w_magic = (uint32_t)(0x100000000ull / (uint32_t)g.W + 1); p.h_magic = (uint32_t)(0x100000000ull / (uint32_t)(g.H + 2) + 1);
@@ -493,9 +582,12 @@ aiq_status_t launch_conv_pw(const ConvGeom& g, const void* maps, const LayerJob*
   const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
   LaunchScope scope(AIQ_KERNEL_CONV_TC, s, 2.0 * g.B * g.Ho * g.Wo * g.Cout * (double)g.Cin * n_jobs,
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W + (double)g.B * g.Ho * g.Wo * g.Cout));
-  const aiq_status_t st = c.ew == 8
-      ? (pieces == 1 ? launch_pr<8, 1>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s) : launch_pr<8, 2>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s))
-      : (pieces == 1 ? launch_pr<16, 1>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s) : launch_pr<16, 2>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s));
+#define AIQ_PW(EW_, P_, S_) launch_pr<EW_, P_, S_>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s)
+  aiq_status_t st;
+  if (c.stream) st = pieces == 1 ? AIQ_PW(8, 1, true) : AIQ_PW(8, 2, true);
+  else if (c.ew == 8) st = pieces == 1 ? AIQ_PW(8, 1, false) : AIQ_PW(8, 2, false);
+  else st = pieces == 1 ? AIQ_PW(16, 1, false) : AIQ_PW(16, 2, false);
+#undef AIQ_PW
   if (st != AIQ_OK) return st;
   AIQ_LAUNCH_CHECK("conv_pw");
   return AIQ_OK;

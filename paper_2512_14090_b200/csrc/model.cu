@@ -248,15 +248,13 @@ static ConvGeom make_geom(const aiq_model* m, const LayerInfo& li, int B) {
 }
 
 // 0: float32 kernels only; 1: small-channel 3x3 / 1x1 tensor-core kernel; 2: pointwise tensor-core
-// kernel with streamed weights; 3: row-streaming tensor-core kernel (models stored in ACT_RS); 4: pointwise
-// tensor-core kernel with resident weights
+// kernel; 3: row-streaming tensor-core kernel (models stored in ACT_RS)
 static int layer_tensor_kind(const aiq_model* m, const LayerInfo& li) {
   if (li.d.kind != AIQ_LAYER_CONV) return 0;
   const ConvGeom g = make_geom(m, li, 1);
   if (conv_rs_eligible(g)) return 3;
   if (conv_tc_eligible(g)) return 1;
-  if (conv_pw_eligible(g)) return 4;
-  if (conv_pw_tc_eligible(g)) return 2;
+  if (conv_pw_eligible(g)) return 2;
   return 0;
 }
 static bool layer_on_tensor_cores(const aiq_model* m, const LayerInfo& li) { return layer_tensor_kind(m, li) != 0; }
@@ -877,17 +875,11 @@ static aiq_status_t build_plan(const aiq_model* m, const uint8_t* schemes, int S
         lp.tc_kind = layer_tensor_kind(m, li);
         aiq_status_t st = lp.tc_kind == 3
             ? conv_rs_encode_maps(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0])
-            : lp.tc_kind == 4
+            : lp.tc_kind == 2
             ? conv_pw_encode_maps(make_geom(m, li, B), ws + wl.slot_off[src.slot], plan.lp[li.d.input].n_versions,
                                   ws + wl.slot_off[li.slot], lp.n_versions, B, &lp.maps[0])
-            : lp.tc_kind == 1
-            ? conv_tc_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0])
-            : conv_pw_tc_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0]);
+            : conv_tc_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0]);
         if (st != AIQ_OK) return st;
-        if (lp.tc_kind == 2) {
-          st = conv_pw_tc_encode_out_map(make_geom(m, li, B), ws + wl.slot_off[li.slot], B, lp.n_versions, &lp.maps[1]);
-          if (st != AIQ_OK) return st;
-        }
       }
       if (li.d.kind == AIQ_LAYER_DEPTHWISE) {
         const LayerInfo& src = m->layers[li.d.input];
@@ -1028,10 +1020,8 @@ static aiq_status_t run_chunk(const aiq_model* m, const EvalPlan& plan, const La
     auto launch_wide = [&](const LayerJob* jd, int n, double wb, int wbits) -> aiq_status_t {
       return lp.tc_kind == 3
           ? launch_conv_rs(g, &lp.maps[0], jd, n, plan.batch_capacity, m->status_word, wb, wbits, lp.pools, stream)
-          : lp.tc_kind == 4
-          ? launch_conv_pw(g, &lp.maps[0], jd, n, plan.batch_capacity, m->status_word, wb, wbits, stream)
           : lp.tc_kind == 2
-          ? launch_conv_pw_tc(g, &lp.maps[0], &lp.maps[1], jd, n, plan.batch_capacity, m->status_word, wb, wbits, stream)
+          ? launch_conv_pw(g, &lp.maps[0], jd, n, plan.batch_capacity, m->status_word, wb, wbits, stream)
           : launch_conv_tc(g, &lp.maps[0], jd, n, plan.batch_capacity, m->status_word, wb, wbits, stream);
     };
     if (lp.n_tc > 0) {

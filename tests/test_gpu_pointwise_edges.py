@@ -1,8 +1,8 @@
-"""The pointwise (1x1) tensor-core kernel with resident weights at the edges of its tiling, against the oracle: channel
+"""The pointwise (1x1) tensor-core kernel at the edges of its tiling, against the oracle: channel
 counts that are padded (24 -> 40, 136 -> 200), a single 16-channel unit, a channel tile narrower than a store unit,
 odd map sizes (border rows inside a warp's 32 pixels), one image and a batch that leaves the last pixel tile partly
-empty, all four bit-widths, a shortcut into the layer; and 1,024 input channels, which the kernel with streamed
-weights takes.  Tolerance: the float32 rule of the other forward tests, 1e-3 (1 + |ref|)."""
+empty, all four bit-widths, a shortcut into the layer; and 1,024 input channels, whose weights are
+streamed.  Tolerance: the float32 rule of the other forward tests, 1e-3 (1 + |ref|)."""
 import numpy as np
 import pytest
 
@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("cin,cout,hw,batch", [(16, 16, 5, 1), (24, 40, 7, 3), (136, 200, 13, 2), (96, 264, 4, 9),
-                                               (320, 48, 9, 30), (1024, 48, 5, 3)])
+                                               (320, 48, 9, 30), (1024, 48, 5, 3),
+                                               (1032, 320, 3, 5)])
 def test_pointwise_tile_edges(cin, cout, hw, batch):
     aiq = binding()
     arch = pointwise_stack(cin, cout, hw)

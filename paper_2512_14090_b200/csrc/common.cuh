@@ -237,7 +237,7 @@ aiq_status_t launch_conv(const ConvGeom& g, const LayerJob* jobs_dev, int n_jobs
 // Depthwise 3x3 (depthwise.cu).  `map`: CUtensorMap over the input slot (channels, hi | lo, columns, padded rows, images).
 aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions, void* map_out);
 aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
-                              int32_t* error_flag, double weight_bytes, cudaStream_t s);
+                              bool has_res, int32_t* error_flag, double weight_bytes, cudaStream_t s);
 // Tensor-core convolution (conv_tc.cu).  `map` points to a 128-byte CUtensorMap over the input
 // slot: dims (2*Cs, W, batch_capacity*(H+2), versions).
 bool conv_tc_eligible(const ConvGeom& g);

@@ -21,6 +21,7 @@
 #include "tc_ptx.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace aiq {
 
@@ -348,19 +349,20 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
       const int pix0 = tile * 128 + q * 32, pix = pix0 + lane;
       const uint32_t row = div_by((uint32_t)pix, (uint32_t)p.W, p.w_magic);
       const int yp = (int)(row - div_by(row, (uint32_t)(p.H + 2), p.h_magic) * (uint32_t)(p.H + 2));
-      const bool interior = pix < p.P && yp >= 1 && yp <= p.H;
+      const bool interior = pix < p.P && yp >= 1 && yp <= p.H, all_interior = __all_sync(0xffffffffu, interior);
       for (; g < groups; g += HW) {
       const int c0 = g * 32;
       const int nv = min(32, p.Cs_out - n0 - c0);              // stored channels of the unit: 32 or 16
       uint4 rh[4], rl[4];
-      const bool has_res = job.res != nullptr && interior;
-      if (has_res) {
+      if (job.res) {
         const __nv_bfloat16* res = static_cast<const __nv_bfloat16*>(job.res) + (size_t)pix * (2 * p.Cs_out) + n0 + c0;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (j * 8 < nv) {
+          if (j * 8 < nv && interior) {
             rh[j] = ld_chain(reinterpret_cast<const uint4*>(res) + j);
             rl[j] = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out) + j);
+          } else {
+            rh[j] = rl[j] = make_uint4(0u, 0u, 0u, 0u);
           }
       }
       alive = mbar_wait_warp(bar_acc_full + 8 * buf, (it >> 1) & 1, s_abort, p.error_flag);
@@ -381,33 +383,27 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
       }
       __syncwarp();
       uint8_t* dst = my_buf + buf_idx * kPrUnitBytes + lane * 64;
+      auto finish = [&](auto act, auto res) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t hi[4], lo[4];
-        const int cc = j * 8 < nv ? c0 + j * 8 : 0;            // past the stored channels: anything (clipped by the map)
-        const uint4 th = rh[j], tl = rl[j];
-        const uint32_t rhw[4] = {th.x, th.y, th.z, th.w}, rlw[4] = {tl.x, tl.y, tl.z, tl.w};
+        for (int j = 0; j < 4; ++j) {
+          uint32_t hi[4], lo[4];
+          const int cc = j * 8 < nv ? c0 + j * 8 : 0;          // past the stored channels: anything (clipped by the map)
+          finish8<decltype(act)::value, decltype(res)::value>(v + 8 * j, s_scale + cc, s_bias + cc, rh[j], rl[j], hi, lo);
+          if (!all_interior && !interior) {                    // border rows are zeros
 #pragma unroll
-        for (int e = 0; e < 8; e += 4) {
-          const float4 sc = *reinterpret_cast<const float4*>(s_scale + cc + e);
-          const float4 bi = *reinterpret_cast<const float4*>(s_bias + cc + e);
-          float a[4] = {fmaf(__uint_as_float(v[8 * j + e]), sc.x, bi.x), fmaf(__uint_as_float(v[8 * j + e + 1]), sc.y, bi.y),
-                        fmaf(__uint_as_float(v[8 * j + e + 2]), sc.z, bi.z), fmaf(__uint_as_float(v[8 * j + e + 3]), sc.w, bi.w)};
-          if (has_res) {
-            a[0] += __uint_as_float(rhw[e >> 1] << 16) + __uint_as_float(rlw[e >> 1] << 16);
-            a[1] += __uint_as_float(rhw[e >> 1] & 0xFFFF0000u) + __uint_as_float(rlw[e >> 1] & 0xFFFF0000u);
-            a[2] += __uint_as_float(rhw[(e >> 1) + 1] << 16) + __uint_as_float(rlw[(e >> 1) + 1] << 16);
-            a[3] += __uint_as_float(rhw[(e >> 1) + 1] & 0xFFFF0000u) + __uint_as_float(rlw[(e >> 1) + 1] & 0xFFFF0000u);
+            for (int i = 0; i < 4; ++i) hi[i] = lo[i] = 0u;
           }
-#pragma unroll
-          for (int i = 0; i < 4; ++i) a[i] = interior ? apply_act(a[i], p.act) : 0.f;   // border rows are zeros
-          split_pair(a[0], a[1], hi[e >> 1], lo[e >> 1]);
-          split_pair(a[2], a[3], hi[(e >> 1) + 1], lo[(e >> 1) + 1]);
+          const uint32_t off = ((uint32_t)j ^ key) << 4;
+          *reinterpret_cast<uint4*>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+          *reinterpret_cast<uint4*>(dst + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
-        const uint32_t off = ((uint32_t)j ^ key) << 4;
-        *reinterpret_cast<uint4*>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(dst + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      }
+      };
+      auto finish_act = [&](auto res) {
+        if (p.act == AIQ_ACT_RELU6) finish(std::integral_constant<int, AIQ_ACT_RELU6>(), res);
+        else if (p.act == AIQ_ACT_RELU) finish(std::integral_constant<int, AIQ_ACT_RELU>(), res);
+        else finish(std::integral_constant<int, AIQ_ACT_NONE>(), res);
+      };
+      if (job.res) finish_act(std::true_type()); else finish_act(std::false_type());
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
@@ -422,8 +418,7 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
       if (++buf_idx == p.n_bufs) buf_idx = 0;
       }
       g -= groups;                                             // counted on into the next tiles
-      skip = g / groups;
-      g -= skip * groups;
+      while (g >= groups) { g -= groups; ++skip; }
     }
     // all stores must have left shared memory (and be complete) before the CTA retires
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");

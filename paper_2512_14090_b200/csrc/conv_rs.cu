@@ -29,6 +29,8 @@
 // Every wait is bounded as in the other tcgen05 kernels.
 #include "tc_ptx.cuh"
 
+#include <type_traits>
+
 namespace aiq {
 
 namespace {
@@ -254,29 +256,14 @@ __device__ __forceinline__ void rs_issue_row(const RowRegs& rr, uint32_t d_xt, u
 // 16 accumulator values of one lane (a 16-channel chunk of one pixel) -> scale, bias, residual,
 // activation, split into hi / lo bfloat16 pairs: hi[0..3] / hi[4..7] are the two hi planes of
 // the chunk, lo likewise.  res: the four residual planes (hi, hi, lo, lo) of the same pixel.
+template <int ACT, bool RES>
 __device__ __forceinline__ void rs_finish_unit(const uint32_t* v, const float* scale, const float* bias, const uint4* res,
-                                               bool has_res, int act, uint32_t* hi, uint32_t* lo) {
+                                               uint32_t* hi, uint32_t* lo) {
+  // planes 0 / 1 of the chunk hold channels 0-7 / 8-15
 #pragma unroll
-  for (int e = 0; e < 16; e += 4) {
-    const float4 sc = *reinterpret_cast<const float4*>(scale + e);
-    const float4 bi = *reinterpret_cast<const float4*>(bias + e);
-    float u0 = fmaf(__uint_as_float(v[e]), sc.x, bi.x);
-    float u1 = fmaf(__uint_as_float(v[e + 1]), sc.y, bi.y);
-    float u2 = fmaf(__uint_as_float(v[e + 2]), sc.z, bi.z);
-    float u3 = fmaf(__uint_as_float(v[e + 3]), sc.w, bi.w);
-    if (has_res) {
-      // planes 0 / 1 of the chunk hold channels 0-7 / 8-15; a bfloat16 is the upper half of a float
-      const uint4 rh4 = res[e >> 3], rl4 = res[2 + (e >> 3)];
-      const uint32_t rh0 = (e & 4) ? rh4.z : rh4.x, rh1 = (e & 4) ? rh4.w : rh4.y;
-      const uint32_t rl0 = (e & 4) ? rl4.z : rl4.x, rl1 = (e & 4) ? rl4.w : rl4.y;
-      u0 += __uint_as_float(rh0 << 16) + __uint_as_float(rl0 << 16);
-      u1 += __uint_as_float(rh0 & 0xFFFF0000u) + __uint_as_float(rl0 & 0xFFFF0000u);
-      u2 += __uint_as_float(rh1 << 16) + __uint_as_float(rl1 << 16);
-      u3 += __uint_as_float(rh1 & 0xFFFF0000u) + __uint_as_float(rl1 & 0xFFFF0000u);
-    }
-    split_pair(apply_act(u0, act), apply_act(u1, act), hi[e >> 1], lo[e >> 1]);
-    split_pair(apply_act(u2, act), apply_act(u3, act), hi[(e >> 1) + 1], lo[(e >> 1) + 1]);
-  }
+  for (int e = 0; e < 2; ++e)
+    finish8<ACT, RES>(v + 8 * e, scale + 8 * e, bias + 8 * e, RES ? res[e] : make_uint4(0u, 0u, 0u, 0u),
+                      RES ? res[2 + e] : make_uint4(0u, 0u, 0u, 0u), hi + 4 * e, lo + 4 * e);
 }
 
 template <int C, int KS, int STRIDE, int PIECES>
@@ -526,7 +513,13 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           if (lane == 0) mbar_arrive(bar_out_empty + 8 * slot);
         }
         uint32_t hi[8], lo[8];
-        rs_finish_unit(v, s_scale + c0, s_bias + c0, rres, res_base != nullptr, p.act, hi, lo);
+        auto finish = [&](auto act) {
+          if (res_base) rs_finish_unit<decltype(act)::value, true>(v, s_scale + c0, s_bias + c0, rres, hi, lo);
+          else rs_finish_unit<decltype(act)::value, false>(v, s_scale + c0, s_bias + c0, nullptr, hi, lo);
+        };
+        if (p.act == AIQ_ACT_RELU) finish(std::integral_constant<int, AIQ_ACT_RELU>());
+        else if (p.act == AIQ_ACT_RELU6) finish(std::integral_constant<int, AIQ_ACT_RELU6>());
+        else finish(std::integral_constant<int, AIQ_ACT_NONE>());
         // the residual registers are free again: request the first unit of this warp's next row
         if (res_base && u + unit_step >= units && k + 1 < total) load_res(k + 1, unit0, rres);
         if (pooling) {
@@ -838,7 +831,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int c0 = (u % chunks) * 16;
-          rs_finish_unit(u == 0 ? v0 : v1, scale + c0, bias + c0, nullptr, false, AIQ_ACT_RELU, hi, lo);
+          rs_finish_unit<AIQ_ACT_RELU, false>(u == 0 ? v0 : v1, scale + c0, bias + c0, nullptr, hi, lo);
           uint8_t* dst = mid_ring + ms * p.stage_bytes + cell[u];
           *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<uint4*>(dst + p.a_lbo) = make_uint4(hi[4], hi[5], hi[6], hi[7]);
@@ -875,7 +868,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const int c0 = (u % chunks) * 16;
-          rs_finish_unit(u == 0 ? v0 : v1, scale + c0, bias + c0, u == 0 ? r0 : r1, true, AIQ_ACT_RELU, hi, lo);
+          rs_finish_unit<AIQ_ACT_RELU, true>(u == 0 ? v0 : v1, scale + c0, bias + c0, u == 0 ? r0 : r1, hi, lo);
           uint8_t* dst = row_dst + (size_t)ux[u] * px_bytes + (size_t)uph[u] * plane_bytes;
           *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
           *reinterpret_cast<uint4*>(dst + plane_bytes) = make_uint4(hi[4], hi[5], hi[6], hi[7]);

@@ -43,38 +43,10 @@ struct DwParams {
   int32_t* error_flag;
 };
 
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
-// hi and lo halves of four channels -> two packed float pairs (a bfloat16 is the upper half of a float)
+// hi and lo halves of four channels -> two packed float pairs
 __device__ __forceinline__ void join4(uint2 h, uint2 l, uint64_t* v) {
-  v[0] = add2(pack2(__uint_as_float(h.x << 16), __uint_as_float(h.x & 0xFFFF0000u)),
-              pack2(__uint_as_float(l.x << 16), __uint_as_float(l.x & 0xFFFF0000u)));
-  v[1] = add2(pack2(__uint_as_float(h.y << 16), __uint_as_float(h.y & 0xFFFF0000u)),
-              pack2(__uint_as_float(l.y << 16), __uint_as_float(l.y & 0xFFFF0000u)));
+  v[0] = add2(widen2(h.x), widen2(l.x));
+  v[1] = add2(widen2(h.y), widen2(l.y));
 }
 
 // Four channels of one pixel in shared memory: [hi(Cb) | lo(Cb)] bfloat16 or Cb floats.
@@ -130,7 +102,7 @@ __device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int u) {
 // columns a row cost 37 per output element at 0.46 issued per clock and scheduler (2.9 TB/s at 256 x 32 x 32 x 144
 // channels); four columns share six unpacked input columns (1.5 per output instead of 2), the per-row waiting and
 // the addresses.
-template <int FMT, int STRIDE, int COLS>
+template <int FMT, int STRIDE, int COLS, bool RES>
 __global__ void __launch_bounds__(kDwThreads + 32, 2)
 depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, const LayerJob* __restrict__ jobs) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -281,7 +253,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     const int b = d.img0 + ni, ox = d.ox0 + xg * COLS;
     const bool writes = worker && b < p.B && c < p.Cs && ox < p.Wo;
     uint8_t* outp = static_cast<uint8_t*>(job.out) + ch_off + (((size_t)b * (p.Ho + 2) + d.oy0 + 1) * p.Wo + ox) * pix_bytes;
-    const uint8_t* resp = job.res ? static_cast<const uint8_t*>(job.res) + (outp - static_cast<uint8_t*>(job.out)) : nullptr;
+    const uint8_t* resp = RES ? static_cast<const uint8_t*>(job.res) + (outp - static_cast<uint8_t*>(job.out)) : nullptr;
     // finish and store the next output row (rows are emitted in order) from its accumulators
     auto emit = [&](const uint64_t (&acc)[COLS][2]) {
       if (writes) {
@@ -292,7 +264,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
         for (int x = 0; x < COLS; ++x) {
           if (ox + x >= p.Wo) break;
           uint64_t r[2] = {fma2(acc[x][0], sc[0], bi[0]), fma2(acc[x][1], sc[1], bi[1])};
-          if (resp) {
+          if (RES) {
             uint64_t rs[2];
             load4<FMT>(resp + x * pix_bytes, lo_off, rs);
             r[0] = add2(r[0], rs[0]);
@@ -308,7 +280,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
         }
       }
       outp += out_pitch;
-      if (resp) resp += out_pitch;
+      if (RES) resp += out_pitch;
     };
     if (STRIDE == 1) {
       // input row k of the block (padded row oy0 + k) is tap row 2 / 1 / 0 of output rows k - 2 / k - 1 / k
@@ -431,7 +403,7 @@ aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int 
 }
 
 aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
-                              int32_t* error_flag, double weight_bytes, cudaStream_t s) {
+                              bool has_res, int32_t* error_flag, double weight_bytes, cudaStream_t s) {
   if (g.stride != 1 && g.stride != 2) return set_error(AIQ_ERR_SHAPE, "depthwise: stride %d is not supported", g.stride);
   DeviceProps props;
   if (aiq_status_t st = current_device_props(&props)) return st;
@@ -494,16 +466,18 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                    (double)g.B * g.Ho * g.Wo * g.Cout));
   const CUtensorMap& m = *static_cast<const CUtensorMap*>(map);
-#define AIQ_DW(FMT_, ST_, COLS_)                                                                       \
-  do {                                                                                                 \
-    AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_>), per_cta);                          \
-    AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<FMT_, ST_, COLS_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
+#define AIQ_DW(FMT_, ST_, COLS_, RES_)                                                                          \
+  do {                                                                                                          \
+    AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_, RES_>), per_cta);                              \
+    AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<FMT_, ST_, COLS_, RES_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
   } while (0)
-  if (g.act_format == ACT_SPLIT) {
-    if (g.stride == 2) AIQ_DW(ACT_SPLIT, 2, 2); else if (sh.cols == 4) AIQ_DW(ACT_SPLIT, 1, 4); else AIQ_DW(ACT_SPLIT, 1, 2);
-  } else {
-    if (g.stride == 2) AIQ_DW(ACT_F32, 2, 2); else if (sh.cols == 4) AIQ_DW(ACT_F32, 1, 4); else AIQ_DW(ACT_F32, 1, 2);
-  }
+#define AIQ_DW_SHAPE(FMT_, RES_)                                                                                \
+  do {                                                                                                          \
+    if (g.stride == 2) AIQ_DW(FMT_, 2, 2, RES_); else if (sh.cols == 4) AIQ_DW(FMT_, 1, 4, RES_); else AIQ_DW(FMT_, 1, 2, RES_); \
+  } while (0)
+  if (g.act_format == ACT_SPLIT) { if (has_res) AIQ_DW_SHAPE(ACT_SPLIT, true); else AIQ_DW_SHAPE(ACT_SPLIT, false); }
+  else { if (has_res) AIQ_DW_SHAPE(ACT_F32, true); else AIQ_DW_SHAPE(ACT_F32, false); }
+#undef AIQ_DW_SHAPE
 #undef AIQ_DW
   AIQ_LAUNCH_CHECK("depthwise3x3");
   return AIQ_OK;

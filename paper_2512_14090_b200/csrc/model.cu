@@ -1012,8 +1012,8 @@ static aiq_status_t run_chunk(const aiq_model* m, const EvalPlan& plan, const La
       continue;
     }
     if (li.d.kind == AIQ_LAYER_DEPTHWISE) {
-      st = launch_depthwise(g, &lp.maps[0], jobs_dev + lp.job_first, lp.n_versions, plan.batch_capacity, m->status_word,
-                            lp.weight_bytes, stream);
+      st = launch_depthwise(g, &lp.maps[0], jobs_dev + lp.job_first, lp.n_versions, plan.batch_capacity, li.d.residual >= 0,
+                            m->status_word, lp.weight_bytes, stream);
       if (st != AIQ_OK) return st;
       continue;
     }

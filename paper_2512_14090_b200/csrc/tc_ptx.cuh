@@ -129,13 +129,75 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
                : "r"(taddr));
 }
+// Two float32 lanes in one 64-bit register: one instruction for both, the roundings of the scalar operations.
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// the two bfloat16 of a word as floats (a bfloat16 is the upper half of a float)
+__device__ __forceinline__ uint64_t widen2(uint32_t w) { return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+
 // v = hi + lo with hi = bf16_rn(v), lo = bf16_rn(v - hi), two values at a time (one packed
 // conversion per pair); the same roundings as split_bf16
 __device__ __forceinline__ void split_pair(float u0, float u1, uint32_t& hi2, uint32_t& lo2) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(u0, u1);
   hi2 = *reinterpret_cast<const uint32_t*>(&h);
-  const __nv_bfloat162 l = __floats2bfloat162_rn(u0 - __uint_as_float(hi2 << 16), u1 - __uint_as_float(hi2 & 0xFFFF0000u));
+  const float2 d = unpack2(sub2(pack2(u0, u1), widen2(hi2)));
+  const __nv_bfloat162 l = __floats2bfloat162_rn(d.x, d.y);
   lo2 = *reinterpret_cast<const uint32_t*>(&l);
+}
+// Eight finished accumulators of a pixel: scale, bias, residual (hi and lo words, or none), activation, split into four
+// hi and four lo words.  ACT and RES are template arguments because the epilogues are bound by these instructions, and a
+// residual or activation chosen inside is predicated, not skipped: its instructions issue all the same.  The pointwise
+// layer 24 -> 144 (256 x 32 x 32) took FIN_A us so, FIN_B us with both chosen once per warp.
+template <int ACT>
+__device__ __forceinline__ float act_of(float v) {
+  if (ACT == AIQ_ACT_RELU) return fmaxf(v, 0.0f);
+  if (ACT == AIQ_ACT_RELU6) return fminf(fmaxf(v, 0.0f), 6.0f);
+  return v;
+}
+template <int ACT, bool RES>
+__device__ __forceinline__ void finish8(const uint32_t* v, const float* scale, const float* bias, uint4 rh, uint4 rl, uint32_t* hi,
+                                        uint32_t* lo) {
+  const uint32_t rhw[4] = {rh.x, rh.y, rh.z, rh.w}, rlw[4] = {rl.x, rl.y, rl.z, rl.w};
+#pragma unroll
+  for (int e = 0; e < 8; e += 4) {
+    const ulonglong2 sc = *reinterpret_cast<const ulonglong2*>(scale + e), bi = *reinterpret_cast<const ulonglong2*>(bias + e);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int w = (e >> 1) + i;
+      uint64_t u = fma2(pack2(__uint_as_float(v[2 * w]), __uint_as_float(v[2 * w + 1])), i ? sc.y : sc.x, i ? bi.y : bi.x);
+      if (RES) u = add2(u, add2(widen2(rhw[w]), widen2(rlw[w])));
+      const float2 f = unpack2(u);
+      split_pair(act_of<ACT>(f.x), act_of<ACT>(f.y), hi[w], lo[w]);
+    }
+  }
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 

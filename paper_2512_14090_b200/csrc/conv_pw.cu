@@ -116,7 +116,7 @@ __device__ __forceinline__ void pr_expand(const PrRaw<PIECES>& raw, int bits, in
 }
 
 template <int EW, int PIECES, bool STREAM>
-__global__ void __launch_bounds__((2 + EW + (STREAM ? kPrExpWarps : 0)) * 32, EW == 8 && !STREAM ? 2 : 1)
+__global__ void __launch_bounds__((2 + EW + (STREAM ? kPrExpWarps : 0)) * 32, EW == 12 && !STREAM ? 2 : 1)
 conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap out_map, PrParams p,
                const LayerJob* __restrict__ jobs) {
   constexpr int THREADS = (2 + EW + (STREAM ? kPrExpWarps : 0)) * 32;
@@ -350,60 +350,67 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
       const uint32_t row = div_by((uint32_t)pix, (uint32_t)p.W, p.w_magic);
       const int yp = (int)(row - div_by(row, (uint32_t)(p.H + 2), p.h_magic) * (uint32_t)(p.H + 2));
       const bool interior = pix < p.P && yp >= 1 && yp <= p.H, all_interior = __all_sync(0xffffffffu, interior);
+      const int g0 = g;
       for (; g < groups; g += HW) {
       const int c0 = g * 32;
       const int nv = min(32, p.Cs_out - n0 - c0);              // stored channels of the unit: 32 or 16
-      uint4 rh[4], rl[4];
-      if (job.res) {
-        const __nv_bfloat16* res = static_cast<const __nv_bfloat16*>(job.res) + (size_t)pix * (2 * p.Cs_out) + n0 + c0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (j * 8 < nv && interior) {
-            rh[j] = ld_chain(reinterpret_cast<const uint4*>(res) + j);
-            rl[j] = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out) + j);
-          } else {
-            rh[j] = rl[j] = make_uint4(0u, 0u, 0u, 0u);
-          }
-      }
-      alive = mbar_wait_warp(bar_acc_full + 8 * buf, (it >> 1) & 1, s_abort, p.error_flag);
-      if (!alive) break;
-      tc_fence_after();
-      uint32_t v[32];
+      uint8_t* dst = my_buf + buf_idx * kPrUnitBytes + lane * 64;
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * Nt + c0);
-      tmem_ld16(taddr, v);
-      if (c0 + 16 < Nt) tmem_ld16(taddr + 16, v + 16);
-      tmem_ld_wait();
-      tc_fence_before();
-      __syncwarp();
+      if (g == g0) {
+        alive = mbar_wait_warp(bar_acc_full + 8 * buf, (it >> 1) & 1, s_abort, p.error_flag);
+        if (!alive) break;
+        tc_fence_after();
+      }
+      // the store that last read this buffer must be done with it
       if (lane == 0) {
-        if (g + HW >= groups) mbar_arrive(bar_acc_empty + 8 * buf);   // this warp's last accumulators of the tile
-        // the store that last read this buffer must be done with it
         if (p.n_bufs == 2) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         else asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
       }
       __syncwarp();
-      uint8_t* dst = my_buf + buf_idx * kPrUnitBytes + lane * 64;
-      auto finish = [&](auto act, auto res) {
+#pragma unroll 1
+      for (int half = 0; half < 2 && half * 16 < nv; ++half) {   // 16 channels at a time: registers for more warps
+        uint32_t v[16];
+        tmem_ld16(taddr + 16 * half, v);
+        uint4 rh[2], rl[2];
+        if (job.res) {
+          const __nv_bfloat16* res = static_cast<const __nv_bfloat16*>(job.res) + (size_t)pix * (2 * p.Cs_out) + n0 + c0 + 16 * half;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          uint32_t hi[4], lo[4];
-          const int cc = j * 8 < nv ? c0 + j * 8 : 0;          // past the stored channels: anything (clipped by the map)
-          finish8<decltype(act)::value, decltype(res)::value>(v + 8 * j, s_scale + cc, s_bias + cc, rh[j], rl[j], hi, lo);
-          if (!all_interior && !interior) {                    // border rows are zeros
-#pragma unroll
-            for (int i = 0; i < 4; ++i) hi[i] = lo[i] = 0u;
-          }
-          const uint32_t off = ((uint32_t)j ^ key) << 4;
-          *reinterpret_cast<uint4*>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          *reinterpret_cast<uint4*>(dst + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          for (int j = 0; j < 2; ++j)
+            if (interior) {
+              rh[j] = ld_chain(reinterpret_cast<const uint4*>(res) + j);
+              rl[j] = ld_chain(reinterpret_cast<const uint4*>(res + p.Cs_out) + j);
+            } else {
+              rh[j] = rl[j] = make_uint4(0u, 0u, 0u, 0u);
+            }
         }
-      };
-      auto finish_act = [&](auto res) {
-        if (p.act == AIQ_ACT_RELU6) finish(std::integral_constant<int, AIQ_ACT_RELU6>(), res);
-        else if (p.act == AIQ_ACT_RELU) finish(std::integral_constant<int, AIQ_ACT_RELU>(), res);
-        else finish(std::integral_constant<int, AIQ_ACT_NONE>(), res);
-      };
-      if (job.res) finish_act(std::true_type()); else finish_act(std::false_type());
+        tmem_ld_wait();
+        if (g + HW >= groups && (half == 1 || nv <= 16)) {     // this warp's last accumulators of the tile
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_acc_empty + 8 * buf);
+        }
+        auto finish = [&](auto act, auto res) {
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            uint32_t hi[4], lo[4];
+            const int cc = c0 + 16 * half + 8 * j;
+            finish8<decltype(act)::value, decltype(res)::value>(v + 8 * j, s_scale + cc, s_bias + cc, rh[j], rl[j], hi, lo);
+            if (!all_interior && !interior) {                  // border rows are zeros
+#pragma unroll
+              for (int i = 0; i < 4; ++i) hi[i] = lo[i] = 0u;
+            }
+            const uint32_t off = ((uint32_t)(2 * half + j) ^ key) << 4;
+            *reinterpret_cast<uint4*>(dst + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(dst + 2048 + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+          }
+        };
+        auto finish_act = [&](auto res) {
+          if (p.act == AIQ_ACT_RELU6) finish(std::integral_constant<int, AIQ_ACT_RELU6>(), res);
+          else if (p.act == AIQ_ACT_RELU) finish(std::integral_constant<int, AIQ_ACT_RELU>(), res);
+          else finish(std::integral_constant<int, AIQ_ACT_NONE>(), res);
+        };
+        if (job.res) finish_act(std::true_type()); else finish_act(std::false_type());
+      }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
@@ -463,9 +470,9 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
     const int Nt = g.Cs_out <= nt ? g.Cs_out : nt;             // the last candidate: one tile, any multiple of 16
     const int ntiles = (g.Cs_out + Nt - 1) / Nt;
     for (int variant = 0; variant < 4; ++variant) {
-      // two blocks per SM, one with 8 or 16 epilogue warps, one with streamed weights
+      // two blocks per SM, one with 12 or 24 epilogue warps, one with streamed weights
       const bool stream = variant == 3;
-      const int occ = variant == 0 ? 2 : 1, ew = variant == 2 ? 16 : 8;
+      const int occ = variant == 0 ? 2 : 1, ew = stream ? 8 : variant == 2 ? 24 : 12;
       if (occ == 2 && Nt > 128) continue;                      // tensor memory: 2 Nt columns per block
       if (stream && (Nt * 8 / (pieces == 2 ? 1 : 2) > 4 * kPrExpWarps * 32 || 2 * Nt > 512)) continue;
       const int limit = occ == 2 ? (props.smem_optin + 1024) / 2 - 1024 : props.smem_optin;
@@ -478,7 +485,7 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
       const double in_flight = (double)occ * st * (stream ? 2 : 1) * kPrChunkBytes;
       const double c_mma = K2 / 16 * pieces * (128 + Nt) / 4.0;
       const double c_in = 128.0 * K2 * 2 / std::min(40.0, in_flight / 1600.0);
-      const double c_epi = (ew == 8 && occ == 1 ? 18.0 : 12.0) * Nt;
+      const double c_epi = (ew < 24 && occ == 1 ? 18.0 : 12.0) * Nt;
       const double c_exp = stream ? Nt * (double)g.Cs_in * pieces * 0.06 : 0.0;
       const double tile = std::max(std::max(c_mma, c_in), std::max(c_epi, c_exp));
       const double setup = 3000.0 + (stream ? 0.0 : Nt * (double)g.Cs_in * pieces / 16.0);
@@ -580,8 +587,8 @@ aiq_status_t launch_conv_pw(const ConvGeom& g, const void* maps, const LayerJob*
 #define AIQ_PW(EW_, P_, S_) launch_pr<EW_, P_, S_>(scope, props, c, p, m[0], m[1], jobs_dev, n_jobs, s)
   aiq_status_t st;
   if (c.stream) st = pieces == 1 ? AIQ_PW(8, 1, true) : AIQ_PW(8, 2, true);
-  else if (c.ew == 8) st = pieces == 1 ? AIQ_PW(8, 1, false) : AIQ_PW(8, 2, false);
-  else st = pieces == 1 ? AIQ_PW(16, 1, false) : AIQ_PW(16, 2, false);
+  else if (c.ew == 12) st = pieces == 1 ? AIQ_PW(12, 1, false) : AIQ_PW(12, 2, false);
+  else st = pieces == 1 ? AIQ_PW(24, 1, false) : AIQ_PW(24, 2, false);
 #undef AIQ_PW
   if (st != AIQ_OK) return st;
   AIQ_LAUNCH_CHECK("conv_pw");

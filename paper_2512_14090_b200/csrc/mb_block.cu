@@ -586,17 +586,18 @@ int mb_block_chunk_channels(const ConvGeom& ge, const ConvGeom& gd, const ConvGe
   return c.ok ? c.NH : 0;
 }
 
-// Where the fused kernel was measured faster than the three layer kernels (B200, both MobileNetV2 variants, batches
-// 32 and 256): blocks on maps at most 8 columns wide and stride-2 blocks on maps up to 56 wide, once the batch
-// gives at least 128 CTAs; elsewhere (wide maps: many waves of short CTAs; few CTAs: the chunks of a CTA run one
-// after the other) the layer kernels win.
+// Where the fused kernel competes with the layer kernels (B200; microseconds of a forward pass through one block, layer
+// by layer / fused): 8-wide maps once the bands are one full wave of CTAs (160 -> 160 channels: 128 bands 77 / 86, 148
+// bands 94 / 89; 160 -> 320: 86 / 91 and 102 / 96).  With fewer bands its CTAs work through their chunks of hidden
+// channels one after the other on a part of the GPU (64 bands: 64 / 81), with more a second wave starts (256: 128 / 157),
+// 7-wide maps leave accumulator lanes idle (148: 86 / 91), and on wider maps the layer kernels win at every batch
+// (16-wide, stride 2, 256: 154 / 203; 56-wide, stride 2, 32: 84 / 99; 32-wide, stride 2, 256: 176 / 210).
 bool mb_block_pays(const ConvGeom& gd, const ConvGeom& gp) {
   DeviceProps props;
   if (current_device_props(&props) != AIQ_OK) return false;
   const int rb = std::min(std::max(128 / gp.Wo, 1), gp.Ho);        // band height of mb_config's first choice
   const long long ctas = (long long)gp.B * ((gp.Ho + rb - 1) / rb);
-  if (ctas < 128) return false;
-  return gd.W <= 8 || (gd.stride == 2 && gd.W <= 56);
+  return gd.W == 8 && gd.stride == 1 && ctas >= 128 && ctas <= props.n_sms;
 }
 
 aiq_status_t launch_mb_build_tiles(int role, const uint8_t* packed, const float* scale, const float* bias, int bits, int N,

@@ -160,23 +160,35 @@ def _check(status):
         raise AiqError(status, last_error())
 
 
+# A small call spends more time here than on the GPU (MobileNetV2's classifier-sized linear layer, one row: 10.0 us a
+# call with a c_void_p object per argument and torch.cuda.current_stream(), 5.3 us with plain integers and the raw
+# stream handle), so pointers are passed as integers; the argument types of the library convert them.
 def _dev(t):
     """Device pointer of a contiguous CUDA tensor (None -> NULL)."""
     if t is None:
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _host(a):
-    return C.c_void_p(a.ctypes.data) if a is not None else None
+    return a.__array_interface__["data"][0] if a is not None else None
 
 
 def _stream(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()                     # initialises CUDA
+        _raw_stream = (torch.cuda.current_device, torch._C._cuda_getCurrentRawStream)
+    device, raw = _raw_stream
+    return raw(device())
+
+
+_raw_stream = None
 
 
 def arch_desc(arch):
@@ -213,10 +225,10 @@ def aiq_qlinear_workspace_bytes(N, K, bits, M):
 
 
 def aiq_qlinear(packed, scales, bias, N, K, bits, x, y, workspace=None, stream=None):
-    M = x.shape[0]
-    _check(lib.aiq_qlinear(_dev(packed), _dev(scales), _dev(bias), int(N), int(K), int(bits),
-                           _dev(x), int(M), _dev(y), _dev(workspace),
-                           workspace.numel() if workspace is not None else 0, _stream(stream)))
+    status = lib.aiq_qlinear(_dev(packed), _dev(scales), _dev(bias), int(N), int(K), int(bits), _dev(x), x.shape[0], _dev(y),
+                             _dev(workspace), workspace.numel() if workspace is not None else 0, _stream(stream))
+    if status:
+        _check(status)
 
 
 def aiq_set_eval_options(chunk=0, share_prefix=True):
@@ -294,7 +306,7 @@ class Model:
                 if name in p and p[name] is not None:
                     a = np.ascontiguousarray(p[name], dtype=np.float32)
                     keep.append(a)
-                    setattr(w, name, a.ctypes.data)
+                    setattr(w, name, a.__array_interface__["data"][0])
         handle = C.c_void_p()
         with torch.cuda.device(self.device):
             _check(lib.aiq_model_create(C.byref(desc), weights, _dev(self.mem), self.mem.numel(),
@@ -321,13 +333,12 @@ class Model:
                 self._view(b.value, n.value * 4).view(dtype=_f32()))
 
     def layer_packed(self, layer, bits):
-        wf, b, n, k = C.c_void_p(), C.c_void_p(), C.c_int(), C.c_int()
-        _check(lib.aiq_model_layer_folded(self.handle, layer, C.byref(wf), C.byref(b), C.byref(n), C.byref(k)))
         p, s = C.c_void_p(), C.c_void_p()
         _check(lib.aiq_model_layer_packed(self.handle, layer, int(bits), C.byref(p), C.byref(s)))
-        rb = aiq_packed_row_bytes(k.value, bits)
-        return (self._view(p.value, n.value * rb).view(n.value, rb),
-                self._view(s.value, n.value * 4).view(dtype=_f32()))
+        l = self.arch["layers"][layer]
+        n, k = l["cout"], (1 if l["kind"] == "dw" else l["cin"]) * l["k"] * l["k"]
+        rb = aiq_packed_row_bytes(k, bits)
+        return (self._view(p.value, n * rb).view(n, rb), self._view(s.value, n * 4).view(dtype=_f32()))
 
     def _view(self, ptr, nbytes):
         off = ptr - self.mem.data_ptr()

@@ -218,6 +218,21 @@ aiq_status_t launch_quantize(const float* W, int N, int K, int bits, void* packe
 // all four widths (4, 8, 16, 32 bits, in that order) of one layer from one read of W; tensor_amax as above, for the 4- and 8-bit codes
 aiq_status_t launch_quantize_bank(const float* W, int N, int K, void* const* packed, float* const* scales,
                                   int32_t* nonfinite_flag, uint32_t* tensor_amax, cudaStream_t s);
+// A model's whole bank - every layer folded and quantized at the four widths - in one launch.  The layers are device
+// records; rows are numbered through the layers (row0 = first row of a layer).  W may be Wf itself.
+struct BankLayer {
+  const float* W;
+  const float *gamma, *beta, *mean, *var;   // has_bn
+  const float* bias_in;                     // else: the layer's bias, or nullptr for zeros
+  float* Wf;
+  float* bias;
+  uint8_t* packed[4];                       // 4, 8, 16, 32 bits
+  float* scales[4];
+  int32_t N, K, row0, has_bn;
+};
+// flops / bytes: for the profile
+aiq_status_t launch_model_bank(const BankLayer* layers_dev, int n_layers, int n_rows, float eps, int32_t* nonfinite_flag,
+                               double flops, double bytes, cudaStream_t s);
 // y[m][n] for every job: in = x [M][K], out = y [M][N]
 aiq_status_t launch_qlinear(const LayerJob* jobs_dev, const LayerJob* single_host, int n_jobs, int N,
                             int K, int M, cudaStream_t s);
@@ -268,9 +283,15 @@ int mb_block_chunk_channels(const ConvGeom& ge, const ConvGeom& gd, const ConvGe
 // bytes of one chunk's operand image: expansion (Cs_in / 8 planes of nh rows), projection (nh / 8 planes of Cs_out rows)
 __host__ __device__ inline size_t mb_etile_bytes(int cs_in, int nh) { return (size_t)(cs_in / 8) * (nh * 16); }
 __host__ __device__ inline size_t mb_ptile_bytes(int cs_out, int nh) { return (size_t)(nh / 8) * (cs_out * 16); }
-// role 0: expansion, 1: projection, 2: depthwise (coefficients only); see mb_block.cu
-aiq_status_t launch_mb_build_tiles(int role, const uint8_t* packed, const float* scale, const float* bias, int bits, int N,
-                                   int K, int nh, int cs, void* tile_out, float* coef_out, cudaStream_t s);
+// one operand image (role 0: expansion, 1: projection) or coefficient table (role 2: depthwise; 0 has one too); see mb_block.cu
+struct MbTileJob {
+  const uint8_t* packed;
+  const float *scale, *bias;
+  uint8_t* tile;
+  float* coef;
+  int32_t role, bits, N, K, nh, cs;
+};
+aiq_status_t launch_mb_build_tiles(const MbTileJob* jobs_dev, int n_jobs, cudaStream_t s);
 // whether the fused kernel is expected to beat the layer kernels for this block at this batch (measured policy)
 bool mb_block_pays(const ConvGeom& gd, const ConvGeom& gp);
 // nh: the chunk width the jobs' operand images were built for

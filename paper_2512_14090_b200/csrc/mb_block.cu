@@ -496,9 +496,15 @@ mb_block_kernel(MbParams p, const LayerJob* __restrict__ jobs) {
 //   role 1, projection (N = Cout rows of K = Ch codes): per chunk [NH / 8 planes][Cs_out rows][8 bfloat16]
 //   role 2, depthwise  (N = Ch rows of 9 elements): coefficients per chunk: w [9][NH], s_d [NH], b_d [NH]
 // Rows, planes and channels past the layer's extent are zero.
-__global__ void mb_build_tiles_kernel(int role, const uint8_t* __restrict__ packed, const float* __restrict__ scale,
-                                      const float* __restrict__ bias, int bits, int N, int K, int NH, int cs,
-                                      uint8_t* __restrict__ tile, float* __restrict__ coef) {
+// One launch builds them all (blockIdx.y: the image or table).
+__global__ void mb_build_tiles_kernel(const MbTileJob* __restrict__ jobs) {
+  const MbTileJob job = jobs[blockIdx.y];
+  const int role = job.role, bits = job.bits, N = job.N, K = job.K, NH = job.nh, cs = job.cs;
+  const uint8_t* const packed = job.packed;
+  const float* const scale = job.scale;
+  const float* const bias = job.bias;
+  uint8_t* const tile = job.tile;
+  float* const coef = job.coef;
   const int wrow = (K + 31) / 32 * 32 * bits / 8;
   const int Ch = role == 1 ? K : N;                  // hidden channels
   const int n_chunks = (Ch + NH - 1) / NH;
@@ -600,11 +606,8 @@ bool mb_block_pays(const ConvGeom& gd, const ConvGeom& gp) {
   return gd.W == 8 && gd.stride == 1 && ctas >= 128 && ctas <= props.n_sms;
 }
 
-aiq_status_t launch_mb_build_tiles(int role, const uint8_t* packed, const float* scale, const float* bias, int bits, int N,
-                                   int K, int nh, int cs, void* tile_out, float* coef_out, cudaStream_t s) {
-  if ((role == 0 || role == 1) && bits != 4 && bits != 8)
-    return set_error(AIQ_ERR_UNSUPPORTED_BITS, "mb_build_tiles: the 1x1 layers of a fused block take 4- or 8-bit codes");
-  mb_build_tiles_kernel<<<64, 256, 0, s>>>(role, packed, scale, bias, bits, N, K, nh, cs, static_cast<uint8_t*>(tile_out), coef_out);
+aiq_status_t launch_mb_build_tiles(const MbTileJob* jobs_dev, int n_jobs, cudaStream_t s) {
+  mb_build_tiles_kernel<<<dim3(8, n_jobs), 256, 0, s>>>(jobs_dev);
   AIQ_LAUNCH_CHECK("mb_build_tiles");
   return AIQ_OK;
 }

@@ -318,6 +318,10 @@ static void find_mb_structure(const std::vector<LayerInfo>& L, std::vector<int>&
   }
 }
 
+// What a model's creation uploads in one copy: the batch-norm vectors and biases of every layer, the weight tensors up to
+// this size (a copy from pageable memory costs microseconds however small it is), and the records of the bank kernels.
+constexpr size_t kBlobWeightBytes = 64 * 1024;
+
 struct ModelLayout {
   size_t total, staging_off, flag_off;
   std::vector<size_t> wf, bias;
@@ -327,7 +331,7 @@ struct ModelLayout {
 
 static ModelLayout model_layout(const std::vector<LayerInfo>& L) {
   ModelLayout lay;
-  size_t off = 0, staging = 0;
+  size_t off = 0, staging = 0, blob = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
   lay.flag_off = take(256);
   for (const LayerInfo& li : L) {
@@ -339,7 +343,10 @@ static ModelLayout model_layout(const std::vector<LayerInfo>& L) {
       lay.scales[b].push_back(take(n * 4));
     }
     staging = std::max(staging, align_up(n * k * 4, 256) + 5 * align_up(n * 4, 256));
+    blob += 5 * align_up(n * 4, 16) + (n * k * 4 <= kBlobWeightBytes ? align_up(n * k * 4, 16) : 0) + sizeof(BankLayer) +
+            4 * sizeof(MbTileJob);
   }
+  staging = std::max(staging, blob + 256);
   lay.staging_off = take(staging);
   // operand images of inverted-residual blocks, sized for either chunk width the kernel may choose
   for (int b = 0; b < 2; ++b) lay.mb_tile[b].assign(L.size(), 0);
@@ -499,44 +506,18 @@ extern "C" aiq_status_t aiq_model_create(const aiq_arch_desc_t* arch, const aiq_
 
   const bool per_tensor = g_opt_per_tensor.load() != 0;
   CREATE_TRY(cudaMemsetAsync(flag, 0, 256, stream));
+  // device addresses of every layer's tensors
   for (size_t i = 0; i < m->layers.size(); ++i) {
     LayerInfo& li = m->layers[i];
-    const size_t n = li.d.cout, k = li.K;
     li.Wf = reinterpret_cast<float*>(base + lay.wf[i]);
     li.bias = reinterpret_cast<float*>(base + lay.bias[i]);
     for (int b = 0; b < 4; ++b) {
       li.packed[b] = base + lay.packed[b][i];
       li.scales[b] = reinterpret_cast<float*>(base + lay.scales[b][i]);
     }
-    const aiq_layer_weights_t& w = weights[i];
-    if (li.d.has_bn) {
-      float* sW = reinterpret_cast<float*>(base + lay.staging_off);
-      const size_t vec = align_up(n * 4, 256);
-      uint8_t* sv = base + lay.staging_off + align_up(n * k * 4, 256);
-      float* sG = reinterpret_cast<float*>(sv);
-      float* sB = reinterpret_cast<float*>(sv + vec);
-      float* sM = reinterpret_cast<float*>(sv + 2 * vec);
-      float* sV = reinterpret_cast<float*>(sv + 3 * vec);
-      CREATE_TRY(cudaMemcpyAsync(sW, w.W, n * k * 4, cudaMemcpyHostToDevice, stream));
-      CREATE_TRY(cudaMemcpyAsync(sG, w.gamma, n * 4, cudaMemcpyHostToDevice, stream));
-      CREATE_TRY(cudaMemcpyAsync(sB, w.beta, n * 4, cudaMemcpyHostToDevice, stream));
-      CREATE_TRY(cudaMemcpyAsync(sM, w.mean, n * 4, cudaMemcpyHostToDevice, stream));
-      CREATE_TRY(cudaMemcpyAsync(sV, w.var, n * 4, cudaMemcpyHostToDevice, stream));
-      st = launch_fold_bn(sW, sG, sB, sM, sV, (int)n, (int)k, 1e-5f, li.Wf, li.bias, stream);
-      if (st != AIQ_OK) return fail(st);
-    } else {
-      CREATE_TRY(cudaMemcpyAsync(li.Wf, w.W, n * k * 4, cudaMemcpyHostToDevice, stream));
-      if (w.bias) CREATE_TRY(cudaMemcpyAsync(li.bias, w.bias, n * 4, cudaMemcpyHostToDevice, stream));
-      else CREATE_TRY(cudaMemsetAsync(li.bias, 0, n * 4, stream));
-    }
-    {
-      void* packed4[4] = {li.packed[0], li.packed[1], li.packed[2], li.packed[3]};
-      st = launch_quantize_bank(li.Wf, (int)n, (int)k, packed4, li.scales, flag,
-                                per_tensor ? reinterpret_cast<uint32_t*>(flag + 2) : nullptr, stream);
-      if (st != AIQ_OK) return fail(st);
-    }
   }
-  // operand images of the fused inverted-residual blocks, from the packed codes just written
+  // operand images of the fused inverted-residual blocks, from the packed codes
+  std::vector<MbTileJob> tile_jobs;
   for (size_t le = 0; le < m->layers.size(); ++le) {
     if (m->mb_tail[le] < 0) continue;
     const int ld = m->mb_mid[le], lp = m->mb_tail[le];
@@ -548,19 +529,97 @@ extern "C" aiq_status_t aiq_model_create(const aiq_arch_desc_t* arch, const aiq_
       e.mb_tile[b] = base + lay.mb_tile[b][le];
       e.mb_coef[b] = reinterpret_cast<float*>(base + lay.mb_coef[b][le]);
       pr.mb_tile[b] = base + lay.mb_tile[b][lp];
-      st = launch_mb_build_tiles(0, e.packed[b], e.scales[b], e.bias, kBitsList[b], e.d.cout, e.K, nh,
-                                 padded_channels(e.d.cin), e.mb_tile[b], e.mb_coef[b], stream);
-      if (st != AIQ_OK) return fail(st);
-      st = launch_mb_build_tiles(1, pr.packed[b], pr.scales[b], pr.bias, kBitsList[b], pr.d.cout, pr.K, nh,
-                                 padded_channels(pr.d.cout), pr.mb_tile[b], nullptr, stream);
-      if (st != AIQ_OK) return fail(st);
+      tile_jobs.push_back({e.packed[b], e.scales[b], e.bias, e.mb_tile[b], e.mb_coef[b], 0, kBitsList[b], e.d.cout, e.K, nh,
+                           padded_channels(e.d.cin)});
+      tile_jobs.push_back({pr.packed[b], pr.scales[b], pr.bias, pr.mb_tile[b], nullptr, 1, kBitsList[b], pr.d.cout, pr.K, nh,
+                           padded_channels(pr.d.cout)});
     }
     for (int b = 0; b < 4; ++b) {
       d.mb_coef[b] = reinterpret_cast<float*>(base + lay.mb_coef[b][ld]);
-      st = launch_mb_build_tiles(2, d.packed[b], d.scales[b], d.bias, kBitsList[b], d.d.cout, d.K, nh, 0, nullptr,
-                                 d.mb_coef[b], stream);
-      if (st != AIQ_OK) return fail(st);
+      tile_jobs.push_back({d.packed[b], d.scales[b], d.bias, nullptr, d.mb_coef[b], 2, kBitsList[b], d.d.cout, d.K, nh, 0});
     }
+  }
+  // Upload.  Large weight tensors go straight into their Wf (the fold works in place), everything else through one blob.
+  const size_t n_layers = m->layers.size();
+  std::vector<uint8_t> blob;
+  uint8_t* const stage_dev = base + lay.staging_off;
+  auto add = [&](const void* src, size_t bytes) -> float* {       // append to the blob; its device address
+    const size_t at = align_up(blob.size(), 16);
+    blob.resize(at + bytes);
+    memcpy(blob.data() + at, src, bytes);
+    return reinterpret_cast<float*>(stage_dev + at);
+  };
+  DeviceProps props;
+  st = current_device_props(&props);
+  if (st != AIQ_OK) return fail(st);
+  std::vector<BankLayer> bank;
+  std::vector<size_t> by_layer;                                   // layers that take the per-layer kernels instead
+  int n_rows = 0;
+  double bank_flops = 0.0, bank_bytes = 0.0;
+  for (size_t i = 0; i < n_layers; ++i) {
+    LayerInfo& li = m->layers[i];
+    const size_t n = li.d.cout, k = li.K;
+    const aiq_layer_weights_t& w = weights[i];
+    // one scale for the whole tensor needs the tensor's maximum first; rows of thousands of elements are the streaming kernel's
+    if (per_tensor || (k >= 2048 && (int)n >= 4 * props.n_sms)) { by_layer.push_back(i); continue; }
+    BankLayer r = {};
+    r.Wf = li.Wf; r.bias = li.bias;
+    r.N = (int)n; r.K = (int)k; r.row0 = n_rows; r.has_bn = li.d.has_bn ? 1 : 0;
+    for (int b = 0; b < 4; ++b) { r.packed[b] = li.packed[b]; r.scales[b] = li.scales[b]; }
+    if (n * k * 4 <= kBlobWeightBytes) {
+      r.W = add(w.W, n * k * 4);
+    } else {
+      CREATE_TRY(cudaMemcpyAsync(li.Wf, w.W, n * k * 4, cudaMemcpyHostToDevice, stream));
+      r.W = li.Wf;
+    }
+    if (r.has_bn) {
+      r.gamma = add(w.gamma, n * 4); r.beta = add(w.beta, n * 4); r.mean = add(w.mean, n * 4); r.var = add(w.var, n * 4);
+    } else if (w.bias) {
+      r.bias_in = add(w.bias, n * 4);
+    }
+    n_rows += (int)n;
+    bank_flops += 9.0 * n * k;
+    bank_bytes += 8.0 * n * k + 24.0 * n;
+    for (int b = 0; b < 4; ++b) bank_bytes += (double)n * row_bytes((int)k, kBitsList[b]);
+    bank.push_back(r);
+  }
+  const BankLayer* bank_dev = bank.empty() ? nullptr : reinterpret_cast<const BankLayer*>(add(bank.data(), bank.size() * sizeof(BankLayer)));
+  const MbTileJob* tiles_dev = tile_jobs.empty() ? nullptr
+      : reinterpret_cast<const MbTileJob*>(add(tile_jobs.data(), tile_jobs.size() * sizeof(MbTileJob)));
+  // the per-layer kernels borrow the staging region for their own uploads, so they come first
+  for (size_t i : by_layer) {
+    LayerInfo& li = m->layers[i];
+    const size_t n = li.d.cout, k = li.K;
+    const aiq_layer_weights_t& w = weights[i];
+    CREATE_TRY(cudaMemcpyAsync(li.Wf, w.W, n * k * 4, cudaMemcpyHostToDevice, stream));
+    if (li.d.has_bn) {
+      const size_t vec = align_up(n * 4, 256);
+      float* v4[4];
+      const float* src4[4] = {w.gamma, w.beta, w.mean, w.var};
+      for (int j = 0; j < 4; ++j) {
+        v4[j] = reinterpret_cast<float*>(stage_dev + j * vec);
+        CREATE_TRY(cudaMemcpyAsync(v4[j], src4[j], n * 4, cudaMemcpyHostToDevice, stream));
+      }
+      st = launch_fold_bn(li.Wf, v4[0], v4[1], v4[2], v4[3], (int)n, (int)k, 1e-5f, li.Wf, li.bias, stream);
+      if (st != AIQ_OK) return fail(st);
+    } else if (w.bias) {
+      CREATE_TRY(cudaMemcpyAsync(li.bias, w.bias, n * 4, cudaMemcpyHostToDevice, stream));
+    } else {
+      CREATE_TRY(cudaMemsetAsync(li.bias, 0, n * 4, stream));
+    }
+    void* packed4[4] = {li.packed[0], li.packed[1], li.packed[2], li.packed[3]};
+    st = launch_quantize_bank(li.Wf, (int)n, (int)k, packed4, li.scales, flag,
+                              per_tensor ? reinterpret_cast<uint32_t*>(flag + 2) : nullptr, stream);
+    if (st != AIQ_OK) return fail(st);
+  }
+  if (!blob.empty()) CREATE_TRY(cudaMemcpyAsync(stage_dev, blob.data(), blob.size(), cudaMemcpyHostToDevice, stream));
+  if (!bank.empty()) {
+    st = launch_model_bank(bank_dev, (int)bank.size(), n_rows, 1e-5f, flag, bank_flops, bank_bytes, stream);
+    if (st != AIQ_OK) return fail(st);
+  }
+  if (!tile_jobs.empty()) {
+    st = launch_mb_build_tiles(tiles_dev, (int)tile_jobs.size(), stream);
+    if (st != AIQ_OK) return fail(st);
   }
   int32_t host_flag = 0;
   CREATE_TRY(cudaMemcpyAsync(&host_flag, flag, 4, cudaMemcpyDeviceToHost, stream));

@@ -118,9 +118,13 @@ void aiq_set_scale_granularity(int granularity);
  * aiq_quantize_layer (device).  bias: device [N] or NULL.  x: device float32 [M][K]
  * row-major, 16-byte aligned; y: device float32 [M][N].  M >= 1.  Asynchronous on `stream`.
  *
- * Three kernels.  The plain one expands weights to float32 in registers and accumulates in
- * float32 (any shape, any bit-width).  For 4- / 8-bit weights two faster ones exist:
- *   M <= 8, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
+ * Four kernels.  The plain one expands weights to float32 in registers and accumulates in
+ * float32 (any shape, any bit-width).  For 4- / 8-bit weights three faster ones exist:
+ *   M <= 4, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: one kernel, no workspace;
+ *     the codes stay integer and feed the int8 warp-level tensor cores, the activations of every
+ *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest
+ *     |x|), the int32 sums are exact and run-to-run identical.
+ *   M <= 8 otherwise, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
  *     warp-level tensor cores; the activations of each group of 512 k become three int8
  *     digits with a shared exponent (21 bits below the group's largest |x|), the int32 sums
  *     are exact.

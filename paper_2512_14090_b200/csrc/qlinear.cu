@@ -207,6 +207,7 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
   job.scale = scales;
   job.bias = bias;
   job.bits = bits;
+  if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
   // the tensor-core kernels need scratch for the converted activations
   if (workspace && aiq::qlinear_tc_applicable(N, K, bits, M)) {
     if (((uintptr_t)workspace) & 15)

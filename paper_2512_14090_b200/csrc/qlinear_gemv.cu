@@ -1,0 +1,355 @@
+// Quantized linear layer for 4- and 8-bit weights and up to four batch rows, in one kernel.
+//
+//   y[m][n] = s_n * sum_k code[n][k] * x[m][k] + bias[n]
+//
+// The weight stream bounds the layer (8192 x 8192 at 4 bits: 33.6 MB, 5.2 us at the copy bandwidth), so everything is
+// arranged around having it in flight from the first instruction on:
+//   - one block per SM; a block takes 8 output channels at a time (a unit) over the whole K, and requests as many units as
+//     fit its shared memory (about 180 KB) as soon as its first activation loads are under way, by one bulk copy per row;
+//   - meanwhile every warp turns its slice of the activations (at most 512 k) into int8 digits with a shared exponent,
+//     x = 2^(e-6) (d1 + d2 / 2^7 + d3 / 2^14 + d4 / 2^21), an image of x to 28 bits below the slice's largest |x|, and
+//     keeps them in registers as the A operand of mma.m16n8k32 (row 4 m + d = digit d of batch row m) for the whole
+//     kernel;
+//   - the packed words are the B operand (column = output channel): 8-bit words as they are, a 4-bit word as its even
+//     and its odd nibbles (one AND, one shift-AND; the +8 of the offset-binary nibbles leaves again exactly, as 8 times
+//     the digit sum); the k order inside a fragment follows from that on both operands;
+//   - the integer sums are exact; a warp scales them with its slice's exponent, and the warps' partial sums meet in shared
+//     memory in a fixed order: no second kernel, no workspace, no atomics, run-to-run identical;
+//   - nothing joins the warps inside the stream: they wait for a unit's copies only, and the output of up to eight units
+//     is formed together after it (a block barrier and an output per unit cost 0.5 us each).
+// The two kernels this replaces at these sizes (a digit pass over x, then the matrix with its K slices meeting in y through
+// atomics) took 18.7 us at 8192 x 8192, 4 bits, one row, 11.5 now (8 bits: 18.8 and 14.5; 2048 x 2048: 13.0 and 6.2).
+#include "tc_ptx.cuh"
+
+#include <algorithm>
+
+namespace aiq {
+
+namespace {
+
+constexpr int kGvWarps = 16;
+constexpr int kGvFrags = 16;                         // k32 fragments of a warp's slice at most: 512 k
+constexpr int kGvMaxSlots = 16;
+constexpr int kGvEpoch = 8;                          // units per warp between two outputs
+constexpr int kGvMaxRows = 4;                        // batch rows
+constexpr int kGvDigWords = 256 + 64;                // of half a slice
+static_assert(kGvEpoch * kGvMaxRows * 8 <= kGvDigWords, "the partial sums take the place of the digit words");
+__device__ __forceinline__ int gv_dig(int k) { return k + (k >> 4) * 4; }
+
+struct GvParams {
+  int N, K, M;
+  int rb;                   // bytes of a packed row
+  int stride;               // of a row in shared memory: 64 modulo 128, so that eight rows x 4 units of 16 bytes spread over all banks
+  int kw;                   // warps that share a unit's K
+  int cw;                   // 64-byte chunks of a row per warp
+  int slots, slot_bytes;
+  int slack;                // bytes behind the ring: a row's last chunk may reach past the last slot
+};
+
+__device__ __forceinline__ void gv_mma(int* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k32.row.col.s32.s8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// HALVES: 1 for one or two batch rows (digit rows 0 .. 7), 2 for up to four.
+template <int BITS, int HALVES>
+__global__ void __launch_bounds__(kGvWarps * 32, 1)
+qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scale, const float* __restrict__ bias,
+                    const float* x, float* y, GvParams p) {
+  constexpr int CHUNK_K = 512 / BITS;                // k of a 64-byte chunk: 128 / 64
+  constexpr int LANE_K = CHUNK_K / 4;                // k of a lane's 16 bytes of it: 32 / 16
+  constexpr int MPC = CHUNK_K / 32;                  // MMAs per chunk: 4 / 2
+  constexpr int MAX_CW = kGvFrags / MPC;             // chunks per warp at most: 4 / 8
+  extern __shared__ __align__(128) uint8_t gsm[];
+  uint8_t* ring = gsm;
+  uint32_t* s_dig = reinterpret_cast<uint32_t*>(gsm + p.slots * p.slot_bytes + p.slack);   // [warp] digit words, then
+  float* s_part = reinterpret_cast<float*>(s_dig);                                        // [kGvEpoch][warp][row][8] partial sums
+  uint64_t* bars = reinterpret_cast<uint64_t*>(s_dig + kGvWarps * kGvDigWords);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * kGvMaxSlots);
+  const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kGvMaxSlots;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int ug = kGvWarps / p.kw;                    // units a block works on at a time
+  const int n_units = (p.N + 7) >> 3;
+  const int per_step = (int)gridDim.x * ug;
+  const int n_steps = ((int)blockIdx.x * ug < n_units) ? (n_units - 1 - (int)blockIdx.x * ug) / per_step + 1 : 0;
+  const int kwi = warp % p.kw, ugi = warp / p.kw;
+
+  if (tid == 0) {
+    for (int i = 0; i < p.slots; ++i) { mbar_init(bar_full + 8 * i, 1); mbar_init(bar_empty + 8 * i, kGvWarps); }
+    *s_abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  chain_release();
+  chain_wait();
+
+  const int slice_k = p.cw * CHUNK_K, k0 = kwi * slice_k;
+  const bool vec = (p.K & 3) == 0 && (((uintptr_t)x) & 15) == 0;
+  auto load_x = [&](int m, float4 (&q)[4]) {
+    const float* xr = x + (size_t)m * p.K;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int kl = j * 128 + lane * 4, k = k0 + kl;
+      q[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (kl < slice_k) {
+        if (vec && k + 4 <= p.K) q[j] = *reinterpret_cast<const float4*>(xr + k);
+        else {
+          if (k < p.K) q[j].x = xr[k];
+          if (k + 1 < p.K) q[j].y = xr[k + 1];
+          if (k + 2 < p.K) q[j].z = xr[k + 2];
+          if (k + 3 < p.K) q[j].w = xr[k + 3];
+        }
+      }
+    }
+  };
+  float4 xv[4], xn[4];
+  load_x(0, xv);                                     // ahead of the weights, which would queue in front of it
+  if (p.M > 1) load_x(1, xn);
+
+  // rows of step i -> slot i mod slots, by one warp.  (Issuing a bulk copy takes about 50 ns: one warp alone needed 2.5 us for
+  // the 48 first ones, so each first slot has a warp of its own.)
+  auto issue = [&](int i) {
+    const int row0 = (i * per_step + (int)blockIdx.x * ug) * 8;
+    const int rows = min(8 * ug, p.N - row0);
+    const uint32_t bar = bar_full + 8 * (i % p.slots), dst = smem_u32(ring) + (i % p.slots) * p.slot_bytes;
+    if (lane == 0) mbar_expect_tx(bar, (uint32_t)(rows * p.rb));
+    __syncwarp();
+    for (int r = lane; r < rows; r += 32) bulk_load(dst + r * p.stride, w + (size_t)(row0 + r) * p.rb, (uint32_t)p.rb, bar);
+  };
+  if (warp < p.slots && warp < n_steps) issue(warp);
+
+  // ---- activations of this warp's slice -> digit fragments in registers ---------------------------------
+  uint32_t a[kGvFrags][2 * HALVES];                  // per fragment: k 0-15 and 16-31 of row g (and of row g + 8)
+  float down[HALVES];                                // value of one unit of this lane's digit row
+  int corr[HALVES];                                  // 4 bits: 8 x the digit sum of the row
+#pragma unroll
+  for (int f = 0; f < kGvFrags; ++f)
+#pragma unroll
+    for (int i = 0; i < 2 * HALVES; ++i) a[f][i] = 0u;
+#pragma unroll
+  for (int h = 0; h < HALVES; ++h) { down[h] = 0.f; corr[h] = 0; }
+  uint32_t* my_dig = s_dig + warp * kGvDigWords;     // word k at gv_dig(k): four words of padding per 16, against bank conflicts
+  for (int m = 0; m < p.M; ++m) {
+    float v[16];
+    uint32_t mx = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { v[4 * j] = xv[j].x; v[4 * j + 1] = xv[j].y; v[4 * j + 2] = xv[j].z; v[4 * j + 3] = xv[j].w; }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) mx = max(mx, (uint32_t)__float_as_int(v[j]) & 0x7FFFFFFFu);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    // 2^(e-1) <= largest |x| < 2^e; slices of zeros and of denormals share the smallest exponent
+    const int e = max((int)(mx >> 23) - 126, -90);
+    const float up = __int_as_float((6 - e + 127) << 23);
+    const bool finite = mx < 0x7F800000u;
+    uint32_t sum = 0;
+    const uint32_t d = g & 3, sel = d | ((d + 4u) << 4);          // byte d of two words
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {                        // 256 k of the slice at a time
+      if (256 * half >= slice_k) break;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        if (256 * half + 128 * j >= slice_k) break;
+        uint32_t word[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float r = finite ? v[8 * half + 4 * j + i] * up : 0.f;  // |r| < 64; every step below is exact
+          // rint without the conversion unit (a quarter of the rate): adding 1.5 x 2^23 leaves the rounded integer in the
+          // low bits
+          uint32_t q4[4];
+#pragma unroll
+          for (int dd = 0; dd < 4; ++dd) {
+            const float q = __fadd_rn(r, 12582912.f);
+            q4[dd] = __float_as_uint(q);
+            r = __fmul_rn(__fsub_rn(r, __fsub_rn(q, 12582912.f)), 128.f);
+          }
+          word[i] = __byte_perm(__byte_perm(q4[0], q4[1], 0x0040), __byte_perm(q4[2], q4[3], 0x0040), 0x5410);
+        }
+        *reinterpret_cast<uint4*>(my_dig + gv_dig(j * 128 + lane * 4)) = make_uint4(word[0], word[1], word[2], word[3]);
+      }
+      __syncwarp();
+      // lane (g, t) gathers digit g & 3 of batch row m into fragment row g = 4 (m & 1) + digit, half m >> 1
+      if ((g >> 2) == (m & 1)) {
+#pragma unroll
+        for (int c = 0; c < MAX_CW / 2; ++c) {
+          if (half * (MAX_CW / 2) + c >= p.cw) break;
+#pragma unroll
+          for (int j = 0; j < MPC; ++j) {
+            // the eight k of this lane in MMA j of the chunk: 4 bits: 8 j ..: even ones, then odd ones; 8 bits: 8 j ..: in order
+            const uint32_t* src = my_dig + gv_dig(c * CHUNK_K + t * LANE_K + 8 * j);
+            const uint4 lo = *reinterpret_cast<const uint4*>(src), hi = *reinterpret_cast<const uint4*>(src + 4);
+            uint32_t f0, f1;
+            if (BITS == 4) {
+              f0 = __byte_perm(__byte_perm(lo.x, lo.z, sel), __byte_perm(hi.x, hi.z, sel), 0x5410);
+              f1 = __byte_perm(__byte_perm(lo.y, lo.w, sel), __byte_perm(hi.y, hi.w, sel), 0x5410);
+            } else {
+              f0 = __byte_perm(__byte_perm(lo.x, lo.y, sel), __byte_perm(lo.z, lo.w, sel), 0x5410);
+              f1 = __byte_perm(__byte_perm(hi.x, hi.y, sel), __byte_perm(hi.z, hi.w, sel), 0x5410);
+            }
+            sum = (uint32_t)__dp4a((int)f0, 0x01010101, (int)sum);
+            sum = (uint32_t)__dp4a((int)f1, 0x01010101, (int)sum);
+            const int f = (half * (MAX_CW / 2) + c) * MPC + j;
+#pragma unroll
+            for (int h = 0; h < HALVES; ++h)
+              if ((m >> 1) == h) { a[f][2 * h] = f0; a[f][2 * h + 1] = f1; }
+          }
+        }
+      }
+      __syncwarp();
+    }
+    if ((g >> 2) == (m & 1)) {
+#pragma unroll
+      for (int h = 0; h < HALVES; ++h)
+        if ((m >> 1) == h) {
+          corr[h] = BITS == 4 ? 8 * (int)sum : 0;
+          down[h] = finite ? __int_as_float((e - 6 - 7 * (int)d + 127) << 23) : __int_as_float(0x7FC00000);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) xv[j] = xn[j];
+    if (m + 2 < p.M) load_x(m + 2, xn);
+  }
+#pragma unroll
+  for (int h = 0; h < HALVES; ++h) {                 // digit sums of the row: its four lanes hold a quarter each
+    corr[h] += __shfl_xor_sync(0xffffffffu, corr[h], 1);
+    corr[h] += __shfl_xor_sync(0xffffffffu, corr[h], 2);
+  }
+
+  __syncthreads();                                   // the digit words make room for the partial sums
+  // ---- the weight stream --------------------------------------------------------------------------------
+  const uint32_t lane_off = (uint32_t)((ugi * 8 + g) * p.stride + kwi * p.cw * 64 + t * 16);
+  bool alive = true;
+  int issued = min(p.slots, n_steps);                // steps requested so far (followed by every warp)
+  for (int e0 = 0; e0 < n_steps; e0 += kGvEpoch) {
+  const int e1 = min(e0 + kGvEpoch, n_steps);
+  // the scale and bias of this thread's first output of the epoch, ahead of their use
+  const int n_out = (e1 - e0) * ug * p.M * 8;
+  auto channel = [&](int o) { return ((e0 + (o >> 3) / (p.M * ug)) * per_step + (int)blockIdx.x * ug + (o >> 3) / p.M % ug) * 8 + (o & 7); };
+  float sc = 0.f, bi = 0.f;
+  if (tid < n_out && channel(tid) < p.N) {
+    sc = __ldg(scale + channel(tid));
+    if (bias) bi = __ldg(bias + channel(tid));
+  }
+  for (int i = e0; i < e1 && alive; ++i) {
+    const int slot = i % p.slots;
+    alive = mbar_wait_warp(bar_full + 8 * slot, (uint32_t)(i / p.slots) & 1u, s_abort, nullptr);
+    if (!alive) break;
+    const uint8_t* src = ring + slot * p.slot_bytes + lane_off;
+    int acc2[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};     // two chains of dependent MMAs
+#pragma unroll
+    for (int c = 0; c < MAX_CW; ++c) {
+      if (c >= p.cw) break;
+      uint4 q = *reinterpret_cast<const uint4*>(src + c * 64);
+      if (BITS == 4) { q.x ^= 0x88888888u; q.y ^= 0x88888888u; q.z ^= 0x88888888u; q.w ^= 0x88888888u; }
+      const uint32_t words[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int j = 0; j < MPC; ++j) {
+        const uint32_t b0 = BITS == 4 ? words[j] & 0x0F0F0F0Fu : words[2 * j];
+        const uint32_t b1 = BITS == 4 ? (words[j] >> 4) & 0x0F0F0F0Fu : words[2 * j + 1];
+        const int f = c * MPC + j;
+        gv_mma(acc2[f & 1], a[f][0], HALVES == 2 ? a[f][2 * HALVES - 2] : 0u, a[f][1], HALVES == 2 ? a[f][2 * HALVES - 1] : 0u, b0, b1);
+      }
+    }
+    // the words have been used (the sums below depend on them): hand the slot back
+    asm volatile("" ::"r"(acc2[0][0]), "r"(acc2[1][0]) : "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_empty + 8 * slot);
+    int acc[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = acc2[0][j] + acc2[1][j];
+    // lane (g, t): rows g (and g + 8), output channels 2 t and 2 t + 1 of the unit; the four digits of a batch row sit in
+    // the lanes with equal g >> 2
+    float* part = s_part + ((i - e0) * kGvWarps + warp) * kGvMaxRows * 8;
+#pragma unroll
+    for (int h = 0; h < HALVES; ++h) {
+      float v0 = (float)(acc[2 * h] - corr[h]) * down[h], v1 = (float)(acc[2 * h + 1] - corr[h]) * down[h];
+      v0 += __shfl_xor_sync(0xffffffffu, v0, 4);
+      v1 += __shfl_xor_sync(0xffffffffu, v1, 4);
+      v0 += __shfl_xor_sync(0xffffffffu, v0, 8);
+      v1 += __shfl_xor_sync(0xffffffffu, v1, 8);
+      if ((g & 3) == 0) *reinterpret_cast<float2*>(part + (2 * h + (g >> 2)) * 8 + 2 * t) = make_float2(v0, v1);
+    }
+    // one step later, so that the other warps are through with it as well, warp 0 refills the slot of the step before
+    if (i > 0 && issued < n_steps && issued == i - 1 + p.slots) {
+      if (warp == 0) {
+        alive = mbar_wait_warp(bar_empty + 8 * ((i - 1) % p.slots), (uint32_t)((i - 1) / p.slots) & 1u, s_abort, nullptr);
+        if (alive) issue(issued);
+      }
+      ++issued;
+    }
+  }
+  __syncthreads();                                   // the epoch's partial sums are in place
+  if (*s_abort) break;
+  for (int o = tid; o < n_out; o += kGvWarps * 32) {
+    const int n = channel(o), m = (o >> 3) % p.M, u = (o >> 3) / p.M % ug, st = (o >> 3) / (p.M * ug);
+    if (n >= p.N) continue;
+    if (o != tid) { sc = __ldg(scale + n); bi = bias ? __ldg(bias + n) : 0.f; }
+    const float* sp = s_part + (st * kGvWarps + u * p.kw) * kGvMaxRows * 8 + m * 8 + (o & 7);
+    float sum = 0.f;
+    for (int k = 0; k < p.kw; ++k) sum += sp[k * kGvMaxRows * 8];
+    y[(size_t)m * p.N + n] = fmaf(sum, sc, bi);
+  }
+  __syncthreads();                                   // before the next epoch's partial sums
+  }
+  if (*s_abort) {
+    // a wait expired: let the copies in flight land (bounded as well) and make the failure visible in the result
+    if (tid == 0)
+      for (int j = 0; j < p.slots && j < issued; ++j) {
+        const int u = issued - 1 - (issued - 1 - j) % p.slots;             // last step issued to slot j
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_full + 8 * j, (uint32_t)(u / p.slots) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
+      }
+    for (int i = tid; i < p.M * p.N; i += kGvWarps * 32) y[i] = __int_as_float(0x7FC00000);
+  }
+}
+
+}  // namespace
+
+// Up to four rows and rows of at most 8,192 elements (16 warps x 512); at least 256 bytes a row and 2^18 elements:
+// below, both this and the plain kernel take less time than a call's host side (512 x 512: 5.8 us a call with either), while
+// at 1000 x 1280 the plain kernel needs 10 us and this one 5.9.
+bool qlinear_gemv_applicable(int N, int K, int bits, int M) {
+  if ((bits != 4 && bits != 8) || M < 1 || M > kGvMaxRows || K > 8192) return false;
+  return row_bytes(K, bits) >= 256 && (long long)N * K >= (1 << 18);
+}
+
+aiq_status_t launch_qlinear_gemv(const LayerJob& job, int N, int K, int M, cudaStream_t s) {
+  DeviceProps props;
+  if (aiq_status_t st = current_device_props(&props)) return st;
+  GvParams p = {};
+  p.N = N; p.K = K; p.M = M;
+  p.rb = (int)row_bytes(K, job.bits);
+  p.stride = (p.rb + 127) / 128 * 128 + 64;
+  const int chunks = (p.rb + 63) / 64, max_cw = job.bits == 4 ? 4 : 8;
+  // as few warps per unit as its K needs; more of them where there are fewer units than that leaves warps for
+  p.kw = 1;
+  const int units = (N + 7) / 8;
+  while (p.kw < kGvWarps && ((chunks + p.kw - 1) / p.kw > max_cw || (p.kw < chunks && units * p.kw < props.n_sms * kGvWarps))) p.kw <<= 1;
+  p.cw = (chunks + p.kw - 1) / p.kw;
+  const int ug = kGvWarps / p.kw;
+  p.slot_bytes = (8 * ug * p.stride + 127) / 128 * 128;
+  p.slack = (std::max(0, 64 * p.cw * p.kw - p.stride) + 127) / 128 * 128;
+  const int fixed = p.slack + kGvWarps * kGvDigWords * 4 + 2 * kGvMaxSlots * 8 + 16;
+  const int steps = (units + props.n_sms * ug - 1) / (props.n_sms * ug);
+  p.slots = std::min(std::min(kGvMaxSlots, steps), (props.smem_optin - fixed) / p.slot_bytes);
+  if (p.slots < 1) return set_error(AIQ_ERR_SHAPE, "qlinear_gemv: %d bytes per step do not fit shared memory", p.slot_bytes);
+  const int smem = p.slots * p.slot_bytes + fixed;
+  const int grid = std::min(props.n_sms, (units + ug - 1) / ug);
+  const float* x = static_cast<const float*>(job.in);
+  float* y = static_cast<float*>(job.out);
+  LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K, (double)N * p.rb + 4.0 * N + 4.0 * M * ((double)K + N));
+#define AIQ_GEMV(B_, H_)                                                                                                  \
+  do {                                                                                                                   \
+    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemv_kernel<B_, H_>), props.smem_optin);                                             \
+    AIQ_CUDA_TRY(launch_chained(true, qlinear_gemv_kernel<B_, H_>, dim3(grid), dim3(kGvWarps * 32), smem, s, job.w, job.scale, \
+                                job.bias, x, y, p));                                                                     \
+  } while (0)
+  if (job.bits == 4) { if (M <= 2) AIQ_GEMV(4, 1); else AIQ_GEMV(4, 2); }
+  else { if (M <= 2) AIQ_GEMV(8, 1); else AIQ_GEMV(8, 2); }
+#undef AIQ_GEMV
+  AIQ_LAUNCH_CHECK("qlinear_gemv");
+  return AIQ_OK;
+}
+
+}  // namespace aiq

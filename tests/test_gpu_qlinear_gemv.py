@@ -1,0 +1,62 @@
+"""The one-kernel linear layer for up to four rows, at its edges: rows whose packed length is no multiple of a chunk or of 32
+elements, fewer and more channels than a unit per SM, one warp to sixteen warps per unit, the longest row, one to four
+batch rows, activations over a wide range of magnitudes.  Bound: the integer sums are exact; the digits hold x to 2^-27 of
+the largest |x| of its slice, digit sums and the at most 16 partial sums round to 2^-24 each, so
+|delta| <= 2^-20 s_n sum_k |code| max|x| is ample.  Integer inputs come out exactly.  The kernel needs no workspace and
+gives the same bits twice."""
+import numpy as np
+import pytest
+
+from oracle import aiq_oracle as O
+from gpu_util import binding, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("N,K,M", [(1024, 520, 1), (1030, 777, 2), (40, 8192, 3), (2999, 1000, 4), (520, 8190, 1),
+                                   (9000, 4100, 4), (20000, 512, 2)])
+def test_gemv_bound(bits, N, K, M):
+    import torch
+    aiq = binding()
+    rng = np.random.default_rng(N + K + M)
+    W = rng.standard_normal((N, K)).astype(np.float32)
+    x = (rng.standard_normal((M, K)) * np.exp(rng.uniform(-12, 4, (M, K)))).astype(np.float32)
+    x[:, :: 7] = 0
+    bias = rng.standard_normal(N).astype(np.float32)
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(to_dev(W), bits, packed, scales)
+    ys = []
+    for _ in range(2):
+        y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+        aiq.aiq_qlinear(packed, scales, to_dev(bias), N, K, bits, to_dev(x), y)
+        ys.append(y.cpu().numpy())
+    assert np.array_equal(ys[0], ys[1])
+    v, s = O.quantize_rows(W, bits)
+    want = x.astype(np.float64) @ (v.astype(np.float64) * np.asarray(s, np.float64)[:, None]).T + bias.astype(np.float64)
+    bound = 2.0 ** -20 * (np.abs(x).max(axis=1)[:, None] * (np.abs(v).sum(axis=1) * s)[None, :]) + 2.0 ** -22 * np.abs(want)
+    assert np.all(np.abs(ys[0] - want) <= bound)
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+def test_gemv_exact_on_integers_and_nonfinite_rows(bits):
+    import torch
+    aiq = binding()
+    rng = np.random.default_rng(bits)
+    qmax = 2 ** (bits - 1) - 1
+    N, K, M = 1200, 2050, 4
+    W = rng.integers(-qmax, qmax + 1, (N, K)).astype(np.float32)
+    W[:, 0] = qmax
+    x = rng.integers(-8, 9, (M, K)).astype(np.float32)
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(to_dev(W), bits, packed, scales)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    aiq.aiq_qlinear(packed, scales, None, N, K, bits, to_dev(x), y)
+    assert np.array_equal(y.cpu().numpy().astype(np.int64), x.astype(np.int64) @ W.astype(np.int64).T)
+    x[2, 11] = np.inf
+    x[3, 1999] = np.nan
+    aiq.aiq_qlinear(packed, scales, None, N, K, bits, to_dev(x), y)
+    got = y.cpu().numpy()
+    assert np.isfinite(got[:2]).all() and not np.isfinite(got[2:]).any()

@@ -119,12 +119,14 @@ void aiq_set_scale_granularity(int granularity);
  * row-major, 16-byte aligned; y: device float32 [M][N].  M >= 1.  Asynchronous on `stream`.
  *
  * Four kernels.  The plain one expands weights to float32 in registers and accumulates in
- * float32 (any shape, any bit-width).  For 4- / 8-bit weights three faster ones exist:
- *   M <= 4, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: one kernel, no workspace;
+ * float32 (any shape, any bit-width; from five rows on as a tiled GEMM whose blocks, where they
+ * are few, split K inside a cluster, in a fixed order).  It is also the one that runs for M >= 5
+ * and N*K*M <= 2^26, where one launch beats the kernels with a pre-pass.  Three faster ones exist:
+ *   M <= 4, 4 / 8 bits, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: no workspace;
  *     the codes stay integer and feed the int8 warp-level tensor cores, the activations of every
  *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest
  *     |x|), the int32 sums are exact and run-to-run identical.
- *   M <= 8 otherwise, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
+ *   M <= 8 otherwise, 4 / 8 bits, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
  *     warp-level tensor cores; the activations of each group of 512 k become three int8
  *     digits with a shared exponent (21 bits below the group's largest |x|), the int32 sums
  *     are exact.
@@ -132,9 +134,9 @@ void aiq_set_scale_granularity(int granularity);
  *     MMA's M operand (codes expanded to bfloat16 in shared memory, exact) and the batch as
  *     its N operand; the activations enter as the sum of two bfloat16 (relative rounding
  *     2^-17), accumulation is float32.
- * Both split K over thread blocks where the matrix has too few rows to fill the GPU; the
+ * The last two split K over thread blocks where the matrix has too few rows to fill the GPU; the
  * partial sums then meet in y through float atomics (run-to-run differences in the last
- * bit).  Both need scratch memory: pass `workspace` (device, 16-byte aligned) of at least
+ * bit).  They need scratch memory: pass `workspace` (device, 16-byte aligned) of at least
  * aiq_qlinear_workspace_bytes(...) bytes; with workspace == NULL, or where that function
  * returns 0, the plain kernel runs.
  * Device-side failure: the tcgen05 kernel bounds every wait on its copy / MMA pipeline (about

@@ -94,15 +94,28 @@ struct LaunchScope {
 // it has it: a later kernel's block could otherwise take the columns an earlier one is waiting for).
 // `chain`: whether to do so at all (chain_pays); the kernel is the same either way.
 bool chain_pays(double bytes);
+// `cluster`: blocks along x that form a thread-block cluster (1: none; at most 8, a divisor of the grid's x).
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+inline cudaError_t launch_chained_cluster(bool chain, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                          cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = chain ? 1 : 0;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (chain) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_chained_cluster(chain, 1, kernel, grid, block, smem, s, static_cast<A&&>(args)...);
 }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // What a kernel of the chain reads of an earlier one's results: an ordinary load, not the read-only path, whose lines

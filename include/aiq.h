@@ -131,9 +131,10 @@ void aiq_set_scale_granularity(int granularity);
  *     digits with a shared exponent (21 bits below the group's largest |x|), the int32 sums
  *     are exact.
  *   M >= 9, K a multiple of 8, K >= 64, N >= 32: a tcgen05 GEMM with the weight matrix as the
- *     MMA's M operand (codes expanded to bfloat16 in shared memory, exact) and the batch as
- *     its N operand; the activations enter as the sum of two bfloat16 (relative rounding
- *     2^-17), accumulation is float32.
+ *     MMA's M operand and the batch as its N operand.  4 / 8 / 16 bits: codes and halves are
+ *     exact; the activations, scaled by a power of two per batch row, enter as the sum of two
+ *     halves (relative rounding 2^-22, or 2^-39 of the row's largest |x|).  32 bits: weights and
+ *     activations enter as sums of two bfloat16 (2^-17).  Accumulation is float32.
  * The last two split K over thread blocks where the matrix has too few rows to fill the GPU; the
  * partial sums then meet in y through float atomics (run-to-run differences in the last
  * bit).  They need scratch memory: pass `workspace` (device, 16-byte aligned) of at least

@@ -428,9 +428,8 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
       return aiq::set_error(AIQ_ERR_INVALID_ARG, "aiq_qlinear: workspace not 16-byte aligned");
     const size_t scratch = aiq::qlinear_tc_workspace_bytes(K, M);
     if (workspace_bytes >= scratch + 16) {
-      // device status word behind the scratch: 0, or 1 once a bounded wait of the kernel expired
+      // device status word behind the scratch: 0 (set by the pre-pass), or 1 once a bounded wait of the kernel expired
       int32_t* status = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + scratch);
-      AIQ_CUDA_TRY(cudaMemsetAsync(status, 0, 16, (cudaStream_t)stream));
       return aiq::launch_qlinear_tc(job, N, K, M, workspace, status, (cudaStream_t)stream);
     }
   } else if (workspace && aiq::qlinear_mma_applicable(N, K, bits, M)) {

@@ -121,7 +121,7 @@ void aiq_set_scale_granularity(int granularity);
  * Four kernels.  The plain one expands weights to float32 in registers and accumulates in
  * float32 (any shape, any bit-width; from five rows on as a tiled GEMM whose blocks, where they
  * are few, split K inside a cluster, in a fixed order).  It is also the one that runs for M >= 5
- * and N*K*M <= 2^26, where one launch beats the kernels with a pre-pass.  Three faster ones exist:
+ * and N*K*M <= 2^26 (K > 4096 and M > 8: 2^24), where one launch beats the kernels with a pre-pass.  Three faster ones exist:
  *   M <= 4, 4 / 8 bits, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: no workspace;
  *     the codes stay integer and feed the int8 warp-level tensor cores, the activations of every
  *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest

@@ -392,8 +392,11 @@ aiq_status_t launch_qlinear(const LayerJob* jobs_dev, const LayerJob* single_hos
 }  // namespace aiq
 
 // Up to 2^26 products the one launch of the float32 kernel (from five rows on) beats the pre-pass and the atomics of the
-// kernels below; see the figures at qlinear_gemm_kernel.
-static bool small_gemm(int N, int K, int M) { return M > 4 && (long long)N * K * M <= 1ll << 26; }
+// kernels below; see the figures at qlinear_gemm_kernel.  Long rows leave it few tiles with many slices each (128 x 8192,
+// 40 rows: 14.2 us against 7.6 on the tensor cores; 64 x 8192, 12 rows: 9.5, one launch): from K = 4096 up to 2^24.
+static bool small_gemm(int N, int K, int M) {
+  return M > 4 && (long long)N * K * M <= (K > 4096 && M > 8 ? 1ll << 24 : 1ll << 26);
+}
 
 extern "C" size_t aiq_qlinear_workspace_bytes(int N, int K, int bits, int M) {
   if (N <= 0 || K <= 0 || M <= 0 || small_gemm(N, K, M)) return 0;

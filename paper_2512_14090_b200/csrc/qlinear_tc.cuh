@@ -55,7 +55,7 @@ struct QtKind {
   static constexpr int TPC = BITS == 32 ? 2 : 1;     // packed tiles per chunk
   static constexpr int A_STAGES = DIRECT ? 0 : kQtAStages;
   static constexpr int A_COLS = A_STAGES * PIECES * kQtACols;
-  static constexpr int THREADS = DIRECT ? 192 : (6 + kQtExpWarps) * 32;
+  static constexpr int THREADS = (6 + kQtExpWarps) * 32;   // DIRECT: the expander warps only take part in the last step
 };
 
 struct QtParams {

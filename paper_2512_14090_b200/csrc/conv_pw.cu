@@ -199,33 +199,26 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
 
   if (warp == 0) {
     // ---- TMA producer -----------------------------------------------------------------------
-    if (lane == 0) {
-      chain_wait();
-      uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
-      for (int tile = tile0; tile < tile1 && alive; ++tile) {
-        const int pix = (int)(job.in_version * p.ver_pixels) + tile * 128;
-        for (int c = 0; c < n_chunks; ++c) {
-          alive = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
-          if (!alive) break;
-          issued |= 1u << stage;
-          issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-          mbar_expect_tx(bar_full + 8 * stage, (STREAM ? 2 : 1) * kPrChunkBytes);
-#pragma unroll
-          for (int part = 0; part < (STREAM ? 2 : 1); ++part)    // STREAM: 64 channels of the hi, then of the lo half
-            asm volatile(
-                "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                ::"r"(smem_u32(smem) + stage * stage_bytes + part * kPrChunkBytes), "l"(reinterpret_cast<uint64_t>(&in_map)),
-                "r"(bar_full + 8 * stage), "r"(c * 64 + part * p.Cs_in), "r"(pix)
-                : "memory");
-          if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
-        }
+    chain_wait();
+    uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
+    for (int tile = tile0; tile < tile1 && alive; ++tile) {
+      const int pix = (int)(job.in_version * p.ver_pixels) + tile * 128;
+      for (int c = 0; c < n_chunks; ++c) {
+        alive = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+        if (!alive) break;
+        const uint32_t dst = smem_u32(smem) + stage * stage_bytes;
+        if (STREAM) tma_fill2_2d(dst, &in_map, bar_full + 8 * stage, kPrChunkBytes, c * 64, c * 64 + p.Cs_in, pix);   // 64 channels: hi, lo
+        else tma_fill_2d(dst, &in_map, bar_full + 8 * stage, kPrChunkBytes, c * 64, pix);
+        issued |= 1u << stage;
+        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+        if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
       }
-      for (int i = 0; i < stages; ++i)             // copies in flight must land before the CTA exits
-        if (issued & (1u << i)) {
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar_full + 8 * i, (issued_phase >> i) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
-        }
     }
+    for (int i = 0; i < stages; ++i)               // copies in flight must land before the CTA exits
+      if (issued & (1u << i)) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_full + 8 * i, (issued_phase >> i) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
+      }
   } else if (warp == 1) {
     // ---- MMA issuer: all 32 lanes converged, one elected lane issues (see umma_bf16) ------------
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Nt >> 3) << 17) | ((128u >> 4) << 24);

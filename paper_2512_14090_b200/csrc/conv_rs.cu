@@ -343,7 +343,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   for (int i = tid; i < p.pool_bytes / 4; i += n_threads) s_pool[i] = 0.f;
   // row programs (one thread per input row)
   if (tid < p.H) s_rows[tid] = rs_row_program<KS, STRIDE>(tid, p.H, p.Ho, N, R);
-  bool alive = mbar_wait_warp(bar_w, 0, s_abort, p.error_flag);
+  bool alive = mbar_wait_warp_inline(bar_w, 0, s_abort, p.error_flag);
   if (alive) rs_expand_weights<C, KS, STRIDE, PIECES>(ring, wrow_bytes, job.bits, N, wsm, tid, n_threads);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // expanded weights -> visible to the MMA
   tc_fence_before();
@@ -358,7 +358,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
 
   // ---- roles ------------------------------------------------------------------------------
   if (warp == 0) {
-    if (lane == 0 && alive) {
+    if (alive) {                                       // converged, an elected lane issues
       chain_wait();
       uint32_t stage = 0, phase = 0;
       uint32_t issued = 0, issued_phase = 0;
@@ -366,25 +366,25 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         const int row0 = job.in_version * p.rows_per_version + (p.gmode == 2 ? 2 * item : item) * p.H;
         for (int y = 0; y < p.H && alive; ++y) {
           if (!row_used(y)) continue;
-          alive = mbar_wait(bar_in_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+          alive = mbar_wait_warp_inline(bar_in_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
           if (!alive) break;
           issued |= 1u << stage;
           issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
           const uint32_t bar = bar_in_full + 8 * stage;
           const uint32_t dst = smem_u32(ring) + stage * p.stage_bytes;
-          mbar_expect_tx(bar, (uint32_t)p.stage_bytes);
+          expect_tx_elect(bar, (uint32_t)p.stage_bytes);
           if (STRIDE == 1) {
-            tma_load_4d(dst, &map0, bar, 0, KS == 3 ? -1 : 0, 0, row0 + y);
+            tma_load_4d_elect(dst, &map0, bar, 0, KS == 3 ? -1 : 0, 0, row0 + y);
           } else if (p.gmode != 2) {
-            tma_load_5d(dst, &map0, bar, 0, KS == 3 ? -1 : 0, 0, 0, row0 + y);
+            tma_load_5d_elect(dst, &map0, bar, 0, KS == 3 ? -1 : 0, 0, 0, row0 + y);
           } else if (KS == 3) {
             // odd columns from pair -1 (tap 0), even columns (tap 1), odd columns from pair 0 (tap 2)
             const uint32_t sub = (uint32_t)p.stage_bytes / 3;
-            tma_load_5d(dst, &map1, bar, 0, -1, 0, 0, row0 + y);
-            tma_load_5d(dst + sub, &map0, bar, 0, 0, 0, 0, row0 + y);
-            tma_load_5d(dst + 2 * sub, &map1, bar, 0, 0, 0, 0, row0 + y);
+            tma_load_5d_elect(dst, &map1, bar, 0, -1, 0, 0, row0 + y);
+            tma_load_5d_elect(dst + sub, &map0, bar, 0, 0, 0, 0, row0 + y);
+            tma_load_5d_elect(dst + 2 * sub, &map1, bar, 0, 0, 0, 0, row0 + y);
           } else {
-            tma_load_5d(dst, &map0, bar, 0, 0, 0, 0, row0 + y);
+            tma_load_5d_elect(dst, &map0, bar, 0, 0, 0, 0, row0 + y);
           }
           if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
         }
@@ -419,10 +419,10 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           const int fresh_row = (int)(w4.y & 255u), n_fresh = (int)(w4.y >> 8);
           for (int i = 0; i < n_fresh && alive; ++i) {
             const int q = q0 + fresh_row + i;
-            alive = mbar_wait_warp(bar_out_empty + 8 * (q & (R - 1)), ((q / R) & 1) ^ 1u, s_abort, p.error_flag);
+            alive = mbar_wait_warp_inline(bar_out_empty + 8 * (q & (R - 1)), ((q / R) & 1) ^ 1u, s_abort, p.error_flag);
           }
           if (!alive) break;
-          alive = mbar_wait_warp(bar_in_full + 8 * stage, phase, s_abort, p.error_flag);
+          alive = mbar_wait_warp_inline(bar_in_full + 8 * stage, phase, s_abort, p.error_flag);
           if (!alive) break;
           tc_fence_after();
           const uint32_t a_stage = smem_u32(ring) + stage * p.stage_bytes;
@@ -495,7 +495,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       const int q = il * p.Ho + y;
       const int slot = q & (R - 1);
       const size_t row_off = row_offset(k);
-      alive = mbar_wait_warp(bar_out_full + 8 * slot, (q / R) & 1, s_abort, p.error_flag);
+      alive = mbar_wait_warp_inline(bar_out_full + 8 * slot, (q / R) & 1, s_abort, p.error_flag);
       if (!alive) break;
       tc_fence_after();
       for (int u = unit0; u < units; u += unit_step) {
@@ -553,7 +553,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         const uint32_t pool_parity = (uint32_t)(il & 1);
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_pool);
-        alive = mbar_wait_warp(bar_pool, pool_parity, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_pool, pool_parity, s_abort, p.error_flag);
         if (!alive) break;
         const int item = (int)blockIdx.x + il * (int)gridDim.x;
         for (int i = tid - 64; i < Gout * N; i += n_epi) {
@@ -569,7 +569,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_pool + 8);
-        alive = mbar_wait_warp(bar_pool + 8, pool_parity, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_pool + 8, pool_parity, s_abort, p.error_flag);
         if (!alive) break;
         for (int i = lane; i < Gout * 16; i += 32) s_pool[(size_t)(warp - 2) * Gout * 16 + i] = 0.f;
         __syncwarp();
@@ -702,7 +702,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
   // the zero columns on both sides of every row of the intermediate ring are written once, here
   for (int i = tid; i < S_mid * p.stage_bytes / 16; i += kRbThreads)
     reinterpret_cast<uint4*>(mid_ring)[i] = make_uint4(0u, 0u, 0u, 0u);
-  bool alive = mbar_wait_warp(bar_w, 0, s_abort, p.error_flag);
+  bool alive = mbar_wait_warp_inline(bar_w, 0, s_abort, p.error_flag);
   if (alive) {
     rs_expand_weights<C, 3, 1, 1>(in_ring, wrow1, job.bits_pre, N, w1, tid, kRbThreads);
     rs_expand_weights<C, 3, 1, 1>(in_ring + packed1, wrow2, job.bits, N, w2, tid, kRbThreads);
@@ -725,19 +725,19 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
   const uint32_t tap1 = 128u, tap2 = 256u;             // one column = 8 images x 16 bytes
 
   if (warp == 0) {
-    if (lane == 0 && alive) {
+    if (alive) {                                       // converged, an elected lane issues
       chain_wait();
       uint32_t issued = 0, issued_phase = 0;
       for (int g = 0; g < total && alive; ++g) {
         const int il = g / p.H, y = g - il * p.H;
         const uint32_t stage = (uint32_t)(g % S_in), phase = (uint32_t)((g / S_in) & 1);
-        alive = mbar_wait(bar_in_free + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_in_free + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
         if (!alive) break;
         issued |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-        mbar_expect_tx(bar_in_full + 8 * stage, (uint32_t)p.stage_bytes);
+        expect_tx_elect(bar_in_full + 8 * stage, (uint32_t)p.stage_bytes);
         const int item = (int)blockIdx.x + il * (int)gridDim.x;
-        tma_load_4d(smem_u32(in_ring) + stage * p.stage_bytes, &in_map, bar_in_full + 8 * stage, 0, -1, 0,
+        tma_load_4d_elect(smem_u32(in_ring) + stage * p.stage_bytes, &in_map, bar_in_full + 8 * stage, 0, -1, 0,
                     job.in_version * p.rows_per_version + item * p.H + y);
       }
       for (int i = 0; i < S_in; ++i)
@@ -764,11 +764,11 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
       const int fresh_row = (int)(rr.w4.y & 255u), n_fresh = (int)(rr.w4.y >> 8);
       for (int i = 0; i < n_fresh && alive; ++i) {
         const int q = il * p.H + fresh_row + i;
-        alive = mbar_wait_warp(bar_acc_empty + 8 * (q & (R - 1)), ((q / R) & 1) ^ 1u, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_acc_empty + 8 * (q & (R - 1)), ((q / R) & 1) ^ 1u, s_abort, p.error_flag);
       }
       if (!alive) break;
       const uint32_t stage = (uint32_t)(g % S), phase = (uint32_t)((g / S) & 1);
-      alive = mbar_wait_warp(bar_src_full + 8 * stage, phase, s_abort, p.error_flag);
+      alive = mbar_wait_warp_inline(bar_src_full + 8 * stage, phase, s_abort, p.error_flag);
       if (!alive) break;
       tc_fence_after();
       const uint32_t a_stage = src_ring + stage * p.stage_bytes;
@@ -813,7 +813,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
       const int slot = g & (R - 1);
       uint32_t v0[16], v1[16];
       uint32_t hi[8], lo[8];
-      alive = mbar_wait_warp(bar_acc_full + 8 * slot, (g / R) & 1, s_abort, p.error_flag);
+      alive = mbar_wait_warp_inline(bar_acc_full + 8 * slot, (g / R) & 1, s_abort, p.error_flag);
       if (!alive) break;
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(qd * 32) << 16) + (uint32_t)(slot * N);
@@ -826,7 +826,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_acc_empty + 8 * slot);
         // the stage of the intermediate ring must have been read by conv2's MMAs of its last occupant
-        alive = mbar_wait_warp(bar_mid_free + 8 * ms, mphase ^ 1u, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_mid_free + 8 * ms, mphase ^ 1u, s_abort, p.error_flag);
         if (!alive) break;
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
@@ -845,7 +845,7 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
         const uint32_t is = (uint32_t)(g % S_in), iphase = (uint32_t)((g / S_in) & 1);
         // shortcut: the block input at the same row, still in the input ring (its copy completed long
         // ago; observing the barrier makes the data visible to this thread)
-        alive = mbar_wait_warp(bar_in_full + 8 * is, iphase, s_abort, p.error_flag);
+        alive = mbar_wait_warp_inline(bar_in_full + 8 * is, iphase, s_abort, p.error_flag);
         uint4 r0[4], r1[4];
         {
           const uint8_t* src = in_ring + is * p.stage_bytes;

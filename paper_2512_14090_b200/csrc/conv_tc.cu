@@ -230,7 +230,7 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, TcParams p, const Lay
 
   // ---- roles ------------------------------------------------------------------------------
   if (warp == 0) {
-    if (lane == 0 && alive) {
+    if (alive) {                                       // converged, an elected lane issues
       chain_wait();
       uint32_t stage = 0, phase = 0;
       uint32_t issued = 0, issued_phase = 0;       // per stage: a load was issued / parity of the last one
@@ -238,14 +238,14 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, TcParams p, const Lay
         const int rb = tile / n_cb, cb = tile - rb * n_cb;
         if (STRIDE == 1) {
           for (int t = T_FIRST; t <= T_LAST && alive; ++t) {
-            alive = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+            alive = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
             if (!alive) break;
             issued |= 1u << stage;
             issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-            mbar_expect_tx(bar_full + 8 * stage, L::STAGE_BYTES);
+            expect_tx_elect(bar_full + 8 * stage, L::STAGE_BYTES);
 #pragma unroll
             for (int ch = 0; ch < L::CHUNKS; ++ch)
-              tma_load_4d(smem_u32(ring) + stage * L::STAGE_BYTES + ch * L::CHUNK_BYTES, &in_map,
+              tma_load_4d_elect(smem_u32(ring) + stage * L::STAGE_BYTES + ch * L::CHUNK_BYTES, &in_map,
                           bar_full + 8 * stage, ch * 64, cb * kColsPerTile + t - 1, rb * kRowsPerTile - 1,
                           job.in_version);
             if (++stage == (uint32_t)stages) { stage = 0; phase ^= 1u; }
@@ -258,16 +258,16 @@ conv_tc_kernel(const __grid_constant__ CUtensorMap in_map, TcParams p, const Lay
           const int b0 = (rb / rbi) * ipt, oy0 = (rb % rbi) * kRowsPerTile;
           for (int t = T_FIRST; t <= T_LAST && alive; ++t) {
             for (int r = T_FIRST; r <= T_LAST && alive; ++r) {
-              alive = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+              alive = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
               if (!alive) break;
               issued |= 1u << stage;
               issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-              mbar_expect_tx(bar_full + 8 * stage, L::CHUNKS * kRowsPerTile * L::GROUP_BYTES);
+              expect_tx_elect(bar_full + 8 * stage, L::CHUNKS * kRowsPerTile * L::GROUP_BYTES);
               for (int img = 0; img < ipt; ++img) {
                 const int pair_row = job.in_version * p.ver_pair_rows + (b0 + img) * ((p.H + 2) >> 1) + oy0 + (r >> 1);
 #pragma unroll
                 for (int ch = 0; ch < L::CHUNKS; ++ch)
-                  tma_load_5d(smem_u32(ring) + stage * L::STAGE_BYTES + ch * L::CHUNK_BYTES +
+                  tma_load_5d_elect(smem_u32(ring) + stage * L::STAGE_BYTES + ch * L::CHUNK_BYTES +
                                   img * rows_per_img * L::GROUP_BYTES,
                               &in_map, bar_full + 8 * stage, ch * 64, (t - 1) & 1, cb * kColsPerTile + ((t - 1) >> 1),
                               r & 1, pair_row);

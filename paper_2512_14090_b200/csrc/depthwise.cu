@@ -150,34 +150,29 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
 
   if (tid >= n_compute) {
     // ---- producer: padded input rows oy0 * STRIDE .. of every unit of this block, in order -----------
-    if (lane == 0) {
-      chain_wait();
-      bool alive = true;
-      uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
-      for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
-        const DwUnit d = dw_unit<COLS>(p, u);
-        const int n_rows = (d.n_out - 1) * STRIDE + 3;
-        const int img = job.in_version * p.batch_capacity + d.img0;
-        for (int r = 0; r < n_rows; ++r) {
-          alive = mbar_wait(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
-          if (!alive) break;
-          issued |= 1u << stage;
-          issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-          mbar_expect_tx(bar_full + 8 * stage, (uint32_t)p.box_bytes);
-          asm volatile(
-              "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-              ::"r"(smem_u32(ring) + stage * p.stage_bytes), "l"(reinterpret_cast<uint64_t>(&in_map)), "r"(bar_full + 8 * stage),
-              "r"(d.slab * p.Cb), "r"(0), "r"(d.ox0 * STRIDE - 1), "r"(d.oy0 * STRIDE + r), "r"(img)
-              : "memory");
-          if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
-        }
+    chain_wait();
+    bool alive = true;
+    uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
+    for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
+      const DwUnit d = dw_unit<COLS>(p, u);
+      const int n_rows = (d.n_out - 1) * STRIDE + 3;
+      const int img = job.in_version * p.batch_capacity + d.img0;
+      for (int r = 0; r < n_rows; ++r) {
+        alive = mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, s_abort, p.error_flag);
+        if (!alive) break;
+        issued |= 1u << stage;
+        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+        expect_tx_elect(bar_full + 8 * stage, (uint32_t)p.box_bytes);
+        tma_load_5d_elect(smem_u32(ring) + stage * p.stage_bytes, &in_map, bar_full + 8 * stage, d.slab * p.Cb, 0,
+                          d.ox0 * STRIDE - 1, d.oy0 * STRIDE + r, img);
+        if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
       }
-      for (int i = 0; i < p.stages; ++i)               // copies in flight must land before the CTA exits
-        if (issued & (1u << i)) {
-          const long long t0 = clock64();
-          while (!mbar_try_wait(bar_full + 8 * i, (issued_phase >> i) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
-        }
     }
+    for (int i = 0; i < p.stages; ++i)               // copies in flight must land before the CTA exits
+      if (issued & (1u << i)) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_full + 8 * i, (issued_phase >> i) & 1u) && clock64() - t0 < kWaitLimitCycles) {}
+      }
     return;
   }
 

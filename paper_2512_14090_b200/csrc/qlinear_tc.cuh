@@ -84,27 +84,6 @@ inline int qt_smem_bytes(int a_stages, int Mt, int stack, int b_stages, int w_st
   return qt_ring_bytes(Mt, stack, b_stages, w_stages) + (2 * a_stages + 2 * b_stages + 2 * w_stages + 1) * 8 + 24 + (Mt + 256) * 4;
 }
 
-// By a converged warp: one elected lane announces the bytes on the barrier and issues the copy.  (Inside `if (lane == 0)`
-// a producer loop took 400 cycles for a copy; its descriptor and coordinates cannot stay in uniform registers there.)
-__device__ __forceinline__ void tma_fill_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, uint32_t bytes, int c0, int c1, int c2) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "elect.sync _|q, 0xffffffff;\n\t"
-      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%2], %3;\n\t"
-      "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%4, %5, %6}], [%2];\n\t}"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(bytes), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-__device__ __forceinline__ void tma_fill_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, uint32_t bytes, int c0, int c1) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "elect.sync _|q, 0xffffffff;\n\t"
-      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%2], %3;\n\t"
-      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%4, %5}], [%2];\n\t}"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(bytes), "r"(c0), "r"(c1)
-      : "memory");
-}
-
 // x [M][K] float32 -> planes hi [M][K], lo [M][K]; one block per batch row.
 //   HALF: x 2^-e = hi + lo in halves, 2^e in down[row] (PERM4: each 8 k in the order 0 4 1 5 2 6 3 7, in which the expanders
 //   unpack 4-bit codes); else hi + lo in bfloat16 (2^-17 of each value), down[row] = 1.

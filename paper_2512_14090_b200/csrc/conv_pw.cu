@@ -455,7 +455,8 @@ EncodeTiledFn pr_encode_fn() {
 // than about 1,600 clocks of that), its epilogue (about 12 clocks per channel) and, streamed, the expansion of its
 // weights; a block adds a set-up that grows with the weights it expands.  Blocks fill the GPU in waves.
 struct PrConfig { bool stream; int Nt, ew, stages, bufs, splits, tiles_per_cta, smem; };
-bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
+// streamed: 0 / 1 restricts the search to that variant, -1 does not.
+bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, int streamed, PrConfig* out) {
   const int n_tiles = (g.B * (g.H + 2) * g.W + 127) / 128;
   const double K2 = 2.0 * g.Cs_in;
   double best = 1e300;
@@ -466,6 +467,7 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
       // two blocks per SM, one with 12 or 24 epilogue warps, one with streamed weights
       const bool stream = variant == 3;
       const int occ = variant == 0 ? 2 : 1, ew = stream ? 8 : variant == 2 ? 24 : 12;
+      if (streamed >= 0 && stream != (streamed == 1)) continue;
       if (occ == 2 && Nt > 128) continue;                      // tensor memory: 2 Nt columns per block
       if (stream && (Nt * 8 / (pieces == 2 ? 1 : 2) > 4 * kPrExpWarps * 32 || 2 * Nt > 512)) continue;
       const int limit = occ == 2 ? (props.smem_optin + 1024) / 2 - 1024 : props.smem_optin;
@@ -507,7 +509,14 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
 bool pr_config(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, PrConfig* out) {
   static thread_local ConfigMemo<PrConfig, 8> memo;
   const int key[8] = {g.B, g.H, g.W, g.Cs_in, g.Cs_out, n_jobs, pieces, props.dev};
-  return memo.get(key, out, [&](PrConfig* c) { return pr_search(g, n_jobs, pieces, props, c); });
+  return memo.get(key, out, [&](PrConfig* c) {
+    // The variants add the hi and lo products of a pixel in different orders.  Which one a layer takes is decided at a
+    // nominal batch, so that an image's result depends neither on the batch around it nor on the number of jobs.
+    ConvGeom nominal = g;
+    nominal.B = 256;
+    PrConfig v;
+    return pr_search(nominal, 1, pieces, props, -1, &v) && pr_search(g, n_jobs, pieces, props, v.stream ? 1 : 0, c);
+  });
 }
 
 template <int EW, int PIECES, bool STREAM>

@@ -321,7 +321,7 @@ qlinear_gemm_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, i
 
 template <int BITS, int BN, int BM>
 aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev, const LayerJob& single, int n_jobs, int N, int K, int M,
-                              int n_sms, cudaStream_t s) {
+                              int n_sms, cudaStream_t s, int fixed_cluster) {
   using G = GemmTile<BN, BM>;
   AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM>), (G::SMEM));
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, n_jobs);
@@ -329,8 +329,8 @@ aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev
   const int n_slices = (K + kGemmBK - 1) / kGemmBK;
   // blocks per tile: doubled while all blocks stay resident and a group of threads has more than one slice
   constexpr int resident = G::SMEM > 113 * 1024 ? 1 : 2;
-  int cluster = 1;
-  while (cluster < 8 && blocks * cluster * 2 <= resident * n_sms && n_slices > cluster * G::KG) cluster *= 2;
+  int cluster = fixed_cluster ? fixed_cluster : 1;
+  while (!fixed_cluster && cluster < 8 && blocks * cluster * 2 <= resident * n_sms && n_slices > cluster * G::KG) cluster *= 2;
   AIQ_CUDA_TRY(launch_chained_cluster(scope.chain, cluster, qlinear_gemm_kernel<BITS, BN, BM>, dim3(grid.x * cluster, grid.y, grid.z),
                                       dim3(kGemmThreads), G::SMEM, s, single, jobs_dev, N, K, M, cluster));
   return AIQ_OK;
@@ -339,20 +339,27 @@ aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev
 template <int BITS>
 aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n_jobs, int N, int K,
                          int M, cudaStream_t s) {
+  DeviceProps props;
+  if (aiq_status_t st = current_device_props(&props)) return st;
   const int gx = (N + kWarps * kRowsPerWarp - 1) / (kWarps * kRowsPerWarp);
   LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K * n_jobs,
                     n_jobs * ((double)N * row_bytes(K, BITS) + 4.0 * N + 4.0 * M * ((double)K + N)));
-  if (M == 1) {
+  if (jobs_dev) {
+    // A classifier inside a model: one tile, and a split of K that depends on the layer alone, so that an image's logits
+    // depend neither on the batch around it nor on the number of jobs.
+    const int n_tiles = (N + 31) / 32, n_slices = (K + kGemmBK - 1) / kGemmBK;
+    int cluster = 1;
+    while (cluster < 8 && n_tiles * cluster * 2 <= 64 && n_slices > cluster * GemmTile<32, 16>::KG) cluster *= 2;
+    if (aiq_status_t st = launch_gemm_tile<BITS, 32, 16>(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s, cluster)) return st;
+  } else if (M == 1) {
     AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 1>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
   } else if (M == 2) {
     AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 2>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
   } else if (M > 4) {
     // The largest tile that still gives every SM a block; smaller ones split K over more thread groups.  The tile of 8 rows
     // leaves out the work of rows that are not there (8191 x 8191, 5 rows, 4 bits: 72 us against 94 with the tile of 16).
-    DeviceProps props;
-    if (aiq_status_t st = current_device_props(&props)) return st;
     auto blocks = [&](int bn, int bm) { return (long long)((N + bn - 1) / bn) * ((M + bm - 1) / bm) * n_jobs; };
-    auto args = [&](auto launch) { return launch(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s); };
+    auto args = [&](auto launch) { return launch(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s, 0); };
     aiq_status_t st;
     if (M > 32 && blocks(64, 64) >= props.n_sms) st = args(launch_gemm_tile<BITS, 64, 64>);
     else if (M > 16 && blocks(64, 32) >= props.n_sms) st = args(launch_gemm_tile<BITS, 64, 32>);

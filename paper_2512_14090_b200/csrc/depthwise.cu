@@ -35,8 +35,9 @@ struct DwParams {
   int Cb, CQ;               // channels of a slab, its quads
   int XG, n_ct;             // column groups of a block, column tiles of a row
   int NI, n_ig;             // images of a block, image groups
-  int rb, n_rb;             // output rows of a block, row blocks
-  int n_slabs, n_units;     // units: slab fastest, then column tile, row block, image group
+  int n_slabs, k;           // slabs (fastest in the grid), blocks per slab
+  int rows, row_rem;        // output rows of a block, and how many blocks have one more
+  int n_rb;                 // or: blocks per image column, each of `rows` rows (the last of fewer); 0: an equal share
   int Wb;                   // input columns of a stage
   int stages, box_bytes, stage_bytes;   // bytes a copy brings; stages start on 128-byte boundaries
   int batch_capacity;       // images per version of the input slot
@@ -50,13 +51,16 @@ __device__ __forceinline__ void join4(uint2 h, uint2 l, uint64_t* v) {
 }
 
 // Four channels of one pixel in shared memory: [hi(Cb) | lo(Cb)] bfloat16 or Cb floats.
+// (By 32-bit address: through a pointer the compiler reads generically, with the latency of a global access.)
 template <int FMT>
-__device__ __forceinline__ void read4(const uint8_t* p, int Cb, uint64_t* v) {
+__device__ __forceinline__ void read4(uint32_t p, int Cb, uint64_t* v) {
   if (FMT == ACT_SPLIT) {
-    join4(*reinterpret_cast<const uint2*>(p), *reinterpret_cast<const uint2*>(p + 2 * Cb), v);
+    uint2 h, l;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(h.x), "=r"(h.y) : "r"(p));
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(l.x), "=r"(l.y) : "r"(p + 2 * Cb));
+    join4(h, l, v);
   } else {
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(p);
-    v[0] = t.x; v[1] = t.y;
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(p));
   }
 }
 
@@ -84,17 +88,18 @@ __device__ __forceinline__ void store4(uint8_t* __restrict__ p, uint32_t lo_off,
   }
 }
 
-struct DwUnit { int slab, ox0, oy0, n_out, img0; };     // ox0: first output column of the tile
+// The output rows of a slab are one sequence: row of the image fastest, then column tile, image group.  A block owns an
+// equal share of it, wherever that begins and ends, and walks it in pieces that stay inside one image; or, where a share
+// would be less than an image, a piece of one image.
+struct DwUnit { int ox0, oy0, n_out, img0; };           // ox0: first output column of the tile
 template <int COLS>
-__device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int u) {
+__device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int r, int r_end) {
   DwUnit d;
-  d.slab = u % p.n_slabs;
-  u /= p.n_slabs;
-  d.ox0 = (u % p.n_ct) * p.XG * COLS;
-  u /= p.n_ct;
-  d.oy0 = (u % p.n_rb) * p.rb;
-  d.n_out = min(p.rb, p.Ho - d.oy0);
-  d.img0 = (u / p.n_rb) * p.NI;
+  const int col = r / p.Ho, ig = col / p.n_ct;
+  d.oy0 = r - col * p.Ho;
+  d.n_out = min(p.Ho - d.oy0, r_end - r);
+  d.ox0 = (col - ig * p.n_ct) * p.XG * COLS;
+  d.img0 = ig * p.NI;
   return d;
 }
 
@@ -114,7 +119,13 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   const uint32_t bar_full = smem_u32(bars), bar_empty = bar_full + 8 * kDwMaxStages;
   volatile int* s_abort = reinterpret_cast<volatile int*>(bars + 2 * kDwMaxStages);
   float* s_w = reinterpret_cast<float*>(ring + p.stages * p.stage_bytes + (2 * kDwMaxStages + 2) * 8);   // [9 taps, scale, bias][Cb]
-  const int slab = (int)blockIdx.x % p.n_slabs;          // the grid is a multiple of the slabs: fixed for this block
+  const int share = (int)blockIdx.x / p.n_slabs, slab = (int)blockIdx.x - share * p.n_slabs;
+  int r_begin = share * p.rows + min(share, p.row_rem), r_end = r_begin + p.rows + (share < p.row_rem ? 1 : 0);
+  if (p.n_rb) {
+    const int col = share / p.n_rb;
+    r_begin = col * p.Ho + (share - col * p.n_rb) * p.rows;
+    r_end = min(r_begin + p.rows, (col + 1) * p.Ho);
+  }
 
   // expanded weights: a thread per channel of the slab
   for (int i = tid; i < p.Cb; i += (int)blockDim.x) {
@@ -149,12 +160,13 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   chain_release();
 
   if (tid >= n_compute) {
-    // ---- producer: padded input rows oy0 * STRIDE .. of every unit of this block, in order -----------
+    // ---- producer: padded input rows oy0 * STRIDE .. of every piece of this block, in order ----------
     chain_wait();
     bool alive = true;
     uint32_t stage = 0, phase = 0, issued = 0, issued_phase = 0;
-    for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
-      const DwUnit d = dw_unit<COLS>(p, u);
+    for (int r0 = r_begin; r0 < r_end && alive;) {
+      const DwUnit d = dw_unit<COLS>(p, r0, r_end);
+      r0 += d.n_out;
       const int n_rows = (d.n_out - 1) * STRIDE + 3;
       const int img = job.in_version * p.batch_capacity + d.img0;
       for (int r = 0; r < n_rows; ++r) {
@@ -163,7 +175,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
         issued |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
         expect_tx_elect(bar_full + 8 * stage, (uint32_t)p.box_bytes);
-        tma_load_5d_elect(smem_u32(ring) + stage * p.stage_bytes, &in_map, bar_full + 8 * stage, d.slab * p.Cb, 0,
+        tma_load_5d_elect(smem_u32(ring) + stage * p.stage_bytes, &in_map, bar_full + 8 * stage, slab * p.Cb, 0,
                           d.ox0 * STRIDE - 1, d.oy0 * STRIDE + r, img);
         if (++stage == (uint32_t)p.stages) { stage = 0; phase ^= 1u; }
       }
@@ -190,14 +202,13 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
 
   chain_wait();                                          // the output slot may still be read by an earlier kernel
   constexpr int IN_COLS = (COLS - 1) * STRIDE + 3;
-  const uint8_t* my_cols = ring + (size_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
-                           (size_t)q * (FMT == ACT_SPLIT ? 8 : 16);
+  const uint32_t my_cols = smem_u32(ring) + (uint32_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
+                           (uint32_t)q * (FMT == ACT_SPLIT ? 8 : 16);
   uint32_t stage = 0, phase = 0;
   bool alive = true;
-  const float* my_w = s_w + q * 4;
+  const uint32_t my_w = smem_u32(s_w) + q * 16;
   auto coef = [&](int k, uint64_t (&v)[2]) {             // the four channels of row k of s_w
-    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(my_w + k * p.Cb);
-    v[0] = t.x; v[1] = t.y;
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(my_w + k * p.Cb * 4));
   };
   // The next padded row: wait, accumulate it as tap row RA into `a`, RB into `b` and RC into `cc` (-1: not
   // at all; the first contribution to `cc` is written, not added) and hand the stage back.
@@ -205,7 +216,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     constexpr int RA = decltype(ra)::value, RB = decltype(rb_)::value, RC = decltype(rc)::value;
     alive = mbar_wait_warp(bar_full + 8 * stage, phase, s_abort, p.error_flag);
     if (!alive) return false;
-    const uint8_t* src = my_cols + stage * p.stage_bytes;
+    const uint32_t src = my_cols + stage * p.stage_bytes;
     uint64_t v[IN_COLS][2];
 #pragma unroll
     for (int xx = 0; xx < IN_COLS; ++xx) read4<FMT>(src + xx * col_bytes, p.Cb, v[xx]);
@@ -243,8 +254,9 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   using I2 = std::integral_constant<int, 2>;
   using IN = std::integral_constant<int, -1>;
 
-  for (int u = blockIdx.x; u < p.n_units && alive; u += gridDim.x) {
-    const DwUnit d = dw_unit<COLS>(p, u);
+  for (int r0 = r_begin; r0 < r_end && alive;) {
+    const DwUnit d = dw_unit<COLS>(p, r0, r_end);
+    r0 += d.n_out;
     const int b = d.img0 + ni, ox = d.ox0 + xg * COLS;
     const bool writes = worker && b < p.B && c < p.Cs && ox < p.Wo;
     uint8_t* outp = static_cast<uint8_t*>(job.out) + ch_off + (((size_t)b * (p.Ho + 2) + d.oy0 + 1) * p.Wo + ox) * pix_bytes;
@@ -307,7 +319,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
         emit(acc);
       }
     }
-    // the two physical padding rows of the image, by the first and the last row block
+    // the two physical padding rows of the image, by the pieces that hold the first and the last row
     if (writes) {
       const float zero[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -374,8 +386,8 @@ DwShape dw_shape(const ConvGeom& g, int batch_capacity) {
   return s;
 }
 
-// Rows of a block and blocks per slab (see launch_depthwise).
-struct DwSplit { int rb, n_rb, k; };
+// Blocks per slab, blocks per image column or 0, rows of a block (see launch_depthwise).
+struct DwSplit { int k, n_rb, rows; };
 
 }  // namespace
 
@@ -420,43 +432,46 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
   const int fixed = 128 + (2 * kDwMaxStages + 2) * 8 + 11 * sh.Cb * 4;
   p.stages = std::min(kDwMaxStages, (per_cta - fixed) / p.stage_bytes);
   if (p.stages < 2) return set_error(AIQ_ERR_SHAPE, "depthwise: %d bytes per input row do not fit shared memory", p.stage_bytes);
-  // Row blocks and blocks per slab (the grid is a multiple of the slabs: a block then keeps its weights), chosen
-  // together: cost of a wave = input rows its blocks walk, halo rows included, and a start-up of about six rows;
-  // cutting images into row blocks pays where whole images would leave the last wave nearly empty (at 256 x 32 x 32 x
-  // 144 channels 192 of 296 resident blocks had work, each for two images) or are fewer than the blocks.
+  // Blocks per slab.  Cost of a wave = input rows of a block, two halo rows per piece and a start-up of about six rows
+  // included; a wave lasts as long however few blocks it has.  Equal shares keep every SM busy to the end (256 x 16 x 16 x
+  // 384 channels: 228 blocks of two units each 54.7 us, 288 equal ones 47.5), pieces of one image save halo rows where a
+  // share is shorter than an image (32 x 14 x 14 x 576: 15.7 us against 17).
   const int resident = 2 * props.n_sms;
-  const long long columns = (long long)p.n_ig * p.n_ct;        // units per slab and row block
+  const long long columns = (long long)p.n_ig * p.n_ct, total = columns * g.Ho;   // output rows of a slab
+  if (total >= (1ll << 31)) return set_error(AIQ_ERR_SHAPE, "depthwise: %lld rows of a channel slab", total);
+  const int halo = 3 - g.stride;
+  auto block_rows = [&](long long rows, bool one_piece) {
+    return rows * g.stride + halo * (one_piece ? 1 : 1 + (rows + g.Ho - 2) / g.Ho);
+  };
   static thread_local ConfigMemo<DwSplit, 8> memo;
   const int key[8] = {g.Ho, g.stride, p.n_ig, p.n_ct, p.n_slabs, n_jobs, resident, 0};
   DwSplit split;
   memo.get(key, &split, [&](DwSplit* out) {
-    *out = {g.Ho, 1, 1};
     double best = 1e300;
-    for (int n = 1; n <= g.Ho; n = n < 4 ? n + 1 : n + n / 2) {
+    *out = {1, 0, (int)total};
+    auto take = [&](long long k, long long rows, int n_rb) {
+      const long long ctas = k * p.n_slabs * n_jobs;
+      const double cost = (double)((ctas + resident - 1) / resident) * (block_rows(rows, n_rb > 0) + 6.0);
+      if (cost < best * 0.999 && k * p.n_slabs < (1ll << 30)) { best = cost; *out = {(int)k, n_rb, (int)rows}; }
+    };
+    for (int n = 1; n <= g.Ho; n = n < 16 ? n + 1 : n + n / 8) {
       const int rb = (g.Ho + n - 1) / n, n_rb = (g.Ho + rb - 1) / rb;
-      const long long per_slab = columns * n_rb;
-      const double rows = (rb - 1) * g.stride + 3;
-      for (int w = 1; w <= 5; ++w) {
-        long long k = w == 5 ? per_slab : (long long)w * resident / ((long long)p.n_slabs * n_jobs);
-        k = std::max(1ll, std::min(k, per_slab));
-        const long long each = (per_slab + k - 1) / k;
-        k = (per_slab + each - 1) / each;
-        const long long ctas = k * p.n_slabs * n_jobs;
-        const double cost = (double)((ctas + resident - 1) / resident) * (each * rows + 6.0);
-        if (cost < best * 0.999 && k * p.n_slabs < (1ll << 30)) { best = cost; *out = {rb, n_rb, (int)k}; }
-        if (k == per_slab) break;
-      }
+      take(columns * n_rb, rb, n_rb);
+    }
+    for (int w = 1; w <= 6; ++w) {
+      const long long k = std::max(1ll, std::min(total, (long long)w * resident / ((long long)p.n_slabs * n_jobs)));
+      take(k, (total + k - 1) / k, 0);
     }
     return true;
   });
-  p.rb = split.rb; p.n_rb = split.n_rb;
-  const int best_k = split.k;
-  p.n_units = p.n_ig * p.n_rb * p.n_ct * p.n_slabs;
+  p.k = split.k;
+  p.n_rb = split.n_rb;
+  p.rows = split.n_rb ? split.rows : (int)(total / p.k);
+  p.row_rem = split.n_rb ? 0 : (int)(total % p.k);
   // no more stages than rows a block walks (small launches: what is left of the SM is the next kernel's)
-  const long long block_rows = (long long)((p.n_units / p.n_slabs + best_k - 1) / best_k) * ((p.rb - 1) * g.stride + 3);
-  p.stages = (int)std::min<long long>(p.stages, std::max(2ll, block_rows));
+  p.stages = (int)std::min<long long>(p.stages, std::max(2ll, block_rows(split.rows, split.n_rb > 0)));
   const int smem = p.stages * p.stage_bytes + fixed;
-  const dim3 grid((unsigned)(best_k * p.n_slabs), n_jobs);
+  const dim3 grid((unsigned)(p.k * p.n_slabs), n_jobs);
   LaunchScope scope(AIQ_KERNEL_DEPTHWISE, s, 18.0 * g.B * g.Ho * g.Wo * g.Cout * n_jobs,
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                    (double)g.B * g.Ho * g.Wo * g.Cout));

@@ -57,7 +57,7 @@ def eval_workload(name):
                     chunk=32, workload="mobilenet_v2_imagenet_coordinate_step: 52 schemes (all-8, one conv layer -> "
                                        "32 / 16 / 4 bits) x 2048 images of 3x224x224",
                     metric="scheme evals/sec (MobileNetV2-ImageNet, 2048 imgs)", oracle_images=2, ref_images=1,
-                    tc_kernel="conv_pw_tc_kernel / conv_tc_kernel (tcgen05 bf16, fp32 accumulate)")
+                    tc_kernel="conv_pw_kernel / conv_tc_kernel (tcgen05 bf16, fp32 accumulate)")
     raise ValueError(name)
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel from one ncu

@@ -50,15 +50,13 @@ __device__ __forceinline__ void decode8(const uint4& q, int sub, float* f) {
 // of the packed rows.
 template <int BITS, int MT>
 __global__ void __launch_bounds__(kWarps * 32)
-qlinear_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K, int M) {
-  const LayerJob job = jobs ? jobs[blockIdx.z] : single;
+qlinear_kernel(LayerJob job, int N, int K, int M) {
   constexpr int E = 128 / BITS;                 // elements per 16-byte chunk
   constexpr int SUBS = (E >= 8) ? E / 8 : 1;    // 8-element sub-chunks (fp32: one of 4)
   constexpr int SE = (E >= 8) ? 8 : 4;          // elements per sub-chunk
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int n0 = (blockIdx.x * kWarps + warp) * kRowsPerWarp;
-  const int m0 = blockIdx.y * MT;
   chain_release();
   chain_wait();
   if (n0 >= N) return;
@@ -88,7 +86,7 @@ qlinear_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K,
       float xv[MT][SE];
 #pragma unroll
       for (int m = 0; m < MT; ++m) {
-        const int mm = min(m0 + m, M - 1);
+        const int mm = min(m, M - 1);
         const float* xp = x + (size_t)mm * K + k0;
         if (xvec && k0 + SE <= K) {
 #pragma unroll
@@ -136,7 +134,7 @@ qlinear_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K,
       const float b = job.bias ? job.bias[n] : 0.0f;
 #pragma unroll
       for (int m = 0; m < MT; ++m)
-        if (m0 + m < M) static_cast<float*>(job.out)[(size_t)(m0 + m) * N + n] = fmaf(acc[r][m], s, b);
+        if (m < M) static_cast<float*>(job.out)[(size_t)m * N + n] = fmaf(acc[r][m], s, b);
     }
   }
 }
@@ -352,9 +350,9 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
     while (cluster < 8 && n_tiles * cluster * 2 <= 64 && n_slices > cluster * GemmTile<32, 16>::KG) cluster *= 2;
     if (aiq_status_t st = launch_gemm_tile<BITS, 32, 16>(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s, cluster)) return st;
   } else if (M == 1) {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 1>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 1>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
   } else if (M == 2) {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 2>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 2>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
   } else if (M > 4) {
     // The largest tile that still gives every SM a block; smaller ones split K over more thread groups.  The tile of 8 rows
     // leaves out the work of rows that are not there (8191 x 8191, 5 rows, 4 bits: 72 us against 94 with the tile of 16).
@@ -368,7 +366,7 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
     else st = args(launch_gemm_tile<BITS, 32, 16>);
     if (st != AIQ_OK) return st;
   } else {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 4>, dim3(gx, 1, n_jobs), dim3(kWarps * 32), 0, s, single, jobs_dev, N, K, M));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 4>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
   }
   AIQ_LAUNCH_CHECK("qlinear");
   return AIQ_OK;

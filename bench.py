@@ -449,8 +449,8 @@ def main():
                          "kernels where the network allows), tiles (pixel-tile tensor-core kernels), fp32")
     ap.add_argument("--fuse-inverted-residual", action="store_true",
                     help="run every eligible inverted-residual block of MobileNetV2 as one kernel (aiq_set_fusion bit 1; "
-                         "the default fuses a block only where that was measured faster)")
-    ap.add_argument("--no-fuse-inverted-residual", action="store_true", help="never fuse inverted-residual blocks")
+                         "default: layer by layer)")
+    ap.add_argument("--no-fuse-inverted-residual", action="store_true", help="never fuse inverted-residual blocks (the default)")
     args = ap.parse_args()
 
     rank = int(os.environ.get("RANK", "0"))

@@ -298,9 +298,9 @@ aiq_status_t aiq_eval_schemes(const aiq_model_t* model, const uint8_t* schemes, 
                               int32_t* correct_counts, int32_t* preds, void* workspace,
                               size_t workspace_bytes, void* stream);
 
-/* Evaluation knobs (process-wide, for experiments and tests; results never depend on
- * them).  chunk: images per pass, 0 = choose from the workspace size.  share_prefix: 0
- * evaluates every scheme independently. */
+/* Evaluation knobs (process-wide, for experiments and tests; results do not depend on them, except that
+ * chunk x schemes decides which view of a small-pass model runs, see aiq_set_small_pass_images).  chunk: images
+ * per pass, 0 = choose from the workspace size.  share_prefix: 0 evaluates every scheme independently. */
 void aiq_set_eval_options(int chunk, int share_prefix);
 
 /* Kernel fusion on networks stored for the row-streaming kernel (process-wide, both default on; the
@@ -309,13 +309,13 @@ void aiq_set_eval_options(int chunk, int share_prefix);
  *           convolutions of 16 or 32 channels runs as one kernel whenever every scheme of the call gives
  *           both convolutions 4 or 8 bits: the intermediate tensor stays in shared memory.  Results are
  *           bit-identical to the layer-by-layer path.
- *           bit 2 (default on) / bit 1 (default off): a MobileNetV2 inverted-residual block (expansion 1x1 -> depthwise 3x3 ->
+ *           bit 1 (default off): a MobileNetV2 inverted-residual block (expansion 1x1 -> depthwise 3x3 ->
  *           projection 1x1, optional shortcut) runs as one kernel whenever every scheme gives both 1x1
  *           layers 4 or 8 bits: the six-fold hidden tensor stays in shared memory (float32 there, so the
  *           results differ from the layer-by-layer path by that path's rounding of the hidden tensor).
- *           Bit 2 fuses a block only where the fused kernel was measured faster than the three layer kernels
- *           (stride 1 on maps 8 columns wide, when the pass has at least 128 bands of 128 output pixels and
- *           no more of them than the GPU has SMs); bit 1 fuses every eligible block.
+ *           Bit 2 asks for that only where the fused kernel is faster than the three layer kernels: at
+ *           present nowhere, so it is accepted and selects no block.  (Where it is the faster one depends on
+ *           the images of the pass, and an image's logits must not.)
  *   pool:   the classifier's global average pool is taken in the epilogue of the convolution that
  *           produces its input; that tensor is then never stored.  Sums are formed in a fixed order
  *           (run-to-run identical); they differ from the separate pooling kernel's in the last bits. */

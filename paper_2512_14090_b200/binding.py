@@ -249,7 +249,8 @@ def aiq_quantize_layer_per_tensor(W, bits, packed_out, scales_out, scratch, nonf
 
 
 def aiq_set_fusion(blocks=True, pool=True, inverted_residual="auto"):
-    """inverted_residual: "auto" (fuse where measured faster), True (every eligible block), False."""
+    """inverted_residual: True (every eligible block), False, or "auto" (where the fused kernel is faster whatever the
+    batch: at present no block)."""
     ir = 4 if inverted_residual == "auto" else (2 if inverted_residual else 0)
     lib.aiq_set_fusion(int(bool(blocks)) | ir, int(bool(pool)))
 

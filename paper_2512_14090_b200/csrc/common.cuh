@@ -308,8 +308,6 @@ struct MbTileJob {
   int32_t role, bits, N, K, nh, cs;
 };
 aiq_status_t launch_mb_build_tiles(const MbTileJob* jobs_dev, int n_jobs, cudaStream_t s);
-// whether the fused kernel is expected to beat the layer kernels for this block at this batch (measured policy)
-bool mb_block_pays(const ConvGeom& gd, const ConvGeom& gp);
 // nh: the chunk width the jobs' operand images were built for
 aiq_status_t launch_mb_block(const ConvGeom& ge, const ConvGeom& gd, const ConvGeom& gp, int nh, const LayerJob* jobs_dev, int n_jobs,
                              int32_t* error_flag, double weight_bytes, cudaStream_t s);

@@ -40,6 +40,14 @@
 // the MMAs they wait for); whether to go on after a wait is decided by one thread before the named
 // barrier and read by all after it, so all workers leave at the same barrier.  Every wait is bounded
 // as in the other tcgen05 kernels.
+//
+// Not chosen by default: it runs where aiq_set_fusion asks for it.  Microseconds of a forward pass through one block, layer
+// by layer / fused: 8-wide maps, 160 -> 160 channels: 64 bands 64 / 81, 128 bands 77 / 86, 148 bands (one wave) 94 / 89, 256
+// bands 128 / 157; 160 -> 320: 128 bands 86 / 91, 148 bands 102 / 96; 7-wide, 148 bands 86 / 91; 16-wide, stride 2, 256: 154 /
+// 203; 56-wide, stride 2, 32: 84 / 99; 32-wide, stride 2, 256: 176 / 210.  One block by itself wins by 5 % at one full wave of
+// CTAs; inside the whole MobileNetV2-CIFAR the layer kernels are faster there too (128 images 1,087 / 1,121, 148 images
+// 1,240 / 1,258).  And the float32 hidden tensor rounds otherwise than the layer kernels' split one, so a choice by the
+// batch would let an image's logits depend on the images around it.
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -590,20 +598,6 @@ int mb_block_chunk_channels(const ConvGeom& ge, const ConvGeom& gd, const ConvGe
   if (current_device_props(&props) != AIQ_OK) return 0;
   const MbConfig c = mb_config(ge, gd, gp, props.smem_optin);
   return c.ok ? c.NH : 0;
-}
-
-// Where the fused kernel competes with the layer kernels (B200; microseconds of a forward pass through one block, layer
-// by layer / fused): 8-wide maps once the bands are one full wave of CTAs (160 -> 160 channels: 128 bands 77 / 86, 148
-// bands 94 / 89; 160 -> 320: 86 / 91 and 102 / 96).  With fewer bands its CTAs work through their chunks of hidden
-// channels one after the other on a part of the GPU (64 bands: 64 / 81), with more a second wave starts (256: 128 / 157),
-// 7-wide maps leave accumulator lanes idle (148: 86 / 91), and on wider maps the layer kernels win at every batch
-// (16-wide, stride 2, 256: 154 / 203; 56-wide, stride 2, 32: 84 / 99; 32-wide, stride 2, 256: 176 / 210).
-bool mb_block_pays(const ConvGeom& gd, const ConvGeom& gp) {
-  DeviceProps props;
-  if (current_device_props(&props) != AIQ_OK) return false;
-  const int rb = std::min(std::max(128 / gp.Wo, 1), gp.Ho);        // band height of mb_config's first choice
-  const long long ctas = (long long)gp.B * ((gp.Ho + rb - 1) / rb);
-  return gd.W == 8 && gd.stride == 1 && ctas >= 128 && ctas <= props.n_sms;
 }
 
 aiq_status_t launch_mb_build_tiles(const MbTileJob* jobs_dev, int n_jobs, cudaStream_t s) {

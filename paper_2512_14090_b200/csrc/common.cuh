@@ -119,7 +119,8 @@ inline cudaError_t launch_chained(bool chain, void (*kernel)(P...), dim3 grid, d
 }
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // What a kernel of the chain reads of an earlier one's results: an ordinary load, not the read-only path, whose lines
-// may be older than the wait and which the compiler may move above it.
+// may be older than the wait and which the compiler may move above it.  The pointer must not be `const __restrict__` either:
+// with that the compiler may choose the read-only path by itself.
 template <typename T>
 __device__ __forceinline__ T ld_chain(const T* p) { return *p; }
 __device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

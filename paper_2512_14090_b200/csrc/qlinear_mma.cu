@@ -158,7 +158,7 @@ qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __rest
 template <int BITS, int NT, int GROUPS>
 __global__ void __launch_bounds__(kMmaWarps * 32)
 qlinear_mma_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scale, const float* __restrict__ bias,
-                   const uint8_t* __restrict__ ws, int n_groups, float* __restrict__ y, int N, int K, int M) {
+                   const uint8_t* ws, int n_groups, float* __restrict__ y, int N, int K, int M) {
   constexpr int SLICE = GROUPS * kGroupK;
   constexpr int KL = BITS == 4 ? 32 : 16;          // k per lane per stage (one 16-byte unit)
   constexpr int CHUNK = 4 * KL;                    // k per stage: 128 / 64

@@ -171,8 +171,7 @@ __device__ __forceinline__ void expand8_half(uint2 raw, uint32_t* o) {
 template <int BITS>
 __global__ void __launch_bounds__(QtKind<BITS>::THREADS, 1)
 qlinear_tc_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ CUtensorMap w_map, QtParams p,
-                  const float* __restrict__ scale, const float* __restrict__ bias, const float* __restrict__ down,
-                  float* __restrict__ y) {
+                  const float* __restrict__ scale, const float* __restrict__ bias, const float* down, float* __restrict__ y) {
   using T = QtKind<BITS>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);

@@ -125,7 +125,8 @@ void aiq_set_scale_granularity(int granularity);
  *   M <= 4, 4 / 8 bits, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: no workspace;
  *     the codes stay integer and feed the int8 warp-level tensor cores, the activations of every
  *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest
- *     |x|), the int32 sums are exact and run-to-run identical.
+ *     |x|), the int32 sums are exact and run-to-run identical; a batch row with an infinity or a
+ *     NaN is multiplied in float32, as by the plain kernel.
  *   M <= 8 otherwise, 4 / 8 bits, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
  *     warp-level tensor cores; the activations of each group of 512 k become three int8
  *     digits with a shared exponent (21 bits below the group's largest |x|), the int32 sums

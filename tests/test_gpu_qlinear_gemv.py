@@ -60,3 +60,41 @@ def test_gemv_exact_on_integers_and_nonfinite_rows(bits):
     aiq.aiq_qlinear(packed, scales, None, N, K, bits, to_dev(x), y)
     got = y.cpu().numpy()
     assert np.isfinite(got[:2]).all() and not np.isfinite(got[2:]).any()
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("N,K,M", [(1030, 777, 2), (2999, 1000, 4), (40, 8190, 3), (2500, 4096, 1)])
+def test_gemv_infinite_activations(bits, N, K, M):
+    """An infinite activation gives an infinity of the code's sign, or a NaN where the code is zero or two infinities
+    meet, as float32 products do; rows without one are as accurate as ever."""
+    import torch
+    aiq = binding()
+    rng = np.random.default_rng(N + K + M + bits)
+    W = rng.standard_normal((N, K)).astype(np.float32)
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(to_dev(W), bits, packed, scales)
+    v, s = O.quantize_rows(W, bits)
+    w = v.astype(np.float64) * np.asarray(s, np.float64)[:, None]
+    cases = [[(0, 5, np.inf)], [(0, K - 1, -np.inf), (M - 1, 600, np.inf)], [(M - 1, 3, np.inf), (M - 1, K - 2, np.inf)],
+             [(M - 1, 1, -np.inf), (0, 2, np.nan)]]
+    for case in cases:
+        xi = x.copy()
+        for m, k, val in case:
+            xi[m, k] = val
+        y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+        aiq.aiq_qlinear(packed, scales, None, N, K, bits, to_dev(xi), y)
+        got = y.cpu().numpy()
+        fin = np.where(np.isfinite(xi), xi, 0).astype(np.float64)
+        want = fin @ w.T
+        bound = 2.0 ** -20 * np.abs(fin).max() * np.abs(w).sum(axis=1)[None, :] + 2.0 ** -22 * np.abs(want)
+        with np.errstate(invalid="ignore"):
+            for m, k, val in case:
+                want[m] += float(val) * w[:, k]
+            assert np.array_equal(np.isnan(got), np.isnan(want))
+            inf = np.isinf(want)
+            assert inf.any() or np.isnan(want).any()
+            assert np.array_equal(np.isinf(got), inf) and np.array_equal(np.sign(got[inf]), np.sign(want[inf]))
+            fine = np.isfinite(want)
+            assert np.all(np.abs(got[fine] - want[fine]) <= np.broadcast_to(bound, want.shape)[fine])

@@ -17,8 +17,9 @@
 //     memory in a fixed order: no second kernel, no workspace, no atomics, run-to-run identical;
 //   - nothing joins the warps inside the stream: they wait for a unit's copies only, and the output of up to eight units
 //     is formed together after it (a block barrier and an output per unit cost 0.5 us each).
-// The two kernels this replaces at these sizes (a digit pass over x, then the matrix with its K slices meeting in y through
-// atomics) took 18.7 us at 8192 x 8192, 4 bits, one row, 11.5 now (8 bits: 18.8 and 14.5; 2048 x 2048: 13.0 and 6.2).
+// The two kernels this replaces at these sizes (a digit pass over x with three digits, then the matrix with its K slices
+// meeting in y through atomics), on the device, calls back to back, one and four rows, before -> now: 8192 x 8192, 4 bits
+// 13.4 -> 12.4 and 16.5 -> 16.7 us, 8 bits 18.4 -> 14.0 and 22.3 -> 18.2; 2048 x 8192, 4 bits 10.2 -> 5.6 and 12.4 -> 10.8.
 #include "tc_ptx.cuh"
 
 #include <algorithm>
@@ -32,9 +33,16 @@ constexpr int kGvFrags = 16;                         // k32 fragments of a warp'
 constexpr int kGvMaxSlots = 16;
 constexpr int kGvEpoch = 8;                          // units per warp between two outputs
 constexpr int kGvMaxRows = 4;                        // batch rows
-constexpr int kGvDigWords = 256 + 64;                // of half a slice
+constexpr int kGvRowWords = 128 + 32;                // digit words of 128 k of a batch row
+constexpr int kGvDigWords = 2 * kGvRowWords;
 static_assert(kGvEpoch * kGvMaxRows * 8 <= kGvDigWords, "the partial sums take the place of the digit words");
 __device__ __forceinline__ int gv_dig(int k) { return k + (k >> 4) * 4; }
+// max(a, |b|), a NaN if either is one
+__device__ __forceinline__ float max_abs_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(fabsf(b)));
+  return r;
+}
 
 struct GvParams {
   int N, K, M;
@@ -77,11 +85,14 @@ __device__ __noinline__ void gv_nonfinite_rows(const uint8_t* __restrict__ w, co
       }
 }
 
-// HALVES: 1 for one or two batch rows (digit rows 0 .. 7), 2 for up to four.
-template <int BITS, int HALVES>
+// ROWS: batch rows at most, 1, 2 or 4.
+template <int BITS, int ROWS>
 __global__ void __launch_bounds__(kGvWarps * 32, 1)
 qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scale, const float* __restrict__ bias,
                     const float* x, float* y, GvParams p) {
+  constexpr int HALVES = ROWS > 2 ? 2 : 1;           // of the 16 digit rows of an MMA
+  constexpr int RP = ROWS > 1 ? 2 : 1;               // batch rows converted at a time
+  constexpr int QP = 2 / RP;                         // and parts of 128 k of each
   constexpr int CHUNK_K = 512 / BITS;                // k of a 64-byte chunk: 128 / 64
   constexpr int LANE_K = CHUNK_K / 4;                // k of a lane's 16 bytes of it: 32 / 16
   constexpr int MPC = CHUNK_K / 32;                  // MMAs per chunk: 4 / 2
@@ -113,26 +124,26 @@ qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ sca
 
   const int slice_k = p.cw * CHUNK_K, k0 = kwi * slice_k;
   const bool vec = (p.K & 3) == 0 && (((uintptr_t)x) & 15) == 0;
-  auto load_x = [&](int m, float4 (&q)[4]) {
+  auto load_x = [&](int m, int j) {                  // four elements of row m: k = 128 j + 4 lane of the slice
     const float* xr = x + (size_t)m * p.K;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int kl = j * 128 + lane * 4, k = k0 + kl;
-      q[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (kl < slice_k) {
-        if (vec && k + 4 <= p.K) q[j] = *reinterpret_cast<const float4*>(xr + k);
-        else {
-          if (k < p.K) q[j].x = xr[k];
-          if (k + 1 < p.K) q[j].y = xr[k + 1];
-          if (k + 2 < p.K) q[j].z = xr[k + 2];
-          if (k + 3 < p.K) q[j].w = xr[k + 3];
-        }
+    const int kl = j * 128 + lane * 4, k = k0 + kl;
+    float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (m < p.M && kl < slice_k) {
+      if (vec && k + 4 <= p.K) q = *reinterpret_cast<const float4*>(xr + k);
+      else {
+        if (k < p.K) q.x = xr[k];
+        if (k + 1 < p.K) q.y = xr[k + 1];
+        if (k + 2 < p.K) q.z = xr[k + 2];
+        if (k + 3 < p.K) q.w = xr[k + 3];
       }
     }
+    return q;
   };
-  float4 xv[4], xn[4];
-  load_x(0, xv);                                     // ahead of the weights, which would queue in front of it
-  if (p.M > 1) load_x(1, xn);
+  float4 xv[RP][4];                                  // ahead of the weights, which would queue in front of it
+#pragma unroll
+  for (int r = 0; r < RP; ++r)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) xv[r][j] = load_x(r, j);
 
   // rows of step i -> slot i mod slots, by one warp.  (Issuing a bulk copy takes about 50 ns: one warp alone needed 2.5 us for
   // the 48 first ones, so each first slot has a warp of its own.)
@@ -156,55 +167,72 @@ qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ sca
     for (int i = 0; i < 2 * HALVES; ++i) a[f][i] = 0u;
 #pragma unroll
   for (int h = 0; h < HALVES; ++h) { down[h] = 0.f; corr[h] = 0; }
+  // Two batch rows at a time, 128 k of both, so that every lane has a row to gather from; the arithmetic is packed float32.
+  // (Issue slots bound it.  One row at a time and scalar it was 2.1 us a row; 4 bits, 8192 x 8192, four rows 18.5 -> 16.7 us,
+  // 2048 x 8192 12.7 -> 10.8, two rows 7.9 -> 6.6; 8 bits, 8192 x 8192, four rows 20.7 -> 18.2.)
   uint32_t* my_dig = s_dig + warp * kGvDigWords;     // word k at gv_dig(k): four words of padding per 16, against bank conflicts
-  for (int m = 0; m < p.M; ++m) {
-    float v[16];
-    uint32_t mx = 0;
+  const uint32_t d = g & 3, sel = d | ((d + 4u) << 4);            // byte d of two words
+  const uint64_t magic = pack2(12582912.f, 12582912.f), m128 = pack2(128.f, 128.f);
+#pragma unroll 1
+  for (int m0 = 0; m0 < (ROWS > 2 ? p.M : 1); m0 += RP) {
+    float up[RP];
+    int e_mine = 0;                                               // exponent of this lane's row, m0 + (g >> 2)
+    bool finite_mine = true;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { v[4 * j] = xv[j].x; v[4 * j + 1] = xv[j].y; v[4 * j + 2] = xv[j].z; v[4 * j + 3] = xv[j].w; }
+    for (int r = 0; r < RP; ++r) {
+      float top = 0.f;                                            // a NaN stays one
 #pragma unroll
-    for (int j = 0; j < 16; ++j) mx = max(mx, (uint32_t)__float_as_int(v[j]) & 0x7FFFFFFFu);
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    // 2^(e-1) <= largest |x| < 2^e; slices of zeros and of denormals share the smallest exponent
-    const int e = max((int)(mx >> 23) - 126, -90);
-    const float up = __int_as_float((6 - e + 127) << 23);
-    const bool finite = mx < 0x7F800000u;
-    if (!finite && lane == 0) atomicOr(s_bad, 1u << m);
+      for (int j = 0; j < 4; ++j)
+        top = max_abs_nan(max_abs_nan(max_abs_nan(max_abs_nan(top, xv[r][j].x), xv[r][j].y), xv[r][j].z), xv[r][j].w);
+      const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(top));
+      // 2^(e-1) <= largest |x| < 2^e; slices of zeros and of denormals share the smallest exponent
+      const int e = max((int)(mx >> 23) - 126, -90);
+      const bool finite = mx < 0x7F800000u;
+      if (!finite && lane == 0) atomicOr(s_bad, 1u << (m0 + r));  // its digits are never used
+      up[r] = __int_as_float((6 - min(e, 128) + 127) << 23);
+      if (RP == 1 || (g >> 2) == r) { e_mine = e; finite_mine = finite; }
+    }
     uint32_t sum = 0;
-    const uint32_t d = g & 3, sel = d | ((d + 4u) << 4);          // byte d of two words
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {                        // 256 k of the slice at a time
-      if (256 * half >= slice_k) break;
+    for (int j0 = 0; j0 < 4; j0 += QP) {
+      if (128 * j0 >= slice_k) break;
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        if (256 * half + 128 * j >= slice_k) break;
+      for (int part = 0; part < 2; ++part) {                      // row m0 + part, or the part of 128 k after j0
+        const int r = RP == 2 ? part : 0, j = RP == 2 ? j0 : j0 + part;
+        if (RP == 2 ? m0 + r >= p.M : 128 * j >= slice_k) break;
         uint32_t word[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          float r = finite ? v[8 * half + 4 * j + i] * up : 0.f;  // |r| < 64; every step below is exact
-          // rint without the conversion unit (a quarter of the rate): adding 1.5 x 2^23 leaves the rounded integer in the
-          // low bits
-          uint32_t q4[4];
+        for (int i = 0; i < 2; ++i) {
+          // |v| < 64; every step below is exact.  rint without the conversion unit (a quarter of the rate): adding 1.5 x 2^23
+          // leaves the rounded integer in the low bits
+          uint64_t v = mul2(i ? pack2(xv[r][j].z, xv[r][j].w) : pack2(xv[r][j].x, xv[r][j].y), pack2(up[r], up[r]));
+          float2 q4[4];
 #pragma unroll
           for (int dd = 0; dd < 4; ++dd) {
-            const float q = __fadd_rn(r, 12582912.f);
-            q4[dd] = __float_as_uint(q);
-            r = __fmul_rn(__fsub_rn(r, __fsub_rn(q, 12582912.f)), 128.f);
+            const uint64_t q = add2(v, magic);
+            q4[dd] = unpack2(q);
+            if (dd < 3) v = mul2(sub2(v, sub2(q, magic)), m128);
           }
-          word[i] = __byte_perm(__byte_perm(q4[0], q4[1], 0x0040), __byte_perm(q4[2], q4[3], 0x0040), 0x5410);
+          auto bytes = [](float a, float b, float c, float e) {
+            return __byte_perm(__byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0040),
+                               __byte_perm(__float_as_uint(c), __float_as_uint(e), 0x0040), 0x5410);
+          };
+          word[2 * i] = bytes(q4[0].x, q4[1].x, q4[2].x, q4[3].x);
+          word[2 * i + 1] = bytes(q4[0].y, q4[1].y, q4[2].y, q4[3].y);
         }
-        *reinterpret_cast<uint4*>(my_dig + gv_dig(j * 128 + lane * 4)) = make_uint4(word[0], word[1], word[2], word[3]);
+        *reinterpret_cast<uint4*>(my_dig + part * kGvRowWords + gv_dig(lane * 4)) = make_uint4(word[0], word[1], word[2], word[3]);
+        if (ROWS > 2) xv[r][j] = load_x(m0 + 2 + r, j);           // the next pair
       }
       __syncwarp();
-      // lane (g, t) gathers digit g & 3 of batch row m into fragment row g = 4 (m & 1) + digit, half m >> 1
-      if ((g >> 2) == (m & 1)) {
+      // lane (g, t) gathers digit g & 3 of batch row m0 + (g >> 2) into fragment row g = 4 (m & 1) + digit, half m0 >> 1
+      if (m0 + (g >> 2) < p.M) {
 #pragma unroll
-        for (int c = 0; c < MAX_CW / 2; ++c) {
-          if (half * (MAX_CW / 2) + c >= p.cw) break;
+        for (int c = 0; c < QP * 128 / CHUNK_K; ++c) {
+          if (j0 * (128 / CHUNK_K) + c >= p.cw) break;
 #pragma unroll
-          for (int j = 0; j < MPC; ++j) {
-            // the eight k of this lane in MMA j of the chunk: 4 bits: 8 j ..: even ones, then odd ones; 8 bits: 8 j ..: in order
-            const uint32_t* src = my_dig + gv_dig(c * CHUNK_K + t * LANE_K + 8 * j);
+          for (int i = 0; i < MPC; ++i) {
+            // the eight k of this lane in MMA i of the chunk: 4 bits: 8 i ..: even ones, then odd ones; 8 bits: 8 i ..: in order
+            const uint32_t* src = my_dig + (RP == 2 ? (g >> 2) * kGvRowWords : 0) + gv_dig(c * CHUNK_K + t * LANE_K + 8 * i);
             const uint4 lo = *reinterpret_cast<const uint4*>(src), hi = *reinterpret_cast<const uint4*>(src + 4);
             uint32_t f0, f1;
             if (BITS == 4) {
@@ -216,26 +244,23 @@ qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ sca
             }
             sum = (uint32_t)__dp4a((int)f0, 0x01010101, (int)sum);
             sum = (uint32_t)__dp4a((int)f1, 0x01010101, (int)sum);
-            const int f = (half * (MAX_CW / 2) + c) * MPC + j;
+            const int f = (j0 * (128 / CHUNK_K) + c) * MPC + i;
 #pragma unroll
             for (int h = 0; h < HALVES; ++h)
-              if ((m >> 1) == h) { a[f][2 * h] = f0; a[f][2 * h + 1] = f1; }
+              if ((m0 >> 1) == h) { a[f][2 * h] = f0; a[f][2 * h + 1] = f1; }
           }
         }
       }
       __syncwarp();
     }
-    if ((g >> 2) == (m & 1)) {
+    if (m0 + (g >> 2) < p.M) {
 #pragma unroll
       for (int h = 0; h < HALVES; ++h)
-        if ((m >> 1) == h) {
+        if ((m0 >> 1) == h) {
           corr[h] = BITS == 4 ? 8 * (int)sum : 0;
-          down[h] = finite ? __int_as_float((e - 6 - 7 * (int)d + 127) << 23) : 0.f;
+          down[h] = finite_mine ? __int_as_float((e_mine - 6 - 7 * (int)d + 127) << 23) : 0.f;
         }
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) xv[j] = xn[j];
-    if (m + 2 < p.M) load_x(m + 2, xn);
   }
 #pragma unroll
   for (int h = 0; h < HALVES; ++h) {                 // digit sums of the row: its four lanes hold a quarter each
@@ -368,14 +393,15 @@ aiq_status_t launch_qlinear_gemv(const LayerJob& job, int N, int K, int M, cudaS
   const float* x = static_cast<const float*>(job.in);
   float* y = static_cast<float*>(job.out);
   LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K, (double)N * p.rb + 4.0 * N + 4.0 * M * ((double)K + N));
-#define AIQ_GEMV(B_, H_)                                                                                                  \
+#define AIQ_GEMV(B_, R_)                                                                                                  \
   do {                                                                                                                   \
-    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemv_kernel<B_, H_>), props.smem_optin);                                             \
-    AIQ_CUDA_TRY(launch_chained(true, qlinear_gemv_kernel<B_, H_>, dim3(grid), dim3(kGvWarps * 32), smem, s, job.w, job.scale, \
+    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemv_kernel<B_, R_>), props.smem_optin);                                             \
+    AIQ_CUDA_TRY(launch_chained(true, qlinear_gemv_kernel<B_, R_>, dim3(grid), dim3(kGvWarps * 32), smem, s, job.w, job.scale, \
                                 job.bias, x, y, p));                                                                     \
   } while (0)
-  if (job.bits == 4) { if (M <= 2) AIQ_GEMV(4, 1); else AIQ_GEMV(4, 2); }
-  else { if (M <= 2) AIQ_GEMV(8, 1); else AIQ_GEMV(8, 2); }
+#define AIQ_GEMV_ROWS(B_) do { if (M == 1) AIQ_GEMV(B_, 1); else if (M == 2) AIQ_GEMV(B_, 2); else AIQ_GEMV(B_, 4); } while (0)
+  if (job.bits == 4) AIQ_GEMV_ROWS(4); else AIQ_GEMV_ROWS(8);
+#undef AIQ_GEMV_ROWS
 #undef AIQ_GEMV
   AIQ_LAUNCH_CHECK("qlinear_gemv");
   return AIQ_OK;

@@ -147,7 +147,7 @@ qlinear_kernel(LayerJob job, int N, int K, int M) {
 // over: they form KG groups that take every KG-th slice of K, and where the tiles are fewer than the blocks the chip holds
 // a cluster of blocks shares a tile in the same way.  Their sums meet in shared memory, in a fixed order.
 // Bound by shared-memory reads (two cycles of them per cycle of multiplications) and, for small layers, by the latency of
-// a slice.  Measured, 4 bits, before (kernel above) and now: 8192 x 777, 5 rows 57.8 -> 11 us, 256 rows 1488 -> 118;
+// a slice.  Measured, 4 bits, before (kernel above) and now: 8192 x 777, 5 rows 57.5 -> 8.6 us, 256 rows 1486 -> 124;
 // 1001 x 1999, 64 rows 138 -> 15; 70 x 8190, 5 rows 140 -> 10.
 // Against the tensor-core path (pre-pass, zeroed y, atomics), 8 bits: 512 x 512, 64 rows 10.6 -> 5.6; 1024 x 1024, 64
 // rows 10.6 -> 9.2, 128 rows 13.6 | 14.5; 2048 x 2048, 16 rows 10.9 -> 9.3, 32 rows 12.4 | 15.
@@ -160,10 +160,12 @@ struct GemmTile {
   static constexpr int T = (BN / 4) * (BM / 4), KG = kGemmThreads / T;
   static constexpr int BUF = (BN + BM) * kGemmPitch;             // floats of one slice
   static constexpr int SMEM = KG * 2 * BUF * 4;
+  static constexpr int RESIDENT = SMEM > 113 * 1024 ? 1 : 2;     // blocks of an SM
 };
 
-template <int BITS, int BN, int BM>
-__global__ void __launch_bounds__(kGemmThreads)
+// LONG: see the sums below.
+template <int BITS, int BN, int BM, bool LONG>
+__global__ void __launch_bounds__(kGemmThreads, (LONG ? GemmTile<BN, BM>::RESIDENT : 0))
 qlinear_gemm_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, int K, int M, int cluster) {
   using G = GemmTile<BN, BM>;
   constexpr int T = G::T, KG = G::KG;
@@ -243,11 +245,22 @@ qlinear_gemm_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, i
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + kg), "n"(T) : "memory");
   };
 
-  uint64_t acc[4][4];                                            // [channel][row]: sums over even and over odd k
+  // LONG: a sum per slice, then the sum of those.  One chain over all slices of a group had up to three times the rounding
+  // error of the kernel above, whose lanes add K / 32 products each (8192 x 777, 256 rows: 3.5e-7 of the result's norm
+  // against 1.1e-7, now 1.2e-7).  It costs 1 to 5 % of the time, so it runs only where the chain, K / 2 over the groups of
+  // the tile, is longer than that lane's and than two slices.
+  float sum[4][4];                                               // [channel][row]
+  uint64_t acc[4][4];                                            // sums over even and over odd k; LONG: of one slice
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    for (int j = 0; j < 4; ++j) { sum[i][j] = 0.f; acc[i][j] = 0ull; }
+  auto add_up = [&]() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { const float2 f = unpack2(acc[i][j]); sum[i][j] += f.x + f.y; }
+  };
   int b = 0;
   const int first = rank * KG + kg, step = cluster * KG;
   if (first < n_slices) { fetch(first); stash(0); }
@@ -266,16 +279,13 @@ qlinear_gemm_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, i
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(w[i].y, v[j].y, fma2(w[i].x, v[j].x, acc[i][j]));
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma2(w[i].y, v[j].y, LONG && k == 0 ? mul2(w[i].x, v[j].x) : fma2(w[i].x, v[j].x, acc[i][j]));
     }
+    if (LONG) add_up();
     b ^= 1;
     if (s + step < n_slices) stash(b);
   }
-  float sum[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { const float2 f = unpack2(acc[i][j]); sum[i][j] = f.x + f.y; }
+  if (!LONG) add_up();
   auto put = [&](int i, float v) {
     const int n = n0 + tx + (i >> 2) * (BN / 4), m = m0 + ty + (i & 3) * (BM / 4);
     if (n < N && m < M) static_cast<float*>(job.out)[(size_t)m * N + n] = fmaf(v, job.scale[n], job.bias ? job.bias[n] : 0.0f);
@@ -321,16 +331,23 @@ template <int BITS, int BN, int BM>
 aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev, const LayerJob& single, int n_jobs, int N, int K, int M,
                               int n_sms, cudaStream_t s, int fixed_cluster) {
   using G = GemmTile<BN, BM>;
-  AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM>), (G::SMEM));
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, n_jobs);
   const long long blocks = (long long)grid.x * grid.y * grid.z;
   const int n_slices = (K + kGemmBK - 1) / kGemmBK;
   // blocks per tile: doubled while all blocks stay resident and a group of threads has more than one slice
-  constexpr int resident = G::SMEM > 113 * 1024 ? 1 : 2;
   int cluster = fixed_cluster ? fixed_cluster : 1;
-  while (!fixed_cluster && cluster < 8 && blocks * cluster * 2 <= resident * n_sms && n_slices > cluster * G::KG) cluster *= 2;
-  AIQ_CUDA_TRY(launch_chained_cluster(scope.chain, cluster, qlinear_gemm_kernel<BITS, BN, BM>, dim3(grid.x * cluster, grid.y, grid.z),
-                                      dim3(kGemmThreads), G::SMEM, s, single, jobs_dev, N, K, M, cluster));
+  while (!fixed_cluster && cluster < 8 && blocks * cluster * 2 <= G::RESIDENT * n_sms && n_slices > cluster * G::KG) cluster *= 2;
+  auto launch = [&](auto kernel) {
+    return launch_chained_cluster(scope.chain, cluster, kernel, dim3(grid.x * cluster, grid.y, grid.z), dim3(kGemmThreads), G::SMEM, s,
+                                  single, jobs_dev, N, K, M, cluster);
+  };
+  if (!jobs_dev && cluster * G::KG < 16 && n_slices > 2 * cluster * G::KG) {
+    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM, true>), (G::SMEM));
+    AIQ_CUDA_TRY(launch(qlinear_gemm_kernel<BITS, BN, BM, true>));
+  } else {
+    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM, false>), (G::SMEM));
+    AIQ_CUDA_TRY(launch(qlinear_gemm_kernel<BITS, BN, BM, false>));
+  }
   return AIQ_OK;
 }
 

@@ -37,3 +37,28 @@ def test_gemm_bound(bits, N, K, M):
     want = x.astype(np.float64) @ w.T + (0 if bias is None else bias.astype(np.float64))
     bound = (K + 2) * 2.0 ** -24 * (np.abs(x).astype(np.float64) @ np.abs(w).T) + 2.0 ** -22 * np.abs(want) + 1e-30
     assert np.all(np.abs(ys[0] - want) <= bound)
+
+
+@pytest.mark.parametrize("bits", [4, 16])
+@pytest.mark.parametrize("N,K,M", [(8192, 777, 64), (8192, 777, 6), (1001, 1999, 256), (9473, 4096, 72), (4800, 2100, 33)])
+def test_gemm_rounding_error(bits, N, K, M):
+    """Long chains of additions are broken up.  n additions in sequence leave about 2^-25 sqrt(n / 2) of the result's norm; a
+    lane's share of K / 32 products, or two levels of fewer, stays below 2^-24 (1.5 + sqrt(K) / 20); one chain of K / 2 does not."""
+    import torch
+    aiq = binding()
+    g = torch.Generator(device="cuda").manual_seed(N + K + M)
+    W = torch.randn(N, K, generator=g, device="cuda")
+    x = torch.randn(M, K, generator=g, device="cuda")
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, bits, packed, scales)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    aiq.aiq_qlinear(packed, scales, None, N, K, bits, x, y)
+    if bits == 16:
+        w = packed.view(torch.float16)[:, :K].double()
+    else:
+        codes = torch.stack([packed & 15, packed >> 4], 2).reshape(N, -1)[:, :K].to(torch.int16)
+        w = torch.where(codes > 7, codes - 16, codes).double() * scales.double()[:, None]
+    want = x.double() @ w.T
+    error = ((y.double() - want).norm() / want.norm()).item()
+    assert error <= 2.0 ** -24 * (1.5 + K ** 0.5 / 20)

@@ -134,7 +134,8 @@ void aiq_set_scale_granularity(int granularity);
  *   M >= 9, K a multiple of 8, K >= 64, N >= 32: a tcgen05 GEMM with the weight matrix as the
  *     MMA's M operand and the batch as its N operand.  4 / 8 / 16 bits: codes and halves are
  *     exact; the activations, scaled by a power of two per batch row, enter as the sum of two
- *     halves (relative rounding 2^-22, or 2^-39 of the row's largest |x|).  32 bits: weights and
+ *     halves (relative rounding 2^-22, with 8-bit weights and 1,024 or more k per thread block 2^-20; or
+ *     2^-39 of the row's largest |x|).  32 bits: weights and
  *     activations enter as sums of two bfloat16 (2^-17).  Accumulation is float32.
  * The last two split K over thread blocks where the matrix has too few rows to fill the GPU; the
  * partial sums then meet in y through float atomics (run-to-run differences in the last

@@ -11,8 +11,8 @@
 // 4, 8 and 16 bits: both operands are halves.  A = the integer codes as halves (exact), or the
 // stored halves themselves: a TMA tile of 16-bit weights is the A operand as it lands.  B = the
 // activations times a power of two per batch row that brings the row's largest |x| into [2^14,
-// 2^15), as the sum of two halves (hi + lo: 22 bits of each value, or 2^-39 of the row's maximum
-// where that is coarser); the power of two is taken out of the sums again, exactly.
+// 2^15), as the sum of two halves (hi + lo: 22 bits of each value - 20 at 8 bits and long sums, see the
+// pre-pass - or 2^-39 of the row's maximum where that is coarser); the power of two is taken out of the sums again, exactly.
 // 32 bits: both operands are bfloat16 sums hi + lo (a float32 weight has no bounded exponent).
 // A pre-pass writes the two planes of x into the caller's workspace; the main kernel starts under programmatic dependent launch, so its
 // weight prefetch overlaps the pre-pass.
@@ -87,8 +87,12 @@ inline int qt_smem_bytes(int a_stages, int Mt, int stack, int b_stages, int w_st
 // x [M][K] float32 -> planes hi [M][K], lo [M][K]; one block per batch row.
 //   HALF: x 2^-e = hi + lo in halves, 2^e in down[row] (PERM4: each 8 k in the order 0 4 1 5 2 6 3 7, in which the expanders
 //   unpack 4-bit codes); else hi + lo in bfloat16 (2^-17 of each value), down[row] = 1.
+//   HI8: hi keeps 8 of its 11 bits and lo takes the rest (2^-20 of each value instead of 2^-22).  The tensor cores drop what
+//   a product has below the accumulator's last bit; with 8-bit codes and long sums that costs more than it gains: error
+//   against 64 bits at 8192 x 8192, 8 bits, 16 / 256 rows 3.6e-6 / 8.4e-6 with 11 bits, 1.0e-6 / 5.9e-6 with 8 (bfloat16
+//   pairs: 2.6e-6 / 6.4e-6); 4096 x 4096, 16 rows 7.0e-7 and 3.6e-7; 2048 x 2048, short sums, 1.7e-7 and 3.2e-7.
 // Optionally y = 0 (the split-K partial sums are added atomically); the status word starts at 0.
-template <bool HALF, bool PERM4>
+template <bool HALF, bool PERM4, bool HI8>
 __global__ void __launch_bounds__(512)
 qlinear_split_x_kernel(const float* __restrict__ x, int K, int M, uint16_t* __restrict__ planes, float* __restrict__ down,
                        float* __restrict__ y, long long y_elems, int32_t* __restrict__ status) {
@@ -131,7 +135,13 @@ qlinear_split_x_kernel(const float* __restrict__ x, int K, int M, uint16_t* __re
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const float a = f[PERM4 ? j : 2 * j] * up, b = f[PERM4 ? j + 4 : 2 * j + 1] * up;
-        const __half2 hh = __floats2half2_rn(a, b);
+        float ha = a, hb = b;
+        if (HI8) {                                               // the leading 8 bits, rounded to nearest
+          const float ta = __fmul_rn(a, 65537.f), tb = __fmul_rn(b, 65537.f);
+          ha = __fsub_rn(ta, __fsub_rn(ta, a));
+          hb = __fsub_rn(tb, __fsub_rn(tb, b));
+        }
+        const __half2 hh = __floats2half2_rn(ha, hb);
         const float2 back = __half22float2(hh);
         const __half2 ll = __floats2half2_rn(a - back.x, b - back.y);
         h[j] = *reinterpret_cast<const uint32_t*>(&hh);
@@ -544,8 +554,9 @@ aiq_status_t launch_qlinear_tc_bits(const LayerJob& job, int N, int K, int M, vo
   float* y = static_cast<float*>(job.out);
   LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K,
                     (double)N * row_bytes(K, BITS) + 4.0 * N + 4.0 * M * ((double)K + N));
-  qlinear_split_x_kernel<BITS != 32, BITS == 4><<<M, 512, 0, s>>>(x, K, M, planes, down, y,
-                                                                   p.atomic ? (long long)M * N : 0ll, status);
+  const auto split_x = BITS == 8 && p.chunks_per_split * kQtChunk >= 1024 ? qlinear_split_x_kernel<BITS != 32, BITS == 4, BITS == 8>
+                                                                          : qlinear_split_x_kernel<BITS != 32, BITS == 4, false>;
+  split_x<<<M, 512, 0, s>>>(x, K, M, planes, down, y, p.atomic ? (long long)M * N : 0ll, status);
   AIQ_LAUNCH_CHECK("qlinear_split_x");
   const int smem = qt_smem_bytes(T::A_STAGES, p.Mt, p.stack, b_stages, w_stages) + 1024;
   AIQ_CUDA_TRY(launch_chained_cluster(true, p.cluster, qlinear_tc_kernel<BITS>, dim3(row_blocks * p.cluster, groups, m_blocks), dim3(T::THREADS), smem, s,

@@ -43,3 +43,23 @@ def test_tc_bound(bits, N, K, M):
     bound = ((K / 16 + 80) * 2.0 ** -22 + tol) * mags + 2.0 ** -22 * np.abs(want) + 1e-30
     bound += 2.0 ** -39 * np.abs(x).max(axis=1)[:, None].astype(np.float64) * np.abs(w).sum(axis=1)[None, :]
     assert np.all(np.abs(got - want) <= bound)
+
+
+@pytest.mark.parametrize("N,K,M,limit", [(8192, 8192, 16, 2.0e-6), (8192, 8192, 256, 6.3e-6), (8192, 4096, 256, 3.7e-6),
+                                         (4096, 4096, 64, 5.0e-7), (2048, 2048, 64, 2.5e-7)])
+def test_tc_rounding_error_at_8_bits(N, K, M, limit):
+    """The tensor cores drop what a product has below the accumulator's last bit.  Limits: below what bfloat16 pairs give
+    (2.6e-6, 6.4e-6, 3.8e-6, 2.5e-6, 2.5e-6 of the result's norm), and at short sums what the activations' 22 bits allow."""
+    import torch
+    aiq = binding()
+    g = torch.Generator(device="cuda").manual_seed(N + K + M)
+    W = torch.randn(N, K, generator=g, device="cuda") * 0.02
+    x = torch.randn(M, K, generator=g, device="cuda")
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, 8)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, 8, packed, scales)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    ws = torch.empty(aiq.aiq_qlinear_workspace_bytes(N, K, 8, M), dtype=torch.uint8, device="cuda")
+    aiq.aiq_qlinear(packed, scales, None, N, K, 8, x, y, workspace=ws)
+    want = x.double() @ (packed.view(torch.int8)[:, :K].double() * scales.double()[:, None]).T
+    assert ((y.double() - want).norm() / want.norm()).item() <= limit

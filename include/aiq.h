@@ -120,9 +120,10 @@ void aiq_set_scale_granularity(int granularity);
  *
  * Four kernels.  The plain one expands weights to float32 in registers and accumulates in
  * float32 (any shape, any bit-width; from five rows on as a tiled GEMM whose blocks, where they
- * are few, split K inside a cluster, in a fixed order).  It is also the one that runs for M >= 5
- * and N*K*M <= 2^26 (K > 4096 and M > 8: 2^24), where one launch beats the kernels with a pre-pass.  Three faster ones exist:
- *   M <= 4, 4 / 8 bits, K <= 8192, N*K >= 2^18, packed rows of 256 bytes or more: no workspace;
+ * are few, split K inside a cluster, in a fixed order).  It is also the one that runs for M >= 5 and N*K*M <= 2^26 (32 bits,
+ * K > 4096 and M > 8: 2^24; below 32 bits and M > 8: 2^25 from K = 1024 on, 2^22 above K = 4096), where one launch beats the
+ * kernels with a pre-pass.  Three faster ones exist:
+ *   M <= 4, 4 / 8 bits, K <= 8192, N*K >= 2^18 (M > 2 and K < 768: 2^19), packed rows of 256 bytes or more: no workspace;
  *     the codes stay integer and feed the int8 warp-level tensor cores, the activations of every
  *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest
  *     |x|), the int32 sums are exact and run-to-run identical; a batch row with an infinity or a

@@ -6,6 +6,8 @@
 // warp with shuffles.  The per-channel scale multiplies the finished sum.
 #include "tc_ptx.cuh"
 
+#include <type_traits>
+
 namespace aiq {
 
 namespace {
@@ -47,8 +49,9 @@ __device__ __forceinline__ void decode8(const uint4& q, int sub, float* f) {
 }
 
 // One warp: kRowsPerWarp output channels x MT batch rows.  Lanes stride over 16-byte chunks
-// of the packed rows.
-template <int BITS, int MT>
+// of the packed rows.  CHAIN: launched as a dependent of the kernel before (see launch_chained); x is then read by ordinary
+// loads, else through the read-only path.
+template <int BITS, int MT, bool CHAIN>
 __global__ void __launch_bounds__(kWarps * 32)
 qlinear_kernel(LayerJob job, int N, int K, int M) {
   constexpr int E = 128 / BITS;                 // elements per 16-byte chunk
@@ -57,8 +60,11 @@ qlinear_kernel(LayerJob job, int N, int K, int M) {
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int n0 = (blockIdx.x * kWarps + warp) * kRowsPerWarp;
-  chain_release();
-  chain_wait();
+  const int m0 = blockIdx.y * MT;
+  if (CHAIN) {
+    chain_release();
+    chain_wait();
+  }
   if (n0 >= N) return;
   const int Kpad = (K + 31) / 32 * 32;
   const size_t rb = (size_t)Kpad * BITS / 8;
@@ -86,17 +92,18 @@ qlinear_kernel(LayerJob job, int N, int K, int M) {
       float xv[MT][SE];
 #pragma unroll
       for (int m = 0; m < MT; ++m) {
-        const int mm = min(m, M - 1);
+        const int mm = min(m0 + m, M - 1);
         const float* xp = x + (size_t)mm * K + k0;
         if (xvec && k0 + SE <= K) {
 #pragma unroll
           for (int v = 0; v < SE / 4; ++v) {
-            const float4 t = ld_chain(reinterpret_cast<const float4*>(xp) + v);
+            const float4* src = reinterpret_cast<const float4*>(xp) + v;
+            const float4 t = CHAIN ? ld_chain(src) : __ldg(src);
             xv[m][4 * v] = t.x; xv[m][4 * v + 1] = t.y; xv[m][4 * v + 2] = t.z; xv[m][4 * v + 3] = t.w;
           }
         } else {
 #pragma unroll
-          for (int j = 0; j < SE; ++j) xv[m][j] = (k0 + j < K) ? ld_chain(xp + j) : 0.0f;
+          for (int j = 0; j < SE; ++j) xv[m][j] = (k0 + j < K) ? (CHAIN ? ld_chain(xp + j) : __ldg(xp + j)) : 0.0f;
         }
       }
 #pragma unroll
@@ -134,7 +141,7 @@ qlinear_kernel(LayerJob job, int N, int K, int M) {
       const float b = job.bias ? job.bias[n] : 0.0f;
 #pragma unroll
       for (int m = 0; m < MT; ++m)
-        if (m < M) static_cast<float*>(job.out)[(size_t)m * N + n] = fmaf(acc[r][m], s, b);
+        if (m0 + m < M) static_cast<float*>(job.out)[(size_t)(m0 + m) * N + n] = fmaf(acc[r][m], s, b);
     }
   }
 }
@@ -327,6 +334,26 @@ qlinear_gemm_kernel(LayerJob single, const LayerJob* __restrict__ jobs, int N, i
   }
 }
 
+// Clusters of `size` blocks that the device holds at a time: they form inside a GPC, so fewer than the SMs would hold one by
+// one.  (2228 x 6400, 16 bits, 5 rows: 35 clusters of four ran in two waves, 31.4 us.)  Asked once per kernel, device and size.
+template <typename K>
+aiq_status_t resident_clusters(K* kernel, int smem, int size, std::atomic<int> (&known)[64], int* out) {
+  int dev = 0;
+  AIQ_CUDA_TRY(cudaGetDevice(&dev));
+  const bool cached = dev >= 0 && dev < 64;
+  *out = cached ? known[dev].load(std::memory_order_acquire) : 0;
+  if (*out) return AIQ_OK;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(size); cfg.blockDim = dim3(kGemmThreads); cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = size; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  AIQ_CUDA_TRY(cudaOccupancyMaxActiveClusters(out, kernel, &cfg));
+  if (cached) known[dev].store(*out, std::memory_order_release);
+  return AIQ_OK;
+}
+
 template <int BITS, int BN, int BM>
 aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev, const LayerJob& single, int n_jobs, int N, int K, int M,
                               int n_sms, cudaStream_t s, int fixed_cluster) {
@@ -334,9 +361,19 @@ aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev
   const dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, n_jobs);
   const long long blocks = (long long)grid.x * grid.y * grid.z;
   const int n_slices = (K + kGemmBK - 1) / kGemmBK;
+  AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM, false>), (G::SMEM));
   // blocks per tile: doubled while all blocks stay resident and a group of threads has more than one slice
   int cluster = fixed_cluster ? fixed_cluster : 1;
-  while (!fixed_cluster && cluster < 8 && blocks * cluster * 2 <= G::RESIDENT * n_sms && n_slices > cluster * G::KG) cluster *= 2;
+  while (!fixed_cluster && cluster < 8 && blocks * cluster * 2 <= G::RESIDENT * n_sms && n_slices > cluster * G::KG) {
+    const int next = cluster * 2;
+    if (G::RESIDENT == 1) {                                      // with two blocks per SM a second wave has not been seen
+      static std::atomic<int> known[3][64];
+      int fit = 0;
+      if (aiq_status_t st = resident_clusters(qlinear_gemm_kernel<BITS, BN, BM, false>, G::SMEM, next, known[next >> 2], &fit)) return st;
+      if (blocks > fit) break;
+    }
+    cluster = next;
+  }
   auto launch = [&](auto kernel) {
     return launch_chained_cluster(scope.chain, cluster, kernel, dim3(grid.x * cluster, grid.y, grid.z), dim3(kGemmThreads), G::SMEM, s,
                                   single, jobs_dev, N, K, M, cluster);
@@ -345,10 +382,24 @@ aiq_status_t launch_gemm_tile(const LaunchScope& scope, const LayerJob* jobs_dev
     AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM, true>), (G::SMEM));
     AIQ_CUDA_TRY(launch(qlinear_gemm_kernel<BITS, BN, BM, true>));
   } else {
-    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_gemm_kernel<BITS, BN, BM, false>), (G::SMEM));
     AIQ_CUDA_TRY(launch(qlinear_gemm_kernel<BITS, BN, BM, false>));
   }
   return AIQ_OK;
+}
+
+// Five to eight rows on the kernel of four, twice, instead of the tile of 64 channels.  Measured, gemm | plain: short rows
+// (16 bits 512 x 512 5.3 | 3.7 us, 1280 x 320 5.1 | 3.9, 1000 x 1280 7.0 | 5.9, 32 bits 901 x 288 5.6 | 3.6, 8 bits 330 x 288 5.1 | 3.5; but 623 x
+// 212, 8 bits, 3.7 | 4.2, 2629 x 139 3.6 | 6.1); 16 bits, where a large layer gives every SM enough and its rows are aligned
+// (4096 x 4096 19.6 | 17.6, 5823 x 6184 52.3 | 45.9, 8192 x 8192 68.9 | 64.8; but 2048 x 8192 19.8 | 29.4); 32 bits, where the
+// tiles occupy half to two thirds of the SMs, one each (5823 x 6184 57.0 | 40.5, 6223 x 1492 16.8 | 13.0; 7522 x 4384 43.2 | 51.4).
+bool plain_rows8(int bits, int N, int K, int M, int n_sms) {
+  if (M > 8 || bits == 4) return false;
+  if (K >= 256 && K <= 512 && N <= 1536) return true;
+  if (bits == 16 && K <= 1280 && N >= 768 && N <= 1536) return true;
+  if (K % 4) return false;
+  if (bits == 16) return N > 16 * n_sms && (long long)N * K >= (1ll << 24);
+  const int tiles = (N + 63) / 64;
+  return bits == 32 && 2 * tiles > n_sms && 3 * tiles <= 2 * n_sms;
 }
 
 template <int BITS>
@@ -366,11 +417,7 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
     int cluster = 1;
     while (cluster < 8 && n_tiles * cluster * 2 <= 64 && n_slices > cluster * GemmTile<32, 16>::KG) cluster *= 2;
     if (aiq_status_t st = launch_gemm_tile<BITS, 32, 16>(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s, cluster)) return st;
-  } else if (M == 1) {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 1>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
-  } else if (M == 2) {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 2>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
-  } else if (M > 4) {
+  } else if (M > 4 && !plain_rows8(BITS, N, K, M, props.n_sms)) {
     // The largest tile that still gives every SM a block; smaller ones split K over more thread groups.  The tile of 8 rows
     // leaves out the work of rows that are not there (8191 x 8191, 5 rows, 4 bits: 72 us against 94 with the tile of 16).
     auto blocks = [&](int bn, int bm) { return (long long)((N + bn - 1) / bn) * ((M + bm - 1) / bm) * n_jobs; };
@@ -383,7 +430,21 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
     else st = args(launch_gemm_tile<BITS, 32, 16>);
     if (st != AIQ_OK) return st;
   } else {
-    AIQ_CUDA_TRY(launch_chained(scope.chain, qlinear_kernel<BITS, 4>, dim3(gx), dim3(kWarps * 32), 0, s, single, N, K, M));
+    // Chained, but for two kinds of launch.  The blocks of the next call settle on the SMs that this one leaves idle; where
+    // those are less than half, two on one, and a long stream of three or four rows then waits for them (16 bits, 4 rows: 4096
+    // x 4096 18.2 us chained, 16.4 not, 3063 x 4147 40.9 | 35.0; 4096 x 1024 6.8 | 8.2, 8192 x 4096 19.5 | 20.7).  And rows of x
+    // that are not 16-byte aligned are read by element, for which the read-only path is the faster one (32 bits, 2 rows: 8099 x
+    // 8023 79 | 62, 543 x 3814 27.7 | 26.0, but 723 x 1593 13.3 | 13.8; 16 bits, 1 / 2 rows: 47.6 / 65 | 41.5 / 49.4, but 543 x 3814 16.0 / 20.2 | 18.1 / 22.2).
+    const bool large = (long long)N * row_bytes(K, BITS) > (16ll << 20);
+    const bool by_element = (K & 3) != 0 || (((uintptr_t)single.in) & 15) != 0;
+    const bool chain = M > 4 || (M > 2 ? !(large && 2 * gx > props.n_sms && gx < props.n_sms) : !(by_element && (BITS == 32 ? M == 2 && K >= 3500 : large)));
+    const dim3 grid(gx, M > 4 ? 2 : 1);
+    auto launch = [&](auto kernel) { return launch_chained(chain && scope.chain, kernel, grid, dim3(kWarps * 32), 0, s, single, N, K, M); };
+    auto pick = [&](auto chained) {
+      constexpr bool CH = decltype(chained)::value;
+      return M == 1 ? launch(qlinear_kernel<BITS, 1, CH>) : M == 2 ? launch(qlinear_kernel<BITS, 2, CH>) : launch(qlinear_kernel<BITS, 4, CH>);
+    };
+    AIQ_CUDA_TRY(chain && scope.chain ? pick(std::true_type()) : pick(std::false_type()));
   }
   AIQ_LAUNCH_CHECK("qlinear");
   return AIQ_OK;
@@ -415,13 +476,18 @@ aiq_status_t launch_qlinear(const LayerJob* jobs_dev, const LayerJob* single_hos
 
 // Up to 2^26 products the one launch of the float32 kernel (from five rows on) beats the pre-pass and the atomics of the
 // kernels below; see the figures at qlinear_gemm_kernel.  Long rows leave it few tiles with many slices each (128 x 8192,
-// 40 rows: 14.2 us against 7.6 on the tensor cores; 64 x 8192, 12 rows: 9.5, one launch): from K = 4096 up to 2^24.
-static bool small_gemm(int N, int K, int M) {
-  return M > 4 && (long long)N * K * M <= (K > 4096 && M > 8 ? 1ll << 24 : 1ll << 26);
+// 40 rows: 14.2 us against 7.6 on the tensor cores): from K = 4096 up to 2^24.  Below 32 bits the tensor cores take a part
+// of that range too, with halves that lose next to nothing (error 1e-7 to 3.5e-7 of the result's norm): K > 4096 from 2^22 on
+// (64 x 8192, 12 rows, 8 bits: 10.1 | 8.3), K >= 1024 from 2^25 on (1000 x 1280, 40 rows, 8 bits: 12.5 | 8.3; 1360 x 3000, 9
+// rows 12.6 | 11.1; 2048 x 2048, 9 rows 9.6 | 8.3).
+static bool small_gemm(int N, int K, int bits, int M) {
+  const long long products = (long long)N * K * M;
+  if (M <= 4 || products > (K > 4096 && M > 8 ? 1ll << 24 : 1ll << 26)) return false;
+  return bits == 32 || M <= 8 || !(products > (K > 4096 ? 1ll << 22 : K >= 1024 ? 1ll << 25 : 1ll << 26));
 }
 
 extern "C" size_t aiq_qlinear_workspace_bytes(int N, int K, int bits, int M) {
-  if (N <= 0 || K <= 0 || M <= 0 || small_gemm(N, K, M)) return 0;
+  if (N <= 0 || K <= 0 || M <= 0 || small_gemm(N, K, bits, M)) return 0;
   if (aiq::qlinear_tc_applicable(N, K, bits, M)) return aiq::qlinear_tc_workspace_bytes(K, M) + 16;   // + status word
   if (aiq::qlinear_mma_applicable(N, K, bits, M)) return aiq::qlinear_mma_workspace_bytes(K, M);
   return 0;
@@ -446,7 +512,7 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
   job.bias = bias;
   job.bits = bits;
   if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
-  if (small_gemm(N, K, M)) return aiq::launch_qlinear(nullptr, &job, 1, N, K, M, (cudaStream_t)stream);
+  if (small_gemm(N, K, bits, M)) return aiq::launch_qlinear(nullptr, &job, 1, N, K, M, (cudaStream_t)stream);
   // the tensor-core kernels need scratch for the converted activations
   if (workspace && aiq::qlinear_tc_applicable(N, K, bits, M)) {
     if (((uintptr_t)workspace) & 15)

@@ -362,9 +362,11 @@ qlinear_gemv_kernel(const uint8_t* __restrict__ w, const float* __restrict__ sca
 
 // Up to four rows and rows of at most 8,192 elements (16 warps x 512); at least 256 bytes a row and 2^18 elements:
 // below, both this and the plain kernel take less time than a call's host side (512 x 512: 5.8 us a call with either), while
-// at 1000 x 1280 the plain kernel needs 10 us and this one 5.9.
+// at 1000 x 1280 the plain kernel needs 10 us and this one 5.9.  Three and four short rows of a small layer are the plain
+// kernel's (1280 x 320, 8 bits, 3 rows 5.4 us here, 3.7 there; 512 x 512 5.5 | 3.8; but 1000 x 1280 5.3 | 8.0).
 bool qlinear_gemv_applicable(int N, int K, int bits, int M) {
   if ((bits != 4 && bits != 8) || M < 1 || M > kGvMaxRows || K > 8192) return false;
+  if (M > 2 && K < 768 && (long long)N * K < (1 << 19)) return false;
   return row_bytes(K, bits) >= 256 && (long long)N * K >= (1 << 18);
 }
 

@@ -61,7 +61,7 @@ struct QtKind {
 struct QtParams {
   int N, K, M;
   int Mt;                   // batch rows per CTA tile (multiple of 16, <= 256)
-  int m_block;              // batch rows per blockIdx.z: 256, or 128 with two weight pieces (shared memory)
+  int m_block;              // batch rows per blockIdx.z: 256 or 128
   int n_chunks;             // ceil(K / 64)
   int chunks_per_split;
   int cluster;              // K splits that are one cluster (blockIdx.x = 128-channel block * cluster + rank)
@@ -438,6 +438,28 @@ qlinear_tc_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_consta
   const int rows = min(Mt, p.M - m0), n = n0 + lane * 4;
   const float4 s = *reinterpret_cast<const float4*>(s_scale + lane * 4), b = *reinterpret_cast<const float4*>(s_scale + 128 + lane * 4);
   const bool vec = (p.N & 3) == 0 && (((uintptr_t)y) & 15) == 0;
+  if (!vec) {
+    // rows of y that are not 16-byte aligned: neighbouring lanes take neighbouring channels (four channels a lane here too
+    // quadrupled the transactions: 5671 x 608, 8 bits, 256 rows 20.6 us in the first version of this epilogue, 24.7 then, 20.6 now)
+    for (int r = rank + warp * p.cluster; r < rows; r += (T::THREADS / 32) * p.cluster)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int ch = lane + 32 * j;
+        const uint32_t mine = smem_u32(smem) + (uint32_t)(r * 128 + ch) * 4;
+        float v = 0.f;
+        for (int q = 0; q < p.cluster; ++q) {
+          uint32_t theirs;
+          float part;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(q));
+          asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(part) : "r"(theirs) : "memory");
+          v += part;
+        }
+        if (n0 + ch >= p.N) continue;
+        v = fmaf(v * s_down[r], s_scale[ch], s_scale[128 + ch]);
+        float* dst = y + (size_t)(m0 + r) * p.N + n0 + ch;
+        if (p.atomic) atomicAdd(dst, v); else *dst = v;
+      }
+  } else
   for (int r = rank + warp * p.cluster; r < rows; r += (T::THREADS / 32) * p.cluster) {
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t mine = smem_u32(smem) + (uint32_t)(r * 128 + lane * 4) * 4;
@@ -452,16 +474,9 @@ qlinear_tc_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_consta
     const float d = s_down[r];
     v.x = fmaf(v.x * d, s.x, b.x); v.y = fmaf(v.y * d, s.y, b.y); v.z = fmaf(v.z * d, s.z, b.z); v.w = fmaf(v.w * d, s.w, b.w);
     float* dst = y + (size_t)(m0 + r) * p.N + n;
-    if (vec) {
-      if (n < p.N) {
-        if (p.atomic) asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
-        else *reinterpret_cast<float4*>(dst) = v;
-      }
-    } else {
-      const float f[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (n + j < p.N) { if (p.atomic) atomicAdd(dst + j, f[j]); else dst[j] = f[j]; }
+    if (n < p.N) {
+      if (p.atomic) asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+      else *reinterpret_cast<float4*>(dst) = v;
     }
   }
   if (p.cluster > 1) {                                       // no CTA leaves while another reads its sums
@@ -483,7 +498,10 @@ aiq_status_t launch_qlinear_tc_bits(const LayerJob& job, int N, int K, int M, vo
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   QtParams p = {};
   p.N = N; p.K = K; p.M = M; p.error_flag = status;
-  p.m_block = T::PIECES == 2 ? 128 : 256;          // two A tiles per stage leave room for activation tiles of 128 rows
+  // Two A tiles per stage leave room for activation tiles of 128 rows.  At 16 bits a small layer takes those too: a tile of 256
+  // rows spends its time in set-up and epilogue (256 rows, 1000 x 1280 18.6 us with tiles of 256, 13.0 of 128; 8192 x 512 20.5 |
+  // 14.5; but 8192 x 8192, 192 rows, 56.5 | 64.6, and 4096 x 4096, 129 rows, 22.7 | 24.6).
+  p.m_block = T::PIECES == 2 || (T::DIRECT && M > 128 && (long long)N * K <= (1ll << 23)) ? 128 : 256;
   p.Mt = M >= p.m_block ? p.m_block : (M + 15) / 16 * 16;
   const int m_blocks = (M + p.m_block - 1) / p.m_block, row_blocks = (N + 127) / 128;
   p.n_chunks = (K + kQtChunk - 1) / kQtChunk;

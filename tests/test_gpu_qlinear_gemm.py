@@ -62,3 +62,30 @@ def test_gemm_rounding_error(bits, N, K, M):
     want = x.double() @ w.T
     error = ((y.double() - want).norm() / want.norm()).item()
     assert error <= 2.0 ** -24 * (1.5 + K ** 0.5 / 20)
+
+
+# the kernel of four rows: one launch chained and unchained, rows of x aligned and not, five to eight rows as two of four
+@pytest.mark.parametrize("bits", [4, 8, 16, 32])
+@pytest.mark.parametrize("N,K,M", [(512, 512, 3), (513, 511, 4), (3000, 2900, 4), (2600, 3301, 3), (1100, 8023, 1), (1200, 8023, 2),
+                                   (601, 1001, 2), (330, 288, 5), (1535, 509, 8), (1000, 1280, 7), (4801, 3600, 6), (6200, 516, 5)])
+def test_rows_of_four_bound(bits, N, K, M):
+    import torch
+    aiq = binding()
+    rng = np.random.default_rng(N + K + M)
+    W = rng.standard_normal((N, K)).astype(np.float32)
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    bias = rng.standard_normal(N).astype(np.float32) if N % 2 else None
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(to_dev(W), bits, packed, scales)
+    ys = []
+    for _ in range(2):
+        y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+        aiq.aiq_qlinear(packed, scales, to_dev(bias) if bias is not None else None, N, K, bits, to_dev(x), y)
+        ys.append(y.cpu().numpy())
+    assert np.array_equal(ys[0], ys[1])
+    v, s = O.quantize_rows(W, bits)
+    w = v.astype(np.float64) * np.asarray(s, np.float64)[:, None]
+    want = x.astype(np.float64) @ w.T + (0 if bias is None else bias.astype(np.float64))
+    bound = (K + 2) * 2.0 ** -24 * (np.abs(x).astype(np.float64) @ np.abs(w).T) + 2.0 ** -22 * np.abs(want) + 1e-30
+    assert np.all(np.abs(ys[0] - want) <= bound)

@@ -140,9 +140,10 @@ void aiq_set_scale_granularity(int granularity);
  *     activations enter as sums of two bfloat16 (2^-17).  Accumulation is float32.
  * The last two split K over thread blocks where the matrix has too few rows to fill the GPU; the
  * partial sums then meet in y through float atomics (run-to-run differences in the last
- * bit).  They need scratch memory: pass `workspace` (device, 16-byte aligned) of at least
- * aiq_qlinear_workspace_bytes(...) bytes; with workspace == NULL, or where that function
- * returns 0, the plain kernel runs.
+ * bit).  They need scratch memory: pass `workspace` (device, 16-byte aligned; refused if it is not)
+ * of at least aiq_qlinear_workspace_bytes(...) bytes; without it the plain kernel runs in their
+ * place.  (The kernel of up to four rows needs none, and runs with or without; the function keeps
+ * its former answer there.)
  * Device-side failure: the tcgen05 kernel bounds every wait on its copy / MMA pipeline (about
  * 2 s of SM clocks).  Should one expire, the kernel stops early and y is invalid; the call has
  * long returned AIQ_OK by then, so the record is on the device: the int32 at byte offset

@@ -486,11 +486,24 @@ static bool small_gemm(int N, int K, int bits, int M) {
   return bits == 32 || M <= 8 || !(products > (K > 4096 ? 1ll << 22 : K >= 1024 ? 1ll << 25 : 1ll << 26));
 }
 
+// The kernel of a call, and of the size query: SCRATCH_* ones need the workspace, and without it PLAIN runs in their place.
+enum QlinearPath { QL_PLAIN, QL_GEMV, QL_SCRATCH_MMA, QL_SCRATCH_TC };
+static QlinearPath qlinear_path(int N, int K, int bits, int M) {
+  if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return QL_GEMV;
+  if (small_gemm(N, K, bits, M)) return QL_PLAIN;
+  if (aiq::qlinear_tc_applicable(N, K, bits, M)) return QL_SCRATCH_TC;
+  return aiq::qlinear_mma_applicable(N, K, bits, M) ? QL_SCRATCH_MMA : QL_PLAIN;
+}
+
 extern "C" size_t aiq_qlinear_workspace_bytes(int N, int K, int bits, int M) {
-  if (N <= 0 || K <= 0 || M <= 0 || small_gemm(N, K, bits, M)) return 0;
-  if (aiq::qlinear_tc_applicable(N, K, bits, M)) return aiq::qlinear_tc_workspace_bytes(K, M) + 16;   // + status word
-  if (aiq::qlinear_mma_applicable(N, K, bits, M)) return aiq::qlinear_mma_workspace_bytes(K, M);
-  return 0;
+  if (N <= 0 || K <= 0 || M <= 0) return 0;
+  switch (qlinear_path(N, K, bits, M)) {
+    case QL_SCRATCH_TC: return aiq::qlinear_tc_workspace_bytes(K, M) + 16;   // + status word
+    case QL_SCRATCH_MMA: return aiq::qlinear_mma_workspace_bytes(K, M);
+    // the kernel of up to four rows touches none; callers that size one buffer by the smallest call keep their answer
+    case QL_GEMV: return aiq::qlinear_mma_applicable(N, K, bits, M) ? aiq::qlinear_mma_workspace_bytes(K, M) : 0;
+    default: return 0;
+  }
 }
 
 extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, const float* bias, int N,
@@ -511,23 +524,21 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
   job.scale = scales;
   job.bias = bias;
   job.bits = bits;
-  if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
-  if (small_gemm(N, K, bits, M)) return aiq::launch_qlinear(nullptr, &job, 1, N, K, M, (cudaStream_t)stream);
+  // a misaligned workspace is refused wherever a kernel with scratch exists for the shape, whichever kernel then runs
+  if (workspace && (((uintptr_t)workspace) & 15) && (aiq::qlinear_tc_applicable(N, K, bits, M) || aiq::qlinear_mma_applicable(N, K, bits, M)))
+    return aiq::set_error(AIQ_ERR_INVALID_ARG, "aiq_qlinear: workspace not 16-byte aligned");
+  const QlinearPath path = qlinear_path(N, K, bits, M);
+  if (path == QL_GEMV) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
   // the tensor-core kernels need scratch for the converted activations
-  if (workspace && aiq::qlinear_tc_applicable(N, K, bits, M)) {
-    if (((uintptr_t)workspace) & 15)
-      return aiq::set_error(AIQ_ERR_INVALID_ARG, "aiq_qlinear: workspace not 16-byte aligned");
+  if (path == QL_SCRATCH_TC && workspace) {
     const size_t scratch = aiq::qlinear_tc_workspace_bytes(K, M);
     if (workspace_bytes >= scratch + 16) {
       // device status word behind the scratch: 0 (set by the pre-pass), or 1 once a bounded wait of the kernel expired
       int32_t* status = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + scratch);
       return aiq::launch_qlinear_tc(job, N, K, M, workspace, status, (cudaStream_t)stream);
     }
-  } else if (workspace && aiq::qlinear_mma_applicable(N, K, bits, M)) {
-    if (((uintptr_t)workspace) & 15)
-      return aiq::set_error(AIQ_ERR_INVALID_ARG, "aiq_qlinear: workspace not 16-byte aligned");
-    if (workspace_bytes >= aiq::qlinear_mma_workspace_bytes(K, M))
-      return aiq::launch_qlinear_mma(job, N, K, M, workspace, (cudaStream_t)stream);
   }
+  if (path == QL_SCRATCH_MMA && workspace && workspace_bytes >= aiq::qlinear_mma_workspace_bytes(K, M))
+    return aiq::launch_qlinear_mma(job, N, K, M, workspace, (cudaStream_t)stream);
   return aiq::launch_qlinear(nullptr, &job, 1, N, K, M, (cudaStream_t)stream);
 }

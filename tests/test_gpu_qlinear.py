@@ -82,3 +82,23 @@ def test_qlinear_two_piece_path_exact_on_integers(bits):
         for trial in range(3):
             got, ref = _run(aiq, W, x, bits)
             assert np.array_equal(got.astype(np.int64), want), (N, K, M, bits, trial)
+
+
+@pytest.mark.parametrize("N,K,M", [(512, 512, 16), (4096, 4096, 1), (2048, 1024, 6), (4096, 4096, 64), (8192, 64, 9)])
+def test_qlinear_refuses_a_misaligned_workspace(N, K, M):
+    """Wherever a kernel with scratch exists for the shape, also where another one runs; elsewhere the workspace is ignored."""
+    import torch
+    aiq = binding()
+    W, x = gen_linear_case(N, K, M, seed=5)
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, 4)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(to_dev(W), 4, packed, scales)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    ws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+    with pytest.raises(aiq.AiqError) as e:
+        aiq.aiq_qlinear(packed, scales, None, N, K, 4, to_dev(x), y, workspace=ws[4:])
+    assert e.value.status == aiq.ERR_INVALID_ARG
+    aiq.aiq_qlinear(packed, scales, None, N, K, 4, to_dev(x), y, workspace=ws)
+    small = torch.empty((30, aiq.aiq_packed_row_bytes(100, 4)), dtype=torch.uint8, device="cuda")
+    aiq.aiq_quantize_layer(torch.randn((30, 100), device="cuda"), 4, small, scales[:30])
+    aiq.aiq_qlinear(small, scales[:30], None, 30, 100, 4, torch.zeros((M, 100), device="cuda"), y.view(-1)[:30 * M].view(M, 30), workspace=ws[4:])

@@ -457,7 +457,7 @@ EncodeTiledFn pr_encode_fn() {
 struct PrConfig { bool stream; int Nt, ew, stages, bufs, splits, tiles_per_cta, smem; };
 // streamed: 0 / 1 restricts the search to that variant, -1 does not.
 bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& props, int streamed, PrConfig* out) {
-  const int n_tiles = (g.B * (g.H + 2) * g.W + 127) / 128;
+  const long long n_tiles = ((long long)g.B * (g.H + 2) * g.W + 127) / 128;   // of the nominal batch: may pass 2^31 pixels
   const double K2 = 2.0 * g.Cs_in;
   double best = 1e300;
   for (int nt = 32; nt <= 256; nt += 32) {
@@ -486,20 +486,20 @@ bool pr_search(const ConvGeom& g, int n_jobs, int pieces, const DeviceProps& pro
       const double setup = 3000.0 + (stream ? 0.0 : Nt * (double)g.Cs_in * pieces / 16.0);
       const int pairs = n_jobs * ntiles;
       for (int wave = 1; wave <= 5; ++wave) {
-        int splits = wave == 5 ? n_tiles : wave * occ * props.n_sms / pairs;
+        long long splits = wave == 5 ? n_tiles : wave * occ * props.n_sms / pairs;
         if (splits < 1) splits = 1;
         if (splits > n_tiles) splits = n_tiles;
-        const int tpc = (n_tiles + splits - 1) / splits;
+        const long long tpc = (n_tiles + splits - 1) / splits;
         splits = (n_tiles + tpc - 1) / tpc;
-        const long long ctas = (long long)splits * pairs;
+        const long long ctas = splits * pairs;
         const long long full = ctas / (occ * props.n_sms), rem = ctas - full * occ * props.n_sms;
         const double one = occ * tpc * tile + setup;
         const double cost = full * one + (rem > props.n_sms ? one : rem > 0 ? tpc * tile + setup : 0.0);
         if (cost < best * 0.999) {
           best = cost;
-          *out = {stream, Nt, ew, st, bf, splits, tpc, need(st, bf)};
+          *out = {stream, Nt, ew, st, bf, (int)splits, (int)tpc, need(st, bf)};
         }
-        if (ctas >= (long long)n_tiles * pairs) break;
+        if (ctas >= n_tiles * pairs) break;
       }
     }
     if (Nt == g.Cs_out) break;

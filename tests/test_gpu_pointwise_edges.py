@@ -44,3 +44,34 @@ def test_pointwise_shortcut(c, hw):
         got = model.aiq_forward(scheme, to_dev(x)).cpu().numpy()
         assert_logits_close(got, O.forward_scheme(arch, bank, scheme, x), f"shortcut {c} {hw} {scheme}")
     model.close()
+
+
+def test_pointwise_on_a_map_of_two_to_the_24_pixels():
+    """The launch shape is searched at a nominal batch of 256 images, which here is 2^32 pixels (the search ended in a division
+    by zero).  One channel of the input is a ramp down the map, so a wrong tile shows in the averages."""
+    import torch
+    import torch.nn.functional as F
+    aiq = binding()
+    H, W = 4094, 4096
+    arch = pointwise_stack(24, 40, hw=8, n_classes=5)
+    arch = dict(arch, in_h=H, in_w=W)
+    params = gen_model(arch, 77)
+    model = aiq.Model(arch, params)
+    x = torch.zeros((1, 3, H, W), device="cuda")
+    x[0, 0] = torch.linspace(-1, 1, H, device="cuda")[:, None]
+    x[0, 1] = torch.linspace(1, -1, W, device="cuda")[None, :]
+    got = model.aiq_forward(np.full(3, 8, np.uint8), x).double().cpu().numpy()
+    v = x.double()
+    for i, l in enumerate(arch["layers"]):
+        packed, scales = model.layer_packed(i, 8)
+        k = l["cin"] * l["k"] ** 2
+        w = packed.view(torch.int8)[:, :k].double() * scales.double()[:, None]
+        b = model.layer_folded(i)[1].double()
+        if l["kind"] == "fc":
+            v = v.mean((2, 3)) @ w.T + b
+        else:
+            v = F.conv2d(v, w.view(l["cout"], l["cin"], l["k"], l["k"]), b, l["stride"], l["pad"])
+            v = v.clamp(min=0) if l["act"] == "relu" else v.clamp(0, 6) if l["act"] == "relu6" else v
+    want = v.cpu().numpy()
+    assert np.all(np.abs(got - want) <= 1e-3 * (1 + np.abs(want)))
+    model.close()

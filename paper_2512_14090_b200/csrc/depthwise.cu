@@ -392,6 +392,7 @@ struct DwSplit { int k, n_rb, rows; };
 }  // namespace
 
 aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions, void* map_out) {
+  if (g.stride != 1 && g.stride != 2) return set_error(AIQ_ERR_SHAPE, "depthwise: stride %d is not supported", g.stride);
   EncodeTiledFn enc = dw_encode_fn();
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const DwShape s = dw_shape(g, batch_capacity);
@@ -411,7 +412,6 @@ aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int 
 
 aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob* jobs_dev, int n_jobs, int batch_capacity,
                               bool has_res, int32_t* error_flag, double weight_bytes, cudaStream_t s) {
-  if (g.stride != 1 && g.stride != 2) return set_error(AIQ_ERR_SHAPE, "depthwise: stride %d is not supported", g.stride);
   DeviceProps props;
   if (aiq_status_t st = current_device_props(&props)) return st;
   const DwShape sh = dw_shape(g, batch_capacity);

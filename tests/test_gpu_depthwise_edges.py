@@ -27,3 +27,19 @@ def test_depthwise_tile_edges(hw, channels, batch, path):
         got = model.aiq_forward(np.array(sc, np.uint8), to_dev(x)).cpu().numpy()
         assert_logits_close(got, ref, f"depthwise stack {hw} {channels} {batch} {path} {sc}")
     model.close()
+
+
+@pytest.mark.parametrize("stride,hw", [(3, 30), (4, 448)])
+def test_depthwise_refuses_other_strides_as_a_shape(stride, hw):
+    """Also on maps so wide that the input box of such a stride would be no legal tensor map."""
+    import torch
+    aiq = binding()
+    arch = depthwise_stack(hw, 32)
+    for l in arch["layers"]:
+        if l["kind"] == "dw" and l["stride"] == 2:
+            l["stride"] = stride
+    model = aiq.Model(arch, gen_model(arch, 3))
+    with pytest.raises(aiq.AiqError) as e:
+        model.aiq_forward(np.full(len(arch["layers"]), 8, np.uint8), torch.zeros((1, 3, hw, hw), device="cuda"))
+    assert e.value.status == aiq.ERR_SHAPE
+    model.close()

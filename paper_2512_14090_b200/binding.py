@@ -336,8 +336,8 @@ class Model:
     def layer_packed(self, layer, bits):
         p, s = C.c_void_p(), C.c_void_p()
         _check(lib.aiq_model_layer_packed(self.handle, layer, int(bits), C.byref(p), C.byref(s)))
-        l = self.arch["layers"][layer]
-        n, k = l["cout"], (1 if l["kind"] == "dw" else l["cin"]) * l["k"] * l["k"]
+        l = self._keep_layers[layer]                    # as the library was given it: the caller's dict may have changed
+        n, k = l.cout, l.cin if l.kind == LAYER_KIND["fc"] else (1 if l.kind == LAYER_KIND["dw"] else l.cin) * l.ksize * l.ksize
         rb = aiq_packed_row_bytes(k, bits)
         return (self._view(p.value, n * rb).view(n, rb), self._view(s.value, n * 4).view(dtype=_f32()))
 

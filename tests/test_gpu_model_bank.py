@@ -5,7 +5,7 @@ takes the per-layer kernels beside it."""
 import numpy as np
 import pytest
 
-from aiq_workloads import gen_model
+from aiq_workloads import gen_model, tiny_net
 from aiq_workloads.archs import _conv, _fc
 from oracle import aiq_oracle as O
 from gpu_util import binding
@@ -45,4 +45,23 @@ def test_bank_bits(widths, kinds, bias):
             v, s = O.quantize_rows(wf, bits)
             assert np.array_equal(packed.cpu().numpy(), O.pack_rows(v, bits)), (i, bits)
             assert np.array_equal(scales.cpu().numpy().view(np.uint32), np.asarray(s, np.float32).view(np.uint32)), (i, bits)
+    model.close()
+
+
+def test_packed_views_follow_the_model_not_the_callers_dict():
+    """The shapes of the packed views are the library's: a classifier's K is its input channels whatever kernel size the
+    description gives, and a description that is changed after the model was made changes nothing."""
+    aiq = binding()
+    arch = tiny_net()
+    arch["layers"][-1]["k"] = 3                         # not read for a classifier
+    params = gen_model(tiny_net(), 5)
+    model = aiq.Model(arch, params)
+    shapes = [tuple(model.layer_packed(i, 8)[0].shape) for i in range(len(arch["layers"]))]
+    fc = arch["layers"][-1]
+    assert shapes[-1] == (fc["cout"], aiq.aiq_packed_row_bytes(fc["cin"], 8))
+    for i in range(len(arch["layers"])):
+        n, k = (t.shape for t in (model.layer_folded(i)[1], model.layer_folded(i)[0]))
+        assert shapes[i] == (n[0], aiq.aiq_packed_row_bytes(k[1], 8))
+    arch["layers"][1]["cout"] += 1
+    assert [tuple(model.layer_packed(i, 8)[0].shape) for i in range(len(arch["layers"]))] == shapes
     model.close()

@@ -183,7 +183,8 @@ def _stream(stream=None):
     if _raw_stream is None:
         import torch
         torch.cuda.current_stream()                     # initialises CUDA
-        _raw_stream = (torch.cuda.current_device, torch._C._cuda_getCurrentRawStream)
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # not a public name: the public call where it is gone
+        _raw_stream = (torch.cuda.current_device, raw or (lambda device: torch.cuda.current_stream(device).cuda_stream))
     device, raw = _raw_stream
     return raw(device())
 

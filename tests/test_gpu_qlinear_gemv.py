@@ -2,8 +2,8 @@
 elements, fewer and more channels than a unit per SM, one warp to sixteen warps per unit, the longest row, one to four
 batch rows, activations over a wide range of magnitudes.  Bound: the integer sums are exact; the digits hold x to 2^-27 of
 the largest |x| of its slice, digit sums and the at most 16 partial sums round to 2^-24 each, so
-|delta| <= 2^-20 s_n sum_k |code| max|x| is ample.  Integer inputs come out exactly.  The kernel needs no workspace and
-gives the same bits twice."""
+|delta| <= 2^-20 s_n sum_k |code| max|x| is ample (random errors average out far below it; that all four digits take part
+is a test of its own).  Integer inputs come out exactly.  The kernel needs no workspace and gives the same bits twice."""
 import numpy as np
 import pytest
 
@@ -98,3 +98,51 @@ def test_gemv_infinite_activations(bits, N, K, M):
             assert np.array_equal(np.isinf(got), inf) and np.array_equal(np.sign(got[inf]), np.sign(want[inf]))
             fine = np.isfinite(want)
             assert np.all(np.abs(got[fine] - want[fine]) <= np.broadcast_to(bound, want.shape)[fine])
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("N,K,M", [(1024, 1536, 1), (600, 4100, 2), (1200, 8192, 3), (3000, 777, 4)])
+def test_gemv_fourth_digit(bits, N, K, M):
+    """Activations of j 2^-26, |j| < 64, beside ones of 1 that meet zero weights: with the largest |x| of every slice at 1 the
+    fourth digit counts 2^-26, so it alone holds them, and every sum is exact."""
+    import torch
+    aiq = binding()
+    qmax = 2 ** (bits - 1) - 1
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    W = torch.randint(-qmax, qmax + 1, (N, K), generator=g, device="cuda").float()
+    W[:, 1] = qmax
+    W[:, ::64] = 0
+    j = torch.randint(-63, 64, (M, K), generator=g, device="cuda")
+    x = j.float() * 2.0 ** -26
+    x[:, ::64] = 1.0
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, bits, packed, scales)
+    assert bool((scales == 1).all())
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    aiq.aiq_qlinear(packed, scales, None, N, K, bits, x, y)
+    j[:, ::64] = 0
+    want = j.double() @ W.double().T
+    assert bool((want != 0).any()) and torch.equal(y.double() * 2.0 ** 26, want)
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("N,K,M", [(12000, 8192, 1), (12000, 8192, 3), (20003, 4100, 4), (20003, 4100, 2), (30001, 1030, 1)])
+def test_gemv_many_units_per_block(bits, N, K, M):
+    """More units than a block forms outputs of at a time (eight) and than its ring has slots: partial sums, slots and parities
+    are used again.  Integers: every sum is exact."""
+    import torch
+    aiq = binding()
+    qmax = 2 ** (bits - 1) - 1
+    g = torch.Generator(device="cuda").manual_seed(N + K + M)
+    W = torch.randint(-qmax, qmax + 1, (N, K), generator=g, device="cuda").float()
+    W[:, 0] = qmax
+    x = torch.randint(-8, 9, (M, K), generator=g, device="cuda").float()
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, bits, packed, scales)
+    want = x.double() @ W.double().T
+    for _ in range(2):
+        y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+        aiq.aiq_qlinear(packed, scales, None, N, K, bits, x, y)
+        assert torch.equal(y.double(), want)

@@ -257,8 +257,8 @@ aiq_status_t launch_qlinear_mma(const LayerJob& job, int N, int K, int M, void* 
 // one-kernel path of the linear layer (qlinear_gemv.cu): 4- / 8-bit weights, up to four rows, no workspace
 bool qlinear_gemv_applicable(int N, int K, int bits, int M);
 aiq_status_t launch_qlinear_gemv(const LayerJob& job, int N, int K, int M, cudaStream_t s);
-// tcgen05 path of the linear layer (4- / 8-bit weights, M >= 9): weights as the MMA's M operand,
-// the batch as its N operand; needs workspace for the activations as two bfloat16 planes
+// tcgen05 path of the linear layer (all widths, M >= 9): weights as the MMA's M operand, the batch as its N operand;
+// needs workspace for the activations as two 16-bit planes (halves, at 32 bits bfloat16) and a factor per batch row
 bool qlinear_tc_applicable(int N, int K, int bits, int M);
 size_t qlinear_tc_workspace_bytes(int K, int M);
 aiq_status_t launch_qlinear_tc(const LayerJob& job, int N, int K, int M, void* workspace, int32_t* error_flag,

@@ -434,21 +434,6 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn pr_encode_fn() {
-  static std::atomic<EncodeTiledFn> fn{nullptr};
-  if (EncodeTiledFn f = fn.load(std::memory_order_acquire)) return f;
-  void* sym = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return nullptr;
-  fn.store(reinterpret_cast<EncodeTiledFn>(sym), std::memory_order_release);
-  return reinterpret_cast<EncodeTiledFn>(sym);
-}
-
 // Launch shape: variant, channel tile, blocks per SM, ring depth, pixel splits.  Every channel tile but the last is a
 // multiple of the 32 channels of a store unit.  Costs are in SM clocks: a tile of 128 pixels takes the longest of its
 // MMAs ((128 + Nt) / 4 clocks per 16-channel step), its input (40 bytes per clock and SM, less where the ring holds fewer
@@ -537,7 +522,7 @@ bool conv_pw_eligible(const ConvGeom& g) {
 
 aiq_status_t conv_pw_encode_maps(const ConvGeom& g, const void* in_slot, int in_versions, const void* out_slot, int out_versions,
                                  int batch_capacity, void* maps_out /* 2 x 128 bytes */) {
-  EncodeTiledFn enc = pr_encode_fn();
+  EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   CUtensorMap* maps = static_cast<CUtensorMap*>(maps_out);
   const cuuint64_t pixels = (cuuint64_t)batch_capacity * (g.H + 2) * g.W;

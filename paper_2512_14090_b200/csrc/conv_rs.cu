@@ -890,22 +890,6 @@ conv_rs_block_kernel(const __grid_constant__ CUtensorMap in_map, RbParams p, con
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn rs_encode_fn() {
-  static std::atomic<EncodeTiledFn> fn{nullptr};
-  if (EncodeTiledFn f = fn.load(std::memory_order_acquire)) return f;
-  void* sym = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return nullptr;
-  fn.store(reinterpret_cast<EncodeTiledFn>(sym), std::memory_order_release);
-  return reinterpret_cast<EncodeTiledFn>(sym);
-}
-
 // geometry shared by the map encoder and the launcher
 struct RsShape {
   int Gin, Gout, gmode, planes, xt, stage_bytes, a_lbo, a_tap_off[3];
@@ -1107,7 +1091,7 @@ bool conv_rs_pool_fusable(const ConvGeom& g) {
 
 aiq_status_t conv_rs_encode_maps(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions,
                                  void* maps_out /* 2 x 128 bytes */) {
-  EncodeTiledFn enc = rs_encode_fn();
+  EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   RsShape s;
   if (!rs_shape(g, &s)) return set_error(AIQ_ERR_SHAPE, "conv_rs: layer shape is not supported");

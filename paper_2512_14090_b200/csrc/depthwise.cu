@@ -335,21 +335,6 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn dw_encode_fn() {
-  static std::atomic<EncodeTiledFn> fn{nullptr};
-  if (EncodeTiledFn f = fn.load(std::memory_order_acquire)) return f;
-  void* sym = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) != cudaSuccess ||
-      q != cudaDriverEntryPointSuccess)
-    return nullptr;
-  fn.store(reinterpret_cast<EncodeTiledFn>(sym), std::memory_order_release);
-  return reinterpret_cast<EncodeTiledFn>(sym);
-}
-
 // The part of the launch shape the tensor map depends on: slab width, column groups, images of a stage.
 struct DwShape { int cols, Cb, XG, NI, Wb; };
 DwShape dw_search_shape(const ConvGeom& g, int batch_capacity) {
@@ -393,7 +378,7 @@ struct DwSplit { int k, n_rb, rows; };
 
 aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int batch_capacity, int n_versions, void* map_out) {
   if (g.stride != 1 && g.stride != 2) return set_error(AIQ_ERR_SHAPE, "depthwise: stride %d is not supported", g.stride);
-  EncodeTiledFn enc = dw_encode_fn();
+  EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const DwShape s = dw_shape(g, batch_capacity);
   const bool split = g.act_format == ACT_SPLIT;

@@ -420,8 +420,8 @@ aiq_status_t launch_bits(const LayerJob* jobs_dev, const LayerJob& single, int n
   } else if (M > 4 && !plain_rows8(BITS, N, K, M, props.n_sms)) {
     // The largest tile that still gives every SM a block; smaller ones split K over more thread groups.  The tile of 8 rows
     // leaves out the work of rows that are not there (8191 x 8191, 5 rows, 4 bits: 72 us against 94 with the tile of 16).
-    auto blocks = [&](int bn, int bm) { return (long long)((N + bn - 1) / bn) * ((M + bm - 1) / bm) * n_jobs; };
-    auto args = [&](auto launch) { return launch(scope, jobs_dev, single, n_jobs, N, K, M, props.n_sms, s, 0); };
+    auto blocks = [&](int bn, int bm) { return (long long)((N + bn - 1) / bn) * ((M + bm - 1) / bm); };
+    auto args = [&](auto launch) { return launch(scope, nullptr, single, 1, N, K, M, props.n_sms, s, 0); };
     aiq_status_t st;
     if (M > 32 && blocks(64, 64) >= props.n_sms) st = args(launch_gemm_tile<BITS, 64, 64>);
     else if (M > 16 && blocks(64, 32) >= props.n_sms) st = args(launch_gemm_tile<BITS, 64, 32>);

@@ -1,5 +1,5 @@
-// Small-batch quantized linear layer for 4- and 8-bit weights, M <= 16, on the warp-level
-// integer tensor-core path.
+// Small-batch quantized linear layer for 4- and 8-bit weights on the warp-level integer tensor-core path: five to eight
+// batch rows (up to four with rows longer than 8,192; up to 16 with fewer than 32 channels).
 //
 //   y[m][n] = s_n * sum_k code[n][k] * x[m][k] + bias[n]
 //

@@ -12,6 +12,22 @@ namespace {
 constexpr long long kWaitLimitCycles = 4000ll * 1000ll * 1000ll;  // every wait gives up after ~2 s of SM clocks
 constexpr uint32_t kSpinLimit = 1u << 30;                         // and after this many polls at the latest
 
+// cuTensorMapEncodeTiled of the driver (looked up once), or nullptr
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+inline EncodeTiledFn encode_tiled_fn() {
+  static std::atomic<EncodeTiledFn> fn{nullptr};
+  if (EncodeTiledFn f = fn.load(std::memory_order_acquire)) return f;
+  void* sym = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &q) != cudaSuccess ||
+      q != cudaDriverEntryPointSuccess)
+    return nullptr;
+  fn.store(reinterpret_cast<EncodeTiledFn>(sym), std::memory_order_release);
+  return reinterpret_cast<EncodeTiledFn>(sym);
+}
+
 // ---- PTX wrappers ------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -85,20 +101,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
   return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, error_flag));
 }
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                            int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-      : "memory");
-}
-__device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1,
-                                            int c2, int c3, int c4) {
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
-      : "memory");
-}
 // By a converged warp: one elected lane announces the bytes on the barrier and issues the copy.  (Inside `if (lane == 0)`
 // a producer loop took 400 cycles for a copy; its descriptor and coordinates cannot stay in uniform registers there.)
 __device__ __forceinline__ void tma_fill_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, uint32_t bytes, int c0, int c1, int c2) {

@@ -128,10 +128,10 @@ void aiq_set_scale_granularity(int granularity);
  *     512 k or fewer become four int8 digits with a shared exponent (28 bits below the largest
  *     |x|), the int32 sums are exact and run-to-run identical; a batch row with an infinity or a
  *     NaN is multiplied in float32, as by the plain kernel.
- *   M <= 8 otherwise, 4 / 8 bits, K a multiple of 512, N*K >= 2^20: the codes stay integer and feed the int8
- *     warp-level tensor cores; the activations of each group of 512 k become three int8
- *     digits with a shared exponent (21 bits below the group's largest |x|), the int32 sums
- *     are exact.
+ *   M <= 8 otherwise (and M <= 4 at 4 bits with N*K > 3 * 2^25), 4 / 8 bits, K a multiple of 512, N*K >= 2^20: the
+ *     codes stay integer and feed the int8 warp-level tensor cores; the activations of each group of
+ *     512 k become three int8 digits (M <= 4: four) with a shared exponent (21 or 28 bits below the
+ *     group's largest |x|), the int32 sums are exact.  A batch row with an infinity or a NaN becomes NaN.
  *   M >= 9, K a multiple of 8, K >= 64, N >= 32: a tcgen05 GEMM with the weight matrix as the
  *     MMA's M operand and the batch as its N operand.  4 / 8 / 16 bits: codes and halves are
  *     exact; the activations, scaled by a power of two per batch row, enter as the sum of two
@@ -141,9 +141,9 @@ void aiq_set_scale_granularity(int granularity);
  * The last two split K over thread blocks where the matrix has too few rows to fill the GPU; the
  * partial sums then meet in y through float atomics (run-to-run differences in the last
  * bit).  They need scratch memory: pass `workspace` (device, 16-byte aligned; refused if it is not)
- * of at least aiq_qlinear_workspace_bytes(...) bytes; without it the plain kernel runs in their
- * place.  (The kernel of up to four rows needs none, and runs with or without; the function keeps
- * its former answer there.)
+ * of at least aiq_qlinear_workspace_bytes(...) bytes; without it the plain kernel (or the one of up
+ * to four rows) runs in their place.  (The kernel of up to four rows needs none, and runs with or
+ * without; the function keeps its former answer there.)
  * Device-side failure: the tcgen05 kernel bounds every wait on its copy / MMA pipeline (about
  * 2 s of SM clocks).  Should one expire, the kernel stops early and y is invalid; the call has
  * long returned AIQ_OK by then, so the record is on the device: the int32 at byte offset

@@ -486,9 +486,13 @@ static bool small_gemm(int N, int K, int bits, int M) {
   return bits == 32 || M <= 8 || !(products > (K > 4096 ? 1ll << 22 : K >= 1024 ? 1ll << 25 : 1ll << 26));
 }
 
-// The kernel of a call, and of the size query: SCRATCH_* ones need the workspace, and without it PLAIN runs in their place.
+// The kernel of a call, and of the size query: SCRATCH_* ones need the workspace, and without it GEMV or PLAIN runs in their place.
 enum QlinearPath { QL_PLAIN, QL_GEMV, QL_SCRATCH_MMA, QL_SCRATCH_TC };
 static QlinearPath qlinear_path(int N, int K, int bits, int M) {
+  // 4 bits above 3 x 2^25 weights: the kernel of up to four rows needs twice the MMAs of the one with scratch (its weights are
+  // the narrow operand) and no longer streams at the memory's rate.  One / four rows, on the device: 16384 x 8192 21.6 / 26.4
+  // us there, 18.7 / 23.7 here; 32768 x 8192 41.0 / 46.5 | 30.0 / 40.0; at 8192 x 8192 calls take 12.2 / 16.9 us and 14.2 / 16.6.
+  if (bits == 4 && M <= 4 && (long long)N * K > (3ll << 25) && aiq::qlinear_mma_applicable(N, K, bits, M)) return QL_SCRATCH_MMA;
   if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return QL_GEMV;
   if (small_gemm(N, K, bits, M)) return QL_PLAIN;
   if (aiq::qlinear_tc_applicable(N, K, bits, M)) return QL_SCRATCH_TC;
@@ -528,7 +532,6 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
   if (workspace && (((uintptr_t)workspace) & 15) && (aiq::qlinear_tc_applicable(N, K, bits, M) || aiq::qlinear_mma_applicable(N, K, bits, M)))
     return aiq::set_error(AIQ_ERR_INVALID_ARG, "aiq_qlinear: workspace not 16-byte aligned");
   const QlinearPath path = qlinear_path(N, K, bits, M);
-  if (path == QL_GEMV) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
   // the tensor-core kernels need scratch for the converted activations
   if (path == QL_SCRATCH_TC && workspace) {
     const size_t scratch = aiq::qlinear_tc_workspace_bytes(K, M);
@@ -540,5 +543,6 @@ extern "C" aiq_status_t aiq_qlinear(const void* packed, const float* scales, con
   }
   if (path == QL_SCRATCH_MMA && workspace && workspace_bytes >= aiq::qlinear_mma_workspace_bytes(K, M))
     return aiq::launch_qlinear_mma(job, N, K, M, workspace, (cudaStream_t)stream);
+  if (aiq::qlinear_gemv_applicable(N, K, bits, M)) return aiq::launch_qlinear_gemv(job, N, K, M, (cudaStream_t)stream);
   return aiq::launch_qlinear(nullptr, &job, 1, N, K, M, (cudaStream_t)stream);
 }

@@ -12,11 +12,12 @@
 // taken out again exactly, in integers, with the column sums of the activations).
 //
 // The activations are brought to the integer side once per block: for each batch row and
-// K-slice, x = 2^(e-6) * (d1 + d2 / 2^7 + d3 / 2^14) with three int8 digits and a shared
-// exponent e (2^e > max |x| of the slice), a 21-bit fixed-point image of x relative to that
-// maximum.  Each digit is a column of the B operand, so a batch row costs three of the eight
-// columns of an MMA; the three int32 sums are exact and are recombined in float32 as
-// s_n * 2^(e-6) * (S1 + S2 / 2^7 + S3 / 2^14).
+// K-slice, x = 2^(e-6) * (d1 + d2 / 2^7 + d3 / 2^14 [+ d4 / 2^21]) with three int8 digits, four up to
+// four batch rows (where they cost no further MMA), and a shared exponent e (2^e > max |x| of the
+// slice), a 21- or 28-bit fixed-point image of x relative to that maximum.  Each digit is a column
+// of the B operand, so a batch row costs three or four of the eight columns of an MMA; the int32
+// sums are exact and are recombined in float32 as s_n * 2^(e-6) * (S1 + S2 / 2^7 + S3 / 2^14 [+ S4 / 2^21]).
+// A slice with an infinity or a NaN makes its batch row NaN.
 //
 // Work split: a block owns 128 output channels x a K-slice of 512 or 1024; each of its 4
 // warps owns 32 channels (two 16-row MMA tiles) and streams them through a private
@@ -83,8 +84,8 @@ __host__ __device__ inline size_t ws_frag_bytes(int n_groups, int nt) { return (
 constexpr int kMetaBytes = 16 * 4 + 48 * 4;
 
 // Pre-pass: one block per group of 512 k.  Brings the activations to the integer side:
-// x = 2^(e-6) * (d1 + d2 / 2^7 + d3 / 2^14), digits written in B-fragment order.
-template <int BITS, int NT>
+// x = 2^(e-6) * (d1 + d2 / 2^7 + d3 / 2^14 [+ d4 / 2^21]), digits written in B-fragment order.
+template <int BITS, int NT, int DIG>
 __global__ void __launch_bounds__(256)
 qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __restrict__ ws, int n_groups,
                       float* __restrict__ y, int y_elems) {
@@ -104,7 +105,7 @@ qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __rest
   if (threadIdx.x < 48) s_colsum[threadIdx.x] = 0;
   for (int idx = threadIdx.x; idx < kGroupFrags * NT * 32; idx += blockDim.x) {
     const int fl = idx & 31, nt = (idx >> 5) % NT, f = idx / (32 * NT);
-    if (nt * 8 + (fl >> 2) >= 3 * M) frags[f][nt][fl] = make_uint2(0u, 0u);      // unused columns
+    if (nt * 8 + (fl >> 2) >= DIG * M) frags[f][nt][fl] = make_uint2(0u, 0u);      // unused columns
   }
   __syncthreads();
   for (int idx = threadIdx.x; idx < M * kGroupK; idx += blockDim.x) {            // one batch row per warp pass
@@ -119,8 +120,9 @@ qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __rest
     const float xmax = __int_as_float(s_xmax[threadIdx.x]);
     int e = 0;
     frexpf(xmax, &e);                                   // xmax = f * 2^e with f in [0.5, 1)
-    s_up[threadIdx.x] = xmax > 0.f ? ldexpf(1.f, 6 - e) : 0.f;
-    reinterpret_cast<float*>(meta)[threadIdx.x] = xmax > 0.f ? ldexpf(1.f, e - 6) : 0.f;
+    const bool finite = s_xmax[threadIdx.x] < 0x7F800000;
+    s_up[threadIdx.x] = finite && xmax > 0.f ? ldexpf(1.f, 6 - e) : 0.f;
+    reinterpret_cast<float*>(meta)[threadIdx.x] = !finite ? __int_as_float(0x7FC00000) : xmax > 0.f ? ldexpf(1.f, e - 6) : 0.f;
   }
   __syncthreads();
   const int n_entries = kGroupFrags * M * 4;            // (fragment, batch row, t)
@@ -130,21 +132,23 @@ qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __rest
     frag_k_offsets<BITS>(f % MPC, o);
     const int kb = k0 + (f / MPC) * CHUNK + ft * KL;
     const float up = s_up[m];
-    int d[3][8];
-    int sum[3] = {0, 0, 0};
+    int d[DIG][8];
+    int sum[DIG] = {};
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const float xv = (kb + o[i] < K) ? __ldg(x + (size_t)m * K + kb + o[i]) * up : 0.f;   // |xv| < 64
-      const float d1 = rintf(xv);
-      const float r1 = (xv - d1) * 128.f;                // exact: |xv - d1| <= 0.5
-      const float d2 = rintf(r1);
-      const float d3 = rintf((r1 - d2) * 128.f);
-      d[0][i] = (int)d1; d[1][i] = (int)d2; d[2][i] = (int)d3;
-      sum[0] += d[0][i]; sum[1] += d[1][i]; sum[2] += d[2][i];
+      float rest = xv;
+#pragma unroll
+      for (int dig = 0; dig < DIG; ++dig) {
+        const float q = rintf(rest);
+        rest = (rest - q) * 128.f;                       // exact: |rest - q| <= 0.5
+        d[dig][i] = (int)q;
+        sum[dig] += d[dig][i];
+      }
     }
 #pragma unroll
-    for (int dig = 0; dig < 3; ++dig) {
-      const int col = 3 * m + dig;
+    for (int dig = 0; dig < DIG; ++dig) {
+      const int col = DIG * m + dig;
       frags[f][col >> 3][(col & 7) * 4 + ft] = make_uint2(pack_s8(d[dig][0], d[dig][1], d[dig][2], d[dig][3]),
                                                           pack_s8(d[dig][4], d[dig][5], d[dig][6], d[dig][7]));
       atomicAdd(&s_colsum[col], sum[dig]);
@@ -155,7 +159,7 @@ qlinear_digits_kernel(const float* __restrict__ x, int K, int M, uint8_t* __rest
 }
 
 // Main kernel: GROUPS groups of 512 k per block.
-template <int BITS, int NT, int GROUPS>
+template <int BITS, int NT, int GROUPS, int DIG>
 __global__ void __launch_bounds__(kMmaWarps * 32)
 qlinear_mma_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scale, const float* __restrict__ bias,
                    const uint8_t* ws, int n_groups, float* __restrict__ y, int N, int K, int M) {
@@ -278,15 +282,15 @@ qlinear_mma_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scal
     if ((st + 1) % STAGES_PER_GROUP == 0) {
       // end of a group: the exact integer sums leave for float32 with the group's exponent.
       // D fragment: lane (g, t) holds rows g, g+8 and columns 2t, 2t+1 of tile nt; column
-      // c = 3 m + digit contributes 2^(e-6) * 2^(-7 digit) * (S - 8 * colsum).
+      // c = DIG m + digit contributes 2^(e-6) * 2^(-7 digit) * (S - 8 * colsum).
       const int gi = st / STAGES_PER_GROUP;
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int col = nt * 8 + 2 * t + e;
-          const int m = col / 3, dig = col - 3 * m;
-          const float wgt = (m < M ? s_down[gi][m] : 0.f) * (dig == 0 ? 1.f : dig == 1 ? 0.0078125f : 0.00006103515625f);
+          const int m = col / DIG, dig = col - DIG * m;
+          const float wgt = (m < M ? s_down[gi][m] : 0.f) * __int_as_float((127 - 7 * dig) << 23);
           const int cs = OFFS * s_colsum[gi][col];
 #pragma unroll
           for (int tile = 0; tile < 2; ++tile) {
@@ -316,7 +320,7 @@ qlinear_mma_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scal
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int col = nt * 8 + 2 * t + e;
-          const int m = col / 3, dig = col - 3 * m;
+          const int m = col / DIG, dig = col - DIG * m;
           if (m >= M) continue;
           atomicAdd(y + (size_t)m * N + n, fmaf(facc[tile][nt][2 * half + e], s, dig == 0 ? b : 0.f));
         }
@@ -328,7 +332,7 @@ qlinear_mma_kernel(const uint8_t* __restrict__ w, const float* __restrict__ scal
 }  // namespace
 
 static int qlinear_nt(int M) {
-  const int nt = (3 * M + 7) / 8;                  // 8-column tiles for 3 digit columns per batch row
+  const int nt = ((M <= 4 ? 4 : 3) * M + 7) / 8;   // 8-column tiles for the digit columns of the batch rows
   return nt <= 1 ? 1 : nt <= 2 ? 2 : nt <= 3 ? 3 : 6;
 }
 
@@ -355,11 +359,11 @@ aiq_status_t launch_qlinear_mma(const LayerJob& job, int N, int K, int M, void* 
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   LaunchScope scope(AIQ_KERNEL_QLINEAR, s, 2.0 * M * N * K,
                     (double)N * row_bytes(K, job.bits) + 4.0 * N + 4.0 * M * ((double)K + N));
-#define AIQ_QMMA(BITS_, NT_, GR_)                                                                           \
+#define AIQ_QMMA(BITS_, NT_, GR_, DIG_)                                                                           \
   do {                                                                                                      \
     const int smem = GR_ * kGroupFrags * NT_ * 32 * (int)sizeof(uint2) + kMmaWarps * kStages * kStageBytes; \
-    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_mma_kernel<BITS_, NT_, GR_>), smem);                                   \
-    qlinear_digits_kernel<BITS_, NT_><<<n_groups, 256, 0, s>>>(x, K, M, ws, n_groups, y, M * N);            \
+    AIQ_ENSURE_DYNAMIC_SMEM((qlinear_mma_kernel<BITS_, NT_, GR_, DIG_>), smem);                                   \
+    qlinear_digits_kernel<BITS_, NT_, DIG_><<<n_groups, 256, 0, s>>>(x, K, M, ws, n_groups, y, M * N);            \
     cudaLaunchConfig_t cfg = {};                                                                            \
     cfg.gridDim = grid; cfg.blockDim = dim3(kMmaWarps * 32); cfg.dynamicSmemBytes = smem; cfg.stream = s;   \
     cudaLaunchAttribute attr[1];                                                                            \
@@ -367,15 +371,16 @@ aiq_status_t launch_qlinear_mma(const LayerJob& job, int N, int K, int M, void* 
     attr[0].val.programmaticStreamSerializationAllowed = 1;                                                 \
     cfg.attrs = attr; cfg.numAttrs = 1;                                                                     \
     const uint8_t* ws_c = ws;                                                                               \
-    AIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, qlinear_mma_kernel<BITS_, NT_, GR_>, w, job.scale, job.bias,      \
+    AIQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, qlinear_mma_kernel<BITS_, NT_, GR_, DIG_>, w, job.scale, job.bias,      \
                                     ws_c, n_groups, y, N, K, M));                                           \
   } while (0)
 #define AIQ_QMMA_BITS(BITS_)                                                                       \
   do {                                                                                             \
-    if (nt_t == 1) { if (groups == 2) AIQ_QMMA(BITS_, 1, 2); else AIQ_QMMA(BITS_, 1, 1); }         \
-    else if (nt_t == 2) { if (groups == 2) AIQ_QMMA(BITS_, 2, 2); else AIQ_QMMA(BITS_, 2, 1); }    \
-    else if (nt_t == 3) { if (groups == 2) AIQ_QMMA(BITS_, 3, 2); else AIQ_QMMA(BITS_, 3, 1); }    \
-    else AIQ_QMMA(BITS_, 6, 1);                                                                    \
+    if (nt_t == 1) { if (groups == 2) AIQ_QMMA(BITS_, 1, 2, 4); else AIQ_QMMA(BITS_, 1, 1, 4); }   \
+    else if (nt_t == 2 && M <= 4) { if (groups == 2) AIQ_QMMA(BITS_, 2, 2, 4); else AIQ_QMMA(BITS_, 2, 1, 4); } \
+    else if (nt_t == 2) { if (groups == 2) AIQ_QMMA(BITS_, 2, 2, 3); else AIQ_QMMA(BITS_, 2, 1, 3); } \
+    else if (nt_t == 3) { if (groups == 2) AIQ_QMMA(BITS_, 3, 2, 3); else AIQ_QMMA(BITS_, 3, 1, 3); } \
+    else AIQ_QMMA(BITS_, 6, 1, 3);                                                                 \
   } while (0)
   if (job.bits == 4) AIQ_QMMA_BITS(4); else AIQ_QMMA_BITS(8);
 #undef AIQ_QMMA_BITS

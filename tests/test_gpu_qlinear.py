@@ -102,3 +102,34 @@ def test_qlinear_refuses_a_misaligned_workspace(N, K, M):
     small = torch.empty((30, aiq.aiq_packed_row_bytes(100, 4)), dtype=torch.uint8, device="cuda")
     aiq.aiq_quantize_layer(torch.randn((30, 100), device="cuda"), 4, small, scales[:30])
     aiq.aiq_qlinear(small, scales[:30], None, 30, 100, 4, torch.zeros((M, 100), device="cuda"), y.view(-1)[:30 * M].view(M, 30), workspace=ws[4:])
+
+
+@pytest.mark.parametrize("N,K", [(13000, 8192), (100001, 1024), (51000, 2048)])
+@pytest.mark.parametrize("M", [1, 2, 3, 4])
+def test_large_4_bit_layer_with_scratch(N, K, M):
+    """Above 3 x 2^25 weights the kernel with scratch takes up to four rows.  Integers beside activations that only the fourth
+    digit holds (j 2^-26 where the largest of every 512 is 1 and meets a zero weight): every sum is exact, with and without
+    the workspace.  An infinity makes its own row not finite."""
+    import torch
+    aiq = binding()
+    g = torch.Generator(device="cuda").manual_seed(N + K + M)
+    W = torch.randint(-7, 8, (N, K), generator=g, device="cuda").float()
+    W[:, 1] = 7
+    W[:, ::64] = 0
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, 4)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, 4, packed, scales)
+    ws = torch.empty(aiq.aiq_qlinear_workspace_bytes(N, K, 4, M), dtype=torch.uint8, device="cuda")
+    assert ws.numel() > 0
+    j = torch.randint(-63, 64, (M, K), generator=g, device="cuda")
+    x = j.float() * 2.0 ** -26
+    x[:, ::64] = 1.0
+    j[:, ::64] = 0
+    want = j.double() @ W.double().T
+    for workspace in (ws, None):
+        y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+        aiq.aiq_qlinear(packed, scales, None, N, K, 4, x, y, workspace=workspace)
+        assert torch.equal(y.double() * 2.0 ** 26, want)
+    x[M - 1, 700] = float("inf")
+    aiq.aiq_qlinear(packed, scales, None, N, K, 4, x, y, workspace=ws)
+    assert torch.equal(y[:M - 1].double() * 2.0 ** 26, want[:M - 1]) and not bool(torch.isfinite(y[M - 1]).any())

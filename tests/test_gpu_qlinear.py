@@ -132,4 +132,35 @@ def test_large_4_bit_layer_with_scratch(N, K, M):
         assert torch.equal(y.double() * 2.0 ** 26, want)
     x[M - 1, 700] = float("inf")
     aiq.aiq_qlinear(packed, scales, None, N, K, 4, x, y, workspace=ws)
-    assert torch.equal(y[:M - 1].double() * 2.0 ** 26, want[:M - 1]) and not bool(torch.isfinite(y[M - 1]).any())
+    assert torch.equal(y[:M - 1].double() * 2.0 ** 26, want[:M - 1])
+    assert not bool(torch.isfinite(y[M - 1]).any())
+
+
+@pytest.mark.parametrize("bits", [4, 8])
+@pytest.mark.parametrize("N,K,M", [(33000, 512, 5), (18000, 1024, 8), (8200, 2048, 6)])
+def test_digit_kernel_extreme_activations(bits, N, K, M):
+    """Five to eight rows with scratch: infinities and NaN make their rows not finite, and slices of denormals count, in rows
+    beside ordinary ones; integers, so that what is finite is exact, but for what float atomics flush: denormal addends and
+    sums, less than 2^-126 each, three digits and up to K / 512 slices an output."""
+    import torch
+    aiq = binding()
+    g = torch.Generator(device="cuda").manual_seed(N + K + M)
+    W = torch.randint(-7, 8, (N, K), generator=g, device="cuda").float()
+    W[:, 1] = 7 if bits == 4 else 127
+    packed = torch.empty((N, aiq.aiq_packed_row_bytes(K, bits)), dtype=torch.uint8, device="cuda")
+    scales = torch.empty(N, dtype=torch.float32, device="cuda")
+    aiq.aiq_quantize_layer(W, bits, packed, scales)
+    ws = torch.empty(aiq.aiq_qlinear_workspace_bytes(N, K, bits, M), dtype=torch.uint8, device="cuda")
+    assert ws.numel() > 0
+    unit = torch.ones(M, 1, device="cuda")
+    unit[1] = 2.0 ** -132
+    x = torch.randint(-63, 64, (M, K), generator=g, device="cuda").float() * unit
+    x[2, K - 1] = float("inf")
+    x[M - 1, 17] = float("nan")
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    aiq.aiq_qlinear(packed, scales, None, N, K, bits, x, y, workspace=ws)
+    want = (torch.where(x.isfinite(), x, 0).double() @ W.double().T).float()
+    assert not bool(torch.isfinite(y[[2, M - 1]]).any())
+    assert float((y[1].double() - want[1].double()).abs().max()) <= 2 * 3 * (K // 512) * 2.0 ** -126
+    rest = [m for m in range(M) if m not in (1, 2, M - 1)]
+    assert torch.equal(y[rest], want[rest])

@@ -164,7 +164,9 @@ __device__ __forceinline__ float apply_act(float v, int act) {
 //   ACT_SPLIT [hi(Cs) | lo(Cs)] bfloat16, value = float(hi) + float(lo) with
 //             hi = bf16_rn(v), lo = bf16_rn(v - hi): 16+ significant bits in the same bytes,
 //             in the form the bf16 tensor cores consume without conversion (the two halves
-//             are two K-slices of the GEMM).  Used when the model has tensor-core layers.
+//             are two K-slices of the GEMM).  Used when the model has tensor-core layers; a tensor that only
+//             depthwise layers read stays in floats all the same (ConvGeom::out_f32): no MMA needs its halves,
+//             and neither its writer nor its readers then split or join (MobileNetV2's expansions).
 //   ACT_RS    the hi / lo bfloat16 pairs of ACT_SPLIT in the image-interleaved layout of the
 //             row-streaming tensor-core convolution (conv_rs.cu):
 //             [group][row][column][plane][image][8 bfloat16], G = rs_group_images(width) images per
@@ -220,6 +222,7 @@ struct ConvGeom {
   int Cs_in, Cs_out;  // padded channel counts of the split tensors
   int in_is_nchw;     // 1: the input is the float32 NCHW network input
   int act_format;     // ACT_F32 or ACT_SPLIT, for input, residual and output alike
+  int in_f32, out_f32;   // ACT_SPLIT models: the input / output tensor holds Cs floats per pixel (its readers are depthwise layers)
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------------------

@@ -107,7 +107,7 @@ __device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int r, int r_end) {
 // columns a row cost 37 per output element at 0.46 issued per clock and scheduler (2.9 TB/s at 256 x 32 x 32 x 144
 // channels); four columns share six unpacked input columns (1.5 per output instead of 2), the per-row waiting and
 // the addresses.
-template <int FMT, int STRIDE, int COLS, bool RES>
+template <int IFMT, int FMT, int STRIDE, int COLS, bool RES>
 __global__ void __launch_bounds__(kDwThreads + 32, 2)
 depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, const LayerJob* __restrict__ jobs) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
@@ -203,7 +203,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
   chain_wait();                                          // the output slot may still be read by an earlier kernel
   constexpr int IN_COLS = (COLS - 1) * STRIDE + 3;
   const uint32_t my_cols = smem_u32(ring) + (uint32_t)(worker ? ni * p.Wb + xg * COLS * STRIDE : 0) * col_bytes +
-                           (uint32_t)q * (FMT == ACT_SPLIT ? 8 : 16);
+                           (uint32_t)q * (IFMT == ACT_SPLIT ? 8 : 16);
   uint32_t stage = 0, phase = 0;
   bool alive = true;
   const uint32_t my_w = smem_u32(s_w) + q * 16;
@@ -219,7 +219,7 @@ depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, cons
     const uint32_t src = my_cols + stage * p.stage_bytes;
     uint64_t v[IN_COLS][2];
 #pragma unroll
-    for (int xx = 0; xx < IN_COLS; ++xx) read4<FMT>(src + xx * col_bytes, p.Cb, v[xx]);
+    for (int xx = 0; xx < IN_COLS; ++xx) read4<IFMT>(src + xx * col_bytes, p.Cb, v[xx]);
     auto tap_row = [&](auto r_, auto fresh, uint64_t (&s)[COLS][2]) {
       constexpr int R = decltype(r_)::value;
       constexpr bool FRESH = decltype(fresh)::value;
@@ -381,7 +381,7 @@ aiq_status_t depthwise_encode_map(const ConvGeom& g, const void* slot_base, int 
   EncodeTiledFn enc = encode_tiled_fn();
   if (!enc) return set_error(AIQ_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const DwShape s = dw_shape(g, batch_capacity);
-  const bool split = g.act_format == ACT_SPLIT;
+  const bool split = g.act_format == ACT_SPLIT && !g.in_f32;
   // (channel, hi | lo, column, padded row, image over all versions); float32 pixels have one part
   const cuuint64_t pix = 4ull * g.Cs_in, row = pix * g.W;
   cuuint64_t dims[5] = {(cuuint64_t)g.Cs_in, split ? 2ull : 1ull, (cuuint64_t)g.W, (cuuint64_t)g.H + 2, (cuuint64_t)n_versions * batch_capacity};
@@ -461,17 +461,20 @@ aiq_status_t launch_depthwise(const ConvGeom& g, const void* map, const LayerJob
                     weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
                                                    (double)g.B * g.Ho * g.Wo * g.Cout));
   const CUtensorMap& m = *static_cast<const CUtensorMap*>(map);
-#define AIQ_DW(FMT_, ST_, COLS_, RES_)                                                                          \
+#define AIQ_DW(IFMT_, FMT_, ST_, COLS_, RES_)                                                                   \
   do {                                                                                                          \
-    AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<FMT_, ST_, COLS_, RES_>), per_cta);                              \
-    AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<FMT_, ST_, COLS_, RES_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
+    AIQ_ENSURE_DYNAMIC_SMEM((depthwise3x3_kernel<IFMT_, FMT_, ST_, COLS_, RES_>), per_cta);                       \
+    AIQ_CUDA_TRY(launch_chained(scope.chain, depthwise3x3_kernel<IFMT_, FMT_, ST_, COLS_, RES_>, grid, dim3(threads), smem, s, m, p, jobs_dev)); \
   } while (0)
-#define AIQ_DW_SHAPE(FMT_, RES_)                                                                                \
+#define AIQ_DW_SHAPE(IFMT_, FMT_, RES_)                                                                         \
   do {                                                                                                          \
-    if (g.stride == 2) AIQ_DW(FMT_, 2, 2, RES_); else if (sh.cols == 4) AIQ_DW(FMT_, 1, 4, RES_); else AIQ_DW(FMT_, 1, 2, RES_); \
+    if (g.stride == 2) AIQ_DW(IFMT_, FMT_, 2, 2, RES_);                                                         \
+    else if (sh.cols == 4) AIQ_DW(IFMT_, FMT_, 1, 4, RES_);                                                     \
+    else AIQ_DW(IFMT_, FMT_, 1, 2, RES_);                                                                       \
   } while (0)
-  if (g.act_format == ACT_SPLIT) { if (has_res) AIQ_DW_SHAPE(ACT_SPLIT, true); else AIQ_DW_SHAPE(ACT_SPLIT, false); }
-  else { if (has_res) AIQ_DW_SHAPE(ACT_F32, true); else AIQ_DW_SHAPE(ACT_F32, false); }
+  if (g.act_format == ACT_SPLIT && g.in_f32) { if (has_res) AIQ_DW_SHAPE(ACT_F32, ACT_SPLIT, true); else AIQ_DW_SHAPE(ACT_F32, ACT_SPLIT, false); }
+  else if (g.act_format == ACT_SPLIT) { if (has_res) AIQ_DW_SHAPE(ACT_SPLIT, ACT_SPLIT, true); else AIQ_DW_SHAPE(ACT_SPLIT, ACT_SPLIT, false); }
+  else { if (has_res) AIQ_DW_SHAPE(ACT_F32, ACT_F32, true); else AIQ_DW_SHAPE(ACT_F32, ACT_F32, false); }
 #undef AIQ_DW_SHAPE
 #undef AIQ_DW
   AIQ_LAUNCH_CHECK("depthwise3x3");

@@ -134,6 +134,7 @@ struct LayerInfo {
   uint8_t* mb_tile[2];
   float* mb_coef[4];
   int mb_nh;
+  int out_f32;             // ConvGeom::out_f32
 };
 
 struct aiq_model {
@@ -243,6 +244,8 @@ static ConvGeom make_geom(const aiq_model* m, const LayerInfo& li, int B) {
   g.Cs_in = padded_channels(li.d.cin); g.Cs_out = padded_channels(li.d.cout);
   g.in_is_nchw = li.d.input < 0 ? 1 : 0;          // the network input is float32 NCHW
   g.act_format = m->act_format;
+  g.out_f32 = li.out_f32;
+  g.in_f32 = li.d.input >= 0 ? m->layers[li.d.input].out_f32 : 0;
   return g;
 }
 
@@ -449,6 +452,25 @@ static void derive_format(aiq_model* m, int opt_path) {
       m->mb_mid[le] = mid[le];
       m->mb_tail[le] = tail[le];
       e.mb_nh = d.mb_nh = pr.mb_nh = nh;
+    }
+  }
+  // Tensors that only depthwise layers read, and whose writer (a pointwise layer, or the layer on the network input) can
+  // leave them in floats: the same bytes, but no splitting there, no joining here, and no rounding.  Before / after, us:
+  // MobileNetV2-CIFAR 1 image 286 / 273, 256 images 2,118 / 2,062; ImageNet shapes, 32 images 623 / 593; 52 candidates x
+  // 512 images 113.5 / 110.6 ms.
+  for (LayerInfo& li : m->layers) li.out_f32 = 0;
+  if (m->act_format == ACT_SPLIT) {
+    std::vector<int> uses(m->layers.size(), 0), dw_uses(m->layers.size(), 0);
+    for (const LayerInfo& li : m->layers) {
+      if (li.d.input >= 0) uses[li.d.input]++;
+      if (li.d.residual >= 0) uses[li.d.residual]++;
+      if (li.d.input >= 0 && li.d.kind == AIQ_LAYER_DEPTHWISE) dw_uses[li.d.input]++;
+    }
+    for (size_t l = 0; l < m->layers.size(); ++l) {
+      const LayerInfo& li = m->layers[l];
+      const int tkind = layer_tensor_kind(m, li);
+      if (uses[l] > 0 && uses[l] == dw_uses[l] && li.d.kind == AIQ_LAYER_CONV && li.d.residual < 0 && (tkind == 2 || (tkind == 0 && li.d.input < 0)))
+        m->layers[l].out_f32 = 1;
     }
   }
   assign_slots(m);
@@ -1096,7 +1118,9 @@ static aiq_status_t run_chunk(const aiq_model* m, const EvalPlan& plan, const La
       done += lp.n_tc32;
     }
     if (lp.n_versions > done) {
-      st = launch_conv(g, jobs_dev + lp.job_first + done, lp.n_versions - done, x_chunk, lp.weight_bytes, stream);
+      ConvGeom gf = g;
+      if (g.out_f32) gf.act_format = ACT_F32;     // a layer on the network input: only the output has a format
+      st = launch_conv(gf, jobs_dev + lp.job_first + done, lp.n_versions - done, x_chunk, lp.weight_bytes, stream);
       if (st != AIQ_OK) return st;
     }
   }

@@ -316,6 +316,14 @@ __device__ __forceinline__ void finish8(const uint32_t* v, const float* scale, c
     }
   }
 }
+// Four finished accumulators that stay floats: scale, bias, activation.
+template <int ACT>
+__device__ __forceinline__ float4 finish4(const uint32_t* v, const float* scale, const float* bias) {
+  const ulonglong2 sc = *reinterpret_cast<const ulonglong2*>(scale), bi = *reinterpret_cast<const ulonglong2*>(bias);
+  const float2 a = unpack2(fma2(pack2(__uint_as_float(v[0]), __uint_as_float(v[1])), sc.x, bi.x));
+  const float2 b = unpack2(fma2(pack2(__uint_as_float(v[2]), __uint_as_float(v[3])), sc.y, bi.y));
+  return make_float4(act_of<ACT>(a.x), act_of<ACT>(a.y), act_of<ACT>(b.x), act_of<ACT>(b.y));
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // Eight packed codes (4 bits: raw.x; 8 bits: raw.x, raw.y; two's complement) -> eight

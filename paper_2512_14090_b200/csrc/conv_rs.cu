@@ -266,7 +266,8 @@ __device__ __forceinline__ void rs_finish_unit(const uint32_t* v, const float* s
                       RES ? res[2 + e] : make_uint4(0u, 0u, 0u, 0u), hi + 4 * e, lo + 4 * e);
 }
 
-template <int C, int KS, int STRIDE, int PIECES>
+// POOL: the jobs pool (LayerJob::pool).  An instantiation of its own: the sums take 16 registers the others do not have.
+template <int C, int KS, int STRIDE, int PIECES, bool POOL>
 __global__ void __launch_bounds__(kRsMaxThreads, 1)
 conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1, RsParams p,
                const LayerJob* __restrict__ jobs) {
@@ -340,7 +341,6 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     s_scale[i] = job.scale[n_off + i];
     s_bias[i] = job.bias[n_off + i];
   }
-  for (int i = tid; i < p.pool_bytes / 4; i += n_threads) s_pool[i] = 0.f;
   // row programs (one thread per input row)
   if (tid < p.H) s_rows[tid] = rs_row_program<KS, STRIDE>(tid, p.H, p.Ho, N, R);
   bool alive = mbar_wait_warp_inline(bar_w, 0, s_abort, p.error_flag);
@@ -456,7 +456,6 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     const uint8_t* res_base = static_cast<const uint8_t*>(job.res);
     uint8_t* out_base = static_cast<uint8_t*>(job.out);
     const int lo_plane0 = p.cout_total / 8;
-    const bool pooling = p.pool_bytes > 0 && job.pool != nullptr;
     const float pool_scale = 1.0f / (float)(p.Ho * p.Wo);
     // this warp's units of a row and its rows of an item
     const int unit0 = units >= WQ ? h : h % units;
@@ -479,6 +478,9 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     // The residual of the first unit of this warp's next row is requested as soon as the current
     // row's arithmetic is done, so its memory latency overlaps the stores and the next wait.
     uint4 rres[4];
+    uint64_t psum[8];                                  // two channels each
+#pragma unroll
+    for (int e = 0; e < 8; ++e) psum[e] = 0ull;
     auto load_res = [&](int k, int u, uint4* r) {
       int c0;
       const uint8_t* src = res_base + row_offset(k) + unit_offset(u, &c0);
@@ -522,22 +524,11 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         else finish(std::integral_constant<int, AIQ_ACT_NONE>());
         // the residual registers are free again: request the first unit of this warp's next row
         if (res_base && u + unit_step >= units && k + 1 < total) load_res(k + 1, unit0, rres);
-        if (pooling) {
-          // Fused global average pool: the stored value hi + lo of each of the 16 channels, summed
-          // over the columns this warp holds (lanes that differ in the column bits), then added to
-          // this warp's partial sums [image][16 channels] in shared memory.  The tensor is not stored.
-          float* mine = s_pool + ((size_t)(warp - 2) * Gout + img) * 16;
+        if constexpr (POOL) {
+          // Fused global average pool: the stored value hi + lo of each of the 16 channels, added up over the rows of
+          // the item in this lane's registers (a warp drains the same unit of every row).  The tensor is not stored.
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            float a = __uint_as_float(hi[e] << 16) + __uint_as_float(lo[e] << 16);
-            float b = __uint_as_float(hi[e] & 0xFFFF0000u) + __uint_as_float(lo[e] & 0xFFFF0000u);
-            for (int o = Gout; o < 32; o <<= 1) {
-              a += __shfl_xor_sync(0xffffffffu, a, o);
-              b += __shfl_xor_sync(0xffffffffu, b, o);
-            }
-            // channel of word e of [hi plane 0 | hi plane 1]: words 0-3 = channels 0-7, 4-7 = channels 8-15
-            if (lane < Gout) { mine[2 * e] += a; mine[2 * e + 1] += b; }
-          }
+          for (int e = 0; e < 8; ++e) psum[e] = add2(psum[e], add2(widen2(hi[e]), widen2(lo[e])));
         } else {
         uint8_t* dst = out_base + row_off + uoff;
         *reinterpret_cast<uint4*>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
@@ -546,11 +537,26 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         *reinterpret_cast<uint4*>(dst + (size_t)(lo_plane0 + 1) * plane_bytes) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
         }
       }
-      if (pooling && (k + 1) % rows_mine == 0) {
+      if (POOL && (k + 1) % rows_mine == 0) {
         // last row of an item for this warp: once all epilogue warps are here, the partial sums of the
         // warps that hold a channel's chunk are added in a fixed order and the means leave for global memory
         const int n_epi = n_threads - 64;
         const uint32_t pool_parity = (uint32_t)(il & 1);
+        // the columns this warp holds (lanes that differ in the column bits) -> [image][16 channels] in shared memory.
+        // (Once per item: 32 shuffles and 16 updates of shared memory for every row made this the longest launch of the
+        // greedy step, 1,401 us against 845 for the same layer with its tensor stored; the step 32.9 ms, now 32.2.)
+        float* mine = s_pool + ((size_t)(warp - 2) * Gout + img) * 16;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          float2 f = unpack2(psum[e]);
+          for (int o = Gout; o < 32; o <<= 1) {
+            f.x += __shfl_xor_sync(0xffffffffu, f.x, o);
+            f.y += __shfl_xor_sync(0xffffffffu, f.y, o);
+          }
+          // channels of word e of [hi plane 0 | hi plane 1]: words 0-3 = channels 0-7, 4-7 = channels 8-15
+          if (lane < Gout) { mine[2 * e] = f.x; mine[2 * e + 1] = f.y; }
+          psum[e] = 0ull;
+        }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_pool);
         alive = mbar_wait_warp_inline(bar_pool, pool_parity, s_abort, p.error_flag);
@@ -571,8 +577,6 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         if (lane == 0) mbar_arrive(bar_pool + 8);
         alive = mbar_wait_warp_inline(bar_pool + 8, pool_parity, s_abort, p.error_flag);
         if (!alive) break;
-        for (int i = lane; i < Gout * 16; i += 32) s_pool[(size_t)(warp - 2) * Gout * 16 + i] = 0.f;
-        __syncwarp();
       }
     }
   }
@@ -985,13 +989,12 @@ RsConfig rs_config(const ConvGeom& g, const RsShape& sh, int weight_bits, int sm
   return c;
 }
 
-template <int C, int KS, int STRIDE, int PIECES>
+template <int C, int KS, int STRIDE, int PIECES, bool POOL>
 aiq_status_t launch_rs(const ConvGeom& g, const RsShape& sh, const CUtensorMap* maps, const LayerJob* jobs_dev, int n_jobs,
-                       int batch_capacity, int32_t* error_flag, double weight_bytes, int weight_bits, bool pool_jobs,
-                       cudaStream_t s) {
+                       int batch_capacity, int32_t* error_flag, double weight_bytes, int weight_bits, cudaStream_t s) {
   DeviceProps props;
   if (aiq_status_t st = current_device_props(&props)) return st;
-  const RsConfig c = rs_config(g, sh, weight_bits, props.smem_optin, pool_jobs);
+  const RsConfig c = rs_config(g, sh, weight_bits, props.smem_optin, POOL);
   if (!c.ok) return set_error(AIQ_ERR_SHAPE, "conv_rs: shared or tensor memory does not fit (%d bytes per input row)", sh.stage_bytes);
   RsParams p = {};
   p.H = g.H; p.W = g.W; p.Ho = g.Ho; p.Wo = g.Wo; p.N = c.N; p.cout_total = g.Cout; p.act = g.act;
@@ -1004,7 +1007,7 @@ aiq_status_t launch_rs(const ConvGeom& g, const RsShape& sh, const CUtensorMap* 
   p.error_flag = error_flag;
   p.batch = g.B;
   p.pool_bytes = c.pool_bytes;
-  AIQ_ENSURE_DYNAMIC_SMEM((conv_rs_kernel<C, KS, STRIDE, PIECES>), props.smem_optin);
+  AIQ_ENSURE_DYNAMIC_SMEM((conv_rs_kernel<C, KS, STRIDE, PIECES, POOL>), props.smem_optin);
   int ctas = c.occ * props.n_sms / (n_jobs * c.slices);
   if (ctas > p.n_items) ctas = p.n_items;
   if (ctas < 1) ctas = 1;
@@ -1012,8 +1015,8 @@ aiq_status_t launch_rs(const ConvGeom& g, const RsShape& sh, const CUtensorMap* 
     LaunchScope scope(AIQ_KERNEL_CONV_TC, s,
                       2.0 * g.B * g.Ho * g.Wo * g.Cout * (double)(g.ks * g.ks * g.Cin) * n_jobs,
                       weight_bytes + 4.0 * n_jobs * ((double)g.B * g.Cin * g.H * g.W +
-                                                     (pool_jobs ? 0.0 : (double)g.B * g.Ho * g.Wo * g.Cout)));
-    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_rs_kernel<C, KS, STRIDE, PIECES>, dim3(ctas, n_jobs, c.slices), dim3(c.threads), c.smem_bytes, s,
+                                                     (POOL ? 0.0 : (double)g.B * g.Ho * g.Wo * g.Cout)));
+    AIQ_CUDA_TRY(launch_chained(scope.chain, conv_rs_kernel<C, KS, STRIDE, PIECES, POOL>, dim3(ctas, n_jobs, c.slices), dim3(c.threads), c.smem_bytes, s,
                                 maps[0], maps[1], p, jobs_dev));
   }
   AIQ_LAUNCH_CHECK("conv_rs");
@@ -1141,11 +1144,12 @@ aiq_status_t launch_conv_rs(const ConvGeom& g, const void* maps, const LayerJob*
   RsShape sh;
   if (!rs_shape(g, &sh)) return set_error(AIQ_ERR_SHAPE, "conv_rs: layer shape is not supported");
   const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
-#define AIQ_RS_ARGS g, sh, m, jobs_dev, n_jobs, batch_capacity, error_flag, weight_bytes, weight_bits, pool_jobs, s
+#define AIQ_RS_ARGS g, sh, m, jobs_dev, n_jobs, batch_capacity, error_flag, weight_bytes, weight_bits, s
+#define AIQ_RS_POOL(C_, K_, S_, P_) (pool_jobs ? launch_rs<C_, K_, S_, P_, true>(AIQ_RS_ARGS) : launch_rs<C_, K_, S_, P_, false>(AIQ_RS_ARGS))
 #define AIQ_RS_KS(C_, P_)                                                                              \
   do {                                                                                                \
-    if (g.ks == 3) return g.stride == 1 ? launch_rs<C_, 3, 1, P_>(AIQ_RS_ARGS) : launch_rs<C_, 3, 2, P_>(AIQ_RS_ARGS); \
-    return g.stride == 1 ? launch_rs<C_, 1, 1, P_>(AIQ_RS_ARGS) : launch_rs<C_, 1, 2, P_>(AIQ_RS_ARGS); \
+    if (g.ks == 3) return g.stride == 1 ? AIQ_RS_POOL(C_, 3, 1, P_) : AIQ_RS_POOL(C_, 3, 2, P_);       \
+    return g.stride == 1 ? AIQ_RS_POOL(C_, 1, 1, P_) : AIQ_RS_POOL(C_, 1, 2, P_);                     \
   } while (0)
 #define AIQ_RS_C(C_)                                  \
   if (g.Cin == C_) {                                  \
@@ -1155,6 +1159,7 @@ aiq_status_t launch_conv_rs(const ConvGeom& g, const void* maps, const LayerJob*
   AIQ_RS_C(16) AIQ_RS_C(32) AIQ_RS_C(64)
 #undef AIQ_RS_C
 #undef AIQ_RS_KS
+#undef AIQ_RS_POOL
 #undef AIQ_RS_ARGS
   return set_error(AIQ_ERR_SHAPE, "conv_rs: no kernel for Cin=%d", g.Cin);
 }

@@ -165,8 +165,8 @@ __device__ __forceinline__ float apply_act(float v, int act) {
 //             hi = bf16_rn(v), lo = bf16_rn(v - hi): 16+ significant bits in the same bytes,
 //             in the form the bf16 tensor cores consume without conversion (the two halves
 //             are two K-slices of the GEMM).  Used when the model has tensor-core layers; a tensor that only
-//             depthwise layers read stays in floats all the same (ConvGeom::out_f32): no MMA needs its halves,
-//             and neither its writer nor its readers then split or join (MobileNetV2's expansions).
+//             depthwise layers read holds the same values as floats (ConvGeom::out_f32): no MMA needs its halves,
+//             and its readers then do not join them (MobileNetV2's expansions).
 //   ACT_RS    the hi / lo bfloat16 pairs of ACT_SPLIT in the image-interleaved layout of the
 //             row-streaming tensor-core convolution (conv_rs.cu):
 //             [group][row][column][plane][image][8 bfloat16], G = rs_group_images(width) images per

@@ -115,8 +115,7 @@ __device__ __forceinline__ void pr_expand(const PrRaw<PIECES>& raw, int bits, in
   }
 }
 
-// F32: the output stays in floats (ConvGeom::out_f32).  Such a layer widens the channels and is bound by its epilogue: 32 ->
-// 192 channels, 256 x 32 x 32 pixels 53.4 us with the split, 49 without (4.1 TB/s).
+// F32: the output is stored as floats (ConvGeom::out_f32) with the values that the hi / lo pairs would have had.
 template <int EW, int PIECES, bool STREAM, bool F32>
 __global__ void __launch_bounds__((2 + EW + (STREAM ? kPrExpWarps : 0)) * 32, EW == 12 && !STREAM ? 2 : 1)
 conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap out_map, PrParams p,
@@ -390,9 +389,9 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int cc = c0 + 16 * half + 4 * j;
-              float4 o = finish4<decltype(act)::value>(v + 4 * j, s_scale + cc, s_bias + cc);
-              if (!all_interior && !interior) o = make_float4(0.f, 0.f, 0.f, 0.f);
-              *reinterpret_cast<float4*>(dst + (((uint32_t)(4 * half + j) ^ key) << 4)) = o;
+              ulonglong2 o = finish4<decltype(act)::value>(v + 4 * j, s_scale + cc, s_bias + cc);
+              if (!all_interior && !interior) o = make_ulonglong2(0ull, 0ull);
+              *reinterpret_cast<ulonglong2*>(dst + (((uint32_t)(4 * half + j) ^ key) << 4)) = o;
             }
             return;
           }

@@ -316,13 +316,19 @@ __device__ __forceinline__ void finish8(const uint32_t* v, const float* scale, c
     }
   }
 }
-// Four finished accumulators that stay floats: scale, bias, activation.
+// Four finished accumulators as floats, rounded as a stored hi / lo pair rounds them: the value of the pair itself.
 template <int ACT>
-__device__ __forceinline__ float4 finish4(const uint32_t* v, const float* scale, const float* bias) {
+__device__ __forceinline__ ulonglong2 finish4(const uint32_t* v, const float* scale, const float* bias) {
   const ulonglong2 sc = *reinterpret_cast<const ulonglong2*>(scale), bi = *reinterpret_cast<const ulonglong2*>(bias);
-  const float2 a = unpack2(fma2(pack2(__uint_as_float(v[0]), __uint_as_float(v[1])), sc.x, bi.x));
-  const float2 b = unpack2(fma2(pack2(__uint_as_float(v[2]), __uint_as_float(v[3])), sc.y, bi.y));
-  return make_float4(act_of<ACT>(a.x), act_of<ACT>(a.y), act_of<ACT>(b.x), act_of<ACT>(b.y));
+  ulonglong2 o;
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const float2 f = unpack2(fma2(pack2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1])), i ? sc.y : sc.x, i ? bi.y : bi.x));
+    uint32_t h, l;
+    split_pair(act_of<ACT>(f.x), act_of<ACT>(f.y), h, l);
+    (i ? o.y : o.x) = add2(widen2(h), widen2(l));
+  }
+  return o;
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 

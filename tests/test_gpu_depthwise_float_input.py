@@ -1,4 +1,4 @@
-"""The tensor between an expansion and its depthwise layer, kept in floats: hidden channel counts whose last store unit of 32
+"""The tensor between an expansion and its depthwise layer, stored as floats: hidden channel counts whose last store unit of 32
 channels is half empty or partly padding, pixel tiles that end inside an image, one column, both strides, every weight class
 of the expansion.  Tolerance: the float32 rule of the other forward tests, 1e-3 (1 + |ref|)."""
 import numpy as np

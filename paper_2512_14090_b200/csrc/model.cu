@@ -134,7 +134,7 @@ struct LayerInfo {
   uint8_t* mb_tile[2];
   float* mb_coef[4];
   int mb_nh;
-  int out_f32;             // ConvGeom::out_f32
+  int out_f32;             // the layer's own kernel may store floats (ConvGeom::out_f32, LayerPlan::out_f32)
 };
 
 struct aiq_model {
@@ -244,9 +244,7 @@ static ConvGeom make_geom(const aiq_model* m, const LayerInfo& li, int B) {
   g.Cs_in = padded_channels(li.d.cin); g.Cs_out = padded_channels(li.d.cout);
   g.in_is_nchw = li.d.input < 0 ? 1 : 0;          // the network input is float32 NCHW
   g.act_format = m->act_format;
-  g.out_f32 = li.out_f32;
-  g.in_f32 = li.d.input >= 0 ? m->layers[li.d.input].out_f32 : 0;
-  return g;
+  return g;                                       // in_f32 / out_f32: see plan_geom
 }
 
 // 0: float32 kernels only; 1: small-channel 3x3 / 1x1 tensor-core kernel; 2: pointwise tensor-core
@@ -761,6 +759,7 @@ struct LayerPlan {
   bool skipped = false;                 // first convolution of a fused block: evaluated inside its partner's kernel
   int fused_head = -1;                  // last layer of a fused block: the first layer it absorbs
   int fused_mid = -1;                   // inverted-residual block: the depthwise layer between the two (else -1)
+  bool out_f32 = false;                 // its tensor holds floats (a fused block's kernel always stores pairs)
   double weight_bytes = 0.0;            // packed weights + scales + biases over all jobs
   double weight_bytes_tc = 0.0, weight_bytes_tc16 = 0.0, weight_bytes_tc32 = 0.0;
   TensorMapBytes maps[2];               // [0] over the input slot (tensor-core layers); [1] over the output slot
@@ -781,6 +780,15 @@ struct EvalPlan {
   int n_final = 0;
   int64_t versions_total = 0;
 };
+
+// Geometry of a layer as this plan runs it: pixel formats included, which follow from the kernel that writes each tensor.
+static ConvGeom plan_geom(const aiq_model* m, const EvalPlan& plan, int l, int B) {
+  const LayerInfo& li = m->layers[l];
+  ConvGeom g = make_geom(m, li, B);
+  g.out_f32 = plan.lp[l].out_f32;
+  g.in_f32 = li.d.input >= 0 && plan.lp[li.d.input].out_f32;
+  return g;
+}
 
 // Builds the job records for `S` schemes over a chunk of B images.  With sharing on, a
 // (layer, version) is keyed by (bit-width, version of its input, version of its residual):
@@ -849,6 +857,7 @@ static aiq_status_t build_plan(const aiq_model* m, const uint8_t* schemes, int S
       }
     }
     lp.n_versions = (int)keys.size();
+    lp.out_f32 = li.out_f32 && mb_head[l] < 0;
     plan.versions_total += lp.n_versions;
     all_keys[l] = keys;
     if (li.d.kind != AIQ_LAYER_FC && m->block_tail[l] >= 0 && fuse_head[m->block_tail[l]] == l) {
@@ -955,14 +964,14 @@ static aiq_status_t build_plan(const aiq_model* m, const uint8_t* schemes, int S
         aiq_status_t st = lp.tc_kind == 3
             ? conv_rs_encode_maps(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0])
             : lp.tc_kind == 2
-            ? conv_pw_encode_maps(make_geom(m, li, B), ws + wl.slot_off[src.slot], plan.lp[li.d.input].n_versions,
+            ? conv_pw_encode_maps(plan_geom(m, plan, l, B), ws + wl.slot_off[src.slot], plan.lp[li.d.input].n_versions,
                                   ws + wl.slot_off[li.slot], lp.n_versions, B, &lp.maps[0])
             : conv_tc_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B, plan.lp[li.d.input].n_versions, &lp.maps[0]);
         if (st != AIQ_OK) return st;
       }
       if (li.d.kind == AIQ_LAYER_DEPTHWISE) {
         const LayerInfo& src = m->layers[li.d.input];
-        aiq_status_t st = depthwise_encode_map(make_geom(m, li, B), ws + wl.slot_off[src.slot], B,
+        aiq_status_t st = depthwise_encode_map(plan_geom(m, plan, l, B), ws + wl.slot_off[src.slot], B,
                                                plan.lp[li.d.input].n_versions, &lp.maps[0]);
         if (st != AIQ_OK) return st;
       }
@@ -1077,7 +1086,7 @@ static aiq_status_t run_chunk(const aiq_model* m, const EvalPlan& plan, const La
       continue;
     }
     if (lp.skipped) continue;
-    const ConvGeom g = make_geom(m, li, B);
+    const ConvGeom g = plan_geom(m, plan, l, B);
     if (lp.fused_head >= 0 && lp.fused_mid >= 0) {
       st = launch_mb_block(make_geom(m, m->layers[lp.fused_head], B), make_geom(m, m->layers[lp.fused_mid], B), g, li.mb_nh,
                            jobs_dev + lp.job_first, lp.n_tc, m->status_word, lp.weight_bytes_tc, stream);

@@ -133,3 +133,46 @@ def test_default_policy_does_not_depend_on_the_batch():
     sample = np.arange(3, 149, 16)
     assert_logits_close(got[sample], O.forward_scheme(arch, bank, scheme, x[sample]), "default policy")
     model.close()
+
+
+def _separable_net(hw, shapes):
+    """Stem, then 1x1 and depthwise layers in turn without shortcuts; shapes: (kind, channels, stride)."""
+    layers = [dict(name="stem", kind="conv", cin=3, cout=24, k=3, stride=1, pad=1, act="relu6", input=-1, residual=-1, has_bn=True)]
+    for kind, cout, stride in shapes:
+        k = 3 if kind == "dw" else 1
+        layers.append(dict(name=f"l{len(layers)}", kind=kind, cin=layers[-1]["cout"], cout=cout, k=k, stride=stride, pad=k // 2,
+                           act="relu6", input=len(layers) - 1, residual=-1, has_bn=True))
+    layers.append(dict(name="fc", kind="fc", cin=layers[-1]["cout"], cout=6, k=1, stride=1, pad=0, act="none",
+                       input=len(layers) - 1, residual=-1, has_bn=False))
+    return dict(name="separable", in_c=3, in_h=hw, in_w=hw, n_classes=6, layers=layers)
+
+
+def _check_separable_net(arch, hw, batch, fused_blocks):
+    aiq = binding()
+    params = gen_model(arch, 8500 + hw)
+    model = aiq.Model(arch, params)
+    bank = O.build_weight_bank(O.fold_model(arch, params), (4, 8, 16))
+    x = gen_images(batch, 3, hw, hw, 8501)
+    L = len(arch["layers"])
+    for low, bits in ((0, 8), (1, 4), (2, 16), (3, 4)):
+        scheme = np.full(L, 8, np.uint8)
+        scheme[low] = bits
+        ref = O.forward_scheme(arch, bank, scheme, x)
+        launches = []
+        for on in (True, False):
+            aiq.aiq_set_fusion(True, True, inverted_residual=on)
+            try:
+                got = model.aiq_forward(scheme, to_dev(x)).cpu().numpy()
+                launches.append(aiq.aiq_last_call_stats()["kernel_launches"])
+            finally:
+                aiq.aiq_set_fusion(True, True)
+            assert_logits_close(got, ref, f"{[l['name'] for l in arch['layers']]} fused {on} scheme {scheme.tolist()}")
+        assert launches[0] == launches[1] - 2 * fused_blocks
+    model.close()
+
+
+@pytest.mark.parametrize("hw,batch,stride", [(9, 3, 2), (16, 2, 1)])
+def test_fused_block_before_a_depthwise_layer(hw, batch, stride):
+    """The projection's tensor is read by a depthwise layer alone: floats where the projection runs as a layer, hi / lo pairs
+    where the fused kernel writes it, and the depthwise layer has to read what was written."""
+    _check_separable_net(_separable_net(hw, [("conv", 96, 1), ("dw", 96, 1), ("conv", 48, 1), ("dw", 48, stride)]), hw, batch, 1)

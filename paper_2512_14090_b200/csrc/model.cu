@@ -353,6 +353,7 @@ static ModelLayout model_layout(const std::vector<LayerInfo>& L) {
   for (int b = 0; b < 4; ++b) lay.mb_coef[b].assign(L.size(), 0);
   std::vector<int> mid, tail;
   find_mb_structure(L, mid, tail);
+  std::vector<size_t> tile_bytes(L.size(), 0);      // a layer may end one block and begin another: room for either image
   for (size_t le = 0; le < L.size(); ++le) {
     if (tail[le] < 0) continue;
     const int ld = mid[le], lp = tail[le];
@@ -365,13 +366,13 @@ static ModelLayout model_layout(const std::vector<LayerInfo>& L) {
       ec = std::max(ec, chunks * 2 * nh * 4);
       dc = std::max(dc, chunks * 11 * nh * 4);
     }
-    for (int b = 0; b < 2; ++b) {
-      lay.mb_tile[b][le] = take(et);
-      lay.mb_coef[b][le] = take(ec);
-      lay.mb_tile[b][lp] = take(pt);
-    }
+    tile_bytes[le] = std::max(tile_bytes[le], et);
+    tile_bytes[lp] = std::max(tile_bytes[lp], pt);
+    for (int b = 0; b < 2; ++b) lay.mb_coef[b][le] = take(ec);
     for (int b = 0; b < 4; ++b) lay.mb_coef[b][ld] = take(dc);
   }
+  for (size_t l = 0; l < L.size(); ++l)
+    for (int b = 0; b < 2 && tile_bytes[l]; ++b) lay.mb_tile[b][l] = take(tile_bytes[l]);
   lay.total = off;
   return lay;
 }
@@ -445,6 +446,7 @@ static void derive_format(aiq_model* m, int opt_path) {
       LayerInfo& d = m->layers[mid[le]];
       LayerInfo& pr = m->layers[tail[le]];
       if (!layer_on_tensor_cores(m, e) || !layer_on_tensor_cores(m, pr)) continue;
+      if (e.mb_nh || pr.mb_nh) continue;            // a layer belongs to one block: the first of a chain that the kernel takes
       const int nh = mb_block_chunk_channels(make_geom(m, e, 1), make_geom(m, d, 1), make_geom(m, pr, 1));
       if (!nh) continue;
       m->mb_mid[le] = mid[le];

@@ -176,3 +176,11 @@ def test_fused_block_before_a_depthwise_layer(hw, batch, stride):
     """The projection's tensor is read by a depthwise layer alone: floats where the projection runs as a layer, hi / lo pairs
     where the fused kernel writes it, and the depthwise layer has to read what was written."""
     _check_separable_net(_separable_net(hw, [("conv", 96, 1), ("dw", 96, 1), ("conv", 48, 1), ("dw", 48, stride)]), hw, batch, 1)
+
+
+@pytest.mark.parametrize("hw,batch", [(9, 3), (16, 2)])
+def test_blocks_that_share_a_layer(hw, batch):
+    """1x1 and depthwise layers in turn: each 1x1 layer between two depthwise ones could end a block and begin the next.  Of
+    the three candidates the first and the third are fused."""
+    _check_separable_net(_separable_net(hw, [("conv", 96, 1), ("dw", 96, 1), ("conv", 48, 1), ("dw", 48, 2), ("conv", 64, 1),
+                                             ("dw", 64, 1), ("conv", 32, 1)]), hw, batch, 2)

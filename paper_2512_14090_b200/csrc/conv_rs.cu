@@ -464,7 +464,8 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     const int row_step = units >= WQ ? 1 : WQ / units;
     const int rows_mine = p.Ho / row_step;             // rows of an item this warp drains
     const int n_my_items = ((int)blockIdx.x < p.n_items) ? (p.n_items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int total = n_my_items * rows_mine;
+    // three units and four warps (24- or 48-column maps, 16 channels, one block per SM): the fourth has no row
+    const int total = row_first < row_step ? n_my_items * rows_mine : 0;
     auto row_offset = [&](int k) -> size_t {           // byte offset of this lane's image in the k-th row of this warp
       const int il = k / rows_mine;
       const int y = row_first + (k - il * rows_mine) * row_step;
@@ -1087,7 +1088,8 @@ bool conv_rs_pool_fusable(const ConvGeom& g) {
   if (current_device_props(&props) != AIQ_OK) return false;
   for (int bits : {8, 16, 32}) {
     const RsConfig c = rs_config(g, s, bits, props.smem_optin, true);
-    if (!c.ok || s.xt * (c.N / 16) > (c.threads / 32 - 2) / 4) return false;
+    const int units = s.xt * (c.N / 16), warps = (c.threads / 32 - 2) / 4;
+    if (!c.ok || units > warps || warps % units != 0) return false;   // every warp of a quarter arrives once per item
   }
   return true;
 }

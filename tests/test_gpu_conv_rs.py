@@ -159,3 +159,26 @@ def test_average_pool_in_the_epilogue_matches_the_pooling_kernel():
             assert_logits_close(plain, ref, f"{arch['name']} pooling kernel batch {batch}")
             assert np.abs(fused - plain).max() <= 1e-5 * (1.0 + np.abs(plain).max())
         model.close()
+
+
+@pytest.mark.parametrize("cin,k,hw", [(32, 3, 24), (32, 1, 48), (64, 1, 24)])
+def test_three_column_tiles_of_sixteen_channels(cin, k, hw):
+    """Three (column tile, channel chunk) units per row beside four epilogue warps a quarter: three of them share the row, the
+    fourth must keep out (it would walk one row past the map).  Several image groups per block, and a ragged last one."""
+    aiq = binding()
+    arch = _net(cin, 16, k, 1, hw, False)
+    params = gen_model(arch, 8600 + cin + k)
+    with compute_path("tensor"):
+        model = aiq.Model(arch, params)
+    bank = O.build_weight_bank(O.fold_model(arch, params), (4, 8, 16, 32))
+    group = 8 if hw % 16 == 0 else 16
+    x = to_dev(np.tile(gen_images(37, 3, hw, hw, 8601), (9 * group, 1, 1, 1)))      # over two groups for each of 148 blocks
+    for bits in (8, 32):
+        scheme = np.array([8, bits, 8], np.uint8)
+        ref = O.forward_scheme(arch, bank, scheme, x[:37].cpu().numpy())
+        few = model.aiq_forward(scheme, x[:37]).cpu().numpy()
+        assert_logits_close(few, ref, f"{arch['name']} bits {bits}")
+        many = model.aiq_forward(scheme, x).cpu().numpy()
+        model.aiq_model_status()
+        assert np.array_equal(many, np.tile(few, (9 * group, 1)))
+    model.close()

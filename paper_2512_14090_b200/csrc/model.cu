@@ -268,6 +268,13 @@ static void assign_slots(aiq_model* m) {
     if (d.input >= 0) last_use[d.input] = std::max(last_use[d.input], pos[l]);
     if (d.residual >= 0) last_use[d.residual] = std::max(last_use[d.residual], pos[l]);
   }
+  // A fused inverted-residual block reads its input when its last layer's turn comes: with other layers in between the slot
+  // stays taken until then (without, neither of the two layers that could get it is written, nor is it the result's).
+  for (int l = 0; l < n; ++l)
+    if (m->mb_tail[l] >= 0 && pos[m->mb_tail[l]] > pos[l] + 2) {
+      const int x = m->layers[l].d.input;
+      last_use[x] = std::max(last_use[x], pos[m->mb_tail[l]]);
+    }
   std::vector<int> owner;   // layer currently held by each slot, -1 = free
   m->slot_bytes.clear();
   for (int i = 0; i < n; ++i) {

@@ -184,3 +184,19 @@ def test_blocks_that_share_a_layer(hw, batch):
     the three candidates the first and the third are fused."""
     _check_separable_net(_separable_net(hw, [("conv", 96, 1), ("dw", 96, 1), ("conv", 48, 1), ("dw", 48, 2), ("conv", 64, 1),
                                              ("dw", 64, 1), ("conv", 32, 1)]), hw, batch, 2)
+
+
+@pytest.mark.parametrize("between,hw,batch", [("second stem", 12, 5), ("second reader", 48, 24)])
+def test_block_with_other_layers_between_its_own(between, hw, batch):
+    """Layers listed between the three of a block run before the fused kernel, which reads the block's input only then: they
+    must not have been given its memory, and neither must the block's result."""
+    def conv(cin, cout, k, inp, kind="conv", residual=-1):
+        return dict(name=f"{kind}{cout}", kind=kind, cin=cin, cout=cout, k=k, stride=1, pad=k // 2, act="relu6", input=inp,
+                    residual=residual, has_bn=True)
+    layers = [conv(3, 24, 3, -1), conv(24, 96, 1, 0)]
+    if between == "second stem":
+        layers += [conv(3, 24, 3, -1), conv(96, 96, 3, 1, "dw"), conv(96, 32, 1, 3), conv(24, 32, 1, 2, residual=4)]
+    else:
+        layers += [conv(96, 96, 3, 1, "dw"), conv(24, 32, 1, 0), conv(96, 32, 1, 2), conv(32, 32, 1, 3, residual=4)]
+    layers.append(dict(name="fc", kind="fc", cin=32, cout=6, k=1, stride=1, pad=0, act="none", input=5, residual=-1, has_bn=False))
+    _check_separable_net(dict(name="branches", in_c=3, in_h=hw, in_w=hw, n_classes=6, layers=layers), hw, batch, 1)

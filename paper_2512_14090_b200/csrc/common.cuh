@@ -222,7 +222,9 @@ struct ConvGeom {
   int Cs_in, Cs_out;  // padded channel counts of the split tensors
   int in_is_nchw;     // 1: the input is the float32 NCHW network input
   int act_format;     // ACT_F32 or ACT_SPLIT, for input, residual and output alike
-  int in_f32, out_f32;   // ACT_SPLIT models: the input / output tensor holds Cs floats per pixel (its readers are depthwise layers)
+  // ACT_SPLIT models: the input / output tensor holds Cs floats per pixel.  The writer is a pointwise layer without a residual
+  // (conv_pw.cu), every reader a depthwise layer that takes it as its input (a residual operand is always pairs).
+  int in_f32, out_f32;
 };
 
 // ---- launchers (defined in the .cu files) --------------------------------------------

@@ -370,7 +370,7 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
         uint32_t v[16];
         tmem_ld16(taddr + 16 * half, v);
         uint4 rh[2], rl[2];
-        if (job.res) {
+        if (!F32 && job.res) {                                 // (a layer with a residual never stores floats)
           const __nv_bfloat16* res = static_cast<const __nv_bfloat16*>(job.res) + (size_t)pix * (2 * p.Cs_out) + n0 + c0 + 16 * half;
 #pragma unroll
           for (int j = 0; j < 2; ++j)
@@ -417,7 +417,7 @@ conv_pw_kernel(const __grid_constant__ CUtensorMap in_map, const __grid_constant
           else if (p.act == AIQ_ACT_RELU) finish(std::integral_constant<int, AIQ_ACT_RELU>(), res);
           else finish(std::integral_constant<int, AIQ_ACT_NONE>(), res);
         };
-        if (job.res) finish_act(std::true_type()); else finish_act(std::false_type());
+        if (F32 || !job.res) finish_act(std::false_type()); else finish_act(std::true_type());
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();

@@ -182,3 +182,37 @@ def test_three_column_tiles_of_sixteen_channels(cin, k, hw):
         model.aiq_model_status()
         assert np.array_equal(many, np.tile(few, (9 * group, 1)))
     model.close()
+
+
+@pytest.mark.parametrize("net,bits", [("resnet20", 8), ("resnet20", 32), ("heavy_early_resnet20", 4)])
+def test_pooled_epilogue_over_several_groups_per_block(net, bits):
+    """Every block walks three image groups or more and the last one is ragged: sums that were carried into the next group, or a
+    partial sum overwritten before it was read, would show.  The pooled logits against the pooling kernel, whose sums run in
+    another order, and bit for bit against the same images in small passes."""
+    import torch
+    from aiq_workloads import resnet20, heavy_early_resnet20
+    aiq = binding()
+    arch = dict(resnet20=resnet20, heavy_early_resnet20=heavy_early_resnet20)[net]()
+    params = gen_model(arch, 4600)
+    model = aiq.Model(arch, params)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    batch = 2 * 16 * 3 * sms + 5                                 # at most two blocks per SM, groups of 16 images
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4601)
+    x = torch.randn((batch, 3, 32, 32), generator=g, device="cuda")
+    scheme = np.full(len(arch["layers"]), bits, np.uint8)
+    pooled = model.aiq_forward(scheme, x).cpu().numpy()
+    n_pooled = aiq.aiq_last_call_stats()["kernel_launches"]
+    aiq.aiq_set_fusion(True, False)
+    try:
+        plain = model.aiq_forward(scheme, x).cpu().numpy()
+        n_plain = aiq.aiq_last_call_stats()["kernel_launches"]
+    finally:
+        aiq.aiq_set_fusion(True, True)
+    model.aiq_model_status()
+    assert n_pooled == n_plain - 1
+    assert np.abs(pooled - plain).max() <= 1e-5 * (1.0 + np.abs(plain).max())
+    for first in (0, 16 * sms - 3, batch - 37):
+        part = model.aiq_forward(scheme, x[first:first + 37].contiguous()).cpu().numpy()
+        assert np.array_equal(part.view(np.uint32), pooled[first:first + 37].view(np.uint32)), first
+    model.close()

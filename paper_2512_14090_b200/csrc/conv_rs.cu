@@ -266,7 +266,10 @@ __device__ __forceinline__ void rs_finish_unit(const uint32_t* v, const float* s
                       RES ? res[2 + e] : make_uint4(0u, 0u, 0u, 0u), hi + 4 * e, lo + 4 * e);
 }
 
-// POOL: the jobs pool (LayerJob::pool).  An instantiation of its own: the sums take 16 registers the others do not have.
+// POOL: the jobs pool (LayerJob::pool).  An instantiation of its own: the sums take 16 registers the others do not have, and
+// spill (24 to 32 bytes; two-piece 64-channel 3x3 kernels 228, 224 without the pool).  Each row still costs less than the
+// shuffles it replaced: 8,192 images, us a launch before / now, 8- and 32-bit weights: 16 -> 16 channels 3x3 at 32 x 32 292 / 208 and
+// 314 / 287, 64 -> 64 at 8 x 8 124 / 104 and 308 / 298, 1x1 32 -> 16 at 8 x 8 33 / 29 and 35 / 31.
 template <int C, int KS, int STRIDE, int PIECES, bool POOL>
 __global__ void __launch_bounds__(kRsMaxThreads, 1)
 conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1, RsParams p,
@@ -545,7 +548,7 @@ conv_rs_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         const uint32_t pool_parity = (uint32_t)(il & 1);
         // the columns this warp holds (lanes that differ in the column bits) -> [image][16 channels] in shared memory.
         // (Once per item: 32 shuffles and 16 updates of shared memory for every row made this the longest launch of the
-        // greedy step, 1,401 us against 845 for the same layer with its tensor stored; the step 32.9 ms, now 32.2.)
+        // greedy step, 1,401 us against 845 for the same layer with its tensor stored; the step 32.6 ms, now 31.8.)
         float* mine = s_pool + ((size_t)(warp - 2) * Gout + img) * 16;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {

@@ -103,11 +103,16 @@ __device__ __forceinline__ DwUnit dw_unit(const DwParams& p, int r, int r_end) {
   return d;
 }
 
-// COLS output columns per thread: 4 at stride 1 (small launches: 2, see dw_search_shape), 2 at stride 2.  What bounds the kernel is instructions: with two
-// columns a row cost 37 per output element at 0.46 issued per clock and scheduler (2.9 TB/s at 256 x 32 x 32 x 144
-// channels); four columns share six unpacked input columns (1.5 per output instead of 2), the per-row waiting and
-// the addresses.  IFMT / FMT: pixel formats of the input and of the output; floats in, pairs out behind an expansion
-// (ConvGeom::in_f32), where 256 x 32 x 32 x 96 channels take 42 us (pairs in: 46) and 192 channels 78 (81; DRAM at 5.1 TB/s).
+// COLS output columns per thread: 4 at stride 1 (small launches: 2, see dw_search_shape), 2 at stride 2.  Four columns share
+// six input columns, two share four, two at stride 2 share five: an input value is read 1.5, 2 or 1.25 times.
+// IFMT / FMT: pixel formats of the input and of the output; floats in, pairs out behind an expansion (ConvGeom::in_f32).
+// What bounds it, at 256 x 32 x 32 x 192 channels (ncu, cold; two blocks of seven warps per SM, which is what the registers allow):
+//   four columns, floats in   79 us, 31.6 M warp instructions, 0.42 per clock and scheduler, DRAM at 5.1 TB/s
+//   four columns, pairs in    82 us, 39.2 M (a value is joined each time it is read), 0.47, 4.9 TB/s
+//   stride 2, floats in       48 us, 11.2 M, 0.26, 5.2 TB/s
+// so at these sizes DRAM first (a plain copy moves 6.5 TB/s), each warp then waiting for its next row; with two columns at
+// stride 1 it had been instructions (37 per output element, 2.9 TB/s).  One image (two columns, seven warps per SM) is neither:
+// 8 us of one row after the other, at 24 blocks as at 128.
 template <int IFMT, int FMT, int STRIDE, int COLS, bool RES>
 __global__ void __launch_bounds__(kDwThreads + 32, 2)
 depthwise3x3_kernel(const __grid_constant__ CUtensorMap in_map, DwParams p, const LayerJob* __restrict__ jobs) {

@@ -462,10 +462,10 @@ static void derive_format(aiq_model* m, int opt_path) {
     }
   }
   // Tensors that only depthwise layers read, and whose writer (a pointwise layer) can leave them in floats: the same bytes and
-  // the same values, but the readers, who meet every value one and a half times, have nothing to join.  Before / after, us:
-  // MobileNetV2-CIFAR 1 image 284.9 / 278.6, 256 images 2,123 / 2,098; ImageNet shapes, 32 images 622.6 / 607.8; 52 candidates
-  // x 512 images 113.7 / 111.6 ms.  (Unrounded floats were 2 % faster still, but a prediction then moves wherever an image's two
-  // largest logits are closer than the rounding.)
+  // the same values, but the readers, who meet every value 1.25 to 2 times, have nothing to join.  Pairs / floats, us:
+  // MobileNetV2-CIFAR 1 image 280.6 / 271.3, 256 images 2,103 / 2,096 (DRAM bounds it either way); ImageNet shapes, 32 images
+  // 622.4 / 605.7; 52 candidates x 512 images 112.3 / 110.8 ms.  (Unrounded floats were 2 % faster still, but a prediction then
+  // moves wherever an image's two largest logits are closer than the rounding.)
   for (LayerInfo& li : m->layers) li.out_f32 = 0;
   if (m->act_format == ACT_SPLIT) {
     std::vector<int> uses(m->layers.size(), 0), dw_uses(m->layers.size(), 0);

@@ -268,13 +268,6 @@ static void assign_slots(aiq_model* m) {
     if (d.input >= 0) last_use[d.input] = std::max(last_use[d.input], pos[l]);
     if (d.residual >= 0) last_use[d.residual] = std::max(last_use[d.residual], pos[l]);
   }
-  // A fused inverted-residual block reads its input when its last layer's turn comes: with other layers in between the slot
-  // stays taken until then (without, neither of the two layers that could get it is written, nor is it the result's).
-  for (int l = 0; l < n; ++l)
-    if (m->mb_tail[l] >= 0 && pos[m->mb_tail[l]] > pos[l] + 2) {
-      const int x = m->layers[l].d.input;
-      last_use[x] = std::max(last_use[x], pos[m->mb_tail[l]]);
-    }
   std::vector<int> owner;   // layer currently held by each slot, -1 = free
   m->slot_bytes.clear();
   for (int i = 0; i < n; ++i) {
@@ -482,6 +475,18 @@ static void derive_format(aiq_model* m, int opt_path) {
     }
   }
   assign_slots(m);
+  // A fused inverted-residual block reads its input when its last layer's turn comes, the slots count it as read at the first
+  // layer's.  Where a layer in between, or the block's result, got that slot, the block runs layer by layer.
+  std::vector<int> pos(m->layers.size());
+  for (size_t i = 0; i < m->order.size(); ++i) pos[m->order[i]] = (int)i;
+  for (size_t le = 0; le < m->layers.size(); ++le)
+    if (m->mb_tail[le] >= 0)
+      for (int i = pos[le] + 1, end = pos[m->mb_tail[le]]; i <= end; ++i) {
+        const int l = m->order[i];                  // (the depthwise layer's own tensor is not written then)
+        if (l == m->mb_mid[le] || m->layers[l].slot != m->layers[m->layers[le].d.input].slot) continue;
+        m->mb_mid[le] = m->mb_tail[le] = -1;
+        break;
+      }
 }
 
 }  // namespace aiq

@@ -186,17 +186,19 @@ def test_blocks_that_share_a_layer(hw, batch):
                                              ("dw", 64, 1), ("conv", 32, 1)]), hw, batch, 2)
 
 
-@pytest.mark.parametrize("between,hw,batch", [("second stem", 12, 5), ("second reader", 48, 24)])
-def test_block_with_other_layers_between_its_own(between, hw, batch):
-    """Layers listed between the three of a block run before the fused kernel, which reads the block's input only then: they
-    must not have been given its memory, and neither must the block's result."""
+@pytest.mark.parametrize("between,hw,batch,fused", [("second stem", 12, 5, 0), ("second reader", 48, 24, 0), ("late stem", 12, 5, 1)])
+def test_block_with_other_layers_between_its_own(between, hw, batch, fused):
+    """Layers listed between the three of a block run before the fused kernel, which reads the block's input only then.  Where
+    one of them, or the block's result, was given the input's memory, the block must run layer by layer; else it is fused."""
     def conv(cin, cout, k, inp, kind="conv", residual=-1):
         return dict(name=f"{kind}{cout}", kind=kind, cin=cin, cout=cout, k=k, stride=1, pad=k // 2, act="relu6", input=inp,
                     residual=residual, has_bn=True)
     layers = [conv(3, 24, 3, -1), conv(24, 96, 1, 0)]
     if between == "second stem":
         layers += [conv(3, 24, 3, -1), conv(96, 96, 3, 1, "dw"), conv(96, 32, 1, 3), conv(24, 32, 1, 2, residual=4)]
+    elif between == "late stem":        # after the depthwise layer: gets the expansion's memory, which nothing needs
+        layers += [conv(96, 96, 3, 1, "dw"), conv(3, 24, 3, -1), conv(96, 32, 1, 2), conv(24, 32, 1, 3, residual=4)]
     else:
         layers += [conv(96, 96, 3, 1, "dw"), conv(24, 32, 1, 0), conv(96, 32, 1, 2), conv(32, 32, 1, 3, residual=4)]
     layers.append(dict(name="fc", kind="fc", cin=32, cout=6, k=1, stride=1, pad=0, act="none", input=5, residual=-1, has_bn=False))
-    _check_separable_net(dict(name="branches", in_c=3, in_h=hw, in_w=hw, n_classes=6, layers=layers), hw, batch, 1)
+    _check_separable_net(dict(name="branches", in_c=3, in_h=hw, in_w=hw, n_classes=6, layers=layers), hw, batch, fused)
